@@ -22,12 +22,27 @@
 //              that is still its session's latest and whose session holds
 //              blocks (a passed entry never becomes valid again, so the front
 //              only moves forward).
-// A request's blocks go 32 at a time, one per lane.  The lanes of a chunk
-// settle together up to the first miss that would take the cache past C (or
-// the second copy of a repeated block); lane 0 brings that block in and
-// evicts, and the lanes after it are tested again, since an eviction can drop
-// a later block of the same chunk.  Session epochs sit in shared memory when
-// there are at most 16,384 sessions.
+// The replay of one capacity is a serial chain, so what bounds it is the
+// latency of a step.  One warp (the replayer) settles a window of up to 256
+// accesses of one request per step, eight per lane: owners, then epochs, then
+// one ballot per 32 accesses.  All misses that fit settle together; a miss
+// that takes the cache past C evicts (the queue is searched 32 requests at a
+// time) and the accesses after it are tested again from the owners in
+// registers, since an eviction can drop a later block of the window.  Once
+// the current session is alone and above C, every later block of the window
+// misses, and they settle in closed form.  Eight other warps read ahead: the
+// ids of the next 2,048 accesses into shared memory, and the owner words of
+// those ids into L1, so that the replayer's owner reads hit L1 (its own
+// stores go through the same L1) instead of waiting for DRAM: the owner table
+// takes 8 bytes per block and capacity.  Epochs, counts and latest requests
+// sit in shared memory when there are at most 16,384 sessions.
+//
+// Ids of prefix chains rise strictly within a request (a prefix first occurs
+// no later than its extensions).  A window where they do not may hold a block
+// twice; it is settled 32 accesses at a time, a second copy after the first.
+//
+// Measured on the 9.3M-access chat trace, 64 capacities: 486 ms with one warp per
+// capacity, 32 accesses a step and owners read from DRAM as they came; 116 ms so.
 #include "ptc_internal.h"
 
 namespace ptc {
@@ -70,124 +85,336 @@ __global__ void k_ses_check(const uint64_t* __restrict__ blk_off, uint32_t R, ui
   if (b < a || b > n || (r == 0 && a != 0) || (r + 1 == R && b != n) || ses[r] >= S) raise_err(st, kErrInvalid);
 }
 
-constexpr uint32_t kSesSmemSessions = 16384;  // session epochs kept in shared memory up to this many (64 KB)
+constexpr uint32_t kSesSmemSessions = 16384;  // session state kept in shared memory up to this many (192 KB)
+constexpr uint32_t kSesPer = 8;                // accesses per lane and window
+constexpr uint32_t kSesWin = 32 * kSesPer;
+constexpr uint32_t kSesAhead = 8;              // warps that read ahead, one window each
+constexpr uint32_t kSesBatch = kSesAhead * kSesWin;
+constexpr uint32_t kSesThreads = 32 * (1 + kSesAhead);
 
-__global__ void __launch_bounds__(32) k_ses_sim(SesArgs a, SesCaps caps) {
-  extern __shared__ uint32_t s_epoch[];
-  grid_dep_sync();
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t g = blockIdx.x;
-  if (g >= a.G || a.st->err) return;  // malformed offsets or labels: nothing to replay
-  uint64_t* owner = a.owner + g * a.sD;
-  uint32_t* count = a.count + g * a.sS;
-  uint32_t* last = a.last + g * a.sS;
-  const bool in_smem = a.n_session <= kSesSmemSessions;
-  volatile uint32_t* ep = in_smem ? s_epoch : a.epoch + g * a.sS;  // one warp owns it: plain accesses
-  if (in_smem)
-    for (uint32_t t = lane; t < a.n_session; t += 32) s_epoch[t] = 0;
-  __syncwarp();
-  const uint64_t C = caps.c[g];
-  uint64_t total = 0, hits = 0, sv_lo = 0, sv_hi = 0;
-  uint32_t front = 0;
-  for (uint32_t r = 0; r < a.n_req; ++r) {
-    const uint32_t s = a.ses[r];
-    const uint64_t b = a.blk_off[r], e = a.blk_off[r + 1];
-    if (lane == 0) __stcg(&last[s], r);
-    uint32_t es = ep[s];
-    bool missed = false;
-    uint32_t id_next = b + lane < e ? a.ids[b + lane] : 0u;
-    for (uint64_t c = b; c < e; c += 32) {
-      const bool valid = c + lane < e;
-      uint32_t id = id_next;
-      id_next = c + 32 + lane < e ? a.ids[c + 32 + lane] : 0u;  // in flight while this chunk settles
-      if (valid && id >= a.n_distinct) {
-        raise_err(a.st, kErrInvalid);
-        id = 0;
+// Ids of two batches and, per 32 accesses, whether an id fails to exceed the
+// one before it.
+struct SesRing {
+  uint32_t ids[2][kSesBatch];
+  uint32_t fall[2][kSesBatch / 32];
+};
+
+// One capacity's session state; the pointers go to shared or global memory,
+// and only the replaying warp touches them.
+struct SesState {
+  uint32_t *ep, *count, *last;
+};
+
+// Evict until at most C blocks are resident, after block x came in for
+// session s (whose epoch is es and which holds cnt blocks) in request r.
+// Returns true if session s itself was emptied but for x.
+__device__ __forceinline__ bool ses_evict(const SesArgs& a, const SesState& S, uint64_t* owner, uint32_t lane,
+                                          uint32_t r, uint32_t s, uint32_t x, uint64_t C, uint32_t& front,
+                                          uint64_t& total, uint32_t& cnt, uint32_t& es) {
+  while (total > C) {
+    uint32_t v = kNone;
+    while (front < r) {
+      const uint32_t f = front + lane;
+      uint32_t t = 0;
+      bool ok = f < r;
+      if (ok) {
+        t = a.ses[f];
+        ok = in_bounds(a.st, t, a.n_session) && S.last[t] == f && S.count[t] > 0;
       }
-      uint32_t pending = __ballot_sync(kFull, valid);
-      while (pending) {
-        const bool mine = (pending >> lane) & 1u;
-        bool res = false;
-        if (mine) {
-          const uint64_t o = __ldcg(&owner[id]);
-          res = o != kNoOwner && in_bounds(a.st, o >> 32, a.n_session) && ep[(uint32_t)(o >> 32)] == (uint32_t)o;
+      const uint32_t m = __ballot_sync(kFull, ok);
+      if (m) {
+        const uint32_t b = __ffs(m) - 1;
+        v = __shfl_sync(kFull, t, b);
+        front += b + 1;
+        break;
+      }
+      front = r - front > 32 ? front + 32 : r;
+    }
+    if (v == kNone) {  // the current session alone is above C: it keeps the block just brought in
+      es += 1;
+      cnt = 1;
+      total = 1;
+      __syncwarp();
+      if (lane == 0) {
+        S.ep[s] = es;
+        owner[x] = ((uint64_t)s << 32) | es;
+      }
+      __syncwarp();
+      return true;
+    }
+    // the least recently touched other session goes whole
+    total -= S.count[v];
+    __syncwarp();
+    if (lane == 0) {
+      S.ep[v] = S.ep[v] + 1u;
+      S.count[v] = 0;
+    }
+    __syncwarp();
+  }
+  return false;
+}
+
+// Hits among the first f accesses of a stretch starting at depth d0.
+struct SesSums {
+  uint64_t hits = 0, lo = 0, hi = 0;
+  __device__ __forceinline__ void add(const SesArgs& a, uint64_t d0, uint32_t f) {
+    hits += f;
+    add_mul128(lo, hi, a.alpha, f);
+    add_mul128(lo, hi, a.beta, (uint64_t)f * d0 + (uint64_t)f * (f ? f - 1 : 0) / 2);
+  }
+};
+
+__device__ __forceinline__ bool ses_resident(const SesArgs& a, const SesState& S, uint64_t o) {
+  return o != kNoOwner && in_bounds(a.st, o >> 32, a.n_session) && S.ep[(uint32_t)(o >> 32)] == (uint32_t)o;
+}
+
+__global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps, uint32_t n) {
+  extern __shared__ uint32_t s_dyn[];
+  SesRing& ring = *reinterpret_cast<SesRing*>(s_dyn);
+  grid_dep_sync();
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t g = blockIdx.x;
+  if (g >= a.G) return;
+  // malformed offsets or labels: nothing to replay (one answer for the whole
+  // CTA: another capacity may report a bad id meanwhile)
+  if (__syncthreads_or(threadIdx.x == 0 && ld_relaxed_u32(&a.st->err) != 0)) return;
+  uint64_t* owner = a.owner + g * a.sD;
+  SesState S;
+  if (a.n_session <= kSesSmemSessions) {
+    S.ep = s_dyn + sizeof(SesRing) / 4;
+    S.count = S.ep + a.n_session;
+    S.last = S.count + a.n_session;
+    for (uint32_t t = threadIdx.x; t < a.n_session; t += kSesThreads) {
+      S.ep[t] = 0;
+      S.count[t] = 0;
+      S.last[t] = kNone;
+    }
+  } else {  // cleared by the caller
+    S.ep = a.epoch + g * a.sS;
+    S.count = a.count + g * a.sS;
+    S.last = a.last + g * a.sS;
+  }
+  // Batch `t` of the read-ahead warps: window `warp - 1` of it into the ring.
+  auto read_ahead = [&](uint32_t t) {
+    const uint64_t base = (uint64_t)t * kSesBatch + (warp - 1) * kSesWin;
+    if (base >= n) return;
+    uint32_t id[kSesPer], left[kSesPer];
+#pragma unroll
+    for (uint32_t u = 0; u < kSesPer; ++u) {
+      const uint64_t j = base + 32 * u + lane;
+      id[u] = j < n ? __ldg(&a.ids[j]) : 0u;
+      left[u] = j > 0 && j < n ? __ldg(&a.ids[j - 1]) : 0u;
+    }
+#pragma unroll
+    for (uint32_t u = 0; u < kSesPer; ++u) {
+      const uint32_t k = (warp - 1) * kSesWin + 32 * u + lane;
+      if (id[u] >= a.n_distinct) {
+        raise_err(a.st, kErrInvalid);
+        id[u] = 0;
+      }
+      ring.ids[t & 1][k] = id[u];
+      const uint32_t fall = __ballot_sync(kFull, id[u] <= left[u]);
+      if (lane == 0) ring.fall[t & 1][k >> 5] = fall;
+    }
+    uint64_t o[kSesPer];
+#pragma unroll
+    for (uint32_t u = 0; u < kSesPer; ++u)  // into L1; the values are not used
+      asm volatile("ld.global.ca.u64 %0, [%1];" : "=l"(o[u]) : "l"(owner + id[u]));
+#pragma unroll
+    for (uint32_t u = 0; u < kSesPer; ++u) asm volatile("" ::"l"(o[u]));
+  };
+  const uint64_t C = caps.c[g];
+  uint64_t total = 0;
+  SesSums sums;
+  uint32_t front = 0;
+  // the current request; 32 requests' sessions and ends at a time, one per lane
+  uint32_t r = kNone, s = 0, b = 0, e = 0, es = 0, cnt = 0, q_s = 0, q_e = 0;
+  bool missed = false;
+  const uint32_t batches = (uint32_t)(((uint64_t)n + kSesBatch - 1) / kSesBatch);
+  if (warp) read_ahead(0);
+  __syncthreads();
+  for (uint32_t t = 0; t < batches; ++t) {
+    if (warp) {
+      if (t + 1 < batches) read_ahead(t + 1);
+      __syncthreads();
+      continue;
+    }
+    const uint32_t* ids = ring.ids[t & 1];
+    const uint32_t* fall = ring.fall[t & 1];
+    const uint64_t t0 = (uint64_t)t * kSesBatch;
+    const uint32_t size = n - t0 < kSesBatch ? (uint32_t)(n - t0) : kSesBatch;
+    uint32_t at = 0;  // accesses of this batch settled
+    while (at < size) {
+      while (t0 + at >= e) {  // the next request (one without accesses only touches its session)
+        if (r != kNone && lane == 0) S.count[s] = cnt;
+        ++r;
+        if (r >= a.n_req) break;  // cannot happen: the offsets were checked
+        if ((r & 31) == 0) {
+          q_s = r + lane < a.n_req ? a.ses[r + lane] : 0u;
+          q_e = r + lane < a.n_req ? (uint32_t)a.blk_off[r + lane + 1] : 0u;
         }
-        // a block repeated inside the chunk is settled after its first copy
-        uint32_t same = 0;
-        if (mine) same = __match_any_sync(pending, id);
-        const uint32_t later_copy = __ballot_sync(kFull, mine && (same & ((1u << lane) - 1u)) != 0);
-        const uint32_t miss = __ballot_sync(kFull, mine && !res);
-        // the first miss that would push the cache past C
-        const uint64_t room = C - total;
-        uint32_t over = 32;
-        if ((uint64_t)__popc(miss) > room) {
-          uint32_t m = miss;
-          for (uint64_t k = 0; k < room; ++k) m &= m - 1u;
-          over = (uint32_t)(__ffs(m) - 1);
-        }
-        const uint32_t rep = later_copy ? (uint32_t)(__ffs(later_copy) - 1) : 32u;
-        const uint32_t stop = over < rep ? over : rep;
-        const uint32_t batch = pending & (stop == 32 ? kFull : ((1u << stop) - 1u));
-        // lanes before `stop` settle together: no eviction among them
-        const uint32_t bmiss = miss & batch;
-        if (((batch >> lane) & 1u) && !res) __stcg(&owner[id], ((uint64_t)s << 32) | es);
-        total += __popc(bmiss);
-        if (lane == 0 && bmiss) __stcg(&count[s], __ldcg(&count[s]) + __popc(bmiss));
-        if (!missed && batch) {
-          const uint32_t lo = __ffs(batch) - 1;
-          const uint32_t f = (bmiss ? (uint32_t)(__ffs(bmiss) - 1) : 32u - __clz(batch)) - lo;
-          const uint64_t d0 = c + lo - b;
-          hits += f;
-          add_mul128(sv_lo, sv_hi, a.alpha, f);
-          add_mul128(sv_lo, sv_hi, a.beta, (uint64_t)f * d0 + (uint64_t)f * (f ? f - 1 : 0) / 2);
-          missed = bmiss != 0;
-        }
-        pending &= ~batch;
-        if (stop == 32 || stop == rep) continue;  // done, or a repeated block: test it again
-        // lane `stop` misses and overflows: lane 0 brings it in and evicts
+        s = __shfl_sync(kFull, q_s, r & 31);
+        b = e;
+        e = __shfl_sync(kFull, q_e, r & 31);
         __syncwarp();
-        const uint32_t x = __shfl_sync(kFull, id, stop);
-        if (lane == 0) {
-          __stcg(&owner[x], ((uint64_t)s << 32) | es);
-          __stcg(&count[s], __ldcg(&count[s]) + 1u);
-          total += 1;
-          while (total > C) {
-            uint32_t v = kNone;
-            while (front < r) {
-              const uint32_t t = a.ses[front];
-              if (in_bounds(a.st, t, a.n_session) && __ldcg(&last[t]) == front && __ldcg(&count[t]) > 0) {
-                v = t;
-                break;
-              }
-              ++front;
+        if (lane == 0) S.last[s] = r;
+        __syncwarp();
+        es = S.ep[s];
+        cnt = S.count[s];
+        missed = false;
+      }
+      if (t0 + at >= e) break;
+      const uint32_t w0 = at & ~(kSesWin - 1);  // this window of the batch
+      const uint32_t lo = at - w0;
+      uint32_t hi = size - w0 < kSesWin ? size - w0 : kSesWin;
+      if (e - (t0 + w0) < hi) hi = (uint32_t)(e - (t0 + w0));
+      const uint64_t depth = t0 + at - b;
+      at = w0 + hi;
+      uint32_t id[kSesPer], miss[kSesPer];
+      uint64_t o[kSesPer];
+#pragma unroll
+      for (uint32_t u = 0; u < kSesPer; ++u) id[u] = ids[w0 + 32 * u + lane];
+#pragma unroll
+      for (uint32_t u = 0; u < kSesPer; ++u) {
+        const uint32_t k = 32 * u + lane;
+        o[u] = k >= lo && k < hi ? owner[id[u]] : kNoOwner;
+      }
+      // an id after the first that does not exceed the one before it
+      bool falls = false;
+      if (lane < kSesPer) {
+        const uint32_t k = 32 * lane, w = fall[(w0 >> 5) + lane];
+        const uint32_t from = lo + 1 <= k ? 0u : lo + 1 - k, to = hi <= k ? 0u : hi - k;
+        falls = from < 32 && to > from && ((w >> from) << from & (to >= 32 ? kFull : (1u << to) - 1u)) != 0;
+      }
+      if (__any_sync(kFull, falls)) {
+        // ---- a block may come twice: 32 accesses at a time
+        uint64_t d0 = depth;
+        for (uint32_t c = lo & ~31u; c < hi; c += 32) {
+          const uint32_t k = c + lane;
+          const uint32_t x = ids[w0 + k];
+          uint32_t pending = __ballot_sync(kFull, k >= lo && k < hi);
+          while (pending) {
+            const bool mine = (pending >> lane) & 1u;
+            bool res = false;
+            if (mine) res = ses_resident(a, S, owner[x]);
+            uint32_t same = 0;
+            if (mine) same = __match_any_sync(pending, x);
+            const uint32_t later_copy = __ballot_sync(kFull, mine && (same & lanemask_lt()) != 0);
+            const uint32_t ms = __ballot_sync(kFull, mine && !res);
+            const uint64_t room = C - total;
+            uint32_t over = 32;  // the first miss that would push the cache past C
+            if ((uint64_t)__popc(ms) > room) {
+              uint32_t m = ms;
+              for (uint64_t q = 0; q < room; ++q) m &= m - 1u;
+              over = (uint32_t)(__ffs(m) - 1);
             }
-            if (v != kNone) {  // the least recently touched other session goes whole
-              ep[v] = ep[v] + 1u;
-              total -= __ldcg(&count[v]);
-              __stcg(&count[v], 0u);
-              ++front;
-            } else {  // the current session alone is above C: it keeps the block just brought in
-              es += 1;
-              ep[s] = es;
-              __stcg(&owner[x], ((uint64_t)s << 32) | es);
-              __stcg(&count[s], 1u);
-              total = 1;
+            const uint32_t rep = later_copy ? (uint32_t)(__ffs(later_copy) - 1) : 32u;
+            const uint32_t stop = over < rep ? over : rep;
+            const uint32_t part = pending & (stop == 32 ? kFull : ((1u << stop) - 1u));
+            const uint32_t pm = ms & part;
+            __syncwarp();
+            if ((pm >> lane) & 1u) owner[x] = ((uint64_t)s << 32) | es;
+            total += __popc(pm);
+            cnt += __popc(pm);
+            if (!missed && part) {
+              const uint32_t f0 = __ffs(part) - 1;
+              sums.add(a, d0, (pm ? (uint32_t)(__ffs(pm) - 1) : 32u - __clz(part)) - f0);
+              missed = pm != 0;
             }
+            d0 += __popc(part);
+            pending &= ~part;
+            __syncwarp();
+            if (stop == 32 || stop == rep) continue;  // done, or a repeated block: test it again
+            const uint32_t y = __shfl_sync(kFull, x, stop);
+            if (lane == 0) owner[y] = ((uint64_t)s << 32) | es;
+            total += 1;
+            cnt += 1;
+            ses_evict(a, S, owner, lane, r, s, y, C, front, total, cnt, es);
+            missed = true;
+            d0 += 1;
+            pending &= ~(1u << stop);
           }
         }
-        missed = true;
-        pending &= ~(1u << stop);
+        continue;
+      }
+      uint32_t m_all = 0, first = kSesWin;
+#pragma unroll
+      for (uint32_t u = 0; u < kSesPer; ++u) {
+        const uint32_t k = 32 * u + lane;
+        miss[u] = __ballot_sync(kFull, k >= lo && k < hi && !ses_resident(a, S, o[u]));
+        m_all += __popc(miss[u]);
+      }
+#pragma unroll
+      for (int u = kSesPer - 1; u >= 0; --u)
+        if (miss[u]) first = 32 * u + __ffs(miss[u]) - 1;
+      if (!missed) {  // the hits before the first miss
+        sums.add(a, depth, (m_all ? first : hi) - lo);
+        missed = m_all != 0;
+      }
+      if (m_all == 0) continue;
+      uint64_t stamp = ((uint64_t)s << 32) | es;
+      while (total + m_all > C) {
+        // the misses before the one that overflows settle
+        const uint32_t room = (uint32_t)(C - total);
+        uint32_t x_at = 0, x = 0, seen = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < kSesPer; ++u) {
+          const uint32_t c = __popc(miss[u]);
+          const uint32_t below = seen + __popc(miss[u] & lanemask_lt());
+          const bool mine = (miss[u] >> lane) & 1u;
+          if (mine && below <= room) owner[id[u]] = stamp;  // the overflowing one too
+          const uint32_t hit = __ballot_sync(kFull, mine && below == room);
+          if (hit) {
+            x_at = 32 * u + __ffs(hit) - 1;
+            x = __shfl_sync(kFull, id[u], x_at & 31);
+          }
+          seen += c;
+        }
+        total += room + 1;
+        cnt += room + 1;
+        m_all -= room + 1;
         __syncwarp();
-        total = __shfl_sync(kFull, total, 0);
-        es = __shfl_sync(kFull, es, 0);
+        if (ses_evict(a, S, owner, lane, r, s, x, C, front, total, cnt, es)) {
+          // session s is alone with block x: each later block misses, and
+          // every C-th of them empties the session again
+          const uint32_t rest = hi - 1 - x_at, per = C < kSesWin ? (uint32_t)C : 2 * kSesWin;
+#pragma unroll
+          for (uint32_t u = 0; u < kSesPer; ++u) {
+            const uint32_t k = 32 * u + lane;
+            if (k > x_at && k < hi) owner[id[u]] = ((uint64_t)s << 32) | (es + (k - x_at) / per);
+          }
+          es += rest / per;
+          total = 1 + rest % per;
+          cnt = (uint32_t)total;
+          m_all = 0;
+          __syncwarp();
+          if (lane == 0) S.ep[s] = es;
+          __syncwarp();
+          break;
+        }
+        m_all = 0;
+#pragma unroll
+        for (uint32_t u = 0; u < kSesPer; ++u) {
+          const uint32_t k = 32 * u + lane;
+          miss[u] = __ballot_sync(kFull, k >= lo && k < hi && k > x_at && !ses_resident(a, S, o[u]));
+          m_all += __popc(miss[u]);
+        }
+      }
+      if (m_all) {
+#pragma unroll
+        for (uint32_t u = 0; u < kSesPer; ++u)
+          if ((miss[u] >> lane) & 1u) owner[id[u]] = stamp;
+        total += m_all;
+        cnt += m_all;
       }
       __syncwarp();
     }
+    __syncthreads();
   }
-  if (lane == 0) {
-    a.out[g] = hits;
-    a.out[a.G + 2 * g] = sv_lo;
-    a.out[a.G + 2 * g + 1] = sv_hi;
+  if (threadIdx.x == 0) {
+    a.out[g] = sums.hits;
+    a.out[a.G + 2 * g] = sums.lo;
+    a.out[a.G + 2 * g + 1] = sums.hi;
   }
 }
 
@@ -279,11 +506,11 @@ extern "C" ptc_status ptc_session_lru_curves(const uint32_t* ids, uint64_t n, ui
   a.st = L.st;
   SesCaps caps;
   for (uint32_t g = 0; g < n_cap; ++g) caps.c[g] = cap_host[g];
-  const size_t smem = n_session <= kSesSmemSessions ? sizeof(uint32_t) * n_session : 0;
+  const size_t smem = sizeof(SesRing) + (n_session <= kSesSmemSessions ? 3 * sizeof(uint32_t) * n_session : 0);
   if (smem > 48 * 1024 &&
       cudaFuncSetAttribute(k_ses_sim, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
     return PTC_ERR_CUDA;
-  PTC_KERNEL("k_ses_sim", s, k_ses_sim, n_cap, 32, smem, a, caps);
+  PTC_KERNEL("k_ses_sim", s, k_ses_sim, n_cap, kSesThreads, smem, a, caps, (uint32_t)n);
   HostStage* hs = host_stage();
   if (copy_to_host_async(hs->out, L.out, sizeof(uint64_t) * 3 * n_cap, s) != PTC_OK) return PTC_ERR_CUDA;
   DevStatus h;
