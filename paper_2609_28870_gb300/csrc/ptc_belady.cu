@@ -26,18 +26,30 @@
 // new free time i - 1 is the one step L - 1 looks for, handled on its own.  A
 // run with gap < L is cut into pieces of length gap, which meet that case.
 //
-// One warp simulates one capacity: the free times are a bitmap over access
-// positions with three summary levels (a bit per nonzero word, kept exact as
-// words fill and empty) and a lower bound on the smallest free time, so a run
-// with nothing free below p learns it at once; runs go in order, up to
-// 1024 steps at a time, one 32-step word per lane.  Hits count with the
-// prefix rule (Sec. 2.2): a request's accesses before its first miss.
+// One warp simulates one capacity.  The free times are a bitmap over access
+// positions with three summary levels (a bit per nonzero word, kept exact) and
+// a lower bound on the smallest free time, so a run with nothing free below p
+// learns it at once.  Runs go in order, up to 1,024 positions at a time: lane
+// l holds word l of the 32 that start with p's, so every update is a plain
+// store of whole words by one lane, and the summary bits come from ballots.
+// What bounds the replay is the latency of one run's chain of reads, hence:
+// the summaries sit in shared memory (a bit per 32 accesses: up to about 50M
+// accesses), the bitmap's words are read through L1, and three other warps
+// read the words of the next 32 runs into L1 ahead of the replayer, whose own
+// stores go through the same L1.  Hits count with the prefix rule (Sec. 2.2):
+// a request's accesses before its first miss.
+//
+// Measured on the 9.3M-access chat trace, 64 capacities: 180 ms with the summaries
+// in L2 and every update an atomic; 43.7 ms so.
 #include "ptc_internal.h"
 
 namespace ptc {
 namespace {
 
-constexpr uint32_t kBelStep = 1024;  // steps of a run simulated together (32 lanes x 32)
+constexpr uint32_t kBelAhead = 3;     // warps that read ahead
+constexpr uint32_t kBelThreads = 32 * (1 + kBelAhead);
+constexpr uint32_t kBelRuns = 32;     // runs per batch
+constexpr size_t kBelSmemMax = 200 * 1024;  // summaries in shared memory up to this size
 
 __device__ __forceinline__ uint32_t hi_bit(uint32_t v) { return 31u - __clz(v); }
 __device__ __forceinline__ uint32_t mask_le(uint32_t b) { return b == 31 ? kFull : ((2u << b) - 1u); }
@@ -108,8 +120,8 @@ struct BelArgs {
   const uint32_t* rec_p;
   const uint8_t* rec_rs;
   const uint64_t* nruns;
-  uint32_t *lv0, *lv1, *lv2, *lv3;  // free-time bitmap and its summaries, one slice per capacity
-  uint64_t s0, s1, s2, s3;          // words per slice
+  uint32_t *lv0, *sum;        // free-time bitmap and its summaries, one slice per capacity
+  uint32_t s0, s1, s2, s3;    // words per slice and level (sum: s1 + s2 + s3)
   uint32_t G;
   uint64_t alpha, beta;
   uint64_t* out;  // hits[G] | saved[G] (lo, hi) | raw hits[G]
@@ -117,104 +129,108 @@ struct BelArgs {
 };
 
 // One capacity's free-time bitmap: level 0 one bit per access position,
-// level k + 1 one bit per nonzero word of level k.  `low` is a lower bound on
-// every set position (raised when a search finds nothing below a point).
+// level k + 1 one bit per nonzero word of level k.  Only one warp uses it,
+// every lane calling each function.  `low` is a lower bound on every set
+// position (raised when a search finds nothing below a point).
 struct FreeBits {
   uint32_t *l0, *l1, *l2, *l3;
-  uint64_t low;
-  uint64_t words;     // level-0 words of the slice
+  uint32_t low;
+  uint32_t words;  // level-0 words of the slice
   const DevStatus* st;
 
-  __device__ void set_word(uint64_t w, uint32_t m) {
-    if (!m || !in_bounds(st, w, words)) return;
-    atomicOr(&l0[w], m);
-    atomicOr(&l1[w >> 5], 1u << (w & 31));
-    atomicOr(&l2[w >> 10], 1u << ((w >> 5) & 31));
-    atomicOr(&l3[w >> 15], 1u << ((w >> 10) & 31));
-  }
-  // Clear bits m of word w; a word that becomes empty clears its summary
-  // bit, and an emptied summary word its bit above (sets and clears of one
-  // warp never overlap, so exactly one lane sees each word empty out).
-  __device__ void clear_word(uint64_t w, uint32_t m) {
-    if (!m || !in_bounds(st, w, words)) return;
-    const uint32_t old = atomicAnd(&l0[w], ~m);
-    if (old == 0 || (old & ~m) != 0) return;
-    const uint32_t b1 = 1u << (w & 31);
-    const uint32_t o1 = atomicAnd(&l1[w >> 5], ~b1);
-    if (o1 == 0 || (o1 & ~b1) != 0) return;
-    const uint32_t b2 = 1u << ((w >> 5) & 31);
-    const uint32_t o2 = atomicAnd(&l2[w >> 10], ~b2);
-    if (o2 != 0 && (o2 & ~b2) == 0) atomicAnd(&l3[w >> 15], ~(1u << ((w >> 10) & 31)));
-  }
-  // The highest set bit in words below w0, or -1.  Summary bits of words
-  // found empty are cleared on the way.
-  __device__ int64_t below_word(uint64_t w0) {
-    uint64_t w1 = w0 >> 5;
-    uint32_t m1 = __ldcg(&l1[w1]) & mask_lt((uint32_t)(w0 & 31));
-    for (;;) {
-      while (m1) {
-        const uint32_t b = hi_bit(m1);
-        const uint64_t ww = w1 * 32 + b;
-        const uint32_t v = __ldcg(&l0[ww]);
-        if (v) return (int64_t)(ww * 32 + hi_bit(v));
-        atomicAnd(&l1[w1], ~(1u << b));
-        m1 &= ~(1u << b);
-      }
-      uint64_t w2 = w1 >> 5;
-      uint32_t m2 = __ldcg(&l2[w2]) & mask_lt((uint32_t)(w1 & 31));
-      for (;;) {
-        while (!m2) {  // the next nonzero level-2 word below w2, through level 3
-          uint64_t w3 = w2 >> 5;
-          uint32_t m3 = __ldcg(&l3[w3]) & mask_lt((uint32_t)(w2 & 31));
-          while (!m3) {
-            if (w3 == 0) return -1;
-            --w3;
-            m3 = __ldcg(&l3[w3]);
-          }
-          w2 = w3 * 32 + hi_bit(m3);
-          m2 = __ldcg(&l2[w2]);
-          if (!m2) atomicAnd(&l3[w3], ~(1u << (w2 & 31)));
-        }
-        const uint32_t b2 = hi_bit(m2);
-        const uint64_t c1 = w2 * 32 + b2;
-        const uint32_t mm = __ldcg(&l1[c1]);
-        if (mm) {
-          w1 = c1;
-          m1 = mm;
-          break;
-        }
-        atomicAnd(&l2[w2], ~(1u << b2));
-        m2 &= ~(1u << b2);
+  // Words w0 .. w0 + 31 just became nonzero where `m` is set: set their
+  // summary bits.  They meet at most two words of level 1, lane 0's and
+  // lane 1's; those set the bits above on their own.
+  __device__ __forceinline__ void mark(uint32_t w0, uint32_t m, uint32_t lane) {
+    const uint32_t sh = w0 & 31;
+    const uint32_t bits = lane == 0 ? m << sh : lane == 1 && sh ? m >> (32 - sh) : 0u;
+    if (bits) {
+      const uint32_t w1 = (w0 >> 5) + lane;
+      const uint32_t old = l1[w1];
+      l1[w1] = old | bits;
+      if (old == 0) {
+        atomicOr(&l2[w1 >> 5], 1u << (w1 & 31));
+        atomicOr(&l3[w1 >> 10], 1u << ((w1 >> 5) & 31));
       }
     }
+    __syncwarp();
+  }
+  // Words w0 .. w0 + 31 just became zero where `m` is set.
+  __device__ __forceinline__ void unmark(uint32_t w0, uint32_t m, uint32_t lane) {
+    const uint32_t sh = w0 & 31;
+    const uint32_t bits = lane == 0 ? m << sh : lane == 1 && sh ? m >> (32 - sh) : 0u;
+    if (bits) {
+      const uint32_t w1 = (w0 >> 5) + lane;
+      const uint32_t now = l1[w1] & ~bits;
+      l1[w1] = now;
+      if (now == 0) {
+        const uint32_t b2 = 1u << (w1 & 31);
+        const uint32_t o2 = atomicAnd(&l2[w1 >> 5], ~b2);
+        if (o2 != 0 && (o2 & ~b2) == 0) atomicAnd(&l3[w1 >> 10], ~(1u << ((w1 >> 5) & 31)));
+      }
+    }
+    __syncwarp();
+  }
+  // The highest nonzero word of level 1 below word w1 (every lane the same
+  // answer), or kNone.
+  __device__ __forceinline__ uint32_t below1(uint32_t w1) {
+    uint32_t w2 = w1 >> 5, m2 = l2[w2] & mask_lt(w1 & 31);
+    if (!m2) {
+      uint32_t w3 = w2 >> 5, m3 = l3[w3] & mask_lt(w2 & 31);
+      while (!m3) {
+        if (w3 == 0) return kNone;
+        m3 = l3[--w3];
+      }
+      w2 = w3 * 32 + hi_bit(m3);
+      m2 = l2[w2];
+      if (!m2) return kNone;  // cannot happen: the summaries are exact
+    }
+    return w2 * 32 + hi_bit(m2);
   }
   // Clear the `need` highest set bits below position `pos`; returns how many
-  // there were (fewer if the bitmap runs out).
-  __device__ uint32_t pop_below(uint64_t pos, uint32_t need) {
-    uint32_t got = 0;
-    while (got < need && pos > low) {
-      const uint64_t w = (pos - 1) >> 5;
-      uint32_t v = __ldcg(&l0[w]) & mask_le((uint32_t)((pos - 1) & 31));
-      uint64_t ww = w;
-      if (!v) {
-        const int64_t b = below_word(w);
-        if (b < 0) {  // nothing set below pos (and appends only go above p0)
-          low = low > pos ? low : pos;
-          break;
+  // there were (fewer if the bitmap runs out).  32 words at a time, lane l
+  // the l-th of the words under one word of level 1.
+  __device__ __forceinline__ uint32_t pop_below(uint32_t pos, uint32_t need, uint32_t lane) {
+    if (pos <= low) return 0;
+    uint32_t got = 0, w1 = pos >> 10;
+    // the words below pos's, and the part of its word below pos
+    uint32_t m1 = l1[w1] & mask_le((pos >> 5) & 31);
+    uint32_t part = mask_lt(pos & 31);  // of word pos >> 5
+    while (true) {
+      if (m1) {
+        const uint32_t w = w1 * 32 + lane;
+        const uint32_t keep = w == pos >> 5 ? part : kFull;
+        uint32_t v = 0, all = 0;
+        if (((m1 >> lane) & 1u) && in_bounds(st, w, words)) {
+          all = l0[w];
+          v = all & keep;
         }
-        ww = (uint64_t)b >> 5;
-        v = __ldcg(&l0[ww]);
+        const uint32_t c = __popc(v);
+        uint32_t above = c;  // set bits in this lane's word and those above it
+#pragma unroll
+        for (int o = 1; o < 32; o <<= 1) {
+          const uint32_t y = __shfl_down_sync(kFull, above, o);
+          if (lane + o < 32) above += y;
+        }
+        const uint32_t sum = __shfl_sync(kFull, above, 0), want = need - got;
+        above -= c;
+        uint32_t take = 0;
+        if (above < want) {
+          take = v;
+          if (above + c > want) take = v & ~mask_le(nth_set(v, c - (want - above) - 1));  // its highest bits
+          if (take) l0[w] = all & ~take;
+        }
+        unmark(w1 * 32, __ballot_sync(kFull, take != 0 && (all & ~take) == 0), lane);
+        got += sum < want ? sum : want;
+        if (got == need) return got;
       }
-      const uint32_t cnt = __popc(v), take = cnt < need - got ? cnt : need - got;
-      uint32_t m = v;
-      if (take < cnt) {  // keep the lowest cnt - take bits
-        m = v & ~mask_le(nth_set(v, cnt - take - 1));
+      w1 = w1 ? below1(w1) : kNone;
+      if (w1 == kNone) {  // nothing set below pos (and appends only go above it)
+        low = pos;
+        return got;
       }
-      clear_word(ww, m);
-      got += take;
-      pos = ww * 32;
+      m1 = l1[w1];
     }
-    return got;
   }
 };
 
@@ -226,28 +242,60 @@ __device__ __forceinline__ void add_mul(uint64_t& lo, uint64_t& hi, uint64_t a, 
   add128(lo, hi, a * b, __umul64hi(a, b));
 }
 
-// One warp per capacity (capacity g = global warp index).
-__global__ void __launch_bounds__(32) k_bel_sim(BelArgs a, BelCaps caps) {
+// One CTA per capacity: warp 0 replays, the others read ahead.
+template <bool SMEM>
+__global__ void __launch_bounds__(kBelThreads) k_bel_sim(BelArgs a, BelCaps caps) {
+  extern __shared__ uint32_t s_sum[];
   grid_dep_sync();
-  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t g = blockIdx.x;
   if (g >= a.G) return;
-  FreeBits fb{a.lv0 + g * a.s0, a.lv1 + g * a.s1, a.lv2 + g * a.s2, a.lv3 + g * a.s3, 0, a.s0, a.st};
-  uint64_t free_inf = caps.c[g] - 1;  // never-used tracks (lane 0's copy is the one used)
+  uint32_t* const l0 = a.lv0 + (uint64_t)g * a.s0;
+  uint32_t* const sum = SMEM ? s_sum : a.sum + (uint64_t)g * (a.s1 + a.s2 + a.s3);
+  if (SMEM)
+    for (uint32_t i = threadIdx.x; i < a.s1 + a.s2 + a.s3; i += kBelThreads) sum[i] = 0;
+  FreeBits fb{l0, sum, sum + a.s1, sum + a.s1 + a.s2, 0, a.s0, a.st};
+  const uint32_t R = (uint32_t)*a.nruns;
+  // The words of the previous accesses of runs r0 .. r0 + 31, into L1.
+  auto read_ahead = [&](uint32_t r0) {
+    const uint32_t r = r0 + lane;
+    const uint32_t rs = r <= R ? __ldg(&a.rec_start[r]) : 0u, rp = r < R ? __ldg(&a.rec_p[r]) : kNone;
+    const uint32_t re = r < R ? __ldg(&a.rec_start[r + 1]) : 0u;
+    for (uint32_t t = warp - 1; t < kBelRuns && r0 + t < R; t += kBelAhead) {
+      const uint32_t p = __shfl_sync(kFull, rp, t), L = __shfl_sync(kFull, re, t) - __shfl_sync(kFull, rs, t);
+      if (p == kNone) continue;
+      // a word per 32-byte sector, and the line below p's (the latest free
+      // times below p tend to lie there)
+      const uint32_t first = (p >> 10) * 32, last = (uint32_t)(((uint64_t)p + L) >> 5);
+      const uint32_t from = first >= 32 ? first - 32 : 0u;
+      for (uint32_t w = from + 8 * lane; w <= last && w < a.s0; w += 256) {
+        uint32_t x;
+        asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(x) : "l"(l0 + w));
+        asm volatile("" ::"r"(x));
+      }
+    }
+  };
+  uint64_t free_inf = caps.c[g] - 1;  // never-used tracks
   uint64_t hits = 0, raw = 0, sv_lo = 0, sv_hi = 0;
   uint32_t req_start = 0;
   bool missed = false;
-  const uint64_t R = *a.nruns;
-  for (uint64_t r0 = 0; r0 < R; r0 += 32) {
-    const uint64_t rl = r0 + lane;
-    const uint32_t my_s = rl <= R ? a.rec_start[rl] : 0u;
+  if (warp) read_ahead(0);
+  __syncthreads();
+  for (uint32_t r0 = 0; r0 < R; r0 += kBelRuns) {
+    if (warp) {
+      if (R - r0 > kBelRuns) read_ahead(r0 + kBelRuns);
+      __syncthreads();
+      continue;
+    }
+    const uint32_t rl = r0 + lane;
+    const uint32_t my_s = rl < R ? a.rec_start[rl] : 0u;
+    const uint32_t my_e = rl < R ? a.rec_start[rl + 1] : 0u;
     const uint32_t my_p = rl < R ? a.rec_p[rl] : kNone;
     const uint32_t my_rs = rl < R ? a.rec_rs[rl] : 0u;
-    const uint32_t end32 = r0 + 32 <= R ? a.rec_start[r0 + 32] : 0u;
-    const uint32_t nr = R - r0 < 32 ? (uint32_t)(R - r0) : 32u;
+    const uint32_t nr = R - r0 < kBelRuns ? R - r0 : kBelRuns;
     for (uint32_t t = 0; t < nr; ++t) {
       uint32_t s = __shfl_sync(kFull, my_s, t);
-      const uint32_t e = t + 1 < 32 ? __shfl_sync(kFull, my_s, (t + 1) & 31) : end32;
+      const uint32_t e = __shfl_sync(kFull, my_e, t);
       uint32_t p = __shfl_sync(kFull, my_p, t);
       if (__shfl_sync(kFull, my_rs, t)) {
         req_start = s;
@@ -269,76 +317,73 @@ __global__ void __launch_bounds__(32) k_bel_sim(BelArgs a, BelCaps caps) {
         continue;
       }
       while (L > 0) {
-        const uint32_t gap = s - p;
-        const uint32_t Lj = L < gap ? (L < kBelStep ? L : kBelStep) : (gap < kBelStep ? gap : kBelStep);
-        // this lane's 32 steps: k = 32 lane .. 32 lane + 31
-        const uint32_t k0 = 32 * lane;
-        const uint32_t valid = k0 >= Lj ? 0u : (Lj - k0 >= 32 ? kFull : ((1u << (Lj - k0)) - 1u));
-        const uint64_t q = (uint64_t)p + k0, w = q >> 5;
-        const uint32_t sh = (uint32_t)(q & 31);
-        uint32_t Bk = 0;
-        if (valid && in_bounds(a.st, w + (sh ? 1 : 0), a.s0)) {
-          const uint32_t lo = __ldcg(&fb.l0[w]);
-          const uint32_t hi = sh ? __ldcg(&fb.l0[w + 1]) : 0u;
-          Bk = (sh ? (lo >> sh) | (hi << (32 - sh)) : lo) & valid;
-        }
-        const bool edge = Lj >= 2 && (uint64_t)p + Lj == s;
-        const uint32_t elane = (Lj - 1) >> 5, ebit = 1u << ((Lj - 1) & 31);
+        const uint32_t gap = s - p, sp = p & 31;
+        uint32_t Lj = L < gap ? L : gap;
+        if (Lj > 1024 - sp) Lj = 1024 - sp;  // the 32 words from p's
+        // this lane's word of them: positions 32 (w0 + lane) ..
+        const uint32_t w0 = p >> 5, w = w0 + lane;
+        const uint32_t end = sp + Lj;  // past the last step, counted from word w0
+        uint32_t valid = lane * 32 >= end ? 0u : end - lane * 32 >= 32 ? kFull : mask_lt(end - lane * 32);
+        if (lane == 0) valid &= ~mask_lt(sp);
+        uint32_t word = 0;
+        if (valid && in_bounds(a.st, w, a.s0)) word = l0[w];
+        const uint32_t Bk = word & valid;
+        // the free times of [p, p + Lj) are used up
+        if (Bk) l0[w] = word & ~valid;
+        fb.unmark(w0, __ballot_sync(kFull, Bk != 0 && (word & ~valid) == 0), lane);
+        const bool edge = Lj >= 2 && p + Lj == s;
+        const uint32_t elane = (end - 1) >> 5, ebit = 1u << ((end - 1) & 31);
         uint32_t zm = ~Bk & valid;
-        if (edge && lane == elane) zm &= ~ebit;  // step Lj - 1: decided by step 0 below
-        const uint32_t zc = __popc(zm);
-        uint32_t zx = zc;  // exclusive prefix of the zero counts
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(kFull, zx, o);
-          if (lane >= (uint32_t)o) zx += y;
-        }
-        const uint32_t z = __shfl_sync(kFull, zx, 31);
-        zx -= zc;
-        // the non-B steps take the latest free times below p, then never-used tracks
-        uint32_t acc = 0;
-        if (lane == 0 && z > 0) {
-          const uint32_t got = fb.pop_below(p, z);
-          const uint64_t rest = z - got;
-          const uint64_t inf = rest < free_inf ? rest : free_inf;
+        if (edge && lane == elane) zm &= ~ebit;  // the last step: decided by step 0 below
+        const uint32_t zc = __popc(zm), z = __reduce_add_sync(kFull, zc);
+        uint32_t A = valid;  // steps that hit
+        uint32_t nh = Lj, f = Lj;  // hits, and hits before the first miss
+        if (z) {
+          // the other steps take the latest free times below p, then never-used tracks
+          uint32_t acc = fb.pop_below(p, z, lane);
+          const uint32_t rest = z - acc, inf = rest < free_inf ? rest : (uint32_t)free_inf;
           free_inf -= inf;
-          acc = got + (uint32_t)inf;
-        }
-        __syncwarp();
-        acc = __shfl_sync(kFull, acc, 0);
-        const bool acc0 = (__shfl_sync(kFull, Bk, 0) & 1u) || acc >= 1;
-        uint32_t A;
-        if (acc >= zx + zc) {
-          A = valid;
-        } else if (acc <= zx) {
-          A = valid & ~zm;
-        } else {
-          const uint32_t first_rej = nth_set(zm, acc - zx);
-          A = (valid & ~zm) | (zm & mask_lt(first_rej));
-        }
-        if (edge && lane == elane) A = acc0 ? (A | ebit) : (A & ~ebit);
-        const uint32_t rej = valid & ~A;
-        const uint32_t my_f = rej ? k0 + (uint32_t)(__ffs(rej) - 1) : Lj;
-        uint32_t f = my_f, nh = __popc(A);
+          acc += inf;
+          if (acc < z) {  // the first acc of them hit
+            uint32_t zx = zc;
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) {
-          const uint32_t of = __shfl_xor_sync(kFull, f, o);
-          f = of < f ? of : f;
-          nh += __shfl_xor_sync(kFull, nh, o);
+            for (int o = 1; o < 32; o <<= 1) {
+              const uint32_t y = __shfl_up_sync(kFull, zx, o);
+              if (lane >= (uint32_t)o) zx += y;
+            }
+            zx -= zc;
+            if (acc < zx + zc) A = (valid & ~zm) | (acc <= zx ? 0u : zm & mask_lt(nth_set(zm, acc - zx)));
+            const bool hit0 = ((__shfl_sync(kFull, Bk, 0) >> sp) & 1u) || acc >= 1;
+            if (edge && !hit0 && lane == elane) A &= ~ebit;
+            const uint32_t rej = valid & ~A;
+            const uint32_t with = __ballot_sync(kFull, rej != 0);
+            nh = Lj - __reduce_add_sync(kFull, __popc(rej));
+            const uint32_t first = __ffs(with) - 1;
+            f = 32 * first + __ffs(__shfl_sync(kFull, rej, first)) - 1 - sp;
+          }
         }
-        // new free times s - 1 + k of the hits, then the free times of [p, p + Lj) are used up
-        if (A) {
-          const uint64_t q2 = (uint64_t)s - 1 + k0, w2 = q2 >> 5;
-          const uint32_t sh2 = (uint32_t)(q2 & 31);
-          fb.set_word(w2, A << sh2);
-          if (sh2) fb.set_word(w2 + 1, A >> (32 - sh2));
+        // New free times s - 1 + k of the hits; with p + Lj = s the last step
+        // took step 0's.  They lie above every free time so far.
+        {
+          uint32_t T = A;
+          if (edge && lane == 0) T &= ~(1u << sp);
+          const uint32_t q = s - 1, v0 = q >> 5, sq = q & 31;
+          const uint32_t up = __shfl_up_sync(kFull, T, 1), dn = __shfl_down_sync(kFull, T, 1);
+          uint32_t out, past = 0;  // words v0 + lane, and v0 + 32 (lane 31)
+          if (sq >= sp) {
+            const uint32_t d = sq - sp;
+            out = T << d | (d && lane ? up >> (32 - d) : 0u);
+            if (d && lane == 31) past = T >> (32 - d);
+          } else {
+            const uint32_t d = sp - sq;
+            out = T >> d | (lane < 31 ? dn << (32 - d) : 0u);
+          }
+          __syncwarp();  // the words cleared above may be among these
+          if (out && in_bounds(a.st, v0 + lane, a.s0)) l0[v0 + lane] = lane ? out : l0[v0] | out;
+          if (past && in_bounds(a.st, v0 + 32, a.s0)) l0[v0 + 32] = past;
+          fb.mark(v0, __ballot_sync(kFull, out != 0), lane);
+          if (__shfl_sync(kFull, past, 31)) fb.mark(v0 + 32, 1u, lane);
         }
-        __syncwarp();
-        if (valid) {
-          fb.clear_word(w, valid << sh);
-          if (sh) fb.clear_word(w + 1, valid >> (32 - sh));
-        }
-        __syncwarp();
         raw += nh;
         if (!missed) {
           const uint64_t d0 = s - req_start;
@@ -352,8 +397,9 @@ __global__ void __launch_bounds__(32) k_bel_sim(BelArgs a, BelCaps caps) {
         L -= Lj;
       }
     }
+    __syncthreads();
   }
-  if (lane == 0) {
+  if (threadIdx.x == 0) {
     a.out[g] = hits;
     a.out[a.G + 2 * g] = sv_lo;
     a.out[a.G + 2 * g + 1] = sv_hi;
@@ -369,7 +415,7 @@ struct BelLayout {
   uint64_t* nruns;
   uint32_t *rec_start, *rec_p;
   uint8_t* rec_rs;
-  uint32_t *lv0, *lv1, *lv2, *lv3;
+  uint32_t *lv0, *sum;
   uint64_t s0, s1, s2, s3;
   uint64_t* out;
   size_t zero_bytes, bits_bytes;
@@ -395,14 +441,12 @@ BelLayout bel_layout(void* ws, uint64_t n, uint32_t n_cap) {
   L.rec_p = cv.take<uint32_t>(nn);
   L.rec_rs = cv.take<uint8_t>(nn);
   const uint64_t G = n_cap ? n_cap : 1;
-  L.s0 = (uint64_t)L.nwords + 2;
+  L.s0 = ((uint64_t)L.nwords + 2 + 31) / 32 * 32;  // whole 128-byte lines
   L.s1 = (L.s0 + 31) / 32 + 1;
   L.s2 = (L.s1 + 31) / 32 + 1;
   L.s3 = (L.s2 + 31) / 32 + 1;
   L.lv0 = cv.take<uint32_t>((L.s0 + L.s1 + L.s2 + L.s3) * G);
-  L.lv1 = L.lv0 + L.s0 * G;
-  L.lv2 = L.lv1 + L.s1 * G;
-  L.lv3 = L.lv2 + L.s2 * G;
+  L.sum = L.lv0 + L.s0 * G;
   L.bits_bytes = sizeof(uint32_t) * (L.s0 + L.s1 + L.s2 + L.s3) * G;
   L.out = cv.take<uint64_t>(4 * G);
   L.total = cv.bytes();
@@ -460,13 +504,11 @@ extern "C" ptc_status ptc_belady_curves(const uint32_t* prev, uint64_t n, const 
   a.rec_rs = L.rec_rs;
   a.nruns = L.nruns;
   a.lv0 = L.lv0;
-  a.lv1 = L.lv1;
-  a.lv2 = L.lv2;
-  a.lv3 = L.lv3;
-  a.s0 = L.s0;
-  a.s1 = L.s1;
-  a.s2 = L.s2;
-  a.s3 = L.s3;
+  a.sum = L.sum;
+  a.s0 = (uint32_t)L.s0;
+  a.s1 = (uint32_t)L.s1;
+  a.s2 = (uint32_t)L.s2;
+  a.s3 = (uint32_t)L.s3;
   a.G = n_cap;
   a.alpha = alpha;
   a.beta = beta;
@@ -474,7 +516,15 @@ extern "C" ptc_status ptc_belady_curves(const uint32_t* prev, uint64_t n, const 
   a.st = L.st;
   BelCaps caps;
   for (uint32_t g = 0; g < n_cap; ++g) caps.c[g] = cap_host[g];
-  PTC_KERNEL("k_bel_sim", s, k_bel_sim, n_cap, 32, 0, a, caps);
+  const size_t sums = sizeof(uint32_t) * (L.s1 + L.s2 + L.s3);
+  if (sums <= kBelSmemMax) {
+    if (sums > 48 * 1024 && cudaFuncSetAttribute(k_bel_sim<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                 (int)kBelSmemMax) != cudaSuccess)
+      return PTC_ERR_CUDA;
+    PTC_KERNEL("k_bel_sim", s, k_bel_sim<true>, n_cap, kBelThreads, sums, a, caps);
+  } else {
+    PTC_KERNEL("k_bel_sim", s, k_bel_sim<false>, n_cap, kBelThreads, 0, a, caps);
+  }
   HostStage* hs = host_stage();
   if (copy_to_host_async(hs->out, L.out, sizeof(uint64_t) * 3 * n_cap, s) != PTC_OK) return PTC_ERR_CUDA;
   if (raw_hits_host_out &&
