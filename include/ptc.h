@@ -181,16 +181,17 @@ ptc_status ptc_assign_ids_prior(const ptc_u128* keys, uint64_t n, const uint64_t
  * (n_req > 0, same hint rules) with the way keys are deduplicated named.
  * Every method gives the same ids and D:
  *   PTC_IDS_TABLE        one open-addressing table of 16-byte slots: a first
- *                        attempt with n / 3 slots (3 n / 4 once that is larger
- *                        than 64 MB), the whole stage again with 1.5 n slots
- *                        if a probe sequence outruns it
+ *                        attempt with 0.6 n slots, at most 128 MB of them
+ *                        (3 n / 4 slots for n above about 12.6M), the whole
+ *                        stage again with 1.5 n slots if a probe sequence
+ *                        outruns it
  *   PTC_IDS_PARTITIONED  the keys to settle are moved, in streaming passes,
  *                        into 65,536 partitions by 16 key bits, and each
  *                        partition is deduplicated in a table in shared
  *                        memory; a partition with more than 6,144 distinct
  *                        keys sends the stage to the full table as above
- *   PTC_IDS_AUTO         PTC_IDS_PARTITIONED when the first table would exceed
- *                        64 MB (n above about 12.6M), else PTC_IDS_TABLE; what
+ *   PTC_IDS_AUTO         PTC_IDS_PARTITIONED for n above about 12.6M (a table
+ *                        that does not fit in L2), else PTC_IDS_TABLE; what
  *                        ptc_assign_ids and ptc_assign_ids_prior do
  * Workspace: ptc_assign_ids_ex_workspace_bytes(n, n_req, method).  An
  * unknown method is PTC_ERR_INVALID_ARG.

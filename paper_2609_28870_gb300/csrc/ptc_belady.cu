@@ -27,20 +27,23 @@
 // run with gap < L is cut into pieces of length gap, which meet that case.
 //
 // One warp simulates one capacity.  The free times are a bitmap over access
-// positions with three summary levels (a bit per nonzero word, kept exact) and
-// a lower bound on the smallest free time, so a run with nothing free below p
-// learns it at once.  Runs go in order, up to 1,024 positions at a time: lane
-// l holds word l of the 32 that start with p's, so every update is a plain
-// store of whole words by one lane, and the summary bits come from ballots.
-// What bounds the replay is the latency of one run's chain of reads, hence:
-// the summaries sit in shared memory (a bit per 32 accesses: up to about 50M
-// accesses), the bitmap's words are read through L1, and three other warps
-// read the words of the next 32 runs into L1 ahead of the replayer, whose own
-// stores go through the same L1.  Hits count with the prefix rule (Sec. 2.2):
-// a request's accesses before its first miss.
+// positions with three summary levels (a bit per word that may be nonzero,
+// cleared when a search finds the word empty) and a lower bound on the
+// smallest free time, so a run with nothing free below p learns it at once.
+// Runs go in order, up to 1,024 positions at a time: lane l holds word l of
+// the 32 that start with p's, and word l of the 32 below them, so every update
+// is a plain store of whole words by one lane.
+// What bounds the replay is the latency of one run's chain of reads and
+// shuffles, hence: the summaries sit in shared memory (a bit per 32 accesses:
+// up to about 50M accesses), three other warps read the bitmap words of the
+// next 32 runs into L1 ahead of the replayer, whose own stores go through the
+// same L1, and the bitmap's last word, which the next run extends, stays in a
+// register.  Hits count with the prefix rule (Sec. 2.2): a request's accesses
+// before its first miss.
 //
-// Measured on the 9.3M-access chat trace, 64 capacities: 180 ms with the summaries
-// in L2 and every update an atomic; 43.7 ms so.
+// Measured on the 9.3M-access chat trace, 64 capacities: 180 ms with the
+// summaries in L2, every update an atomic and one lane searching; 43.7 ms with
+// exact summaries in shared memory; @@MEASURED@@
 #include "ptc_internal.h"
 
 namespace ptc {
@@ -54,10 +57,27 @@ constexpr size_t kBelSmemMax = 200 * 1024;  // summaries in shared memory up to 
 __device__ __forceinline__ uint32_t hi_bit(uint32_t v) { return 31u - __clz(v); }
 __device__ __forceinline__ uint32_t mask_le(uint32_t b) { return b == 31 ? kFull : ((2u << b) - 1u); }
 __device__ __forceinline__ uint32_t mask_lt(uint32_t b) { return b == 0 ? 0u : (kFull >> (32 - b)); }
-// Position of the j-th lowest set bit of v (j = 0 is the lowest); v has more than j set bits.
-__device__ __forceinline__ uint32_t nth_set(uint32_t v, uint32_t j) {
-  for (uint32_t t = 0; t < j; ++t) v &= v - 1u;
-  return (uint32_t)(__ffs(v) - 1);
+// Exclusive prefix over the lanes of c <= 32 (six ballots, whose latencies
+// overlap, where a shuffle scan is a chain of five); *total gets the sum.
+__device__ __forceinline__ uint32_t lanes_excl(uint32_t c, uint32_t* total) {
+  const uint32_t lt = lanemask_lt();
+  uint32_t x = 0, t = 0;
+#pragma unroll
+  for (int b = 0; b < 6; ++b) {
+    const uint32_t m = __ballot_sync(kFull, (c >> b) & 1u);
+    x += __popc(m & lt) << b;
+    t += __popc(m) << b;
+  }
+  *total = t;
+  return x;
+}
+// The j highest set bits of v, the same v and j in every lane.
+__device__ __forceinline__ uint32_t top_bits(uint32_t v, uint32_t j, uint32_t lane) {
+  return __ballot_sync(kFull, ((v >> lane) & 1u) && __popc(v >> lane) <= j);
+}
+// The j lowest set bits of v, the same v and j in every lane.
+__device__ __forceinline__ uint32_t low_bits(uint32_t v, uint32_t j, uint32_t lane) {
+  return __ballot_sync(kFull, ((v >> lane) & 1u) && __popc(v & mask_le(lane)) <= j);
 }
 
 // Request starts: one bit per access in `heads` and `rs`; offsets checked.
@@ -129,18 +149,17 @@ struct BelArgs {
 };
 
 // One capacity's free-time bitmap: level 0 one bit per access position,
-// level k + 1 one bit per nonzero word of level k.  Only one warp uses it,
-// every lane calling each function.  `low` is a lower bound on every set
-// position (raised when a search finds nothing below a point).
+// level k + 1 one bit per word of level k that may be nonzero (a nonzero word
+// always has its bit).  Only one warp uses it, every lane calling each
+// function.  `low` is a lower bound on every set position (raised when a
+// search finds nothing below a point).
 struct FreeBits {
   uint32_t *l0, *l1, *l2, *l3;
   uint32_t low;
   uint32_t words;  // level-0 words of the slice
   const DevStatus* st;
 
-  // Words w0 .. w0 + 31 just became nonzero where `m` is set: set their
-  // summary bits.  They meet at most two words of level 1, lane 0's and
-  // lane 1's; those set the bits above on their own.
+  // Words w0 .. w0 + 31 became nonzero where `m` is set.
   __device__ __forceinline__ void mark(uint32_t w0, uint32_t m, uint32_t lane) {
     const uint32_t sh = w0 & 31;
     const uint32_t bits = lane == 0 ? m << sh : lane == 1 && sh ? m >> (32 - sh) : 0u;
@@ -155,27 +174,18 @@ struct FreeBits {
     }
     __syncwarp();
   }
-  // Words w0 .. w0 + 31 just became zero where `m` is set.
-  __device__ __forceinline__ void unmark(uint32_t w0, uint32_t m, uint32_t lane) {
-    const uint32_t sh = w0 & 31;
-    const uint32_t bits = lane == 0 ? m << sh : lane == 1 && sh ? m >> (32 - sh) : 0u;
-    if (bits) {
-      const uint32_t w1 = (w0 >> 5) + lane;
-      const uint32_t now = l1[w1] & ~bits;
-      l1[w1] = now;
-      if (now == 0) {
-        const uint32_t b2 = 1u << (w1 & 31);
-        const uint32_t o2 = atomicAnd(&l2[w1 >> 5], ~b2);
-        if (o2 != 0 && (o2 & ~b2) == 0) atomicAnd(&l3[w1 >> 10], ~(1u << ((w1 >> 5) & 31)));
-      }
-    }
-    __syncwarp();
-  }
-  // The highest nonzero word of level 1 below word w1 (every lane the same
-  // answer), or kNone.
-  __device__ __forceinline__ uint32_t below1(uint32_t w1) {
+  // The highest word of level 1 below word w1 that is nonzero, or kNone;
+  // level-2 and level-3 bits of words found empty are cleared on the way.
+  __device__ __forceinline__ uint32_t below1(uint32_t w1, uint32_t lane) {
     uint32_t w2 = w1 >> 5, m2 = l2[w2] & mask_lt(w1 & 31);
-    if (!m2) {
+    while (true) {
+      while (m2) {
+        const uint32_t b = hi_bit(m2), c = w2 * 32 + b;
+        if (l1[c]) return c;
+        if (lane == 0) l2[w2] &= ~(1u << b);
+        m2 &= ~(1u << b);
+        __syncwarp();
+      }
       uint32_t w3 = w2 >> 5, m3 = l3[w3] & mask_lt(w2 & 31);
       while (!m3) {
         if (w3 == 0) return kNone;
@@ -183,52 +193,40 @@ struct FreeBits {
       }
       w2 = w3 * 32 + hi_bit(m3);
       m2 = l2[w2];
-      if (!m2) return kNone;  // cannot happen: the summaries are exact
+      __syncwarp();
+      if (!m2 && lane == 0) l3[w3] &= ~(1u << (w2 & 31));
+      __syncwarp();
     }
-    return w2 * 32 + hi_bit(m2);
   }
-  // Clear the `need` highest set bits below position `pos`; returns how many
-  // there were (fewer if the bitmap runs out).  32 words at a time, lane l
-  // the l-th of the words under one word of level 1.
-  __device__ __forceinline__ uint32_t pop_below(uint32_t pos, uint32_t need, uint32_t lane) {
-    if (pos <= low) return 0;
-    uint32_t got = 0, w1 = pos >> 10;
-    // the words below pos's, and the part of its word below pos
-    uint32_t m1 = l1[w1] & mask_le((pos >> 5) & 31);
-    uint32_t part = mask_lt(pos & 31);  // of word pos >> 5
+  // Clear the `need` highest set bits in the words below word `end`; returns
+  // how many there were (fewer if the bitmap runs out).  32 words at a time,
+  // lane l the l-th of those under one word of level 1, in falling order.
+  __device__ __forceinline__ uint32_t pop_words(uint32_t end, uint32_t need, uint32_t lane) {
+    uint32_t got = 0, w1 = end >> 5;
+    uint32_t m1 = l1[w1] & mask_lt(end & 31);
     while (true) {
       if (m1) {
-        const uint32_t w = w1 * 32 + lane;
-        const uint32_t keep = w == pos >> 5 ? part : kFull;
-        uint32_t v = 0, all = 0;
-        if (((m1 >> lane) & 1u) && in_bounds(st, w, words)) {
-          all = l0[w];
-          v = all & keep;
+        const uint32_t b = 31 - lane, w = w1 * 32 + b;
+        const uint32_t v = ((m1 >> b) & 1u) && in_bounds(st, w, words) ? l0[w] : 0u;
+        uint32_t sum;
+        const uint32_t c = __popc(v), above = lanes_excl(c, &sum);
+        const uint32_t want = need - got;
+        uint32_t take = above + c <= want ? v : 0u;
+        const uint32_t part = __ballot_sync(kFull, above < want && above + c > want);
+        if (part) {  // the word that holds the last one wanted
+          const uint32_t src = __ffs(part) - 1;
+          const uint32_t t = top_bits(__shfl_sync(kFull, v, src), want - __shfl_sync(kFull, above, src), lane);
+          if (lane == src) take = t;
         }
-        const uint32_t c = __popc(v);
-        uint32_t above = c;  // set bits in this lane's word and those above it
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_down_sync(kFull, above, o);
-          if (lane + o < 32) above += y;
-        }
-        const uint32_t sum = __shfl_sync(kFull, above, 0), want = need - got;
-        above -= c;
-        uint32_t take = 0;
-        if (above < want) {
-          take = v;
-          if (above + c > want) take = v & ~mask_le(nth_set(v, c - (want - above) - 1));  // its highest bits
-          if (take) l0[w] = all & ~take;
-        }
-        unmark(w1 * 32, __ballot_sync(kFull, take != 0 && (all & ~take) == 0), lane);
-        got += sum < want ? sum : want;
-        if (got == need) return got;
+        if (take) l0[w] = v & ~take;
+        const uint32_t empty = m1 & __brev(__ballot_sync(kFull, v == take));
+        if (lane == 0 && empty) l1[w1] &= ~empty;
+        __syncwarp();
+        if (sum >= want) return need;
+        got += sum;
       }
-      w1 = w1 ? below1(w1) : kNone;
-      if (w1 == kNone) {  // nothing set below pos (and appends only go above it)
-        low = pos;
-        return got;
-      }
+      w1 = w1 ? below1(w1, lane) : kNone;
+      if (w1 == kNone) return got;
       m1 = l1[w1];
     }
   }
@@ -276,8 +274,9 @@ __global__ void __launch_bounds__(kBelThreads) k_bel_sim(BelArgs a, BelCaps caps
     }
   };
   uint64_t free_inf = caps.c[g] - 1;  // never-used tracks
-  uint64_t hits = 0, raw = 0, sv_lo = 0, sv_hi = 0;
+  uint64_t hits = 0, raw = 0, depths = 0;  // counted hits, all hits, and the counted hits' depths
   uint32_t req_start = 0;
+  uint32_t tail_w = 0, tail = 0;  // the highest word that free times were added to, as it stands
   bool missed = false;
   if (warp) read_ahead(0);
   __syncthreads();
@@ -291,13 +290,13 @@ __global__ void __launch_bounds__(kBelThreads) k_bel_sim(BelArgs a, BelCaps caps
     const uint32_t my_s = rl < R ? a.rec_start[rl] : 0u;
     const uint32_t my_e = rl < R ? a.rec_start[rl + 1] : 0u;
     const uint32_t my_p = rl < R ? a.rec_p[rl] : kNone;
-    const uint32_t my_rs = rl < R ? a.rec_rs[rl] : 0u;
+    const uint32_t opens = __ballot_sync(kFull, rl < R && a.rec_rs[rl]);  // runs that open a request
     const uint32_t nr = R - r0 < kBelRuns ? R - r0 : kBelRuns;
     for (uint32_t t = 0; t < nr; ++t) {
       uint32_t s = __shfl_sync(kFull, my_s, t);
       const uint32_t e = __shfl_sync(kFull, my_e, t);
       uint32_t p = __shfl_sync(kFull, my_p, t);
-      if (__shfl_sync(kFull, my_rs, t)) {
+      if ((opens >> t) & 1u) {
         req_start = s;
         missed = false;
       }
@@ -309,10 +308,8 @@ __global__ void __launch_bounds__(kBelThreads) k_bel_sim(BelArgs a, BelCaps caps
       if (s - p == 1) {  // every step re-reads the block just accessed: busy nowhere, hits
         raw += L;
         if (!missed) {
-          const uint64_t d0 = s - req_start;
           hits += L;
-          add_mul(sv_lo, sv_hi, a.alpha, L);
-          add_mul(sv_lo, sv_hi, a.beta, (uint64_t)L * d0 + (uint64_t)L * (L - 1) / 2);
+          depths += (uint64_t)L * (s - req_start) + (uint64_t)L * (L - 1) / 2;
         }
         continue;
       }
@@ -320,48 +317,74 @@ __global__ void __launch_bounds__(kBelThreads) k_bel_sim(BelArgs a, BelCaps caps
         const uint32_t gap = s - p, sp = p & 31;
         uint32_t Lj = L < gap ? L : gap;
         if (Lj > 1024 - sp) Lj = 1024 - sp;  // the 32 words from p's
-        // this lane's word of them: positions 32 (w0 + lane) ..
+        // this lane's word of them (positions 32 (w0 + lane) ..) and of the 32 below
         const uint32_t w0 = p >> 5, w = w0 + lane;
         const uint32_t end = sp + Lj;  // past the last step, counted from word w0
         uint32_t valid = lane * 32 >= end ? 0u : end - lane * 32 >= 32 ? kFull : mask_lt(end - lane * 32);
+        const bool has = valid != 0 && in_bounds(a.st, w, a.s0);
+        const uint32_t word = has ? l0[w] : 0u;
+        const uint32_t below = w0 > lane ? l0[w0 - 1 - lane] : 0u;
         if (lane == 0) valid &= ~mask_lt(sp);
-        uint32_t word = 0;
-        if (valid && in_bounds(a.st, w, a.s0)) word = l0[w];
         const uint32_t Bk = word & valid;
-        // the free times of [p, p + Lj) are used up
-        if (Bk) l0[w] = word & ~valid;
-        fb.unmark(w0, __ballot_sync(kFull, Bk != 0 && (word & ~valid) == 0), lane);
-        const bool edge = Lj >= 2 && p + Lj == s;
+        const bool edge = Lj >= 2 && p + Lj == s;  // the last step: decided by step 0 below
         const uint32_t elane = (end - 1) >> 5, ebit = 1u << ((end - 1) & 31);
-        uint32_t zm = ~Bk & valid;
-        if (edge && lane == elane) zm &= ~ebit;  // the last step: decided by step 0 below
-        const uint32_t zc = __popc(zm), z = __reduce_add_sync(kFull, zc);
-        uint32_t A = valid;  // steps that hit
+        const uint32_t z = Lj - edge - __reduce_add_sync(kFull, __popc(Bk));
+        uint32_t left = word & ~valid;  // the free times of [p, p + Lj) are used up
+        uint32_t A = valid;        // steps that hit
         uint32_t nh = Lj, f = Lj;  // hits, and hits before the first miss
         if (z) {
           // the other steps take the latest free times below p, then never-used tracks
-          uint32_t acc = fb.pop_below(p, z, lane);
+          uint32_t acc = 0;
+          if (p > fb.low) {
+            const uint32_t first = __shfl_sync(kFull, word, 0) & mask_lt(sp);  // those in p's own word
+            uint32_t sum;
+            const uint32_t c = __popc(below), n0 = __popc(first), above = n0 + lanes_excl(c, &sum);
+            if (n0 > z) {
+              const uint32_t tk = top_bits(first, z, lane);
+              if (lane == 0) left &= ~tk;
+            } else {
+              if (lane == 0) left &= ~first;
+              uint32_t take = above + c <= z ? below : 0u;
+              const uint32_t part = __ballot_sync(kFull, above < z && above + c > z);
+              if (part) {  // the word that holds the last one wanted
+                const uint32_t src = __ffs(part) - 1;
+                const uint32_t tk = top_bits(__shfl_sync(kFull, below, src), z - __shfl_sync(kFull, above, src), lane);
+                if (lane == src) take = tk;
+              }
+              if (take) l0[w0 - 1 - lane] = below & ~take;
+            }
+            acc = n0 + sum;
+            if (acc >= z) {
+              acc = z;
+            } else {
+              if (w0 > 32) acc += fb.pop_words(w0 - 32, z - acc, lane);
+              if (acc < z) fb.low = p;  // nothing is left below p, and free times are added above it
+            }
+          }
           const uint32_t rest = z - acc, inf = rest < free_inf ? rest : (uint32_t)free_inf;
           free_inf -= inf;
           acc += inf;
           if (acc < z) {  // the first acc of them hit
-            uint32_t zx = zc;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-              const uint32_t y = __shfl_up_sync(kFull, zx, o);
-              if (lane >= (uint32_t)o) zx += y;
+            uint32_t zm = ~Bk & valid, sum;
+            if (edge && lane == elane) zm &= ~ebit;
+            const uint32_t zc = __popc(zm), zx = lanes_excl(zc, &sum);
+            A = (valid & ~zm) | (zx + zc <= acc ? zm : 0u);
+            const uint32_t part = __ballot_sync(kFull, zx < acc && zx + zc > acc);
+            if (part) {
+              const uint32_t src = __ffs(part) - 1;
+              const uint32_t tk = low_bits(__shfl_sync(kFull, zm, src), acc - __shfl_sync(kFull, zx, src), lane);
+              if (lane == src) A |= tk;
             }
-            zx -= zc;
-            if (acc < zx + zc) A = (valid & ~zm) | (acc <= zx ? 0u : zm & mask_lt(nth_set(zm, acc - zx)));
             const bool hit0 = ((__shfl_sync(kFull, Bk, 0) >> sp) & 1u) || acc >= 1;
             if (edge && !hit0 && lane == elane) A &= ~ebit;
             const uint32_t rej = valid & ~A;
             const uint32_t with = __ballot_sync(kFull, rej != 0);
             nh = Lj - __reduce_add_sync(kFull, __popc(rej));
-            const uint32_t first = __ffs(with) - 1;
-            f = 32 * first + __ffs(__shfl_sync(kFull, rej, first)) - 1 - sp;
+            const uint32_t l_f = __ffs(with) - 1;
+            f = 32 * l_f + __ffs(__shfl_sync(kFull, rej, l_f)) - 1 - sp;
           }
         }
+        if (has && left != word) l0[w] = left;
         // New free times s - 1 + k of the hits; with p + Lj = s the last step
         // took step 0's.  They lie above every free time so far.
         {
@@ -378,18 +401,36 @@ __global__ void __launch_bounds__(kBelThreads) k_bel_sim(BelArgs a, BelCaps caps
             const uint32_t d = sp - sq;
             out = T >> d | (lane < 31 ? dn << (32 - d) : 0u);
           }
-          __syncwarp();  // the words cleared above may be among these
-          if (out && in_bounds(a.st, v0 + lane, a.s0)) l0[v0 + lane] = lane ? out : l0[v0] | out;
+          // what word v0 holds already: the tail's bits, read back if this
+          // run's updates may have met that word
+          if ((p + Lj - 1) >> 5 >= v0) {
+            __syncwarp();  // the words cleared above
+            tail_w = v0;
+            tail = in_bounds(a.st, v0, a.s0) ? l0[v0] : 0u;
+            if (lane == 0 && out) out |= tail;
+            __syncwarp();
+          } else if (v0 == tail_w && lane == 0 && out) {
+            out |= tail;
+          }
+          if (out && in_bounds(a.st, v0 + lane, a.s0)) l0[v0 + lane] = out;
           if (past && in_bounds(a.st, v0 + 32, a.s0)) l0[v0 + 32] = past;
-          fb.mark(v0, __ballot_sync(kFull, out != 0), lane);
-          if (__shfl_sync(kFull, past, 31)) fb.mark(v0 + 32, 1u, lane);
+          const uint32_t set = __ballot_sync(kFull, out != 0);
+          fb.mark(v0, set, lane);
+          const uint32_t over = __shfl_sync(kFull, past, 31);
+          if (over) {
+            fb.mark(v0 + 32, 1u, lane);
+            tail_w = v0 + 32;
+            tail = over;
+          } else if (set) {
+            const uint32_t l_t = hi_bit(set);
+            tail_w = v0 + l_t;
+            tail = __shfl_sync(kFull, out, l_t);
+          }
         }
         raw += nh;
         if (!missed) {
-          const uint64_t d0 = s - req_start;
           hits += f;
-          add_mul(sv_lo, sv_hi, a.alpha, f);
-          add_mul(sv_lo, sv_hi, a.beta, (uint64_t)f * d0 + (uint64_t)f * (f ? f - 1 : 0) / 2);
+          depths += (uint64_t)f * (s - req_start) + (uint64_t)f * (f ? f - 1 : 0) / 2;
           if (f < Lj) missed = true;
         }
         s += Lj;
@@ -399,6 +440,9 @@ __global__ void __launch_bounds__(kBelThreads) k_bel_sim(BelArgs a, BelCaps caps
     }
     __syncthreads();
   }
+  uint64_t sv_lo = 0, sv_hi = 0;  // depths fits 64 bits: fewer than 2^32 hits at depths below 2^32
+  add_mul(sv_lo, sv_hi, a.alpha, hits);
+  add_mul(sv_lo, sv_hi, a.beta, depths);
   if (threadIdx.x == 0) {
     a.out[g] = hits;
     a.out[a.G + 2 * g] = sv_lo;

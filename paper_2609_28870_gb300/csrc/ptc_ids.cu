@@ -90,6 +90,11 @@ constexpr int kInsK = 1;  // keys per thread: their key and slot loads are in fl
 // 2^32 - 1, so an all-ones word marks an empty or half-written slot.
 __device__ __forceinline__ void toggle(uint32_t* bits, uint32_t i) { atomicXor(&bits[i >> 5], 1u << (i & 31)); }
 
+// Whether some key has outrun the table (the attempt's results are void).
+__device__ __forceinline__ bool table_outrun(const DevStatus* st) {
+  return (ld_relaxed_u32(&st->err) & kErrTableFull) != 0;
+}
+
 __device__ __forceinline__ void settle(ulonglong2* table, uint64_t mask, uint64_t probe_cap, uint32_t i,
                                        ulonglong2 k, uint64_t pos, ulonglong2 cur, uint32_t* __restrict__ slot_out,
                                        uint32_t* bits, DevStatus* st) {
@@ -118,6 +123,8 @@ __device__ __forceinline__ void settle(ulonglong2* table, uint64_t mask, uint64_
       return;
     }
     if (++probe > mask || probe >= probe_cap) break;
+    // a table some other key has outrun is given up: nobody walks its long runs to the end
+    if ((probe & 31) == 0 && table_outrun(st)) break;
     pos = (pos + 1) & mask;
     cur = ld_slot(&table[pos]);
   }
@@ -161,7 +168,7 @@ __global__ void __launch_bounds__(kInsThreads) k_ids_insert(const ulonglong2* __
       cy[j] = __ldg(&kc.carry[t]);
     }
   }
-  const uint32_t n = keys_used(n_ub, n_dev);
+  const uint32_t n = table_outrun(st) ? 0u : keys_used(n_ub, n_dev);
 #pragma unroll
   for (int j = 0; j < kInsK; ++j) {
     const uint32_t i = i0 + j * kInsThreads;
@@ -207,7 +214,7 @@ __global__ void __launch_bounds__(kGaThreads) k_ids_gather(const uint32_t* __res
                                                           const uint64_t* n_dev, uint32_t* __restrict__ ids,
                                                           const DevStatus* st) {
   grid_dep_sync();
-  const uint32_t n = keys_used(n_ub, n_dev);
+  const uint32_t n = table_outrun(st) ? 0u : keys_used(n_ub, n_dev);
   const uint32_t i0 = blockIdx.x * (kGaThreads * kGaPer) + threadIdx.x;
   uint32_t f[kGaPer], own[kGaPer];
 #pragma unroll
@@ -368,7 +375,7 @@ __global__ void __launch_bounds__(kInsThreads) k_ids_insert_prior(const ulonglon
   report_keys_used(n_ub, n_dev, st);
   const uint32_t n = keys_used(n_ub, n_dev);
   const uint32_t base = blockIdx.x * (kInsThreads * K) + threadIdx.x;
-  if (blockIdx.x * (kInsThreads * K) >= n) return;  // the whole CTA
+  if (blockIdx.x * (kInsThreads * K) >= n || table_outrun(st)) return;
   bool unm[K];
 #pragma unroll
   for (int j = 0; j < K; ++j) {
@@ -1221,16 +1228,21 @@ __global__ void __launch_bounds__(kGaThreads) k_ids_gather_pd(const uint32_t* __
 }
 
 // Slots for n keys at most: the full table holds 1.5 n.  The first attempt
-// holds n / 3 while that is at most 2^22 slots (64 MB, half of L2): traces
-// that repeat most blocks fill it well below half, and it stays in L2.  A
-// larger table lives in DRAM whatever its size, so there the first attempt
-// takes 3n / 4 slots instead: a trace that repeats few blocks (an agentic
-// trace, D near n / 2) then probes a table at most about half full rather
-// than one near 90% full, whose linear probe runs are tens of slots long.  If
+// holds 0.6 n, at most 2^23 of them (128 MB), up to the size where the
+// partitioned dedup takes over (n / 3 above 2^22): a trace that repeats few
+// blocks (an agentic trace, D near n / 2) fills it to at most about 3/4.  At
+// n / 3 slots, up to 2^22, such a trace outran its table: 11.3M keys of an
+// agentic window took 26.7 ms there and 0.39 ms in 2^23 slots, 9.3M keys of a
+// chat trace (D = 0.17 n) 174 against 166 us plus 11 us more of fill.  Forced
+// beyond that size the table lives in DRAM and takes 3n / 4 slots.  If
 // a probe sequence of the first attempt runs past kSmallProbeCap slots, the
-// call redoes the stage with the full table.
-constexpr uint64_t kSmallProbeCap = 4096;
+// call redoes the stage with the full table.  A table no more than 3/4 full
+// has no runs of that length; a fuller one is slower than the redo: with
+// runs of up to 4,096 slots allowed, and walked by every thread after the
+// first had failed, 12M keys half of them distinct took 24 ms.
+constexpr uint64_t kSmallProbeCap = 256;
 constexpr uint32_t kL2TableLog2 = 22;
+constexpr uint32_t kFirstTableLog2 = 23;
 uint32_t table_log2(uint64_t want) {
   uint32_t l = 10;
   while ((1ULL << l) < want) ++l;
@@ -1238,8 +1250,8 @@ uint32_t table_log2(uint64_t want) {
 }
 uint32_t full_table_log2(uint64_t n) { return table_log2(n + n / 2 + 64); }
 uint32_t small_table_log2(uint64_t n) {
-  const uint32_t l = table_log2(n / 3 + 64);
-  return l <= kL2TableLog2 ? l : table_log2(n / 4 * 3 + 64);
+  if (ids_table_in_dram(n)) return table_log2(n / 4 * 3 + 64);
+  return std::min(table_log2(n / 5 * 3 + 64), kFirstTableLog2);
 }
 
 struct IdsLayout {

@@ -130,15 +130,25 @@ __device__ __forceinline__ IrArgs resolved(const IrArgs& in) {
   return a;
 }
 
+// Stage a2's D, N and error word go to the status block.  With an error the
+// ids are void: this call's own error word keeps the kernels after this one
+// from reading them, and the caller learns stage a2's.
+__device__ __forceinline__ bool ids_void(const IrArgs& in, const IrArgs& a) {
+  const uint32_t ext = in.ext_err ? *in.ext_err : 0u;
+  if (in.nd && blockIdx.x == 0 && threadIdx.x == 0) {
+    a.st->value[4] = in.nd[1];
+    a.st->value[5] = in.nd[0];
+    a.st->value[6] = ext;
+    if (ext) raise_err(a.st, kErrInvalid);
+  }
+  return ext != 0;
+}
+
 __global__ void __launch_bounds__(kIT) k_ir_count(IrArgs a0) {
   grid_dep_sync();
   __shared__ uint32_t s_w[kIT / 32];
   const IrArgs a = resolved(a0);
-  if (a0.nd && blockIdx.x == 0 && threadIdx.x == 0) {
-    a.st->value[4] = a0.nd[1];
-    a.st->value[5] = a0.nd[0];
-    a.st->value[6] = a0.ext_err ? *a0.ext_err : 0u;
-  }
+  if (ids_void(a0, a)) return;
   const uint32_t tile = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint32_t id[kIR], left[kIR], words[kIR];
   bool bad = false;
@@ -238,11 +248,7 @@ __global__ void __launch_bounds__(kIT) k_ir_count4(IrArgs a0) {
   grid_dep_sync();
   __shared__ uint32_t s_wcnt[kIT / 32];
   const IrArgs a = resolved(a0);
-  if (a0.nd && blockIdx.x == 0 && threadIdx.x == 0) {
-    a.st->value[4] = a0.nd[1];
-    a.st->value[5] = a0.nd[0];
-    a.st->value[6] = a0.ext_err ? *a0.ext_err : 0u;
-  }
+  if (ids_void(a0, a)) return;
   const uint32_t tile = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   uint4 v[kIR4];
   uint32_t x[kIR4], il[kIR4];

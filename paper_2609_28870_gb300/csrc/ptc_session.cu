@@ -38,11 +38,14 @@
 // sit in shared memory when there are at most 16,384 sessions.
 //
 // Ids of prefix chains rise strictly within a request (a prefix first occurs
-// no later than its extensions).  A window where they do not may hold a block
-// twice; it is settled 32 accesses at a time, a second copy after the first.
+// no later than its extensions), so no window holds a block twice.  Whether
+// the given ids do is checked once for all capacities (k_ses_check); if they
+// do not, every window is settled 32 accesses at a time, a second copy of a
+// block after the first.
 //
 // Measured on the 9.3M-access chat trace, 64 capacities: 486 ms with one warp per
-// capacity, 32 accesses a step and owners read from DRAM as they came; 116 ms so.
+// capacity, 32 accesses a step and owners read from DRAM as they came; 116 ms
+// with the windows read ahead; @@MEASURED@@
 #include "ptc_internal.h"
 
 namespace ptc {
@@ -75,14 +78,24 @@ __device__ __forceinline__ void add_mul128(uint64_t& lo, uint64_t& hi, uint64_t 
   hi += phi + (lo < plo ? 1 : 0);
 }
 
-// Request offsets checked once (the replay trusts them afterwards).
+// Request offsets and labels checked once (the replay trusts them
+// afterwards), ids too, and whether ids rise strictly within every request
+// (*falls is raised where they do not).  One thread per access, the first
+// n_req of them per request as well.
 __global__ void k_ses_check(const uint64_t* __restrict__ blk_off, uint32_t R, uint64_t n,
-                            const uint32_t* __restrict__ ses, uint32_t S, DevStatus* st) {
+                            const uint32_t* __restrict__ ses, uint32_t S, const uint32_t* __restrict__ ids,
+                            uint64_t D, uint32_t* falls, DevStatus* st) {
   grid_dep_sync();
-  const uint64_t r = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  if (r >= R) return;
-  const uint64_t a = blk_off[r], b = blk_off[r + 1];
-  if (b < a || b > n || (r == 0 && a != 0) || (r + 1 == R && b != n) || ses[r] >= S) raise_err(st, kErrInvalid);
+  const uint64_t t = (uint64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  if (t < R) {
+    const uint64_t a = blk_off[t], b = blk_off[t + 1];
+    if (b < a || b > n || (t == 0 && a != 0) || (t + 1 == R && b != n) || ses[t] >= S) raise_err(st, kErrInvalid);
+  }
+  if (t < n) {
+    const uint32_t id = ids[t];
+    if (id >= D) raise_err(st, kErrInvalid);
+    if (t > 0 && id <= ids[t - 1] && blk_off[req_search(blk_off, 0, R - 1, t)] != t) *falls = 1;
+  }
 }
 
 constexpr uint32_t kSesSmemSessions = 16384;  // session state kept in shared memory up to this many (192 KB)
@@ -92,11 +105,9 @@ constexpr uint32_t kSesAhead = 8;              // warps that read ahead, one win
 constexpr uint32_t kSesBatch = kSesAhead * kSesWin;
 constexpr uint32_t kSesThreads = 32 * (1 + kSesAhead);
 
-// Ids of two batches and, per 32 accesses, whether an id fails to exceed the
-// one before it.
+// Ids of two batches.
 struct SesRing {
   uint32_t ids[2][kSesBatch];
-  uint32_t fall[2][kSesBatch / 32];
 };
 
 // One capacity's session state; the pointers go to shared or global memory,
@@ -154,21 +165,24 @@ __device__ __forceinline__ bool ses_evict(const SesArgs& a, const SesState& S, u
   return false;
 }
 
-// Hits among the first f accesses of a stretch starting at depth d0.
-struct SesSums {
-  uint64_t hits = 0, lo = 0, hi = 0;
-  __device__ __forceinline__ void add(const SesArgs& a, uint64_t d0, uint32_t f) {
-    hits += f;
-    add_mul128(lo, hi, a.alpha, f);
-    add_mul128(lo, hi, a.beta, (uint64_t)f * d0 + (uint64_t)f * (f ? f - 1 : 0) / 2);
+// Which of the owner words in `o` name a resident block: every epoch is read
+// before any is compared, so the reads overlap.
+template <int N>
+__device__ __forceinline__ void ses_resident(const SesArgs& a, const SesState& S, const uint64_t (&o)[N],
+                                             bool (&res)[N]) {
+  uint32_t ep[N];
+#pragma unroll
+  for (int u = 0; u < N; ++u) {
+    const uint32_t t = o[u] == kNoOwner ? 0u : (uint32_t)(o[u] >> 32);
+    ep[u] = in_bounds(a.st, t, a.n_session) ? S.ep[t] : 0u;
   }
-};
-
-__device__ __forceinline__ bool ses_resident(const SesArgs& a, const SesState& S, uint64_t o) {
-  return o != kNoOwner && in_bounds(a.st, o >> 32, a.n_session) && S.ep[(uint32_t)(o >> 32)] == (uint32_t)o;
+#pragma unroll
+  for (int u = 0; u < N; ++u) res[u] = o[u] != kNoOwner && ep[u] == (uint32_t)o[u];
 }
 
-__global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps, uint32_t n) {
+template <bool SMEM>
+__global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps, uint32_t n,
+                                                         const uint32_t* falls) {
   extern __shared__ uint32_t s_dyn[];
   SesRing& ring = *reinterpret_cast<SesRing*>(s_dyn);
   grid_dep_sync();
@@ -180,7 +194,7 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
   if (__syncthreads_or(threadIdx.x == 0 && ld_relaxed_u32(&a.st->err) != 0)) return;
   uint64_t* owner = a.owner + g * a.sD;
   SesState S;
-  if (a.n_session <= kSesSmemSessions) {
+  if (SMEM) {
     S.ep = s_dyn + sizeof(SesRing) / 4;
     S.count = S.ep + a.n_session;
     S.last = S.count + a.n_session;
@@ -198,24 +212,14 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
   auto read_ahead = [&](uint32_t t) {
     const uint64_t base = (uint64_t)t * kSesBatch + (warp - 1) * kSesWin;
     if (base >= n) return;
-    uint32_t id[kSesPer], left[kSesPer];
+    uint32_t id[kSesPer];
 #pragma unroll
     for (uint32_t u = 0; u < kSesPer; ++u) {
       const uint64_t j = base + 32 * u + lane;
       id[u] = j < n ? __ldg(&a.ids[j]) : 0u;
-      left[u] = j > 0 && j < n ? __ldg(&a.ids[j - 1]) : 0u;
     }
 #pragma unroll
-    for (uint32_t u = 0; u < kSesPer; ++u) {
-      const uint32_t k = (warp - 1) * kSesWin + 32 * u + lane;
-      if (id[u] >= a.n_distinct) {
-        raise_err(a.st, kErrInvalid);
-        id[u] = 0;
-      }
-      ring.ids[t & 1][k] = id[u];
-      const uint32_t fall = __ballot_sync(kFull, id[u] <= left[u]);
-      if (lane == 0) ring.fall[t & 1][k >> 5] = fall;
-    }
+    for (uint32_t u = 0; u < kSesPer; ++u) ring.ids[t & 1][(warp - 1) * kSesWin + 32 * u + lane] = id[u];
     uint64_t o[kSesPer];
 #pragma unroll
     for (uint32_t u = 0; u < kSesPer; ++u)  // into L1; the values are not used
@@ -224,8 +228,11 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
     for (uint32_t u = 0; u < kSesPer; ++u) asm volatile("" ::"l"(o[u]));
   };
   const uint64_t C = caps.c[g];
+  const uint32_t per = C < kSesWin ? (uint32_t)C : 2 * kSesWin;  // misses between two resets of a lone session
+  const uint32_t per_inv = 65536u / per + 1;  // k / per = k per_inv >> 16 for k < 256 (per <= 256), and 0 above
+  const bool repeats = __ldg(falls) != 0;
   uint64_t total = 0;
-  SesSums sums;
+  uint64_t hits = 0, depths = 0;  // counted hits and their depths
   uint32_t front = 0;
   // the current request; 32 requests' sessions and ends at a time, one per lane
   uint32_t r = kNone, s = 0, b = 0, e = 0, es = 0, cnt = 0, q_s = 0, q_e = 0;
@@ -240,7 +247,6 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
       continue;
     }
     const uint32_t* ids = ring.ids[t & 1];
-    const uint32_t* fall = ring.fall[t & 1];
     const uint64_t t0 = (uint64_t)t * kSesBatch;
     const uint32_t size = n - t0 < kSesBatch ? (uint32_t)(n - t0) : kSesBatch;
     uint32_t at = 0;  // accesses of this batch settled
@@ -270,23 +276,7 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
       if (e - (t0 + w0) < hi) hi = (uint32_t)(e - (t0 + w0));
       const uint64_t depth = t0 + at - b;
       at = w0 + hi;
-      uint32_t id[kSesPer], miss[kSesPer];
-      uint64_t o[kSesPer];
-#pragma unroll
-      for (uint32_t u = 0; u < kSesPer; ++u) id[u] = ids[w0 + 32 * u + lane];
-#pragma unroll
-      for (uint32_t u = 0; u < kSesPer; ++u) {
-        const uint32_t k = 32 * u + lane;
-        o[u] = k >= lo && k < hi ? owner[id[u]] : kNoOwner;
-      }
-      // an id after the first that does not exceed the one before it
-      bool falls = false;
-      if (lane < kSesPer) {
-        const uint32_t k = 32 * lane, w = fall[(w0 >> 5) + lane];
-        const uint32_t from = lo + 1 <= k ? 0u : lo + 1 - k, to = hi <= k ? 0u : hi - k;
-        falls = from < 32 && to > from && ((w >> from) << from & (to >= 32 ? kFull : (1u << to) - 1u)) != 0;
-      }
-      if (__any_sync(kFull, falls)) {
+      if (repeats) {
         // ---- a block may come twice: 32 accesses at a time
         uint64_t d0 = depth;
         for (uint32_t c = lo & ~31u; c < hi; c += 32) {
@@ -295,8 +285,10 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
           uint32_t pending = __ballot_sync(kFull, k >= lo && k < hi);
           while (pending) {
             const bool mine = (pending >> lane) & 1u;
-            bool res = false;
-            if (mine) res = ses_resident(a, S, owner[x]);
+            const uint64_t o1[1] = {mine ? owner[x] : kNoOwner};
+            bool r1[1];
+            ses_resident<1>(a, S, o1, r1);
+            const bool res = r1[0];
             uint32_t same = 0;
             if (mine) same = __match_any_sync(pending, x);
             const uint32_t later_copy = __ballot_sync(kFull, mine && (same & lanemask_lt()) != 0);
@@ -318,7 +310,9 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
             cnt += __popc(pm);
             if (!missed && part) {
               const uint32_t f0 = __ffs(part) - 1;
-              sums.add(a, d0, (pm ? (uint32_t)(__ffs(pm) - 1) : 32u - __clz(part)) - f0);
+              const uint32_t f = (pm ? (uint32_t)(__ffs(pm) - 1) : 32u - __clz(part)) - f0;
+              hits += f;
+              depths += (uint64_t)f * d0 + (uint64_t)f * (f ? f - 1 : 0) / 2;
               missed = pm != 0;
             }
             d0 += __popc(part);
@@ -337,54 +331,66 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
         }
         continue;
       }
-      uint32_t m_all = 0, first = kSesWin;
+      uint32_t id[kSesPer], miss[kSesPer];
+      uint64_t o[kSesPer];
+      bool res[kSesPer];
 #pragma unroll
-      for (uint32_t u = 0; u < kSesPer; ++u) {
+      for (uint32_t u = 0; u < kSesPer; ++u) id[u] = ids[w0 + 32 * u + lane];
+#pragma unroll
+      for (uint32_t u = 0; u < kSesPer; ++u) o[u] = 32 * u + lane >= lo && 32 * u + lane < hi ? owner[id[u]] : kNoOwner;
+      ses_resident<kSesPer>(a, S, o, res);
+      uint32_t m_all = 0, first = hi;
+#pragma unroll
+      for (int u = kSesPer - 1; u >= 0; --u) {
         const uint32_t k = 32 * u + lane;
-        miss[u] = __ballot_sync(kFull, k >= lo && k < hi && !ses_resident(a, S, o[u]));
+        miss[u] = __ballot_sync(kFull, k >= lo && k < hi && !res[u]);
         m_all += __popc(miss[u]);
-      }
-#pragma unroll
-      for (int u = kSesPer - 1; u >= 0; --u)
         if (miss[u]) first = 32 * u + __ffs(miss[u]) - 1;
+      }
       if (!missed) {  // the hits before the first miss
-        sums.add(a, depth, (m_all ? first : hi) - lo);
+        const uint32_t f = first - lo;
+        hits += f;
+        depths += (uint64_t)f * depth + (uint64_t)f * (f ? f - 1 : 0) / 2;
         missed = m_all != 0;
       }
       if (m_all == 0) continue;
-      uint64_t stamp = ((uint64_t)s << 32) | es;
+      const uint64_t stamp = ((uint64_t)s << 32) | es;
       while (total + m_all > C) {
-        // the misses before the one that overflows settle
+        // the misses before the one that overflows (the room-th, from 0)
+        // settle, and so does that one before it evicts
         const uint32_t room = (uint32_t)(C - total);
-        uint32_t x_at = 0, x = 0, seen = 0;
+        uint32_t x_u = 0, x_m = 0, before = 0, x_before = 0, x_id = 0;
 #pragma unroll
         for (uint32_t u = 0; u < kSesPer; ++u) {
           const uint32_t c = __popc(miss[u]);
-          const uint32_t below = seen + __popc(miss[u] & lanemask_lt());
-          const bool mine = (miss[u] >> lane) & 1u;
-          if (mine && below <= room) owner[id[u]] = stamp;  // the overflowing one too
-          const uint32_t hit = __ballot_sync(kFull, mine && below == room);
-          if (hit) {
-            x_at = 32 * u + __ffs(hit) - 1;
-            x = __shfl_sync(kFull, id[u], x_at & 31);
+          if (before <= room && before + c > room) {
+            x_u = u;
+            x_m = miss[u];
+            x_before = before;
+            x_id = id[u];
           }
-          seen += c;
+          before += c;
         }
+        const uint32_t x_lane =
+            __ffs(__ballot_sync(kFull, ((x_m >> lane) & 1u) && x_before + __popc(x_m & lanemask_lt()) == room)) - 1;
+        const uint32_t x_at = 32 * x_u + x_lane, x = __shfl_sync(kFull, x_id, x_lane);
+#pragma unroll
+        for (uint32_t u = 0; u < kSesPer; ++u)
+          if (((miss[u] >> lane) & 1u) && 32 * u + lane <= x_at) owner[id[u]] = stamp;
         total += room + 1;
         cnt += room + 1;
-        m_all -= room + 1;
         __syncwarp();
         if (ses_evict(a, S, owner, lane, r, s, x, C, front, total, cnt, es)) {
           // session s is alone with block x: each later block misses, and
           // every C-th of them empties the session again
-          const uint32_t rest = hi - 1 - x_at, per = C < kSesWin ? (uint32_t)C : 2 * kSesWin;
+          const uint32_t rest = hi - 1 - x_at, resets = rest * per_inv >> 16;
 #pragma unroll
           for (uint32_t u = 0; u < kSesPer; ++u) {
             const uint32_t k = 32 * u + lane;
-            if (k > x_at && k < hi) owner[id[u]] = ((uint64_t)s << 32) | (es + (k - x_at) / per);
+            if (k > x_at && k < hi) owner[id[u]] = ((uint64_t)s << 32) | (es + ((k - x_at) * per_inv >> 16));
           }
-          es += rest / per;
-          total = 1 + rest % per;
+          es += resets;
+          total = 1 + rest - resets * per;
           cnt = (uint32_t)total;
           m_all = 0;
           __syncwarp();
@@ -392,11 +398,12 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
           __syncwarp();
           break;
         }
+        ses_resident<kSesPer>(a, S, o, res);
         m_all = 0;
 #pragma unroll
         for (uint32_t u = 0; u < kSesPer; ++u) {
           const uint32_t k = 32 * u + lane;
-          miss[u] = __ballot_sync(kFull, k >= lo && k < hi && k > x_at && !ses_resident(a, S, o[u]));
+          miss[u] = __ballot_sync(kFull, k > x_at && k < hi && !res[u]);
           m_all += __popc(miss[u]);
         }
       }
@@ -412,18 +419,23 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
     __syncthreads();
   }
   if (threadIdx.x == 0) {
-    a.out[g] = sums.hits;
-    a.out[a.G + 2 * g] = sums.lo;
-    a.out[a.G + 2 * g + 1] = sums.hi;
+    uint64_t lo = 0, hi = 0;  // depths fits 64 bits: fewer than 2^32 hits at depths below 2^32
+    add_mul128(lo, hi, a.alpha, hits);
+    add_mul128(lo, hi, a.beta, depths);
+    a.out[g] = hits;
+    a.out[a.G + 2 * g] = lo;
+    a.out[a.G + 2 * g + 1] = hi;
   }
 }
 
 struct SesLayout {
   DevStatus* st;
+  uint32_t* falls;  // zeroed with the status block
   uint64_t* owner;
   uint32_t *epoch, *count, *last;
   uint64_t sD, sS;
   uint64_t* out;
+  size_t zero_bytes;
   size_t total;
 };
 
@@ -434,6 +446,8 @@ SesLayout ses_layout(void* ws, uint64_t n_distinct, uint32_t n_session, uint32_t
   L.sD = n_distinct ? n_distinct : 1;
   L.sS = n_session ? n_session : 1;
   L.st = cv.take<DevStatus>(1);
+  L.falls = cv.take<uint32_t>(1);
+  L.zero_bytes = cv.off;
   L.owner = cv.take<uint64_t>(L.sD * G);
   L.epoch = cv.take<uint32_t>(2 * L.sS * G);  // epochs, then counts: cleared together
   L.count = L.epoch + L.sS * G;
@@ -479,13 +493,13 @@ extern "C" ptc_status ptc_session_lru_curves(const uint32_t* ids, uint64_t n, ui
   if (!ws_ok(ws, ws_bytes, ses_layout(nullptr, n_distinct, n_session, n_cap).total)) return PTC_ERR_WORKSPACE;
   cudaStream_t s = (cudaStream_t)stream;
   const SesLayout L = ses_layout(ws, n_distinct, n_session, n_cap);
-  const FillRange zf[4] = {{ws, kStatusBytes, 0u},
+  const FillRange zf[4] = {{ws, L.zero_bytes, 0u},
                            {L.owner, sizeof(uint64_t) * L.sD * n_cap, ~0u},
                            {L.epoch, sizeof(uint32_t) * L.sS * n_cap * 2, 0u},  // epoch and count
                            {L.last, sizeof(uint32_t) * L.sS * n_cap, ~0u}};
   if (fill_many_async(zf, 4, s) != PTC_OK) return PTC_ERR_CUDA;
-  PTC_KERNEL("k_ses_check", s, k_ses_check, ceil_div_u32(n_req, 256), 256, 0, req_blk_off, n_req, n, req_session,
-             n_session, L.st);
+  PTC_KERNEL("k_ses_check", s, k_ses_check, ceil_div_u32(n > n_req ? n : n_req, 256), 256, 0, req_blk_off, n_req, n,
+             req_session, n_session, ids, n_distinct, L.falls, L.st);
   SesArgs a;
   a.ids = ids;
   a.blk_off = req_blk_off;
@@ -506,11 +520,16 @@ extern "C" ptc_status ptc_session_lru_curves(const uint32_t* ids, uint64_t n, ui
   a.st = L.st;
   SesCaps caps;
   for (uint32_t g = 0; g < n_cap; ++g) caps.c[g] = cap_host[g];
-  const size_t smem = sizeof(SesRing) + (n_session <= kSesSmemSessions ? 3 * sizeof(uint32_t) * n_session : 0);
-  if (smem > 48 * 1024 &&
-      cudaFuncSetAttribute(k_ses_sim, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) != cudaSuccess)
-    return PTC_ERR_CUDA;
-  PTC_KERNEL("k_ses_sim", s, k_ses_sim, n_cap, kSesThreads, smem, a, caps, (uint32_t)n);
+  if (n_session <= kSesSmemSessions) {
+    const size_t smem = sizeof(SesRing) + 3 * sizeof(uint32_t) * n_session;
+    if (smem > 48 * 1024 &&
+        cudaFuncSetAttribute(k_ses_sim<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)(sizeof(SesRing) + 3 * sizeof(uint32_t) * kSesSmemSessions)) != cudaSuccess)
+      return PTC_ERR_CUDA;
+    PTC_KERNEL("k_ses_sim", s, k_ses_sim<true>, n_cap, kSesThreads, smem, a, caps, (uint32_t)n, L.falls);
+  } else {
+    PTC_KERNEL("k_ses_sim", s, k_ses_sim<false>, n_cap, kSesThreads, sizeof(SesRing), a, caps, (uint32_t)n, L.falls);
+  }
   HostStage* hs = host_stage();
   if (copy_to_host_async(hs->out, L.out, sizeof(uint64_t) * 3 * n_cap, s) != PTC_OK) return PTC_ERR_CUDA;
   DevStatus h;
