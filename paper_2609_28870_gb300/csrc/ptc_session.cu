@@ -31,11 +31,11 @@
 // registers, since an eviction can drop a later block of the window.  Once
 // the current session is alone and above C, every later block of the window
 // misses, and they settle in closed form.  Eight other warps read ahead: the
-// ids of the next 2,048 accesses into shared memory, and the owner words of
+// ids of the next 4,096 accesses into shared memory, and the owner words of
 // those ids into L1, so that the replayer's owner reads hit L1 (its own
 // stores go through the same L1) instead of waiting for DRAM: the owner table
 // takes 8 bytes per block and capacity.  Epochs, counts and latest requests
-// sit in shared memory when there are at most 16,384 sessions.
+// sit in shared memory when there are at most 14,336 sessions.
 //
 // Ids of prefix chains rise strictly within a request (a prefix first occurs
 // no later than its extensions), so no window holds a block twice.  Whether
@@ -45,7 +45,9 @@
 //
 // Measured on the 9.3M-access chat trace, 64 capacities: 486 ms with one warp per
 // capacity, 32 accesses a step and owners read from DRAM as they came; 116 ms
-// with the windows read ahead; @@MEASURED@@
+// with the windows read ahead; 55 ms with epochs read together, the check for
+// repeats made once and 4,096 accesses read ahead at a time (33 ms at the
+// largest capacity, 55 at the smallest, which evicts in every window).
 #include "ptc_internal.h"
 
 namespace ptc {
@@ -98,16 +100,17 @@ __global__ void k_ses_check(const uint64_t* __restrict__ blk_off, uint32_t R, ui
   }
 }
 
-constexpr uint32_t kSesSmemSessions = 16384;  // session state kept in shared memory up to this many (192 KB)
+constexpr uint32_t kSesSmemSessions = 14336;  // session state kept in shared memory up to this many
 constexpr uint32_t kSesPer = 8;                // accesses per lane and window
 constexpr uint32_t kSesWin = 32 * kSesPer;
-constexpr uint32_t kSesAhead = 8;              // warps that read ahead, one window each
-constexpr uint32_t kSesBatch = kSesAhead * kSesWin;
+constexpr uint32_t kSesAhead = 8;              // warps that read ahead
+constexpr uint32_t kSesAheadPer = 16;          // accesses per lane that a batch reads ahead
+constexpr uint32_t kSesBatch = kSesAhead * 32 * kSesAheadPer;  // 4,096 accesses
 constexpr uint32_t kSesThreads = 32 * (1 + kSesAhead);
 
-// Ids of two batches.
+// Ids of the batch being replayed and the two after it.
 struct SesRing {
-  uint32_t ids[2][kSesBatch];
+  uint32_t ids[3][kSesBatch];
 };
 
 // One capacity's session state; the pointers go to shared or global memory,
@@ -181,7 +184,7 @@ __device__ __forceinline__ void ses_resident(const SesArgs& a, const SesState& S
 }
 
 template <bool SMEM>
-__global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps, uint32_t n,
+__global__ void __launch_bounds__(kSesThreads, 1) k_ses_sim(SesArgs a, SesCaps caps, uint32_t n,
                                                          const uint32_t* falls) {
   extern __shared__ uint32_t s_dyn[];
   SesRing& ring = *reinterpret_cast<SesRing*>(s_dyn);
@@ -208,24 +211,30 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
     S.count = a.count + g * a.sS;
     S.last = a.last + g * a.sS;
   }
-  // Batch `t` of the read-ahead warps: window `warp - 1` of it into the ring.
-  auto read_ahead = [&](uint32_t t) {
-    const uint64_t base = (uint64_t)t * kSesBatch + (warp - 1) * kSesWin;
-    if (base >= n) return;
-    uint32_t id[kSesPer];
+  // The read-ahead warps' share of a batch: the owner words of batch t_owner
+  // into L1 and the ids of batch t_ids into the ring, all loads in flight
+  // together and once per batch: L1 answers in order, so the replayer's hits
+  // wait while any of these misses is outstanding.
+  auto read_ahead = [&](uint32_t t_owner, uint32_t t_ids) {
+    const uint32_t k0 = (warp - 1) * 32 * kSesAheadPer + lane;
+    const uint64_t owners = (uint64_t)t_owner * kSesBatch, next = (uint64_t)t_ids * kSesBatch;
+    uint32_t id[kSesAheadPer], o[kSesAheadPer];
 #pragma unroll
-    for (uint32_t u = 0; u < kSesPer; ++u) {
-      const uint64_t j = base + 32 * u + lane;
-      id[u] = j < n ? __ldg(&a.ids[j]) : 0u;
+    for (uint32_t u = 0; u < kSesAheadPer; ++u) {
+      const uint32_t k = k0 + 32 * u;
+      id[u] = next + k < n ? __ldg(&a.ids[next + k]) : 0u;
     }
 #pragma unroll
-    for (uint32_t u = 0; u < kSesPer; ++u) ring.ids[t & 1][(warp - 1) * kSesWin + 32 * u + lane] = id[u];
-    uint64_t o[kSesPer];
+    for (uint32_t u = 0; u < kSesAheadPer; ++u) {  // the values are not used
+      const uint32_t k = k0 + 32 * u;
+      o[u] = 0;
+      if (t_owner != kNone && owners + k < n)
+        asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(o[u]) : "l"(owner + ring.ids[t_owner % 3][k]));
+    }
 #pragma unroll
-    for (uint32_t u = 0; u < kSesPer; ++u)  // into L1; the values are not used
-      asm volatile("ld.global.ca.u64 %0, [%1];" : "=l"(o[u]) : "l"(owner + id[u]));
+    for (uint32_t u = 0; u < kSesAheadPer; ++u) ring.ids[t_ids % 3][k0 + 32 * u] = id[u];
 #pragma unroll
-    for (uint32_t u = 0; u < kSesPer; ++u) asm volatile("" ::"l"(o[u]));
+    for (uint32_t u = 0; u < kSesAheadPer; ++u) asm volatile("" ::"r"(o[u]));
   };
   const uint64_t C = caps.c[g];
   const uint32_t per = C < kSesWin ? (uint32_t)C : 2 * kSesWin;  // misses between two resets of a lone session
@@ -238,15 +247,17 @@ __global__ void __launch_bounds__(kSesThreads) k_ses_sim(SesArgs a, SesCaps caps
   uint32_t r = kNone, s = 0, b = 0, e = 0, es = 0, cnt = 0, q_s = 0, q_e = 0;
   bool missed = false;
   const uint32_t batches = (uint32_t)(((uint64_t)n + kSesBatch - 1) / kSesBatch);
-  if (warp) read_ahead(0);
+  if (warp) read_ahead(kNone, 0);
+  __syncthreads();
+  if (warp) read_ahead(0, 1);
   __syncthreads();
   for (uint32_t t = 0; t < batches; ++t) {
     if (warp) {
-      if (t + 1 < batches) read_ahead(t + 1);
+      if (t + 1 < batches) read_ahead(t + 1, t + 2);
       __syncthreads();
       continue;
     }
-    const uint32_t* ids = ring.ids[t & 1];
+    const uint32_t* ids = ring.ids[t % 3];
     const uint64_t t0 = (uint64_t)t * kSesBatch;
     const uint32_t size = n - t0 < kSesBatch ? (uint32_t)(n - t0) : kSesBatch;
     uint32_t at = 0;  // accesses of this batch settled
@@ -526,7 +537,11 @@ extern "C" ptc_status ptc_session_lru_curves(const uint32_t* ids, uint64_t n, ui
         cudaFuncSetAttribute(k_ses_sim<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                              (int)(sizeof(SesRing) + 3 * sizeof(uint32_t) * kSesSmemSessions)) != cudaSuccess)
       return PTC_ERR_CUDA;
-    PTC_KERNEL("k_ses_sim", s, k_ses_sim<true>, n_cap, kSesThreads, smem, a, caps, (uint32_t)n, L.falls);
+    if (n_cap <= (uint32_t)num_sms())
+      PTC_LAUNCH("k_ses_sim", s,
+                 launch_l1(k_ses_sim<true>, n_cap, kSesThreads, smem, s, a, caps, (uint32_t)n, L.falls));
+    else
+      PTC_KERNEL("k_ses_sim", s, k_ses_sim<true>, n_cap, kSesThreads, smem, a, caps, (uint32_t)n, L.falls);
   } else {
     PTC_KERNEL("k_ses_sim", s, k_ses_sim<false>, n_cap, kSesThreads, sizeof(SesRing), a, caps, (uint32_t)n, L.falls);
   }
