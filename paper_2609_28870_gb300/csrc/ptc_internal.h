@@ -46,6 +46,28 @@ inline void launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t s
   (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
 }
 
+// launch_pdl for a kernel whose CTAs each have an SM to themselves and live on
+// L1 hits: asks for no more of the SM's 256 KB as shared memory than `smem`
+// takes (by default the split favours more resident CTAs and leaves as little
+// as 28 KB of L1).  A hint of this launch only.
+template <typename... KArgs, typename... Args>
+inline void launch_l1(void (*kernel)(KArgs...), dim3 grid, dim3 block, size_t smem, cudaStream_t s, Args&&... args) {
+  cudaLaunchAttribute attr[2];
+  attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[0].val.programmaticStreamSerializationAllowed = 1;
+  attr[1].id = cudaLaunchAttributePreferredSharedMemoryCarveout;
+  const size_t pct = (smem + 2048) * 100 / (228 * 1024) + 1;  // 1 KB of each CTA is the system's
+  attr[1].val.sharedMemCarveout = (unsigned)(pct < 100 ? pct : 100);
+  cudaLaunchConfig_t cfg = {};
+  cfg.gridDim = grid;
+  cfg.blockDim = block;
+  cfg.dynamicSmemBytes = smem;
+  cfg.stream = s;
+  cfg.attrs = attr;
+  cfg.numAttrs = 2;
+  (void)cudaLaunchKernelEx(&cfg, kernel, std::forward<Args>(args)...);
+}
+
 // PTC_KERNEL(name, stream, kernel, grid, block, smem, args...): a counted
 // (and, while timing, bracketed) launch_pdl.  A template kernel whose
 // arguments hold a comma goes in parentheses.
