@@ -286,6 +286,14 @@ size_t stack_distance_points_bytes(uint64_t n);
 ptc_status stack_distance_points(const uint32_t* prev, uint64_t n, uint32_t* dist_out, void* ws, size_t ws_bytes,
                                  cudaStream_t s, const uint32_t* wend = nullptr);
 
+// Stage c by counting (ptc_count.cu), for traces without runs of up to 33.5M
+// accesses.  *counted is false if prev takes a value twice (nothing is written
+// then); the bytes are 0 for an n it does not take.
+bool stack_distance_countable(uint64_t n);
+size_t stack_distance_count_bytes(uint64_t n);
+ptc_status stack_distance_count(const uint32_t* prev, uint64_t n, uint32_t* dist_out, void* ws, size_t ws_bytes,
+                                cudaStream_t s, bool* counted);
+
 // Stage b by a radix sort of every access (ptc_sort.cu), and the same sort
 // for any (key, value) pairs; the C entry point in ptc_reuse.cu chooses.
 size_t reuse_by_sort_bytes(uint64_t n);

@@ -81,6 +81,7 @@ struct MarkArgs {
   uint32_t* tpre;     // runs starting before each tile; tpre[ntiles] = R
   uint32_t* done;
   uint32_t* kbits;    // bitmap of the runs' keys (largest values) over [0, n]
+  uint32_t max_runs;  // with more runs than this the matrix over runs is not built: nothing is marked
   DevStatus* st;      // value[1] <- R
 };
 
@@ -149,6 +150,7 @@ __global__ void __launch_bounds__(kMT) k_runs_count(MarkArgs a) {
 // Pass 2: bitmap, run index per word, and the (start, first value) records.
 __global__ void __launch_bounds__(kMT) k_runs_mark(MarkArgs a) {
   grid_dep_sync();
+  if (a.st->value[1] > a.max_runs) return;
   __shared__ uint32_t s_wcnt[kMT / 32];
   const uint32_t tile = blockIdx.x;
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -268,6 +270,7 @@ __global__ void __launch_bounds__(kMT) k_runs_count4(MarkArgs a) {
 
 __global__ void __launch_bounds__(kMT) k_runs_mark4(MarkArgs a) {
   grid_dep_sync();
+  if (a.st->value[1] > a.max_runs) return;
   __shared__ uint32_t s_wcnt[kMT / 32];
   const uint32_t tile = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t base = tile * kMTile + w * (32 * kMR);
@@ -864,6 +867,7 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
   m.tpre = M.tpre;
   m.done = &M.done[63];
   m.kbits = M.kbits;
+  m.max_runs = method == PTC_SD_AUTO ? (uint32_t)(n / 3) : (uint32_t)n;
   m.st = M.st;
   if ((reinterpret_cast<uintptr_t>(prev) & 15) == 0) {
     PTC_KERNEL("k_runs_count", s, k_runs_count4, M.mtiles, kMT, 0, m);
@@ -879,7 +883,16 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
   const uint64_t R = h.value[1];
   const RunsLayout W = runs_layout(ws, n, R);
   const bool fits = R >= 1 && R <= n && ws_bytes >= W.total;
-  if (method == PTC_SD_AUTO && (!fits || R > n / 3)) return stack_distance_points(prev, n, dist_out, ws, ws_bytes, s);
+  if (method == PTC_SD_AUTO && (!fits || R > n / 3)) {
+    // no runs to speak of: by counting, or on the matrix over every access
+    // (more accesses than the count takes, or a prev that repeats values)
+    if (stack_distance_countable(n) && ws_bytes >= stack_distance_count_bytes(n)) {
+      bool counted = false;
+      rc = stack_distance_count(prev, n, dist_out, ws, ws_bytes, s, &counted);
+      if (counted) return rc;
+    }
+    return stack_distance_points(prev, n, dist_out, ws, ws_bytes, s);
+  }
   if (!fits) return PTC_ERR_WORKSPACE;
   const FillRange zf[2] = {{W.acc, W.acc_bytes, 0u}, {W.done, 64 * sizeof(uint32_t), 0u}};
   if (fill_many_async(zf, 2, s) != PTC_OK) return PTC_ERR_CUDA;
@@ -997,8 +1010,9 @@ extern "C" size_t ptc_stack_distance_ex_workspace_bytes(uint64_t n, int method) 
   const size_t pts = stack_distance_points_bytes(n);
   if (method == PTC_SD_POINTS) return pts;
   if (method == PTC_SD_RUNS) return runs_layout(nullptr, n, n).total;
-  const size_t runs = runs_layout(nullptr, n, runs_reserve(n)).total;
-  return pts > runs ? pts : runs;
+  const size_t runs = runs_layout(nullptr, n, runs_reserve(n)).total, count = stack_distance_count_bytes(n);
+  const size_t most = pts > runs ? pts : runs;
+  return most > count ? most : count;
 }
 
 extern "C" size_t ptc_stack_distance_workspace_bytes(uint64_t n) {
