@@ -168,8 +168,8 @@ def kernel_model_bytes(name, T, N, L, D, U=None):
     }
     return {
         "k_hash_local": 4 * T + 16 * N,   # token stream in, block keys out
-        "k_hash16": 4 * T + 16 * N,       # the same, B = 16 path
-        "k_hash_tile": 4 * T + 16 * N,    # the same, other multiples of 16
+        "k_hash_units": 4 * T + 16 * N,   # the same, B a multiple of 16, 12 or 8
+        "k_hash16": 4 * T + 16 * N,       # the same, B = 16 path of an earlier build
         "k_ids_insert": 16 * N,           # keys in
         "k_ids_insert_prior": 16 * N,     # keys in (the same stage, prior-request hint)
         "k_ids_gather": 4 * N,            # ids out
@@ -187,7 +187,7 @@ def kernel_model_bytes(name, T, N, L, D, U=None):
 
 KERNEL_SOURCE = {
     "k_block_offsets": "ptc_hash.cu", "k_pow_tables": "ptc_hash.cu", "k_hash_local": "ptc_hash.cu",
-    "k_hash16": "ptc_hash.cu", "k_hash_tile": "ptc_hash.cu", "k_fill_many": "ptc_abi.cu",
+    "k_hash16": "ptc_hash.cu", "k_hash_units": "ptc_hash.cu", "k_fill_many": "ptc_abi.cu",
     "k_hash_chain": "ptc_hash.cu", "k_ids_insert": "ptc_ids.cu",
     "k_ids_gather": "ptc_ids.cu", "k_ids_insert_prior": "ptc_ids.cu", "k_ids_follow": "ptc_ids.cu",
     "k_tile_req": "ptc_ids.cu", "k_ids_lam": "ptc_ids.cu", "k_session_prior": "ptc_ids.cu", "k_sort_count": "ptc_sort.cu", "k_sort_rowscan": "ptc_sort.cu",

@@ -16,12 +16,11 @@
 //                    validates offsets and timestamp order, max blocks/request
 //   k_pow_tables     u^(B e) for e < 2^32 as two 65,536-entry levels
 //                    (filled up to the longest request)
-//   k_hash16         B = 16, aligned tokens: the tile's request offsets in
-//                    shared memory, one block per thread
-//   k_hash_tile      B any multiple of 16, aligned tokens: one block per
-//                    thread, its 16-token chunks hashed one after another
-//                    with two-limb products, 256-block tiles whatever B
-//   k_hash_local     any other B or tokens not 16-byte aligned: tokens
+//   k_hash_units     B a multiple of 16, 12 or 8: a unit of U = 16, 12 or 8
+//                    tokens per lane, 32 units at a time, then prefix sums over
+//                    the 256 units of a warp's tile, eight units per lane
+//   k_hash_units_wide  the tiles with a token of 2^27 or more
+//   k_hash_local     any other B: tokens
 //                    staged through padded shared memory with 16-byte
 //                    loads; each thread hashes 16 tokens (one "sub-chunk")
 //                    with 3 x 21-bit limbs of u^1..u^16 held as constant
@@ -46,7 +45,7 @@ constexpr int kWinTokens = 8192 + 256;
 constexpr int kWinWords = kWinTokens + kWinTokens / 16;
 
 constexpr int kEpochOffsets = 1;
-constexpr int kEpochWide = 2;  // st->tile_ctr slot counting the tiles of k_hash16_wide
+constexpr int kEpochWide = 2;  // st->tile_ctr slot counting the tiles of k_hash_units_wide
 
 // ---------------------------------------------------------------- block scans
 // Exclusive sum over a CTA of kOffThreads threads; returns the CTA total in *total.
@@ -139,16 +138,17 @@ __global__ void __launch_bounds__(kOffThreads) k_block_offsets(const uint64_t* _
 }
 
 // ---------------------------------------------------------------- powers
-// tables[(b*2 + w) * 65536 + e] for base b in {0,1} and
-//   w = 0: u_b^(B e)          w = 1: u_b^(B 65536 e)
+// tables[(b*2 + w) * 65536 + e] for base b in {0,1} and U tokens per unit
+// (k_hash_local: a unit is a block)
+//   w = 0: u_b^(U e)          w = 1: u_b^(U 65536 e)
 constexpr int kPowChunk = 8;  // powers per thread: short dependent chains
 
 struct PowBases {
   uint64_t base[4];
 };
 
-// Only the entries some block can use are filled: exponents e = k reach at
-// most the longest request's block count minus one (st->value[1]).
+// Only the entries some unit can use are filled: exponents reach at most the
+// longest request's units (st->value[1] blocks of g units).
 // Blocks the key kernels may touch: N as the offsets kernel left it, or none
 // if its look-back gave up (then the offsets are not a prefix sum and must
 // not steer any read; the call reports PTC_ERR_TIMEOUT).
@@ -158,12 +158,12 @@ __device__ __forceinline__ uint64_t blocks_live(const DevStatus* st, uint64_t ke
   return N < keys_cap ? N : keys_cap;
 }
 
-__global__ void k_pow_tables(PowBases pb, uint64_t* __restrict__ tables, const DevStatus* st) {
+__global__ void k_pow_tables(PowBases pb, uint64_t* __restrict__ tables, uint32_t g, const DevStatus* st) {
   grid_dep_sync();
   const uint32_t gid = blockIdx.x * blockDim.x + threadIdx.x;  // 4 tables x 8192 chunks of kPowChunk
   const uint32_t t = gid >> 13, chunk = gid & 8191;
   if (t >= 4) return;
-  const uint64_t kmax = st->value[1];
+  const uint64_t kmax = st->value[1] * g;
   const uint64_t need = (t & 1) ? (kmax >> 16) : (kmax < 65535 ? kmax : 65535);
   const uint64_t base = pb.base[t];
   const uint64_t e0 = (uint64_t)chunk * kPowChunk;
@@ -221,7 +221,8 @@ struct HashArgs {
   uint32_t* tile_lead;   // per tile: blocks before its first request start (keys left normalised)
   DevStatus* st;
   int aligned;
-  uint32_t* wide_list;  // k_hash16: tiles left to k_hash16_wide (their count in st->tile_ctr[kEpochWide])
+  uint32_t* wide_list;  // k_hash_units: tiles left to k_hash_units_wide (their count in st->tile_ctr[kEpochWide])
+  uint32_t g, tb;       // k_hash_units: units per block, blocks per tile
 };
 
 __device__ __forceinline__ uint32_t pad16(uint32_t i) { return i + (i >> 4); }
@@ -232,13 +233,13 @@ __device__ __forceinline__ uint64_t mad_wide(uint32_t a, uint32_t b, uint64_t c)
   return (uint64_t)a * (uint64_t)b + c;
 }
 
-// Sum over the 16 words t[m .. m+15] of t * u^(j + 1) for both bases, as
-// 21-bit limb accumulators (M is the word offset of the first token).
-template <int M, int NW>
-__device__ __forceinline__ void hash16(const uint32_t (&wd)[NW], const HashConsts& c, uint64_t (&acc)[6]) {
-  static_assert(M + 16 <= NW, "chunk words out of range");
+// Sum over the U words wd[M ..] of wd[M + j] u^(j + 1) for both bases, as
+// 21-bit limb accumulators.
+template <int U, int M, int NW>
+__device__ __forceinline__ void unit_sum_3(const uint32_t (&wd)[NW], const HashConsts& c, uint64_t (&acc)[6]) {
+  static_assert(M + U <= NW, "unit words out of range");
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
+  for (int j = 0; j < U; ++j) {
     const uint32_t t = wd[j + M];
     acc[0] = mad_wide(t, c.limb[0][0][j], acc[0]);
     acc[1] = mad_wide(t, c.limb[0][1][j], acc[1]);
@@ -251,11 +252,11 @@ __device__ __forceinline__ void hash16(const uint32_t (&wd)[NW], const HashConst
 
 // The same sum with two limbs (31 + 30 bits), exact when every token is
 // below 2^27: 16 products of at most 2^58 stay below 2^62.
-template <int M, int NW>
-__device__ __forceinline__ void hash16_2(const uint32_t (&wd)[NW], const HashConsts& c, uint64_t (&acc)[4]) {
-  static_assert(M + 16 <= NW, "chunk words out of range");
+template <int U, int M, int NW>
+__device__ __forceinline__ void unit_sum_2(const uint32_t (&wd)[NW], const HashConsts& c, uint64_t (&acc)[4]) {
+  static_assert(M + U <= NW, "unit words out of range");
 #pragma unroll
-  for (int j = 0; j < 16; ++j) {
+  for (int j = 0; j < U; ++j) {
     const uint32_t t = wd[j + M];
     acc[0] = mad_wide(t, c.limb2[0][0][j], acc[0]);
     acc[1] = mad_wide(t, c.limb2[0][1][j], acc[1]);
@@ -488,533 +489,298 @@ __global__ void __launch_bounds__(kHashThreads) k_hash_local(HashArgs a, const _
   hash_finish<G>(a, tile, b0, b_end, h0, h1, k, lb, s);
 }
 
-// B = 16 with 16-byte-aligned tokens: one block per thread, kHashThreads =
-// 256 blocks per tile (as k_hash_local with G = 1), eight CTAs per SM (32
-// registers; a few values spill to L1, which measured faster than six CTAs
-// at 40 registers), so that a CTA waiting at one of its barriers leaves seven
-// others to issue.  The requests that meet the tile are
-// tile_req[tile] .. tile_req[tile + 1]; their block and token offsets are
-// loaded into shared memory once, so a thread finds its request without a
-// dependent chain of global loads, and its token loads and power-table loads
-// all go out together.  Tiles meeting more than kH16Req requests search the
-// global offsets instead.
-constexpr int kH16Req = 256;
+// B = g U with U = 16, 12 or 8 tokens per unit, tokens at any 4-byte
+// alignment.  With units numbered through a request (unit e of it covers its
+// tokens [U e, U e + U)) the key of a block is the sum over the units up to
+// its last one of h_e u^(U e), so units are hashed and summed alike and only
+// every g-th sum is written.
+//
+// One warp per tile of tb blocks (tb g <= 256 units, tb a power of two), no
+// CTA barrier anywhere:
+//   units   32 at a time, one per lane: its 16-byte loads (a unit that does
+//           not start on a 16-byte boundary takes its last words from the next
+//           lane), the limb products, one multiplication by u^(U e); the
+//           result to shared memory
+//   sums    eight consecutive units per lane: a serial sum that starts anew
+//           where a request starts, one segmented scan over the lanes for the
+//           256 units, and the canonical residues back to shared memory
+//   store   the block ends, coalesced
+// What bounds it: integer issue, then DRAM.  The form before this one gave
+// each of 256 threads one block and ran a warp scan, a scan over the warps and
+// the exchange of request starts for every block, with four CTA barriers: 562
+// instructions a block, of which the products are 64.
+// Measured (keys and tokens over the time; the form before in brackets): 844
+// us or 4.5 TB/s on 763M tokens of the agentic trace [3.7 TB/s on the whole
+// one], 186 us on the chat trace [214], 776 us on 724M tokens in blocks of 64
+// that start at an odd word [1,675], 87 us on 55M tokens in blocks of 24 [223].
+// At 64 registers 32 warps an SM are half the latency hiding the loads want;
+// five or six CTAs' worth of warps with spills took 7 and 30% longer, and a
+// separate path for tiles inside one request (a quarter fewer instructions,
+// the next round's tokens loaded ahead) took as long on the agentic trace and a
+// third longer on the chat trace, where both paths' code competes for the
+// instruction cache.
+constexpr uint32_t kUnitTile = 256;                            // units per tile at most
+constexpr uint32_t kUnitWarps = 2;  // per CTA: small, so that few tiles still spread over the SMs
+constexpr uint32_t kUnitThreads = 32 * kUnitWarps;
+constexpr uint32_t kUnitSlots = kUnitTile + kUnitTile / 8;     // one slot of padding per lane's eight
+__device__ __forceinline__ uint32_t unit_slot(uint32_t v) { return v + (v >> 3); }
 
-// One tile of k_hash16.  WIDE = false: two-limb products, exact while every
-// token is below 2^27 (any vocabulary in use); a tile that holds a larger
-// token is left to k_hash16_wide (its index goes to wide_list) and returns
-// before it writes anything.  WIDE = true: three-limb products, exact for
-// every 32-bit token.  Keeping the three-limb code out of the common kernel
-// keeps that kernel's registers free of it (with it the kernel spilled more
-// and took 0.7 ms longer on the mixed 10B-token trace).
-template <bool WIDE>
-__device__ __forceinline__ void hash16_tile(const HashArgs& a, const HashConsts& c, uint32_t tile, uint64_t N) {
-  __shared__ uint64_t s_boff[kH16Req + 1];
-  __shared__ uint64_t s_toff[kH16Req + 1];
-  __shared__ uint32_t s_big;  // some block of the tile needs three limbs
-  constexpr uint32_t TB = kHashThreads;
-  const uint64_t b0 = (uint64_t)tile * TB;
+// x mod p for any 64-bit x.
+__device__ __forceinline__ uint64_t p61_canon(uint64_t x) {
+  const uint64_t y = (x & kP61) + (x >> 61);  // at most p + 7
+  return y >= kP61 ? y - kP61 : y;
+}
+__device__ __forceinline__ uint64_t p61_part(uint64_t x) { return (x & kP61) + (x >> 61); }
+
+// h of a unit whose first token is word M of wd: below 2^62 + 3.
+template <int U, int M, bool WIDE, int NW>
+__device__ __forceinline__ void unit_hash(const uint32_t (&wd)[NW], const HashConsts& c, uint64_t& h0, uint64_t& h1) {
+  if (WIDE) {
+    uint64_t acc[6] = {0, 0, 0, 0, 0, 0};
+    unit_sum_3<U, M>(wd, c, acc);
+    h0 = p61_add(limbs_to_p61(acc[0], acc[1], acc[2]), c.csum[0][U]);
+    h1 = p61_add(limbs_to_p61(acc[3], acc[4], acc[5]), c.csum[1][U]);
+  } else {
+    uint64_t acc[4] = {0, 0, 0, 0};
+    unit_sum_2<U, M>(wd, c, acc);
+    h0 = limbs2_lazy(acc[0], acc[1]) + c.csum[0][U];
+    h1 = limbs2_lazy(acc[2], acc[3]) + c.csum[1][U];
+  }
+}
+
+__device__ __forceinline__ int64_t shfl_i64(int64_t v, uint32_t src) {
+  return (int64_t)__shfl_sync(kFull, (unsigned long long)v, src);
+}
+
+// The sums of a tile: slot[v] (units' values below 2^61 + 8) becomes the
+// canonical sum of the values since the last request start.  `mine` are the
+// starts among this lane's eight units, `opens` the lanes that have one.
+__device__ __forceinline__ void unit_sums(ulonglong2* slot, uint32_t lane, uint32_t mine, uint32_t opens, bool in) {
+  uint64_t p0[8], p1[8];
+  uint64_t s0 = 0, s1 = 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    const ulonglong2 t = in ? slot[9 * lane + j] : make_ulonglong2(0, 0);
+    if ((mine >> j) & 1u) s0 = s1 = 0;
+    s0 += t.x;
+    s1 += t.y;
+    p0[j] = s0;  // below 5 2^61 + 64
+    p1[j] = s1;
+    if (j == 3) {
+      s0 = p61_part(s0);
+      s1 = p61_part(s1);
+    }
+  }
+  s0 = p61_part(s0);
+  s1 = p61_part(s1);
+  // segmented scan over the lanes; from values below 2^61 + 8 two plain steps
+  // stay below 2^63 + 32, so a fold every other step keeps sums below 2^64
+  const uint32_t upto = opens & (lanemask_lt() | (1u << lane));
+  const uint32_t seg = upto ? 31u - __clz(upto) : 0u;  // the sum reaches back to this lane
+#pragma unroll
+  for (int d = 1; d < 32; d <<= 1) {
+    const uint64_t y0 = __shfl_up_sync(kFull, s0, d), y1 = __shfl_up_sync(kFull, s1, d);
+    if (lane >= seg + (uint32_t)d) {
+      s0 += y0;
+      s1 += y1;
+    }
+    if (d == 2 || d == 8) {
+      s0 = p61_part(s0);
+      s1 = p61_part(s1);
+    }
+  }
+  uint64_t c0 = __shfl_up_sync(kFull, s0, 1), c1 = __shfl_up_sync(kFull, s1, 1);
+  c0 = lane ? p61_part(c0) : 0;
+  c1 = lane ? p61_part(c1) : 0;
+#pragma unroll
+  for (int j = 0; j < 8; ++j) {
+    if ((mine >> j) & 1u) c0 = c1 = 0;  // the carry ends at the lane's first start
+    if (in) slot[9 * lane + j] = make_ulonglong2(p61_canon(p0[j] + c0), p61_canon(p1[j] + c1));
+  }
+}
+
+// One tile, by one warp.  WIDE = false: two-limb products, exact while every
+// token is below 2^27 (any vocabulary in use); a tile that holds a larger one
+// writes nothing and is left to k_hash_units_wide.  WIDE = true: three-limb
+// products, exact for every 32-bit token.
+template <int U, bool WIDE>
+__device__ __forceinline__ void hash_units_tile(const HashArgs& a, const HashConsts& c, uint32_t tile, uint64_t N,
+                                                ulonglong2* slot, uint32_t* starts) {
+  constexpr int NV = U / 4;
+  const uint32_t lane = threadIdx.x & 31;
+  const uint64_t b0 = (uint64_t)tile * a.tb;
   if (b0 >= N) return;
-  const uint64_t b_end = b0 + TB < N ? b0 + TB : N;
-  const uint64_t ntiles = (N + TB - 1) / TB;
+  const uint32_t nb = N - b0 < a.tb ? (uint32_t)(N - b0) : a.tb, nu = nb * a.g;
+  const uint64_t ntiles = (N + a.tb - 1) / a.tb;
   const uint32_t r_first = a.tile_req[tile];
   const uint32_t r_last = tile + 1 < ntiles ? a.tile_req[tile + 1] : a.R - 1;  // the last request meeting the tile
-  const uint32_t nreq = r_last - r_first + 1;
-  const bool cached = nreq <= kH16Req;
-  if (cached) {
-    for (uint32_t i = threadIdx.x; i <= nreq; i += kHashThreads) {
-      s_boff[i] = a.blk_off[r_first + i];
-      s_toff[i] = a.tok_off[r_first + i];
-    }
-  }
-  if (threadIdx.x == 0) s_big = 0;
-  __syncthreads();
-  const uint32_t t = threadIdx.x;
-  const uint64_t b = b0 + t;
-  uint64_t h0 = 0, h1 = 0;
-  uint32_t k = 0;
-  uint64_t wd_x = 0;  // token offset of this thread's block
-  uint64_t rstart = 0;  // first block of its request
-  if (b < b_end) {
-    uint64_t x;
-    if (cached) {  // largest i with s_boff[i] <= b
-      uint32_t lo = 0, hi = nreq - 1;
-      while (lo < hi) {
-        const uint32_t mid = (lo + hi + 1) >> 1;
-        if (s_boff[mid] <= b)
-          lo = mid;
-        else
-          hi = mid - 1;
+  // the token array from the 16-byte boundary at or below its start
+  const uint32_t mis = (uint32_t)(reinterpret_cast<uintptr_t>(a.tokens) >> 2) & 3u;
+  const uint32_t* base = a.tokens - mis;
+  const uint64_t n_word = a.n_tok + mis;
+  // A window of 32 requests from rw, one per lane: unit v of the tile that
+  // lies in one of them is unit v + e0 of the request and starts at word
+  // x0 + U v.  `past` is the first unit after the window.
+  uint32_t rw = r_first, wn = 0;
+  int64_t e0 = 0, x0 = 0, past = 0;
+  auto window = [&]() {
+    wn = r_last - rw + 1 < 32 ? r_last - rw + 1 : 32;
+    const uint32_t r = rw + (lane < wn ? lane : wn - 1);
+    e0 = ((int64_t)b0 - (int64_t)a.blk_off[r]) * (int64_t)a.g;
+    x0 = (int64_t)(a.tok_off[r] + mis) + U * e0;
+    past = ((int64_t)a.blk_off[rw + wn] - (int64_t)b0) * (int64_t)a.g;
+  };
+  window();
+  const bool one = r_first == r_last;
+  bool big = false;
+#pragma unroll 1
+  for (uint32_t v0 = 0; v0 < nu; v0 += 32) {
+    const uint32_t v = v0 + lane;
+    const bool live = v < nu;
+    int64_t e = e0, x = x0;  // of this lane's unit
+    if (!one) {
+      const uint32_t last = nu - v0 < 32 ? nu - 1 : v0 + 31;
+      if (past <= (int64_t)last) {  // move the window to the request of this round's first unit
+        const uint32_t in = __popc(__ballot_sync(kFull, lane < wn && -e0 <= (int64_t)v0));
+        rw = past <= (int64_t)v0 ? find_request(a.blk_off, rw, r_last, b0 + v0 / a.g) : rw + (in ? in - 1 : 0);
+        window();
       }
-      rstart = s_boff[lo];
-      k = (uint32_t)(b - rstart);
-      x = s_toff[lo] + 16ULL * k;
-    } else {
-      const uint32_t r = find_request(a.blk_off, r_first, r_last, b);
-      rstart = a.blk_off[r];
-      k = (uint32_t)(b - rstart);
-      x = a.tok_off[r] + 16ULL * k;
+      if (past > (int64_t)last) {
+        uint32_t idx = 0;
+        for (uint32_t i = 1; i < wn; ++i) {
+          const int64_t st = -shfl_i64(e0, i);
+          if (st > (int64_t)last) break;
+          if (st <= (int64_t)v) idx = i;
+        }
+        e = shfl_i64(e0, idx);
+        x = shfl_i64(x0, idx);
+      } else if (live) {  // more requests than the window holds (many without blocks)
+        const uint32_t r = find_request(a.blk_off, rw, r_last, b0 + v / a.g);
+        e = ((int64_t)b0 - (int64_t)a.blk_off[r]) * (int64_t)a.g;
+        x = (int64_t)(a.tok_off[r] + mis) + U * e;
+      }
     }
-    wd_x = x;
-  }
-  // Each lane reads the four aligned 16-byte words that start its 16 tokens;
-  // a block that does not start on a 16-byte boundary also needs the first
-  // one to three words of the next 16, which the next lane holds when its
-  // block follows on directly (the usual case inside a request).
-  const uint32_t m = (uint32_t)(wd_x & 3);
-  const uint64_t x4 = wd_x - m;
-  uint32_t wd[20];
-  const bool live = b < b_end;
-  const bool whole = live && x4 + 16 <= a.n_tok;
-  {
-    const uint4* q4 = reinterpret_cast<const uint4*>(a.tokens + x4);
+    e += v;
+    x += (int64_t)U * v;
+    const uint32_t st = __ballot_sync(kFull, live && e == 0);  // units that open a request
+    if (lane == 0) starts[v0 >> 5] = st;
+    // its words: NV aligned vectors, and for a unit that starts m words into
+    // the first the next vector's m words, which the next lane holds if its
+    // unit follows on
+    const uint32_t m = (uint32_t)x & 3u;
+    const uint64_t x4 = (uint64_t)x - m;
+    const bool whole = live && x4 >= mis && x4 + U <= n_word;
+    const uint32_t full = __ballot_sync(kFull, whole);
+    const bool follows = lane < 31 && ((full & ~st) >> (lane + 1)) & 1u;  // the next lane has the next vector
+    uint32_t wd[U + 4];
+    uint4 nx = make_uint4(0, 0, 0, 0);
 #pragma unroll
-    for (int q = 0; q < 4; ++q) {
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (whole) v = __ldcs(q4 + q);
-      wd[4 * q] = v.x;
-      wd[4 * q + 1] = v.y;
-      wd[4 * q + 2] = v.z;
-      wd[4 * q + 3] = v.w;
+    for (int q = 0; q < NV; ++q) {
+      uint4 t = make_uint4(0, 0, 0, 0);
+      if (whole) t = __ldcs(reinterpret_cast<const uint4*>(base + x4) + q);
+      wd[4 * q] = t.x;
+      wd[4 * q + 1] = t.y;
+      wd[4 * q + 2] = t.z;
+      wd[4 * q + 3] = t.w;
+    }
+    if (live && m != 0 && !follows) {
+      const uint64_t y = x4 + U;
+      if (y + 4 <= n_word) {
+        nx = __ldcs(reinterpret_cast<const uint4*>(base + y));
+      } else {
+        nx.x = y < n_word ? base[y] : 0u;
+        nx.y = y + 1 < n_word ? base[y + 1] : 0u;
+        nx.z = y + 2 < n_word ? base[y + 2] : 0u;
+      }
+    }
+    // the powers go out with the tokens
+    const uint64_t* T = a.tables;
+    uint64_t w0 = 0, w1 = 0;
+    if (live) {
+      w0 = pow_at(T + 0 * 65536, T + 1 * 65536, (uint64_t)e);
+      w1 = pow_at(T + 2 * 65536, T + 3 * 65536, (uint64_t)e);
     }
     if (live && !whole) {
 #pragma unroll
-      for (int q = 0; q < 16; ++q) wd[q] = x4 + q < a.n_tok ? a.tokens[x4 + q] : 0u;
+      for (int q = 0; q < U; ++q) wd[q] = x4 + q >= mis && x4 + q < n_word ? base[x4 + q] : 0u;
     }
-  }
-  const uint64_t x_next = __shfl_down_sync(kFull, wd_x, 1);
-  const uint32_t n0 = __shfl_down_sync(kFull, wd[0], 1), n1 = __shfl_down_sync(kFull, wd[1], 1),
-                 n2 = __shfl_down_sync(kFull, wd[2], 1);
-  const bool follows = (threadIdx.x & 31) != 31 && x_next == wd_x + 16 && whole;
-  wd[16] = n0;
-  wd[17] = n1;
-  wd[18] = n2;
-  wd[19] = 0;
-  if (live && m && !follows) {
-    const uint64_t y = x4 + 16;
-    if (y + 4 <= a.n_tok) {
-      const uint4 v = __ldcs(reinterpret_cast<const uint4*>(a.tokens + y));
-      wd[16] = v.x;
-      wd[17] = v.y;
-      wd[18] = v.z;
-    } else {
-      wd[16] = y < a.n_tok ? a.tokens[y] : 0u;
-      wd[17] = y + 1 < a.n_tok ? a.tokens[y + 1] : 0u;
-      wd[18] = y + 2 < a.n_tok ? a.tokens[y + 2] : 0u;
+    if (__any_sync(kFull, m != 0)) {
+      const uint32_t n0 = __shfl_down_sync(kFull, wd[0], 1), n1 = __shfl_down_sync(kFull, wd[1], 1),
+                     n2 = __shfl_down_sync(kFull, wd[2], 1);
+      if (follows) nx = make_uint4(n0, n1, n2, 0u);
     }
-  }
-  if (live) {
-    if (!WIDE) {  // a token (or a word around the block: that only widens the test) reaching 2^27
+    wd[U] = nx.x;
+    wd[U + 1] = nx.y;
+    wd[U + 2] = nx.z;
+    wd[U + 3] = 0;
+    if (!WIDE) {  // words around the unit only widen the test
       uint32_t any = 0;
 #pragma unroll
-      for (int j = 0; j < 19; ++j) any |= wd[j];
-      if (any >> 27) s_big = 1;
-      uint64_t acc[4] = {0, 0, 0, 0};
+      for (int q = 0; q < U + 3; ++q) any |= wd[q];
+      big |= (any >> 27) != 0;
+    }
+    uint64_t g0 = 0, g1 = 0;
+    if (live) {
+      uint64_t h0, h1;
       switch (m) {
-        case 0: hash16_2<0>(wd, c, acc); break;
-        case 1: hash16_2<1>(wd, c, acc); break;
-        case 2: hash16_2<2>(wd, c, acc); break;
-        default: hash16_2<3>(wd, c, acc); break;
+        case 0: unit_hash<U, 0, WIDE>(wd, c, h0, h1); break;
+        case 1: unit_hash<U, 1, WIDE>(wd, c, h0, h1); break;
+        case 2: unit_hash<U, 2, WIDE>(wd, c, h0, h1); break;
+        default: unit_hash<U, 3, WIDE>(wd, c, h0, h1); break;
       }
-      // lazily reduced (below 2^62 + 3); p61_mul_lazy takes it as it is
-      h0 = limbs2_lazy(acc[0], acc[1]) + c.csum[0][16];
-      h1 = limbs2_lazy(acc[2], acc[3]) + c.csum[1][16];
-    } else {  // three limbs
-      uint64_t acc[6] = {0, 0, 0, 0, 0, 0};
-      switch (m) {
-        case 0: hash16<0>(wd, c, acc); break;
-        case 1: hash16<1>(wd, c, acc); break;
-        case 2: hash16<2>(wd, c, acc); break;
-        default: hash16<3>(wd, c, acc); break;
-      }
-      h0 = p61_add(limbs_to_p61(acc[0], acc[1], acc[2]), c.csum[0][16]);
-      h1 = p61_add(limbs_to_p61(acc[3], acc[4], acc[5]), c.csum[1][16]);
+      g0 = p61_mul_lazy(h0, w0);
+      g1 = p61_mul_lazy(h1, w1);
     }
+    slot[unit_slot(v)] = make_ulonglong2(g0, g1);
   }
-  // g = h u^(16 k), then a plain prefix sum over the tile; a block whose
-  // request starts inside the tile at index s subtracts the prefix before s.
-  const uint64_t* T = a.tables;
-  uint64_t v0 = 0, v1 = 0;  // below 2^61 + 5
-  if (live) {
-    v0 = p61_mul_lazy(h0, pow_at(T + 0 * 65536, T + 1 * 65536, k));
-    v1 = p61_mul_lazy(h1, pow_at(T + 2 * 65536, T + 3 * 65536, k));
-  }
-  __shared__ uint64_t s_p0[kHashThreads], s_p1[kHashThreads];
-  __shared__ uint64_t s_w0[kHashThreads / 32], s_w1[kHashThreads / 32];
-  const uint32_t lane = t & 31, w = t >> 5;
-  // warp scan with lazy reduction: from values below 2^61 + 5, two plain
-  // steps stay below 2^63 + 20; a fold (x & p) + (x >> 61) brings such a sum
-  // back below 2^61 + 4, so folding after d = 2 and d = 8 keeps every sum
-  // below 2^64 and leaves the result below 2^62 + 8
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const uint64_t y0 = __shfl_up_sync(kFull, v0, d), y1 = __shfl_up_sync(kFull, v1, d);
-    if (lane >= (uint32_t)d) {
-      v0 += y0;
-      v1 += y1;
-    }
-    if (d == 2 || d == 8) {
-      v0 = (v0 & kP61) + (v0 >> 61);
-      v1 = (v1 & kP61) + (v1 >> 61);
-    }
-  }
-  if (lane == 31) {
-    s_w0[w] = v0;
-    s_w1[w] = v1;
-  }
-  __syncthreads();
-  if (!WIDE && s_big) {  // the tile goes to k_hash16_wide, which writes all of it
-    if (t == 0) a.wide_list[atomicAdd(&a.st->tile_ctr[kEpochWide], 1u)] = tile;
+  if (!WIDE && __any_sync(kFull, big)) {
+    if (lane == 0) a.wide_list[atomicAdd(&a.st->tile_ctr[kEpochWide], 1u)] = tile;
     return;
   }
-  if (w == 0) {  // exclusive prefix of the warp totals
-    uint64_t z0 = lane < kHashThreads / 32 ? s_w0[lane] : 0, z1 = lane < kHashThreads / 32 ? s_w1[lane] : 0;
-    const uint64_t x0 = z0, x1 = z1;
-#pragma unroll
-    for (int d = 1; d < kHashThreads / 32; d <<= 1) {
-      const uint64_t y0 = __shfl_up_sync(kFull, z0, d), y1 = __shfl_up_sync(kFull, z1, d);
-      if (lane >= (uint32_t)d) {
-        z0 += y0;
-        z1 += y1;
-      }
-      z0 = (z0 & kP61) + (z0 >> 61);
-      z1 = (z1 & kP61) + (z1 >> 61);
-    }
-    if (lane < kHashThreads / 32) {
-      s_w0[lane] = p61_fold(z0 + (kP61 << 2) - x0);  // z < 2^61 + 4, x < 2^62 + 8: stays in (0, 2^64)
-      s_w1[lane] = p61_fold(z1 + (kP61 << 2) - x1);
-    }
-  }
-  __syncthreads();
-  v0 = p61_fold(v0 + s_w0[w]);
-  v1 = p61_fold(v1 + s_w1[w]);
-  // A request starting after b0 inside the tile subtracts the prefix before
-  // its start; when none does (a long request spans the tile), the prefixes
-  // are not exchanged.
-  const bool inner = !cached || (nreq >= 2 && s_boff[1] < b_end);
-  if (inner) {
-    s_p0[t] = v0;
-    s_p1[t] = v1;
-    __syncthreads();
-  }
-  if (live) {
-    const bool own_start = rstart >= b0;  // the request starts in this tile
-    if (inner && own_start && rstart > b0) {
-      const uint32_t sl = (uint32_t)(rstart - b0) - 1;
-      v0 = p61_add(v0, kP61 - s_p0[sl]);
-      v1 = p61_add(v1, kP61 - s_p1[sl]);
-    }
-    a.keys[b] = make_ulonglong2(v0, v1);
-  }
-  // the tile's aggregate for k_hash_chain: the last block's sum since its
-  // request's start, and whether that start is in the tile; and the leading
-  // blocks (before the tile's first request start)
-  if (b + 1 == b_end) {
-    HashCarry agg;
-    agg.f = rstart >= b0;
-    agg.v0 = v0;
-    agg.v1 = v1;
-    a.tile_agg[tile] = agg;
-  }
-  if (t == 0) {
-    uint32_t lead = (uint32_t)(b_end - b0);
-    if (cached) {
-      for (uint32_t i = 0; i < nreq; ++i)
-        if (s_boff[i] >= b0 && s_boff[i] < b_end && s_boff[i + 1] > s_boff[i]) {
-          lead = (uint32_t)(s_boff[i] - b0);
-          break;
-        }
-    } else {
-      for (uint32_t r = r_first; r <= r_last; ++r) {
-        const uint64_t st0 = a.blk_off[r];
-        if (st0 >= b0 && st0 < b_end && a.blk_off[r + 1] > st0) {
-          lead = (uint32_t)(st0 - b0);
-          break;
-        }
-      }
-    }
+  __syncwarp();
+  // ---- sums: this lane's units 8 lane .. 8 lane + 7 (values below 2^61 + 8)
+  const uint32_t rounds = (nu + 31) / 32;
+  const uint32_t mine = (lane >> 2) < rounds ? (starts[lane >> 2] >> (8 * (lane & 3))) & 0xFFu : 0u;
+  const bool in = 8 * lane < 32 * rounds;
+  const uint32_t opens = __ballot_sync(kFull, mine != 0);
+  unit_sums(slot, lane, mine, opens, in);
+  __syncwarp();
+  for (uint32_t i = lane; i < nb; i += 32) a.keys[b0 + i] = slot[unit_slot((i + 1) * a.g - 1)];
+  // the tile's aggregate for the carry: its last unit's sum since its request's
+  // start, and whether a request starts in the tile; and the blocks before the
+  // tile's first request start
+  if (lane == 0) {
+    const ulonglong2 t = slot[unit_slot(nu - 1)];
+    uint32_t lead = nb;
+    for (int q = (int)rounds - 1; q >= 0; --q)
+      if (starts[q]) lead = (32 * q + __ffs(starts[q]) - 1) / a.g;
+    a.tile_agg[tile] = HashCarry{t.x, t.y, opens != 0};
     a.tile_lead[tile] = lead;
   }
 }
 
-__global__ void __launch_bounds__(kHashThreads, 8) k_hash16(HashArgs a, const __grid_constant__ HashConsts c) {
+template <int U>
+__global__ void __launch_bounds__(kUnitThreads, 16) k_hash_units(HashArgs a, const __grid_constant__ HashConsts c) {
   grid_dep_sync();
-  hash16_tile<false>(a, c, blockIdx.x, blocks_live(a.st, a.keys_cap));
+  __shared__ ulonglong2 s_slot[kUnitWarps][kUnitSlots];
+  __shared__ uint32_t s_starts[kUnitWarps][kUnitTile / 32];
+  const uint32_t w = threadIdx.x >> 5;
+  hash_units_tile<U, false>(a, c, blockIdx.x * kUnitWarps + w, blocks_live(a.st, a.keys_cap), s_slot[w], s_starts[w]);
 }
 
-// The tiles k_hash16 left (a token at or above 2^27), a persistent grid over
-// the list it wrote.
-__global__ void __launch_bounds__(kHashThreads) k_hash16_wide(HashArgs a, const __grid_constant__ HashConsts c) {
+// The tiles k_hash_units left, a persistent grid over the list it wrote.
+template <int U>
+__global__ void __launch_bounds__(kUnitThreads) k_hash_units_wide(HashArgs a, const __grid_constant__ HashConsts c) {
   grid_dep_sync();
+  __shared__ ulonglong2 s_slot[kUnitWarps][kUnitSlots];
+  __shared__ uint32_t s_starts[kUnitWarps][kUnitTile / 32];
+  const uint32_t w = threadIdx.x >> 5;
   const uint64_t N = blocks_live(a.st, a.keys_cap);
   const uint32_t n_wide = ld_relaxed_u32(&a.st->tile_ctr[kEpochWide]);
-  for (uint32_t j = blockIdx.x; j < n_wide; j += gridDim.x) {
+  for (uint32_t j = blockIdx.x * kUnitWarps + w; j < n_wide; j += gridDim.x * kUnitWarps) {
     const uint32_t tile = a.wide_list[j];
-    if (in_bounds(a.st, tile, (N + kHashThreads - 1) / kHashThreads)) hash16_tile<true>(a, c, tile, N);
-    __syncthreads();  // the next tile reuses the shared arrays
-  }
-}
-
-// B a multiple of 16 (g = B / 16 chunks of 16 tokens) with 16-byte-aligned
-// tokens: P consecutive blocks per thread (one here; two would suit B = 16,
-// which k_hash16 takes), tiles of kHashThreads = 256 blocks whatever B,
-// kHashThreads / P threads per CTA, 64 registers.
-// The requests that meet the tile are tile_req[tile] .. tile_req[tile + 1];
-// their block and token offsets are loaded into shared memory once, so a
-// thread finds its request without a dependent chain of global loads.  A
-// thread hashes its P g chunks one after another in one loop (four or five
-// 16-byte loads each), so the code of the chunk product exists once and the
-// registers of one chunk are live at a time: h_b = sum over chunks s of
-// h_(b,s) u^(16 s).  The prefix sum then runs over one value per thread.
-// Tiles meeting more than kH16Req requests search the global offsets.
-// The 20 words x4 .. x4 + 19 of a 16-token chunk whose first token is word
-// m of them (the fifth 16-byte load only when m > 0).
-__device__ __forceinline__ void load_chunk(const HashArgs& a, uint64_t x4, uint32_t m, uint32_t (&wd)[20]) {
-  if (x4 + 20 <= a.n_tok) {
-    const uint4* q4 = reinterpret_cast<const uint4*>(a.tokens + x4);
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      uint4 v = make_uint4(0, 0, 0, 0);
-      if (q < 4 || m != 0) v = __ldcs(q4 + q);
-      wd[4 * q] = v.x;
-      wd[4 * q + 1] = v.y;
-      wd[4 * q + 2] = v.z;
-      wd[4 * q + 3] = v.w;
-    }
-  } else {  // within 20 words of the end of the token array
-#pragma unroll
-    for (int q = 0; q < 20; ++q) wd[q] = x4 + q < a.n_tok ? a.tokens[x4 + q] : 0u;
-  }
-}
-
-// h of the 16 tokens wd[M .. M+15] for both bases, every token below 2^27:
-// below 2^62 + 2.
-template <int M>
-__device__ __forceinline__ void chunk_narrow(const uint32_t (&wd)[20], const HashConsts& c, uint64_t& e0, uint64_t& e1) {
-  uint64_t acc[4] = {0, 0, 0, 0};
-  hash16_2<M>(wd, c, acc);
-  e0 = limbs2_lazy(acc[0], acc[1]) + c.csum[0][16];
-  e1 = limbs2_lazy(acc[2], acc[3]) + c.csum[1][16];
-}
-
-// The same for any 32-bit tokens (three limbs), fully reduced.
-template <int M>
-__device__ __forceinline__ void chunk_wide(const uint32_t (&wd)[20], const HashConsts& c, uint64_t& e0, uint64_t& e1) {
-  uint64_t acc[6] = {0, 0, 0, 0, 0, 0};
-  hash16<M>(wd, c, acc);
-  e0 = p61_add(limbs_to_p61(acc[0], acc[1], acc[2]), c.csum[0][16]);
-  e1 = p61_add(limbs_to_p61(acc[3], acc[4], acc[5]), c.csum[1][16]);
-}
-
-// Chunk s of a block into its h: h_s u^(16 s) added to the chunks before,
-// kept below 2^62 + 2 by one fold (the first chunk is taken as it is).
-__device__ __forceinline__ void chunk_add(const HashConsts& c, uint32_t s, uint64_t e0, uint64_t e1, uint64_t& h0,
-                                          uint64_t& h1) {
-  if (s == 0) {
-    h0 = e0;
-    h1 = e1;
-    return;
-  }
-  h0 += p61_mul_lazy(e0, c.sub_mul[0][s]);
-  h1 += p61_mul_lazy(e1, c.sub_mul[1][s]);
-  h0 = (h0 & kP61) + (h0 >> 61);
-  h1 = (h1 & kP61) + (h1 >> 61);
-}
-
-// B a multiple of 16 (g = B / 16 chunks of 16 tokens) with 16-byte-aligned
-// tokens, B > 16: one block per thread, tiles of kHashThreads = 256 blocks
-// whatever B, four CTAs per SM (64 registers).  The requests that meet the
-// tile are tile_req[tile] .. tile_req[tile + 1]; their block and token
-// offsets are loaded into shared memory once, so a thread finds its request
-// without a dependent chain of global loads.  A thread hashes its block's g
-// chunks one after another in one loop (four or five 16-byte loads each), so
-// the code of the chunk product exists once and the registers of one chunk
-// are live at a time: h = sum over chunks s of h_s u^(16 s).  Tiles meeting
-// more than kTileReq requests search the global offsets.
-constexpr int kTileReq = 256;
-
-__global__ void __launch_bounds__(kHashThreads, 4) k_hash_tile(HashArgs a, const __grid_constant__ HashConsts c) {
-  constexpr uint32_t TB = kHashThreads;
-  grid_dep_sync();
-  __shared__ uint64_t s_boff[kTileReq + 1];
-  __shared__ uint64_t s_toff[kTileReq + 1];
-  __shared__ uint64_t s_p0[TB], s_p1[TB];
-  __shared__ uint64_t s_w0[TB / 32], s_w1[TB / 32];
-  const uint32_t tile = blockIdx.x;
-  const uint64_t N = blocks_live(a.st, a.keys_cap);
-  const uint64_t b0 = (uint64_t)tile * TB;
-  if (b0 >= N) return;
-  const uint64_t b_end = b0 + TB < N ? b0 + TB : N;
-  const uint64_t ntiles = (N + TB - 1) / TB;
-  const uint32_t r_first = a.tile_req[tile];
-  const uint32_t r_last = tile + 1 < ntiles ? a.tile_req[tile + 1] : a.R - 1;  // the last request meeting the tile
-  const uint32_t nreq = r_last - r_first + 1;
-  const bool cached = nreq <= kTileReq;
-  if (cached) {
-    for (uint32_t i = threadIdx.x; i <= nreq; i += TB) {
-      s_boff[i] = a.blk_off[r_first + i];
-      s_toff[i] = a.tok_off[r_first + i];
-    }
-  }
-  __syncthreads();
-  const uint32_t t = threadIdx.x, lane = t & 31, w = t >> 5;
-  const uint32_t g = a.B / 16;
-  const uint64_t b = b0 + t;
-  const bool live = b < b_end;
-  // the block's request starts at block rs, the block's tokens at xb
-  uint64_t rs = 0, xb = 0;
-  if (live) {
-    if (cached) {  // largest i with s_boff[i] <= b
-      uint32_t lo = 0, hi = nreq - 1;
-      while (lo < hi) {
-        const uint32_t mid = (lo + hi + 1) >> 1;
-        if (s_boff[mid] <= b)
-          lo = mid;
-        else
-          hi = mid - 1;
-      }
-      rs = s_boff[lo];
-      xb = s_toff[lo] + (uint64_t)a.B * (b - rs);
-    } else {
-      const uint32_t r = find_request(a.blk_off, r_first, r_last, b);
-      rs = a.blk_off[r];
-      xb = a.tok_off[r] + (uint64_t)a.B * (b - rs);
-    }
-  }
-  // h of the block, below 2^62 + 2.  The loop takes every chunk with
-  // two-limb products; a block with a token of 2^27 or more is redone with
-  // three limbs in a second loop (never taken over a real vocabulary), so
-  // the two paths' registers are not live together.  (Loop bounds rather than
-  // an enclosing branch, and the first loop running to its end: this shape
-  // spills the fewest registers at 64.)
-  uint64_t h0 = 0, h1 = 0;
-  bool wide = false;
-  const uint32_t gl = live ? g : 0u;
-  {
-#pragma unroll 1
-    for (uint32_t s = 0; s < gl; ++s) {
-      const uint64_t x = xb + 16ULL * s;
-      const uint32_t m = (uint32_t)(x & 3);
-      uint32_t wd[20];
-      load_chunk(a, x - m, m, wd);
-      uint32_t any = 0;  // words outside the chunk only widen the test
-#pragma unroll
-      for (int q = 0; q < 20; ++q) any |= wd[q];
-      if (any >> 27) {
-        wide = true;
-        continue;
-      }
-      uint64_t e0, e1;
-      switch (m) {
-        case 0: chunk_narrow<0>(wd, c, e0, e1); break;
-        case 1: chunk_narrow<1>(wd, c, e0, e1); break;
-        case 2: chunk_narrow<2>(wd, c, e0, e1); break;
-        default: chunk_narrow<3>(wd, c, e0, e1); break;
-      }
-      chunk_add(c, s, e0, e1, h0, h1);
-    }
-  }
-  if (wide) {
-#pragma unroll 1
-    for (uint32_t s = 0; s < g; ++s) {
-      const uint64_t x = xb + 16ULL * s;
-      const uint32_t m = (uint32_t)(x & 3);
-      uint32_t wd[20];
-      load_chunk(a, x - m, m, wd);
-      uint64_t e0, e1;
-      switch (m) {
-        case 0: chunk_wide<0>(wd, c, e0, e1); break;
-        case 1: chunk_wide<1>(wd, c, e0, e1); break;
-        case 2: chunk_wide<2>(wd, c, e0, e1); break;
-        default: chunk_wide<3>(wd, c, e0, e1); break;
-      }
-      chunk_add(c, s, e0, e1, h0, h1);
-    }
-  }
-  // g = h u^(B k) for the block's depth k (the tables hold u^(B e)), below
-  // 2^61 + 5, then a plain prefix sum over the tile; a block whose request
-  // starts inside the tile at index s subtracts the prefix before s.
-  const uint64_t* T = a.tables;
-  uint64_t v0 = 0, v1 = 0;
-  if (live) {
-    const uint32_t k = (uint32_t)(b - rs);
-    v0 = p61_mul_lazy(h0, pow_at(T + 0 * 65536, T + 1 * 65536, k));
-    v1 = p61_mul_lazy(h1, pow_at(T + 2 * 65536, T + 3 * 65536, k));
-  }
-  // warp scan with lazy reduction: from values below 2^61 + 5, two plain
-  // steps stay below 2^63 + 20; a fold (x & p) + (x >> 61) brings such a sum
-  // back below 2^61 + 4, so folding after d = 2 and d = 8 keeps every sum
-  // below 2^64 and leaves the result below 2^62 + 8
-#pragma unroll
-  for (int d = 1; d < 32; d <<= 1) {
-    const uint64_t y0 = __shfl_up_sync(kFull, v0, d), y1 = __shfl_up_sync(kFull, v1, d);
-    if (lane >= (uint32_t)d) {
-      v0 += y0;
-      v1 += y1;
-    }
-    if (d == 2 || d == 8) {
-      v0 = (v0 & kP61) + (v0 >> 61);
-      v1 = (v1 & kP61) + (v1 >> 61);
-    }
-  }
-  if (lane == 31) {
-    s_w0[w] = v0;
-    s_w1[w] = v1;
-  }
-  __syncthreads();
-  if (w == 0) {  // exclusive prefix of the warp totals
-    constexpr int NW = TB / 32;
-    uint64_t z0 = lane < NW ? s_w0[lane] : 0, z1 = lane < NW ? s_w1[lane] : 0;
-    const uint64_t o0 = z0, o1 = z1;
-#pragma unroll
-    for (int d = 1; d < NW; d <<= 1) {
-      const uint64_t y0 = __shfl_up_sync(kFull, z0, d), y1 = __shfl_up_sync(kFull, z1, d);
-      if (lane >= (uint32_t)d) {
-        z0 += y0;
-        z1 += y1;
-      }
-      z0 = (z0 & kP61) + (z0 >> 61);
-      z1 = (z1 & kP61) + (z1 >> 61);
-    }
-    if (lane < NW) {
-      s_w0[lane] = p61_fold(z0 + (kP61 << 2) - o0);  // z < 2^61 + 4, o < 2^62 + 8: stays in (0, 2^64)
-      s_w1[lane] = p61_fold(z1 + (kP61 << 2) - o1);
-    }
-  }
-  __syncthreads();
-  v0 = p61_fold(v0 + s_w0[w]);
-  v1 = p61_fold(v1 + s_w1[w]);
-  s_p0[t] = v0;
-  s_p1[t] = v1;
-  __syncthreads();
-  if (live && rs > b0) {  // the request starts inside the tile, after its first block
-    const uint32_t sl = (uint32_t)(rs - b0) - 1;
-    v0 = p61_add(v0, kP61 - s_p0[sl]);
-    v1 = p61_add(v1, kP61 - s_p1[sl]);
-  }
-  if (live) a.keys[b] = make_ulonglong2(v0, v1);
-  // the tile's aggregate for the carry: the last block's sum since its
-  // request's start, and whether that start is in the tile; and the leading
-  // blocks (before the tile's first request start)
-  if (live && b + 1 == b_end) a.tile_agg[tile] = HashCarry{v0, v1, rs >= b0};
-  if (t == 0) {
-    uint32_t lead = (uint32_t)(b_end - b0);
-    if (cached) {
-      for (uint32_t i = 0; i < nreq; ++i)
-        if (s_boff[i] >= b0 && s_boff[i] < b_end && s_boff[i + 1] > s_boff[i]) {
-          lead = (uint32_t)(s_boff[i] - b0);
-          break;
-        }
-    } else {
-      for (uint32_t r = r_first; r <= r_last; ++r) {
-        const uint64_t st0 = a.blk_off[r];
-        if (st0 >= b0 && st0 < b_end && a.blk_off[r + 1] > st0) {
-          lead = (uint32_t)(st0 - b0);
-          break;
-        }
-      }
-    }
-    a.tile_lead[tile] = lead;
+    if (in_bounds(a.st, tile, (N + a.tb - 1) / a.tb)) hash_units_tile<U, true>(a, c, tile, N, s_slot[w], s_starts[w]);
+    __syncwarp();  // the next tile reuses the slots
   }
 }
 
@@ -1122,20 +888,27 @@ __global__ void __launch_bounds__(kChainWarps * 32) k_hash_carry(const HashCarry
   }
 }
 
+template <int U>
+void launch_units(uint32_t tiles, cudaStream_t s, const HashArgs& a, const HashConsts& c) {
+  const uint32_t grid = ceil_div_u32(tiles, kUnitWarps);
+  PTC_KERNEL("k_hash_units", s, k_hash_units<U>, grid, kUnitThreads, 0, a, c);
+  const uint32_t wgrid = grid < (uint32_t)(2 * num_sms()) ? grid : (uint32_t)(2 * num_sms());
+  PTC_KERNEL("k_hash_units_wide", s, k_hash_units_wide<U>, wgrid, kUnitThreads, 0, a, c);
+}
+
 template <int G>
 void launch_hash(uint32_t grid, cudaStream_t s, const HashArgs& a, const HashConsts& c, bool full) {
-  if (G == 1 && full && a.aligned) {
-    PTC_KERNEL("k_hash16", s, k_hash16, grid, kHashThreads, 0, a, c);
-    const uint32_t wgrid = grid < (uint32_t)(2 * num_sms()) ? grid : (uint32_t)(2 * num_sms());
-    PTC_KERNEL("k_hash16_wide", s, k_hash16_wide, wgrid, kHashThreads, 0, a, c);
-  }
-  else if (a.aligned && a.B % 16 == 0)
-    PTC_KERNEL("k_hash_tile", s, k_hash_tile, grid, kHashThreads, 0, a, c);
-  else if (full)
+  if (full)
     PTC_KERNEL("k_hash_local", s, (k_hash_local<G, true>), grid, kHashThreads, 0, a, c);
   else
     PTC_KERNEL("k_hash_local", s, (k_hash_local<G, false>), grid, kHashThreads, 0, a, c);
 }
+
+// Tokens per unit of k_hash_units, or 0 for a block size that k_hash_local
+// takes.  Units are whole vectors of four tokens, so that the units of a
+// request share their alignment; the larger the unit, the fewer
+// multiplications and sums per token.
+uint32_t unit_tokens(uint32_t B) { return B % 16 == 0 ? 16 : B % 12 == 0 ? 12 : B % 8 == 0 ? 8 : 0; }
 
 uint32_t chunks_per_block(uint32_t B) {  // G: power of two >= ceil(B / 16)
   uint32_t need = (B + 15) / 16, g = 1;
@@ -1143,14 +916,15 @@ uint32_t chunks_per_block(uint32_t B) {  // G: power of two >= ceil(B / 16)
   return g;
 }
 
-// Blocks per hash tile: kHashThreads for k_hash16 and k_hash_tile (B a
-// multiple of 16 over 16-byte-aligned tokens), one CTA's kHashThreads / G for
-// k_hash_local.  Arrays sized per tile take the smaller (the alignment of the
-// tokens is not known there).
-uint32_t tile_blocks(uint32_t B, bool aligned) {
-  return aligned && B % 16 == 0 ? (uint32_t)kHashThreads : kHashThreads / chunks_per_block(B);
+// Blocks per hash tile, a power of two: as many as make up to 256 units for
+// k_hash_units, one CTA's kHashThreads / G for k_hash_local.
+uint32_t tile_blocks(uint32_t B) {
+  const uint32_t U = unit_tokens(B);
+  if (!U) return kHashThreads / chunks_per_block(B);
+  uint32_t tb = kUnitTile;
+  while (tb * (B / U) > kUnitTile) tb >>= 1;
+  return tb;
 }
-uint32_t min_tile_blocks(uint32_t B) { return tile_blocks(B, false); }
 
 struct HashLayout {
   DevStatus* st;
@@ -1170,7 +944,7 @@ HashLayout hash_layout(void* ws, uint32_t n_req, uint64_t n_tok, uint32_t B, uin
   Carver cv(ws);
   const uint32_t off_tiles = ceil_div_u32(n_req, kOffTile) + 1;
   const uint64_t nb = n_tok / B < keys_cap ? n_tok / B : keys_cap;
-  const uint32_t tb = min_tile_blocks(B);
+  const uint32_t tb = tile_blocks(B);
   const uint32_t hash_tiles = ceil_div_u32(nb, tb) + 1;
   L.st = cv.take<DevStatus>(1);
   L.lb_off = cv.take<uint64_t>(off_tiles);
@@ -1192,7 +966,7 @@ using namespace ptc;
 
 uint64_t ptc::hash_carry_tiles(uint64_t n_tok, uint32_t block_size) {
   if (block_size == 0) block_size = 1;
-  return ceil_div_u32(n_tok / block_size, min_tile_blocks(block_size)) + 1;
+  return ceil_div_u32(n_tok / block_size, tile_blocks(block_size)) + 1;
 }
 
 extern "C" size_t ptc_hash_blocks_workspace_bytes(uint32_t n_req, uint64_t n_tok, uint32_t block_size) {
@@ -1226,7 +1000,7 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
   }
   const uint32_t G = chunks_per_block(block_size);
   const bool aligned = (((uintptr_t)tokens) & 15) == 0;
-  const uint32_t tb = tile_blocks(block_size, aligned);
+  const uint32_t tb = tile_blocks(block_size), U = unit_tokens(block_size);
   PTC_KERNEL("k_block_offsets", s, k_block_offsets, ceil_div_u32(n_req, kOffTile), kOffThreads, 0, req_tok_off, req_ts_us, n_req, n_tok, block_size, tb, req_blk_off_out, L.tile_req, L.hash_tiles, L.lb_off, L.st);
 
   // seeded bases and their derived constants
@@ -1234,13 +1008,13 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
   HashConsts hc;
   for (int b = 0; b < 2; ++b) {
     const uint64_t u = 2 + splitmix64_at(seed, (uint64_t)b) % (kP61 - 3);
-    const uint64_t uB = p61_pow(u, block_size);
-    pb.base[b * 2 + 0] = uB;
-    pb.base[b * 2 + 1] = p61_pow(uB, 65536);
-    uint64_t sum = 0;
+    const uint64_t uU = p61_pow(u, U ? U : block_size);
+    pb.base[b * 2 + 0] = uU;
+    pb.base[b * 2 + 1] = p61_pow(uU, 65536);
+    uint64_t sum = 0, v = 1;
     hc.csum[b][0] = 0;
     for (int j = 0; j < 16; ++j) {
-      const uint64_t v = p61_pow(u, j + 1);
+      v = p61_mul(v, u);
       hc.limb[b][0][j] = (uint32_t)(v & 0x1FFFFF);
       hc.limb[b][1][j] = (uint32_t)((v >> 21) & 0x1FFFFF);
       hc.limb[b][2][j] = (uint32_t)(v >> 42);
@@ -1249,9 +1023,10 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
       sum = p61_add(sum, v);
       hc.csum[b][j + 1] = sum;
     }
-    for (int q = 0; q < 32; ++q) hc.sub_mul[b][q] = p61_pow(u, 16ULL * q);
+    hc.sub_mul[b][0] = 1;
+    for (int q = 1; q < 32; ++q) hc.sub_mul[b][q] = p61_mul(hc.sub_mul[b][q - 1], v);  // v = u^16
   }
-  PTC_KERNEL("k_pow_tables", s, k_pow_tables, (4 * 8192) / 256, 256, 0, pb, L.tables, L.st);
+  PTC_KERNEL("k_pow_tables", s, k_pow_tables, (4 * 8192) / 256, 256, 0, pb, L.tables, U ? block_size / U : 1u, L.st);
 
   HashArgs a;
   a.tokens = tokens;
@@ -1269,11 +1044,19 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
   a.wide_list = L.wide_list;
   a.st = L.st;
   a.aligned = aligned;
+  a.g = U ? block_size / U : 1;
+  a.tb = tb;
   const bool full = block_size == 16 * G;
   const uint64_t nb = n_tok / block_size < keys_cap ? n_tok / block_size : keys_cap;
   const uint32_t grid = ceil_div_u32(nb, tb);
   if (grid > 0) {
-    switch (G) {
+    if (U == 16)
+      launch_units<16>(grid, s, a, hc);
+    else if (U == 12)
+      launch_units<12>(grid, s, a, hc);
+    else if (U == 8)
+      launch_units<8>(grid, s, a, hc);
+    else switch (G) {
       case 1: launch_hash<1>(grid, s, a, hc, full); break;
       case 2: launch_hash<2>(grid, s, a, hc, full); break;
       case 4: launch_hash<4>(grid, s, a, hc, full); break;
