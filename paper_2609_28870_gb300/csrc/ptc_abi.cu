@@ -152,19 +152,6 @@ __global__ void k_copy_words(const uint32_t* __restrict__ src, uint32_t* dst, ui
   for (uint32_t i = quads * 4 + tid; i < words; i += nth) dst[i] = src[i];
 }
 
-// Earlier calls' error words (deferred, see defer_status) join this call's.
-__global__ void k_carry_err(const uint32_t* err, uint32_t n, DevStatus* st) {
-  grid_dep_sync();
-  if (threadIdx.x < n && err[threadIdx.x]) atomicOr(&st->err, err[threadIdx.x]);
-}
-
-__global__ void k_copy_err(const DevStatus* st, uint32_t* slot, uint64_t* value_slot, uint32_t value_index,
-                           uint32_t value_count) {
-  grid_dep_sync();
-  *slot = st->err;
-  if (value_slot)
-    for (uint32_t i = 0; i < value_count; ++i) value_slot[i] = st->value[value_index + i];
-}
 }  // namespace
 
 ptc_status fill_async(void* p, uint32_t pattern, size_t bytes, cudaStream_t s) {
@@ -288,29 +275,60 @@ __global__ void __launch_bounds__(kRkThreads) k_rank_words(const uint32_t* __res
     run += c[k];
   }
 }
+// The ranks of a small bitmap in one launch of one CTA: warp w owns a
+// contiguous stretch, 32 consecutive words per round.  Up to kRankOne words (a
+// quarter of a million positions) it is done in the time of a launch; the two
+// passes of the general form are launches that it saves.
+constexpr uint32_t kRankOne = 8192;
+__global__ void __launch_bounds__(1024) k_rank_one(const uint32_t* __restrict__ bits, uint32_t nwords,
+                                                   uint32_t* __restrict__ pre, uint64_t* total) {
+  grid_dep_sync();
+  __shared__ uint32_t s_w[32];
+  constexpr int kRounds = kRankOne / 1024;
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  uint32_t c[kRounds], sum = 0;
+#pragma unroll
+  for (int k = 0; k < kRounds; ++k) {
+    const uint32_t i = (w * kRounds + k) * 32 + lane;
+    c[k] = i < nwords ? __popc(bits[i]) : 0u;
+    sum += c[k];
+  }
+  sum = __reduce_add_sync(kFull, sum);
+  if (lane == 0) s_w[w] = sum;
+  __syncthreads();
+  uint32_t x = s_w[lane];
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kFull, x, o);
+    if (lane >= (uint32_t)o) x += y;
+  }
+  uint32_t run = __shfl_sync(kFull, x, w) - s_w[w];
+  if (total && threadIdx.x == 1023) *total = x;
+#pragma unroll
+  for (int k = 0; k < kRounds; ++k) {
+    uint32_t y = c[k];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const uint32_t z = __shfl_up_sync(kFull, y, o);
+      if (lane >= (uint32_t)o) y += z;
+    }
+    const uint32_t i = (w * kRounds + k) * 32 + lane;
+    if (i < nwords) pre[i] = run + y - c[k];
+    run += __shfl_sync(kFull, y, 31);
+  }
+}
 }  // namespace
 
 ptc_status bitmap_ranks(const uint32_t* bits, uint32_t nwords, uint32_t* pre, uint32_t* tcnt, uint32_t* tpre,
                         uint32_t* done, uint64_t* total, cudaStream_t s) {
   if (nwords == 0) return PTC_OK;
   const uint32_t T = rank_tiles(nwords);
+  if (nwords <= kRankOne) {
+    PTC_KERNEL("k_rank_one", s, k_rank_one, 1, 1024, 0, bits, nwords, pre, total);
+    return PTC_OK;
+  }
   PTC_KERNEL("k_rank_count", s, k_rank_count, T, kRkThreads, 0, bits, nwords, T, tcnt, tpre, done, total);
   PTC_KERNEL("k_rank_words", s, k_rank_words, T, kRkThreads, 0, bits, nwords, tpre, pre);
-  return PTC_OK;
-}
-
-ptc_status carry_errors(const uint32_t* err, uint32_t n, DevStatus* st, cudaStream_t s) {
-  if (n == 0) return PTC_OK;
-  if (n > 32) return PTC_ERR_INVALID_ARG;
-  PTC_KERNEL("k_carry_err", s, k_carry_err, 1, 32, 0, err, n, st);
-  return PTC_OK;
-}
-
-ptc_status defer_status(const DevStatus* dev, uint32_t* slot, cudaStream_t stream, uint64_t* value_slot,
-                        uint32_t value_index, uint32_t value_count) {
-  if (cudaGetLastError() != cudaSuccess) return PTC_ERR_CUDA;
-  if (value_index + value_count > 8) return PTC_ERR_INVALID_ARG;
-  PTC_KERNEL("k_copy_err", stream, k_copy_err, 1, 1, 0, dev, slot, value_slot, value_index, value_count);
   return PTC_OK;
 }
 

@@ -547,11 +547,15 @@ __device__ __forceinline__ U128 add_u128(U128 a, U128 b) {
   return r;
 }
 
-// out layout: hits[G] | saved[G] (lo, hi) | total (lo, hi).  One CTA of
+// out layout: hits[G] | saved[G] (lo, hi) | total (lo, hi) | slow.  One CTA of
 // 1,024 threads: an inclusive block scan of (count, depth sum) over the bins.
+// The errors of the stages before join this call's; `out` and `st_host` may be
+// the mapped host stage (then the results and the status need no copies).
 __global__ void __launch_bounds__(1024) k_finalize(const unsigned long long* __restrict__ cnt,
                                                    const unsigned long long* __restrict__ ksum, uint32_t G,
-                                                   uint64_t alpha, uint64_t beta, uint64_t* __restrict__ out) {
+                                                   uint64_t alpha, uint64_t beta, uint64_t* __restrict__ out,
+                                                   const uint32_t* slow, DevStatus* st, const DevStatus* earlier,
+                                                   uint32_t n_earlier, DevStatus* st_host) {
   grid_dep_sync();
   __shared__ unsigned long long s_h[32], s_k[32];
   const uint32_t t = threadIdx.x, lane = t & 31, w = t >> 5;
@@ -584,7 +588,16 @@ __global__ void __launch_bounds__(1024) k_finalize(const unsigned long long* __r
     const U128 tc = add_u128(mul_u64(alpha, hn), mul_u64(beta, kn));
     out[3 * G] = tc.lo;
     out[3 * G + 1] = tc.hi;
+    out[3 * G + 2] = *slow;
   }
+  if (t == 0) {
+    uint32_t e = st->err;
+    for (uint32_t q = 0; q < n_earlier; ++q) e |= earlier[q].err;
+    st->err = e;
+  }
+  __syncthreads();
+  if (st_host && t < sizeof(DevStatus) / 4)
+    reinterpret_cast<uint32_t*>(st_host)[t] = reinterpret_cast<const volatile uint32_t*>(st)[t];
 }
 
 struct CurvesLayout {
@@ -612,7 +625,7 @@ CurvesLayout curves_layout(void* ws, uint64_t n, uint32_t G) {
   L.tile_req = cv.take<uint32_t>(tiles + 1);
   L.zero_bytes = cv.off;
   L.lb_agg = cv.take<RunMax>(tiles);
-  L.out = cv.take<uint64_t>(3 * PTC_MAX_CAPACITIES + 2);
+  L.out = cv.take<uint64_t>(3 * PTC_MAX_CAPACITIES + 3);
   L.total = cv.bytes();
   (void)G;
   return L;
@@ -652,11 +665,13 @@ ptc_status ptc::cost_coeffs(const ptc_cost_model* cm, uint32_t block_size, uint6
   return PTC_OK;
 }
 
+size_t ptc::curves_zero_bytes(uint64_t n) { return curves_layout(nullptr, n, 1).zero_bytes; }
+
 ptc_status ptc::curves_impl(const uint32_t* dist, uint64_t n, const uint64_t* req_blk_off, uint32_t n_req,
                             uint32_t block_size, const ptc_cost_model* cm, const uint64_t* cap_host, uint32_t n_cap,
                             uint64_t* hits_host_out, ptc_u128* saved_host_out, ptc_u128* total_cost_host_out,
                             void* ws, size_t ws_bytes, cudaStream_t stream, const RunsView* runs,
-                            const uint32_t* carry_err, uint32_t n_carry) {
+                            const DevStatus* earlier, uint32_t n_earlier) {
   if (n >= (uint64_t)kNone) return PTC_ERR_OVERFLOW;
   if (!cm || !cap_host || !hits_host_out || !saved_host_out || !total_cost_host_out) return PTC_ERR_INVALID_ARG;
   if (n_cap < 1 || n_cap > PTC_MAX_CAPACITIES) return PTC_ERR_INVALID_ARG;
@@ -671,47 +686,67 @@ ptc_status ptc::curves_impl(const uint32_t* dist, uint64_t n, const uint64_t* re
   if (!ws_ok(ws, ws_bytes, curves_layout(nullptr, n, n_cap).total)) return PTC_ERR_WORKSPACE;
   cudaStream_t s = stream;
   const CurvesLayout L = curves_layout(ws, n, n_cap);
-  if (begin_call(ws, L.zero_bytes, s) != PTC_OK) return PTC_ERR_CUDA;
+  if (!earlier && begin_call(ws, L.zero_bytes, s) != PTC_OK) return PTC_ERR_CUDA;
   HostStage* hs = host_stage();
-  if (n_carry && carry_errors(carry_err, n_carry, L.st, s) != PTC_OK) return PTC_ERR_CUDA;
-  if (n > 0) {
-    PTC_KERNEL("k_heads", s, k_heads, ceil_div_u32(n_req, 256), 256, 0, req_blk_off, n_req, n, L.bitmap, L.tile_req, L.st);
-    CurveArgs a;
-    a.dist = dist;
-    a.n = (uint32_t)n;
-    a.bitmap = L.bitmap;
-    for (uint32_t g = 0; g < n_cap; ++g)
-      a.caps[g] = cap_host[g] >= (uint64_t)kNone ? kNone - 1 : (uint32_t)cap_host[g];
-    a.G = n_cap;
-    a.cnt = L.cnt;
-    a.ksum = L.ksum;
-    a.tile_agg = L.lb_agg;
-    a.st = L.st;
-    a.blk_off = req_blk_off;
-    a.tile_req = L.tile_req;
-    a.R = n_req;
-    a.slow = L.slow;
-    if (runs && runs->used) {
-      const RunsArgs ra{runs->rec_s, runs->sd, runs->bits, runs->wpre};
-      const uint32_t g_r = ceil_div_u32(n_req, 256) < (uint32_t)(2 * num_sms()) ? ceil_div_u32(n_req, 256)
-                                                                                  : (uint32_t)(2 * num_sms());
-      PTC_KERNEL("k_curves_runs", s, k_curves_runs, g_r, 256, 0, a, ra);
-    } else {
-      const uint32_t tiles0 = ceil_div_u32(n, kCvTile);
-      const uint32_t grid0 = tiles0 < (uint32_t)(3 * num_sms()) ? tiles0 : (uint32_t)(3 * num_sms());
-      PTC_KERNEL("k_curves_fast", s, k_curves_fast, grid0, kCvThreads, 0, a);
-    }
-    PTC_KERNEL("k_curves_agg", s, k_curves_agg, ceil_div_u32(n, kCvTile), kCvThreads, 0, dist, (uint32_t)n, L.bitmap, L.lb_agg, L.slow, L.cnt, L.ksum, n_cap);
-    const uint32_t tiles = ceil_div_u32(n, kCvTile);
-    const uint32_t grid = tiles < (uint32_t)(3 * num_sms()) ? tiles : (uint32_t)(3 * num_sms());
+  const bool from_runs = n > 0 && runs && runs->used;
+  CurveArgs a;
+  a.dist = dist;
+  a.n = (uint32_t)n;
+  a.bitmap = L.bitmap;
+  for (uint32_t g = 0; g < n_cap; ++g)
+    a.caps[g] = cap_host[g] >= (uint64_t)kNone ? kNone - 1 : (uint32_t)cap_host[g];
+  a.G = n_cap;
+  a.cnt = L.cnt;
+  a.ksum = L.ksum;
+  a.tile_agg = L.lb_agg;
+  a.st = L.st;
+  a.blk_off = req_blk_off;
+  a.tile_req = L.tile_req;
+  a.R = n_req;
+  a.slow = L.slow;
+  const uint32_t tiles = ceil_div_u32(n, kCvTile);
+  const uint32_t grid = tiles < (uint32_t)(3 * num_sms()) ? tiles : (uint32_t)(3 * num_sms());
+  auto heads = [&]() {
+    PTC_KERNEL("k_heads", s, k_heads, ceil_div_u32(n_req, 256), 256, 0, req_blk_off, n_req, n, L.bitmap, L.tile_req,
+               L.st);
+  };
+  // the running maximum per request, where a distance falls inside one
+  auto scans = [&]() {
+    PTC_KERNEL("k_curves_agg", s, k_curves_agg, tiles, kCvThreads, 0, dist, (uint32_t)n, L.bitmap, L.lb_agg, L.slow,
+               L.cnt, L.ksum, n_cap);
     PTC_KERNEL("k_curves", s, k_curves, grid, kCvThreads, 0, a);
-  }
-  PTC_KERNEL("k_finalize", s, k_finalize, 1, 1024, 0, L.cnt, L.ksum, n_cap, alpha, beta, L.out);
-  const uint64_t* host_out = hs->out;
-  if (copy_to_host_async(hs->out, L.out, sizeof(uint64_t) * (3 * n_cap + 2), s) != PTC_OK) return PTC_ERR_CUDA;
+  };
+  // results and status, waited for
   DevStatus h;
-  const ptc_status rc = end_call(L.st, s, &h);
+  auto finish = [&]() -> ptc_status {
+    const bool staged = hs->dev != nullptr;
+    PTC_KERNEL("k_finalize", s, k_finalize, 1, 1024, 0, L.cnt, L.ksum, n_cap, alpha, beta,
+               staged ? hs->dev->out : L.out, L.slow, L.st, earlier, n_earlier, staged ? &hs->dev->st : nullptr);
+    if (staged) return end_call_staged(s, &h);
+    if (copy_to_host_async(hs->out, L.out, sizeof(uint64_t) * (3 * n_cap + 3), s) != PTC_OK) return PTC_ERR_CUDA;
+    return end_call(L.st, s, &h);
+  };
+  if (from_runs) {
+    const RunsArgs ra{runs->rec_s, runs->sd, runs->bits, runs->wpre};
+    const uint32_t g_r = ceil_div_u32(n_req, 256) < (uint32_t)(2 * num_sms()) ? ceil_div_u32(n_req, 256)
+                                                                                : (uint32_t)(2 * num_sms());
+    PTC_KERNEL("k_curves_runs", s, k_curves_runs, g_r, 256, 0, a, ra);
+  } else if (n > 0) {
+    heads();
+    PTC_KERNEL("k_curves_fast", s, k_curves_fast, grid, kCvThreads, 0, a);
+    scans();
+  }
+  const uint64_t* host_out = hs->out;
+  ptc_status rc = finish();
   if (rc != PTC_OK) return rc;
+  if (from_runs && host_out[3 * n_cap + 2]) {
+    // the distances of some request's runs fall (never so for a root-first
+    // trace): the bins are void, and the scans start them afresh
+    heads();
+    scans();
+    rc = finish();
+    if (rc != PTC_OK) return rc;
+  }
   for (uint32_t g = 0; g < n_cap; ++g) {
     hits_host_out[g] = host_out[g];
     saved_host_out[g].lo = host_out[n_cap + 2 * g];

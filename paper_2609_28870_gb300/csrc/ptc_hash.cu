@@ -13,13 +13,13 @@
 //
 // Kernels
 //   k_block_offsets  per-request block counts -> exclusive scan (look-back),
-//                    validates offsets and timestamp order, max blocks/request
-//   k_pow_tables     u^(B e) for e < 2^32 as two 65,536-entry levels
-//                    (filled up to the longest request)
+//                    validates offsets, timestamp order and session labels;
+//                    CTAs beside those of the scan fill the powers u^(U e),
+//                    two levels of 65,536 entries, as far as a request can reach
 //   k_hash_units     B a multiple of 16, 12 or 8: a unit of U = 16, 12 or 8
 //                    tokens per lane, 32 units at a time, then prefix sums over
 //                    the 256 units of a warp's tile, eight units per lane
-//   k_hash_units_wide  the tiles with a token of 2^27 or more
+//                    (three-limb products where a token reaches 2^27)
 //   k_hash_local     any other B: tokens
 //                    staged through padded shared memory with 16-byte
 //                    loads; each thread hashes 16 tokens (one "sub-chunk")
@@ -45,7 +45,6 @@ constexpr int kWinTokens = 8192 + 256;
 constexpr int kWinWords = kWinTokens + kWinTokens / 16;
 
 constexpr int kEpochOffsets = 1;
-constexpr int kEpochWide = 2;  // st->tile_ctr slot counting the tiles of k_hash_units_wide
 
 // ---------------------------------------------------------------- block scans
 // Exclusive sum over a CTA of kOffThreads threads; returns the CTA total in *total.
@@ -75,13 +74,61 @@ __device__ __forceinline__ uint64_t cta_exclusive_sum(uint64_t v, uint64_t* tota
   return warp_excl + x - v;
 }
 
+// ---------------------------------------------------------------- powers
+// tables[(b*2 + w) * 65536 + e] for base b in {0,1} and U tokens per unit
+// (k_hash_local: a unit is a block)
+//   w = 0: u_b^(U e)          w = 1: u_b^(U 65536 e)
+// The first n_lo and n_hi entries are filled: as many as the longest request
+// that the tokens allow can use.
+constexpr int kPowChunk = 8;  // powers per thread: short dependent chains
+
+struct PowArgs {
+  uint64_t base[4];
+  uint64_t* tables;
+  uint32_t n_lo, n_hi;
+  uint32_t off_tiles;  // CTAs of the offsets' scan; the others fill powers
+};
+inline uint32_t pow_chunks(const PowArgs& p) {
+  return 2 * (ceil_div_u32(p.n_lo, kPowChunk) + ceil_div_u32(p.n_hi, kPowChunk));
+}
+
+__device__ __forceinline__ void fill_powers(const PowArgs& p, uint32_t chunk) {
+  const uint32_t c_lo = (p.n_lo + kPowChunk - 1) / kPowChunk, c_hi = (p.n_hi + kPowChunk - 1) / kPowChunk;
+  uint32_t t = 0, n = p.n_lo;
+  if (chunk >= c_lo + c_hi) {
+    t = 2;
+    chunk -= c_lo + c_hi;
+  }
+  if (chunk >= c_lo) {
+    ++t;
+    chunk -= c_lo;
+    n = p.n_hi;
+    if (chunk >= c_hi) return;
+  }
+  const uint64_t base = p.base[t];
+  const uint32_t e0 = chunk * kPowChunk;
+  uint64_t v = p61_pow(base, e0);
+  uint64_t* out = p.tables + (uint64_t)t * 65536 + e0;
+  for (uint32_t i = 0; i < (uint32_t)kPowChunk && e0 + i < n; ++i) {
+    out[i] = v;
+    v = p61_mul(v, base);
+  }
+}
+
 __global__ void __launch_bounds__(kOffThreads) k_block_offsets(const uint64_t* __restrict__ tok_off,
                                                                const int64_t* __restrict__ ts, uint32_t R,
                                                                uint64_t n_tok, uint32_t B, uint32_t tb,
                                                                uint64_t* __restrict__ blk_off,
                                                                uint32_t* __restrict__ tile_req, uint64_t tile_cap,
-                                                               uint64_t* lb, DevStatus* st) {
+                                                               uint64_t* lb, DevStatus* st,
+                                                               const uint32_t* __restrict__ ses,
+                                                               uint32_t n_session,
+                                                               const __grid_constant__ PowArgs pw) {
   grid_dep_sync();
+  if (blockIdx.x >= pw.off_tiles) {
+    fill_powers(pw, (blockIdx.x - pw.off_tiles) * kOffThreads + threadIdx.x);
+    return;
+  }
   const uint32_t tile = next_tile(st, kEpochOffsets);
   const uint64_t r0 = (uint64_t)tile * kOffTile + (uint64_t)threadIdx.x * kOffPer;
   uint64_t cnt[kOffPer];
@@ -99,6 +146,7 @@ __global__ void __launch_bounds__(kOffThreads) k_block_offsets(const uint64_t* _
         cnt[j] = (b - a) / B;
       }
       if (ts != nullptr && r + 1 < R && ts[r + 1] < ts[r]) err |= kErrUnsorted;
+      if (ses != nullptr && ses[r] >= n_session) err |= kErrInvalid;
       local += cnt[j];
       kmax = cnt[j] > kmax ? cnt[j] : kmax;
     }
@@ -137,18 +185,6 @@ __global__ void __launch_bounds__(kOffThreads) k_block_offsets(const uint64_t* _
   }
 }
 
-// ---------------------------------------------------------------- powers
-// tables[(b*2 + w) * 65536 + e] for base b in {0,1} and U tokens per unit
-// (k_hash_local: a unit is a block)
-//   w = 0: u_b^(U e)          w = 1: u_b^(U 65536 e)
-constexpr int kPowChunk = 8;  // powers per thread: short dependent chains
-
-struct PowBases {
-  uint64_t base[4];
-};
-
-// Only the entries some unit can use are filled: exponents reach at most the
-// longest request's units (st->value[1] blocks of g units).
 // Blocks the key kernels may touch: N as the offsets kernel left it, or none
 // if its look-back gave up (then the offsets are not a prefix sum and must
 // not steer any read; the call reports PTC_ERR_TIMEOUT).
@@ -156,24 +192,6 @@ __device__ __forceinline__ uint64_t blocks_live(const DevStatus* st, uint64_t ke
   if (ld_relaxed_u32(&st->err) & kErrTimeout) return 0;
   const uint64_t N = st->value[0];
   return N < keys_cap ? N : keys_cap;
-}
-
-__global__ void k_pow_tables(PowBases pb, uint64_t* __restrict__ tables, uint32_t g, const DevStatus* st) {
-  grid_dep_sync();
-  const uint32_t gid = blockIdx.x * blockDim.x + threadIdx.x;  // 4 tables x 8192 chunks of kPowChunk
-  const uint32_t t = gid >> 13, chunk = gid & 8191;
-  if (t >= 4) return;
-  const uint64_t kmax = st->value[1] * g;
-  const uint64_t need = (t & 1) ? (kmax >> 16) : (kmax < 65535 ? kmax : 65535);
-  const uint64_t base = pb.base[t];
-  const uint64_t e0 = (uint64_t)chunk * kPowChunk;
-  if (e0 > need) return;
-  uint64_t v = p61_pow(base, e0);
-  uint64_t* out = tables + (uint64_t)t * 65536 + e0;
-  for (int i = 0; i < kPowChunk; ++i) {
-    out[i] = v;
-    v = p61_mul(v, base);
-  }
 }
 
 __device__ __forceinline__ uint64_t pow_at(const uint64_t* __restrict__ lo, const uint64_t* __restrict__ hi,
@@ -221,7 +239,6 @@ struct HashArgs {
   uint32_t* tile_lead;   // per tile: blocks before its first request start (keys left normalised)
   DevStatus* st;
   int aligned;
-  uint32_t* wide_list;  // k_hash_units: tiles left to k_hash_units_wide (their count in st->tile_ctr[kEpochWide])
   uint32_t g, tb;       // k_hash_units: units per block, blocks per tile
 };
 
@@ -604,12 +621,12 @@ __device__ __forceinline__ void unit_sums(ulonglong2* slot, uint32_t lane, uint3
 // writes nothing and is left to k_hash_units_wide.  WIDE = true: three-limb
 // products, exact for every 32-bit token.
 template <int U, bool WIDE>
-__device__ __forceinline__ void hash_units_tile(const HashArgs& a, const HashConsts& c, uint32_t tile, uint64_t N,
+__device__ __forceinline__ bool hash_units_tile(const HashArgs& a, const HashConsts& c, uint32_t tile, uint64_t N,
                                                 ulonglong2* slot, uint32_t* starts) {
   constexpr int NV = U / 4;
   const uint32_t lane = threadIdx.x & 31;
   const uint64_t b0 = (uint64_t)tile * a.tb;
-  if (b0 >= N) return;
+  if (b0 >= N) return false;
   const uint32_t nb = N - b0 < a.tb ? (uint32_t)(N - b0) : a.tb, nu = nb * a.g;
   const uint64_t ntiles = (N + a.tb - 1) / a.tb;
   const uint32_t r_first = a.tile_req[tile];
@@ -733,10 +750,7 @@ __device__ __forceinline__ void hash_units_tile(const HashArgs& a, const HashCon
     }
     slot[unit_slot(v)] = make_ulonglong2(g0, g1);
   }
-  if (!WIDE && __any_sync(kFull, big)) {
-    if (lane == 0) a.wide_list[atomicAdd(&a.st->tile_ctr[kEpochWide], 1u)] = tile;
-    return;
-  }
+  if (!WIDE && __any_sync(kFull, big)) return true;
   __syncwarp();
   // ---- sums: this lane's units 8 lane .. 8 lane + 7 (values below 2^61 + 8)
   const uint32_t rounds = (nu + 31) / 32;
@@ -757,30 +771,28 @@ __device__ __forceinline__ void hash_units_tile(const HashArgs& a, const HashCon
     a.tile_agg[tile] = HashCarry{t.x, t.y, opens != 0};
     a.tile_lead[tile] = lead;
   }
+  return false;
+}
+
+// Kept out of line, so that the three-limb code is not part of every tile's
+// path (nor its registers of it).
+template <int U>
+__device__ __noinline__ void hash_units_wide(const HashArgs& a, const HashConsts& c, uint32_t tile, uint64_t N,
+                                             ulonglong2* slot, uint32_t* starts) {
+  hash_units_tile<U, true>(a, c, tile, N, slot, starts);
 }
 
 template <int U>
-__global__ void __launch_bounds__(kUnitThreads, 16) k_hash_units(HashArgs a, const __grid_constant__ HashConsts c) {
+__global__ void __launch_bounds__(kUnitThreads, 16) k_hash_units(const __grid_constant__ HashArgs a,
+                                                                 const __grid_constant__ HashConsts c) {
   grid_dep_sync();
   __shared__ ulonglong2 s_slot[kUnitWarps][kUnitSlots];
   __shared__ uint32_t s_starts[kUnitWarps][kUnitTile / 32];
-  const uint32_t w = threadIdx.x >> 5;
-  hash_units_tile<U, false>(a, c, blockIdx.x * kUnitWarps + w, blocks_live(a.st, a.keys_cap), s_slot[w], s_starts[w]);
-}
-
-// The tiles k_hash_units left, a persistent grid over the list it wrote.
-template <int U>
-__global__ void __launch_bounds__(kUnitThreads) k_hash_units_wide(HashArgs a, const __grid_constant__ HashConsts c) {
-  grid_dep_sync();
-  __shared__ ulonglong2 s_slot[kUnitWarps][kUnitSlots];
-  __shared__ uint32_t s_starts[kUnitWarps][kUnitTile / 32];
-  const uint32_t w = threadIdx.x >> 5;
+  const uint32_t w = threadIdx.x >> 5, tile = blockIdx.x * kUnitWarps + w;
   const uint64_t N = blocks_live(a.st, a.keys_cap);
-  const uint32_t n_wide = ld_relaxed_u32(&a.st->tile_ctr[kEpochWide]);
-  for (uint32_t j = blockIdx.x * kUnitWarps + w; j < n_wide; j += gridDim.x * kUnitWarps) {
-    const uint32_t tile = a.wide_list[j];
-    if (in_bounds(a.st, tile, (N + a.tb - 1) / a.tb)) hash_units_tile<U, true>(a, c, tile, N, s_slot[w], s_starts[w]);
-    __syncwarp();  // the next tile reuses the slots
+  if (hash_units_tile<U, false>(a, c, tile, N, s_slot[w], s_starts[w])) {
+    __syncwarp();
+    hash_units_wide<U>(a, c, tile, N, s_slot[w], s_starts[w]);
   }
 }
 
@@ -890,10 +902,7 @@ __global__ void __launch_bounds__(kChainWarps * 32) k_hash_carry(const HashCarry
 
 template <int U>
 void launch_units(uint32_t tiles, cudaStream_t s, const HashArgs& a, const HashConsts& c) {
-  const uint32_t grid = ceil_div_u32(tiles, kUnitWarps);
-  PTC_KERNEL("k_hash_units", s, k_hash_units<U>, grid, kUnitThreads, 0, a, c);
-  const uint32_t wgrid = grid < (uint32_t)(2 * num_sms()) ? grid : (uint32_t)(2 * num_sms());
-  PTC_KERNEL("k_hash_units_wide", s, k_hash_units_wide<U>, wgrid, kUnitThreads, 0, a, c);
+  PTC_KERNEL("k_hash_units", s, k_hash_units<U>, ceil_div_u32(tiles, kUnitWarps), kUnitThreads, 0, a, c);
 }
 
 template <int G>
@@ -933,7 +942,6 @@ struct HashLayout {
   uint32_t* tile_lead;
   uint64_t* tables;
   uint32_t* tile_req;
-  uint32_t* wide_list;
   uint64_t hash_tiles;
   size_t zero_bytes;
   size_t total;
@@ -953,7 +961,6 @@ HashLayout hash_layout(void* ws, uint32_t n_req, uint64_t n_tok, uint32_t B, uin
   L.tile_lead = cv.take<uint32_t>(hash_tiles);
   L.tables = cv.take<uint64_t>(4 * 65536);
   L.tile_req = cv.take<uint32_t>(hash_tiles + 1);
-  L.wide_list = cv.take<uint32_t>(hash_tiles);
   L.hash_tiles = hash_tiles;
   L.total = cv.bytes();
   return L;
@@ -963,6 +970,8 @@ HashLayout hash_layout(void* ws, uint32_t n_req, uint64_t n_tok, uint32_t B, uin
 }  // namespace ptc
 
 using namespace ptc;
+
+size_t ptc::hash_lb_words(uint32_t n_req) { return ceil_div_u32(n_req, kOffTile) + 1; }
 
 uint64_t ptc::hash_carry_tiles(uint64_t n_tok, uint32_t block_size) {
   if (block_size == 0) block_size = 1;
@@ -977,40 +986,42 @@ extern "C" size_t ptc_hash_blocks_workspace_bytes(uint32_t n_req, uint64_t n_tok
 ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t* req_tok_off,
                          const int64_t* req_ts_us, uint32_t n_req, uint32_t block_size, uint64_t seed,
                          ptc_u128* keys_out, uint64_t keys_cap, uint64_t* req_blk_off_out,
-                         uint64_t* n_access_host_out, void* ws, size_t ws_bytes, cudaStream_t s, uint64_t* n_slot,
-                         uint32_t* err_slot, KeyCarry* carry) {
+                         uint64_t* n_access_host_out, void* ws, size_t ws_bytes, cudaStream_t s, DevStatus* lent,
+                         uint64_t* lent_lb, KeyCarry* carry, const uint32_t* ses, uint32_t n_session) {
   if (block_size < 1 || block_size > PTC_MAX_BLOCK_SIZE) return PTC_ERR_INVALID_ARG;
   if (req_tok_off == nullptr || req_blk_off_out == nullptr || n_access_host_out == nullptr)
     return PTC_ERR_INVALID_ARG;
   if (n_tok > 0 && tokens == nullptr) return PTC_ERR_INVALID_ARG;
   if (keys_cap > 0 && keys_out == nullptr) return PTC_ERR_INVALID_ARG;
-  const bool deferred = n_slot != nullptr && err_slot != nullptr;
   const HashLayout need = hash_layout(nullptr, n_req, n_tok, block_size, ~0ULL);
   if (!ws_ok(ws, ws_bytes, need.total)) return PTC_ERR_WORKSPACE;
-  const HashLayout L = hash_layout(ws, n_req, n_tok, block_size, ~0ULL);
+  HashLayout L = hash_layout(ws, n_req, n_tok, block_size, ~0ULL);
   *n_access_host_out = 0;
-  if (begin_call(ws, L.zero_bytes, s) != PTC_OK) return PTC_ERR_CUDA;
+  if (lent) {
+    L.st = lent;
+    L.lb_off = lent_lb;
+  } else if (begin_call(ws, L.zero_bytes, s) != PTC_OK) {
+    return PTC_ERR_CUDA;
+  }
   const uint32_t wait_test = test_wait_polls();
   if (wait_test && fill_async(&L.st->wait_test, wait_test, sizeof(uint32_t), s) != PTC_OK) return PTC_ERR_CUDA;
   if (n_req == 0) {
     if (fill_async(req_blk_off_out, 0u, sizeof(uint64_t), s) != PTC_OK) return PTC_ERR_CUDA;
-    if (deferred) return defer_status(L.st, err_slot, s, n_slot, 0);
+    if (lent) return cudaGetLastError() == cudaSuccess ? PTC_OK : PTC_ERR_CUDA;
     DevStatus h;
     return end_call(L.st, s, &h);
   }
   const uint32_t G = chunks_per_block(block_size);
   const bool aligned = (((uintptr_t)tokens) & 15) == 0;
   const uint32_t tb = tile_blocks(block_size), U = unit_tokens(block_size);
-  PTC_KERNEL("k_block_offsets", s, k_block_offsets, ceil_div_u32(n_req, kOffTile), kOffThreads, 0, req_tok_off, req_ts_us, n_req, n_tok, block_size, tb, req_blk_off_out, L.tile_req, L.hash_tiles, L.lb_off, L.st);
-
   // seeded bases and their derived constants
-  PowBases pb;
+  PowArgs pw;
   HashConsts hc;
   for (int b = 0; b < 2; ++b) {
     const uint64_t u = 2 + splitmix64_at(seed, (uint64_t)b) % (kP61 - 3);
     const uint64_t uU = p61_pow(u, U ? U : block_size);
-    pb.base[b * 2 + 0] = uU;
-    pb.base[b * 2 + 1] = p61_pow(uU, 65536);
+    pw.base[b * 2 + 0] = uU;
+    pw.base[b * 2 + 1] = p61_pow(uU, 65536);
     uint64_t sum = 0, v = 1;
     hc.csum[b][0] = 0;
     for (int j = 0; j < 16; ++j) {
@@ -1026,7 +1037,14 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
     hc.sub_mul[b][0] = 1;
     for (int q = 1; q < 32; ++q) hc.sub_mul[b][q] = p61_mul(hc.sub_mul[b][q - 1], v);  // v = u^16
   }
-  PTC_KERNEL("k_pow_tables", s, k_pow_tables, (4 * 8192) / 256, 256, 0, pb, L.tables, U ? block_size / U : 1u, L.st);
+  const uint64_t reach = n_tok / (U ? U : block_size);  // units of the longest request there can be
+  pw.tables = L.tables;
+  pw.n_lo = (uint32_t)(reach < 65535 ? reach + 1 : 65536);
+  pw.n_hi = (uint32_t)((reach >> 16) < 65535 ? (reach >> 16) + 1 : 65536);
+  pw.off_tiles = ceil_div_u32(n_req, kOffTile);
+  PTC_KERNEL("k_block_offsets", s, k_block_offsets, pw.off_tiles + ceil_div_u32(pow_chunks(pw), kOffThreads),
+             kOffThreads, 0, req_tok_off, req_ts_us, n_req, n_tok, block_size, tb, req_blk_off_out, L.tile_req,
+             L.hash_tiles, L.lb_off, L.st, ses, n_session, pw);
 
   HashArgs a;
   a.tokens = tokens;
@@ -1041,7 +1059,6 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
   a.tile_req = L.tile_req;
   a.tile_agg = L.tile_agg;
   a.tile_lead = L.tile_lead;
-  a.wide_list = L.wide_list;
   a.st = L.st;
   a.aligned = aligned;
   a.g = U ? block_size / U : 1;
@@ -1073,7 +1090,7 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
                  L.tile_agg, L.tile_lead, tb, L.st, keys_cap);
     }
   }
-  if (deferred) return defer_status(L.st, err_slot, s, n_slot, 0);
+  if (lent) return cudaGetLastError() == cudaSuccess ? PTC_OK : PTC_ERR_CUDA;
   DevStatus h;
   ptc_status rc = end_call(L.st, s, &h);
   *n_access_host_out = h.value[0];

@@ -1384,8 +1384,8 @@ extern "C" size_t ptc_assign_ids_workspace_bytes(uint64_t n) {
 
 ptc_status ptc::ids_impl(const ptc_u128* keys, uint64_t n, const uint64_t* n_dev, uint32_t* ids_out,
                         uint64_t* n_used_host_out, uint64_t* n_distinct_host_out, void* ws, size_t ws_bytes,
-                        cudaStream_t s, const uint32_t* carry_err, uint32_t n_carry, const KeyCarry* kc,
-                        uint64_t* nd_slot, uint32_t* err_slot, bool full_table, const IdsHint* hint, int method) {
+                        cudaStream_t s, const KeyCarry* kc, DevStatus* lent, bool full_table, const IdsHint* hint,
+                        int method) {
   if (hint && (hint->n_req == 0 || !hint->blk_off || !hint->prior)) return PTC_ERR_INVALID_ARG;
   if (kc && (kc->tile_blocks == 0 || (kc->tile_blocks & (kc->tile_blocks - 1)) != 0)) return PTC_ERR_INVALID_ARG;
   if (method != PTC_IDS_AUTO && method != PTC_IDS_TABLE && method != PTC_IDS_PARTITIONED) return PTC_ERR_INVALID_ARG;
@@ -1399,7 +1399,8 @@ ptc_status ptc::ids_impl(const ptc_u128* keys, uint64_t n, const uint64_t* n_dev
   const uint32_t hreq = hint ? hint->n_req : 0;
   const bool pd_layout = ids_partitioned(n, method);
   if (!ws_ok(ws, ws_bytes, ids_layout(nullptr, n, hreq, pd_layout).total)) return PTC_ERR_WORKSPACE;
-  const IdsLayout L = ids_layout(ws, n, hreq, pd_layout);
+  IdsLayout L = ids_layout(ws, n, hreq, pd_layout);
+  if (lent) L.st = lent;
   const PriorHint ph = hint ? PriorHint{hint->blk_off, hint->prior, hint->order, hint->pos, hint->n_req, L.lam, L.tile_req}
                             : PriorHint{nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr};
   const bool pd = pd_layout && !full_table;  // the first attempt deduplicates by partitions
@@ -1411,7 +1412,7 @@ ptc_status ptc::ids_impl(const ptc_u128* keys, uint64_t n, const uint64_t* n_dev
                             {L.table, fill_table ? sizeof(ulonglong2) << log2m : 0, ~0u},
                             {L.bits, n > 0 ? sizeof(uint32_t) * L.nwords : 0, 0u},
                             {L.pd_ubits, L.pd_ubits && n > 0 && !table ? sizeof(uint32_t) * L.nwords : 0, 0u}};
-    return fill_many_async(zf, 4, s) == PTC_OK && carry_errors(carry_err, n_carry, L.st, s) == PTC_OK;
+    return fill_many_async(zf, 4, s) == PTC_OK;
   };
   const ulonglong2* k = reinterpret_cast<const ulonglong2*>(keys);
   const uint32_t n32 = (uint32_t)n;
@@ -1482,10 +1483,10 @@ ptc_status ptc::ids_impl(const ptc_u128* keys, uint64_t n, const uint64_t* n_dev
   const uint32_t first_log2m = full_table ? L.log2m : small_table_log2(n);
   if (!start(first_log2m, !pd)) return PTC_ERR_CUDA;
   DevStatus h{};
-  if (nd_slot && err_slot) {  // one attempt, nothing waits
+  if (lent) {  // one attempt, nothing waits
     const uint32_t lg = first_log2m;
     if (n > 0 && !(pd ? run_pd() : run(lg, lg < L.log2m ? kSmallProbeCap : ~0ULL))) return PTC_ERR_CUDA;
-    return defer_status(L.st, err_slot, s, nd_slot, 0, 2);
+    return cudaGetLastError() == cudaSuccess ? PTC_OK : PTC_ERR_CUDA;
   }
   if (n > 0) {
     const uint32_t small = first_log2m;
@@ -1510,8 +1511,7 @@ ptc_status ptc::ids_impl(const ptc_u128* keys, uint64_t n, const uint64_t* n_dev
 
 extern "C" ptc_status ptc_assign_ids(const ptc_u128* keys, uint64_t n, uint32_t* ids_out, uint64_t* n_distinct_host_out,
                                      void* ws, size_t ws_bytes, void* stream) {
-  return ptc::ids_impl(keys, n, nullptr, ids_out, nullptr, n_distinct_host_out, ws, ws_bytes, (cudaStream_t)stream,
-                       nullptr, 0);
+  return ptc::ids_impl(keys, n, nullptr, ids_out, nullptr, n_distinct_host_out, ws, ws_bytes, (cudaStream_t)stream);
 }
 
 bool ptc::ids_table_in_dram(uint64_t n) { return n / 3 + 64 > (1ULL << kL2TableLog2); }
@@ -1535,7 +1535,7 @@ extern "C" ptc_status ptc_assign_ids_ex(const ptc_u128* keys, uint64_t n, const 
   if (n > 0 && n_req > 0 && (!req_blk_off || !req_prior)) return PTC_ERR_INVALID_ARG;
   const IdsHint h{req_blk_off, req_prior, n_req, nullptr, nullptr};
   return ptc::ids_impl(keys, n, nullptr, ids_out, nullptr, n_distinct_host_out, ws, ws_bytes, (cudaStream_t)stream,
-                       nullptr, 0, nullptr, nullptr, nullptr, false, n > 0 && n_req > 0 ? &h : nullptr, method);
+                       nullptr, nullptr, false, n > 0 && n_req > 0 ? &h : nullptr, method);
 }
 
 extern "C" ptc_status ptc_assign_ids_prior(const ptc_u128* keys, uint64_t n, const uint64_t* req_blk_off,
@@ -1544,10 +1544,10 @@ extern "C" ptc_status ptc_assign_ids_prior(const ptc_u128* keys, uint64_t n, con
   if (n > 0 && (n_req == 0 || !req_blk_off || !req_prior)) return PTC_ERR_INVALID_ARG;
   if (n == 0 || n_req == 0)
     return ptc::ids_impl(keys, n, nullptr, ids_out, nullptr, n_distinct_host_out, ws, ws_bytes,
-                         (cudaStream_t)stream, nullptr, 0);
+                         (cudaStream_t)stream);
   const IdsHint h{req_blk_off, req_prior, n_req, nullptr, nullptr};
   return ptc::ids_impl(keys, n, nullptr, ids_out, nullptr, n_distinct_host_out, ws, ws_bytes, (cudaStream_t)stream,
-                       nullptr, 0, nullptr, nullptr, nullptr, false, &h);
+                       nullptr, nullptr, false, &h);
 }
 
 size_t ptc::session_prior_bytes(uint32_t n_req) {

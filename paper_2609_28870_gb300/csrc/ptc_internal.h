@@ -109,7 +109,7 @@ constexpr size_t kStatsHostWords = sizeof(ptc_trace_summary) / 8 + PTC_MAX_CAPAC
 // had.  Valid until the thread's next call.
 struct HostStage {
   DevStatus st;
-  uint64_t out[3 * PTC_MAX_CAPACITIES + 2];
+  uint64_t out[3 * PTC_MAX_CAPACITIES + 3];
   alignas(16) uint64_t stats[kStatsHostWords];
   HostStage* dev;  // the same memory as seen by kernels (mapped), or null
 };
@@ -151,8 +151,16 @@ inline ptc_status end_call(const DevStatus* dev, cudaStream_t stream, DevStatus*
   return status_of(host_copy->err);
 }
 
-// Instead of waiting for a call's status, queue a copy of its error word to
-// `slot`, for a later call that does wait to fold in (ptc_pipeline).
+// end_call after a kernel that wrote the status block to the (mapped) host
+// stage itself.
+inline ptc_status end_call_staged(cudaStream_t stream, DevStatus* host_copy) {
+  if (cudaGetLastError() != cudaSuccess) return PTC_ERR_CUDA;
+  if (cudaStreamSynchronize(stream) != cudaSuccess) return PTC_ERR_CUDA;
+  *host_copy = host_stage()->st;
+  timer_resolve();
+  return status_of(host_copy->err);
+}
+
 // Ranks over a bitmap (ptc_abi.cu): pre[w] = set bits in words [0, w) for
 // w < nwords, by a count per tile of kRankTile words, the last CTA's prefix
 // over the tiles, then a pass per word.  Scratch: tcnt and tpre of
@@ -162,13 +170,6 @@ constexpr uint32_t kRankTile = 2048;
 inline uint32_t rank_tiles(uint32_t nwords) { return (nwords + kRankTile - 1) / kRankTile; }
 ptc_status bitmap_ranks(const uint32_t* bits, uint32_t nwords, uint32_t* pre, uint32_t* tcnt, uint32_t* tpre,
                         uint32_t* done, uint64_t* total, cudaStream_t s);
-
-// OR the n (at most 32) deferred error words at `err` into st->err.
-ptc_status carry_errors(const uint32_t* err, uint32_t n, DevStatus* st, cudaStream_t s);
-// With `value_slot`, value[value_index .. value_index + value_count) of the
-// status block is copied there too.
-ptc_status defer_status(const DevStatus* dev, uint32_t* slot, cudaStream_t stream, uint64_t* value_slot = nullptr,
-                        uint32_t value_index = 0, uint32_t value_count = 1);
 
 // Streaming multiprocessors of the current device (persistent grids).
 inline int num_sms() {
@@ -204,23 +205,31 @@ struct KeyCarry {
 };
 uint64_t hash_carry_tiles(uint64_t n_tok, uint32_t block_size);
 
-// Stage a1 (ptc_hash.cu).  With `n_slot` and `err_slot` (device memory) the
-// final wait is replaced by defer_status: N goes to *n_slot, the error word
-// to *err_slot, and *n_access_host_out is left 0.  With `carry` the keys are
-// left without the cross-tile carry, which goes to carry's arrays instead.
+// In ptc_pipeline no stage but the last waits for its own status: the stages
+// get status blocks of their own, side by side, which later stages' kernels
+// read (N and D as well as errors), and whatever else of theirs must start at
+// zero lies there too, cleared by one launch for all.
+enum { kStHash = 0, kStSessions = 1, kStIds = 2, kStReuse = 3, kStStack = 4, kStStages = 5 };
+
+// Stage a1 (ptc_hash.cu).  With `lent` (a status block) and `lent_lb`
+// (hash_lb_words() words), both zeroed, nothing is cleared and nothing waits:
+// N is left in lent->value[0], and *n_access_host_out is left 0.  With `carry`
+// the keys are left without the cross-tile carry, which goes to carry's arrays
+// instead.  With `ses` every request's label is checked against n_session.
+size_t hash_lb_words(uint32_t n_req);
 ptc_status hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t* req_tok_off, const int64_t* req_ts_us,
                      uint32_t n_req, uint32_t block_size, uint64_t seed, ptc_u128* keys_out, uint64_t keys_cap,
                      uint64_t* req_blk_off_out, uint64_t* n_access_host_out, void* ws, size_t ws_bytes,
-                     cudaStream_t s, uint64_t* n_slot, uint32_t* err_slot, KeyCarry* carry = nullptr);
+                     cudaStream_t s, DevStatus* lent, uint64_t* lent_lb, KeyCarry* carry = nullptr,
+                     const uint32_t* ses = nullptr, uint32_t n_session = 0);
 // Stage a2 (ptc_ids.cu) over n_ub keys, of which the first min(*n_dev, n_ub)
-// are used when `n_dev` (device memory) is given.  Error words at
-// `carry_err` join the call's own.  Reports the number used and D.  With
-// `kc` each key gets its tile's carry as it is read.
-// With `nd_slot` and `err_slot` (device memory) the call does not wait: it
-// makes one attempt (the partitioned dedup, or the table's small first
-// size) and leaves D in nd_slot[0], the number of keys used in nd_slot[1]
-// and its error word in *err_slot (an attempt that outran its table shows as
-// exactly kErrTableFull; redo the stage then with `full_table`).
+// are used when `n_dev` (device memory) is given.  Reports the number used and
+// D.  With `kc` each key gets its tile's carry as it is read.  With `lent` (a
+// zeroed status block) the call does not wait: it makes one attempt (the
+// partitioned dedup, or the table's small first size) and leaves D in
+// lent->value[0] and the number of keys used in lent->value[1] (an attempt that
+// outran its table shows as exactly kErrTableFull; redo the stage then with
+// `full_table`).
 // The prior-request hint of stage a2 (ptc_assign_ids_prior): prior[r] is an
 // earlier request whose blocks request r is likely to repeat, or PTC_NONE.
 struct IdsHint {
@@ -244,39 +253,59 @@ void session_prior(const uint32_t* req_session, uint32_t n_req, uint32_t n_sessi
                    uint32_t* pos = nullptr);
 ptc_status ids_impl(const ptc_u128* keys, uint64_t n_ub, const uint64_t* n_dev, uint32_t* ids_out,
                     uint64_t* n_used_host_out, uint64_t* n_distinct_host_out, void* ws, size_t ws_bytes,
-                    cudaStream_t s, const uint32_t* carry_err, uint32_t n_carry, const KeyCarry* kc = nullptr,
-                    uint64_t* nd_slot = nullptr, uint32_t* err_slot = nullptr, bool full_table = false,
+                    cudaStream_t s, const KeyCarry* kc = nullptr, DevStatus* lent = nullptr, bool full_table = false,
                     const IdsHint* hint = nullptr, int method = PTC_IDS_AUTO);
+// Stage c with the runs it found in *view; with `lent` (its zeroed status
+// block, counters and key bitmap) it does not wait at its end.
+struct StackLent {
+  DevStatus* st = nullptr;
+  uint32_t* done = nullptr;   // kStackDone counters
+  uint32_t* kbits = nullptr;  // stack_key_words(n) words
+};
+constexpr uint32_t kStackDone = 64;
+inline size_t stack_key_words(uint64_t n) { return n / 32 + 2; }
 ptc_status stack_distance_view(const uint32_t* prev, uint64_t n, uint32_t* dist_out, int method, void* ws,
-                               size_t ws_bytes, cudaStream_t s, RunsView* view, uint32_t* defer_err);
-// Stage b as ptc_reuse_indices does it (ptc_reuse.cu); with `defer_err` the
-// final wait is replaced by defer_status.  With `din`, stage a2 has not
-// waited: n and n_distinct are upper bounds, the kernels before this stage's
-// own wait read the real ones from din->nd (nd[0] = D, nd[1] = accesses),
-// and that wait reports them, with stage a2's error word, in *hout.  If that
-// word is not 0 the call returns PTC_OK at once and its results are void.
+                               size_t ws_bytes, cudaStream_t s, RunsView* view, const StackLent* lent);
+// Stage b as ptc_reuse_indices does it (ptc_reuse.cu); with `lent` (its zeroed
+// status block, counters and cut bitmap) it does not wait at its end.  With
+// `din`, stage a2 has not waited: n and n_distinct are upper bounds, the kernels
+// before this stage's own wait read the real ones from din->nd (nd[0] = D, nd[1]
+// = accesses), and that wait reports them, with the error words of the n_errs
+// status blocks at din->errs, in *hout.  If those are not 0 the call returns
+// PTC_OK at once and its results are void.
+struct ReuseLent {
+  DevStatus* st = nullptr;
+  uint32_t* done = nullptr;  // kReuseDone counters
+  uint32_t* cut = nullptr;   // reuse_cut_words(D) words
+};
+constexpr uint32_t kReuseDone = 64;
+inline size_t reuse_cut_words(uint64_t n_distinct) { return (n_distinct + 1) / 32 + 1; }
 struct ReuseDevIn {
   const uint64_t* nd;
-  const uint32_t* ids_err;
+  const DevStatus* errs;
+  uint32_t n_errs;
 };
 struct ReuseHostOut {
   uint64_t n = 0, D = 0;
   uint32_t ids_err = 0;
 };
 ptc_status reuse_view(const uint32_t* ids, uint64_t n, uint64_t n_distinct, uint32_t* prev_out, uint32_t* next_out,
-                      void* ws, size_t ws_bytes, cudaStream_t s, uint32_t* defer_err, const ReuseDevIn* din = nullptr,
-                      ReuseHostOut* hout = nullptr);
+                      void* ws, size_t ws_bytes, cudaStream_t s, const ReuseLent* lent,
+                      const ReuseDevIn* din = nullptr, ReuseHostOut* hout = nullptr);
 // The per-block cost as cost(k) = alpha + beta k for block size B (R7: every
 // cost kind is affine in the depth k); PTC_ERR_OVERFLOW if a coefficient
 // exceeds 64 bits, PTC_ERR_INVALID_ARG for an unknown kind (ptc_curves.cu).
 ptc_status cost_coeffs(const ptc_cost_model* cm, uint32_t block_size, uint64_t* alpha, uint64_t* beta);
 // Stage d (ptc_curves.cu); with `runs` (from stack_distance_view) the curves
-// come from the runs instead of a pass over every distance.
+// come from the runs instead of a pass over every distance.  With `earlier`
+// (the pipeline) the error words of n_earlier status blocks join the call's,
+// and the first curves_zero_bytes(n) bytes of ws are zero already.
+size_t curves_zero_bytes(uint64_t n);
 ptc_status curves_impl(const uint32_t* dist, uint64_t n, const uint64_t* req_blk_off, uint32_t n_req,
                        uint32_t block_size, const ptc_cost_model* cm, const uint64_t* cap_host, uint32_t n_cap,
                        uint64_t* hits_host_out, ptc_u128* saved_host_out, ptc_u128* total_cost_host_out, void* ws,
-                       size_t ws_bytes, cudaStream_t s, const RunsView* runs, const uint32_t* carry_err = nullptr,
-                       uint32_t n_carry = 0);
+                       size_t ws_bytes, cudaStream_t s, const RunsView* runs, const DevStatus* earlier = nullptr,
+                       uint32_t n_earlier = 0);
 
 // Stage c on the matrix over every access (ptc_wavelet.cu); the C entry
 // points in ptc_runs.cu choose between it and the matrix over runs.  With

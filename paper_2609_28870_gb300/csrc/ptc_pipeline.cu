@@ -19,12 +19,16 @@ struct PipeLayout {
   size_t scratch_bytes;
   void* curves;
   size_t curves_bytes;
-  uint32_t* defer;  // error words of stages a1, prior, b, c and a2, read with a later stage's
   uint32_t* prior;  // previous request of each request's session (sessions given)
   uint32_t* order;  // the requests in session order, and the place of each in it (sessions given)
   uint32_t* pos;
-  uint64_t* n_slot;  // N as stage a1 left it, for stage a2
-  uint64_t* nd_slot;  // D and N as stage a2 left them, for stage b
+  // cleared by one launch: the stages' status blocks and what else of theirs
+  // must start at zero (stage d's lies at the front of `curves`, right after)
+  ptc::DevStatus* st;
+  uint64_t* hash_lb;
+  ptc::ReuseLent reuse;
+  ptc::StackLent stack;
+  size_t zero_bytes;
   ulonglong2* carry;  // per hash tile: the carry stage a2 adds to the keys (when they are not returned)
   uint32_t* lead;
   size_t total;
@@ -52,14 +56,21 @@ PipeLayout pipe_layout(void* ws, uint32_t n_req, uint64_t n_tok, uint32_t B, uin
   L.dist = dist ? nullptr : cv.take<uint32_t>(n);
   L.scratch_bytes = stage_scratch_bytes(n_req, n_tok, B, n_cap);
   L.scratch = cv.take<unsigned char>(L.scratch_bytes);
+  L.st = cv.take<ptc::DevStatus>(ptc::kStStages);
+  const size_t zero_off = cv.off - ptc::kStStages * sizeof(ptc::DevStatus);
+  L.hash_lb = cv.take<uint64_t>(ptc::hash_lb_words(n_req));
+  L.reuse.st = L.st ? L.st + ptc::kStReuse : nullptr;
+  L.reuse.done = cv.take<uint32_t>(ptc::kReuseDone);
+  L.reuse.cut = cv.take<uint32_t>(ptc::reuse_cut_words(n));
+  L.stack.st = L.st ? L.st + ptc::kStStack : nullptr;
+  L.stack.done = cv.take<uint32_t>(ptc::kStackDone);
+  L.stack.kbits = cv.take<uint32_t>(ptc::stack_key_words(n));
   L.curves_bytes = ptc_curves_workspace_bytes(n_tok / B, n_req, n_cap);
   L.curves = cv.take<unsigned char>(L.curves_bytes);
-  L.defer = cv.take<uint32_t>(5);
+  L.zero_bytes = cv.off - L.curves_bytes + ptc::curves_zero_bytes(n_tok / B) - zero_off;
   L.prior = cv.take<uint32_t>(n_req ? n_req : 1);
   L.order = cv.take<uint32_t>(n_req ? n_req : 1);
   L.pos = cv.take<uint32_t>(n_req ? n_req : 1);
-  L.n_slot = cv.take<uint64_t>(1);
-  L.nd_slot = cv.take<uint64_t>(2);
   const uint64_t ct = keys ? 1 : ptc::hash_carry_tiles(n_tok, B);
   L.carry = cv.take<ulonglong2>(ct);
   L.lead = cv.take<uint32_t>(ct);
@@ -102,58 +113,61 @@ extern "C" ptc_status ptc_pipeline(const uint32_t* tokens, uint64_t n_tok, const
   *n_access_host_out = 0;
   *n_distinct_host_out = 0;
   cudaStream_t s = (cudaStream_t)stream;
-  // Stages a1, a2, b and c do not wait for their own status.  a1's error
-  // word and N go to device slots that stage a2 reads (its grids cover N's
-  // upper bound, n_tok / B); a2's error word, N and D go to slots that stage
-  // b's first kernels read, and reach the host with stage b's own wait; b's
-  // and c's error words are read with stage d's.
-  if (ptc::fill_async(L.defer, 0u, 5 * sizeof(uint32_t), s) != PTC_OK) return PTC_ERR_CUDA;
+  // Stages a1, a2, b and c do not wait for their own status: N, D and errors
+  // stay in the stages' status blocks, where later kernels read them (stage
+  // a2's grids cover N's upper bound, n_tok / B); stage b's own wait brings
+  // a1's and a2's to the host, stage d's the others.
+  if (ptc::fill_async(L.st, 0u, L.zero_bytes, s) != PTC_OK) return PTC_ERR_CUDA;
   // with sessions, stage a2 is told the previous request of each request's
   // session, whose blocks the request mostly repeats (computed here, in the
   // scratch region, before stage a1 takes it over); only a DRAM-sized id
-  // table gains from it
-  // (the labels are checked whenever they are given)
+  // table gains from it.  The labels are checked whenever they are given (by
+  // stage a1 where there is no hint).
   const bool hinted = req_session != nullptr && n_req > 0 && ptc::ids_table_in_dram(cap);
-  if (req_session && n_req > 0)
-    ptc::session_prior(req_session, n_req, n_session, L.prior, L.scratch, s, &L.defer[1], L.order, L.pos);
+  if (hinted)
+    ptc::session_prior(req_session, n_req, n_session, L.prior, L.scratch, s, &L.st[ptc::kStSessions].err, L.order,
+                       L.pos);
   const ptc::IdsHint hint{blk, L.prior, n_req, L.order, L.pos};
   const ptc::IdsHint* hp = hinted ? &hint : nullptr;
   // keys the caller does not take skip their carry pass: stage a2 adds the
   // carry as it reads them
   ptc::KeyCarry kc{L.carry, L.lead, 1};
   ptc::KeyCarry* kcp = keys_out ? nullptr : &kc;
+  const uint64_t* n_dev = &L.st[ptc::kStHash].value[0];
   ptc_status rc = ptc::hash_impl(tokens, n_tok, req_tok_off, req_ts_us, n_req, block_size, seed, keys, cap, blk,
-                                 &unused, L.scratch, L.scratch_bytes, s, L.n_slot, &L.defer[0], kcp);
+                                 &unused, L.scratch, L.scratch_bytes, s, &L.st[ptc::kStHash], L.hash_lb, kcp,
+                                 hinted ? nullptr : req_session, n_session);
   if (rc != PTC_OK) return rc;
-  rc = ptc::ids_impl(keys, cap, L.n_slot, ids, &n, &d, L.scratch, L.scratch_bytes, s, &L.defer[0], 2, kcp,
-                     L.nd_slot, &L.defer[4], false, hp);
+  rc = ptc::ids_impl(keys, cap, n_dev, ids, &n, &d, L.scratch, L.scratch_bytes, s, kcp, &L.st[ptc::kStIds], false, hp);
   if (rc != PTC_OK) return rc;
-  const ptc::ReuseDevIn din{L.nd_slot, &L.defer[4]};
+  static_assert(ptc::kStHash == 0 && ptc::kStSessions == 1 && ptc::kStIds == 2, "stage b reads the first three");
+  const ptc::ReuseDevIn din{&L.st[ptc::kStIds].value[0], L.st, 3};
   ptc::ReuseHostOut hout;
-  rc = ptc::reuse_view(ids, cap, cap, prev, next, L.scratch, L.scratch_bytes, s, &L.defer[2], &din, &hout);
+  rc = ptc::reuse_view(ids, cap, cap, prev, next, L.scratch, L.scratch_bytes, s, &L.reuse, &din, &hout);
   *n_access_host_out = n = hout.n;
   *n_distinct_host_out = d = hout.D;
   if (rc != PTC_OK) return rc;
   if (hout.ids_err) {
     // stage a2's first attempt outran its table (or a1 / a2 failed): redo a2
     // with the full table, waiting for it, then stage b with the host's N
-    // and D
+    // and D (its status block holds the word that kept it off the void ids)
     if (hout.ids_err != ptc::kErrTableFull) return ptc::status_of(hout.ids_err);
-    rc = ptc::ids_impl(keys, cap, L.n_slot, ids, &n, &d, L.scratch, L.scratch_bytes, s, &L.defer[0], 2, kcp, nullptr,
-                       nullptr, true, hp);
+    rc = ptc::ids_impl(keys, cap, n_dev, ids, &n, &d, L.scratch, L.scratch_bytes, s, kcp, nullptr, true, hp);
     *n_access_host_out = n;
     *n_distinct_host_out = d;
     if (rc != PTC_OK) return rc;
-    if (n > 0) rc = ptc::reuse_view(ids, n, d, prev, next, L.scratch, L.scratch_bytes, s, &L.defer[2]);
+    if (ptc::fill_async(L.reuse.st, 0u, sizeof(ptc::DevStatus), s) != PTC_OK) return PTC_ERR_CUDA;
+    if (n > 0) rc = ptc::reuse_view(ids, n, d, prev, next, L.scratch, L.scratch_bytes, s, nullptr);
     if (rc != PTC_OK) return rc;
   }
   ptc::RunsView runs;
   if (n > 0) {
-    rc = ptc::stack_distance_view(prev, n, dist, PTC_SD_AUTO, L.scratch, L.scratch_bytes, s, &runs, &L.defer[3]);
+    rc = ptc::stack_distance_view(prev, n, dist, PTC_SD_AUTO, L.scratch, L.scratch_bytes, s, &runs, &L.stack);
     if (rc != PTC_OK) return rc;
   }
+  static_assert(ptc::kStStack == ptc::kStReuse + 1, "stage d reads both");
   return ptc::curves_impl(dist, n, blk, n_req, block_size, cm, cap_host, n_cap, hits_host_out, saved_host_out,
-                          total_cost_host_out, L.curves, L.curves_bytes, s, &runs, &L.defer[2], 2);
+                          total_cost_host_out, L.curves, L.curves_bytes, s, &runs, &L.st[ptc::kStReuse], 2);
 }
 
 // ptc_pipeline_host: the same path for a trace in host memory.  The trace is

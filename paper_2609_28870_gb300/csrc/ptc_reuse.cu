@@ -46,7 +46,8 @@ struct IrArgs {
   const uint32_t* ids;
   uint32_t n, D, ntiles;  // with nd: n is an upper bound, and D and the used n come from nd
   const uint64_t* nd;     // device: nd[0] = D, nd[1] = accesses (stage a2 did not wait), or null
-  const uint32_t* ext_err;  // device: stage a2's error word, reported in value[6], or null
+  const DevStatus* errs;  // device: the n_errs status blocks of stages a1 and a2, whose errors go to value[6]
+  uint32_t n_errs;
   uint32_t* tcnt;
   uint32_t* tpre;     // runs before each tile; tpre[ntiles] = number of runs
   uint32_t* done;
@@ -131,11 +132,12 @@ __device__ __forceinline__ IrArgs resolved(const IrArgs& in) {
   return a;
 }
 
-// Stage a2's D, N and error word go to the status block.  With an error the
-// ids are void: this call's own error word keeps the kernels after this one
-// from reading them, and the caller learns stage a2's.
+// Stage a2's D and N and the errors so far go to the status block.  With an
+// error the ids are void: this call's own error word keeps the kernels after
+// this one from reading them, and the caller learns the earlier ones.
 __device__ __forceinline__ bool ids_void(const IrArgs& in, const IrArgs& a) {
-  const uint32_t ext = in.ext_err ? *in.ext_err : 0u;
+  uint32_t ext = 0;
+  for (uint32_t q = 0; q < in.n_errs; ++q) ext |= in.errs[q].err;
   if (in.nd && blockIdx.x == 0 && threadIdx.x == 0) {
     a.st->value[4] = in.nd[1];
     a.st->value[5] = in.nd[0];
@@ -487,17 +489,17 @@ struct ReuseLayout {
 // (all of them when the run path is forced: there are at most n).
 uint64_t incidence_cap(uint64_t n, bool forced) { return forced ? n + 64 : n / 4 + 64; }
 
-ReuseLayout reuse_layout(void* ws, uint64_t n, uint64_t D, bool forced) {
+ReuseLayout reuse_layout(void* ws, uint64_t n, uint64_t D, bool forced, const ReuseLent* lent = nullptr) {
   ReuseLayout L;
   Carver cv(ws);
   const uint64_t nn = n ? n : 1;
   L.ntiles = ceil_div_u32(nn, kITile);
-  L.nwords = (uint32_t)((D + 1) / 32 + 1);
+  L.nwords = (uint32_t)reuse_cut_words(D);
   L.btiles = ceil_div_u32(L.nwords, kBmTile);
   L.rtiles_max = ceil_div_u32(nn, kRunTile);
   L.kcap = incidence_cap(nn, forced);
   L.st = cv.take<DevStatus>(1);
-  L.done = cv.take<uint32_t>(64);
+  L.done = cv.take<uint32_t>(kReuseDone);
   L.zero_bytes = cv.off;
   L.tcnt = cv.take<uint32_t>(L.ntiles + 1);
   L.tpre = cv.take<uint32_t>(L.ntiles + 1);
@@ -518,6 +520,11 @@ ReuseLayout reuse_layout(void* ws, uint64_t n, uint64_t D, bool forced) {
   L.in0 = cv.take<uint32_t>(L.kcap);
   L.sort_ws = cv.take<unsigned char>(sort_pairs_bytes(L.kcap));
   L.total = cv.bytes();
+  if (lent) {
+    L.st = lent->st;
+    L.done = lent->done;
+    L.cut = lent->cut;
+  }
   return L;
 }
 
@@ -528,12 +535,14 @@ uint32_t bits_for(uint64_t v) {  // bits to hold values below v
 }
 
 ptc_status reuse_by_runs(const uint32_t* ids, uint64_t n, uint64_t D, uint32_t* prev_out, uint32_t* next_out, void* ws,
-                         size_t ws_bytes, cudaStream_t s, bool forced, uint32_t* defer_err = nullptr,
+                         size_t ws_bytes, cudaStream_t s, bool forced, const ReuseLent* lent = nullptr,
                          const ReuseDevIn* din = nullptr, ReuseHostOut* hout = nullptr) {
-  const ReuseLayout L = reuse_layout(ws, n, D, forced);
+  const ReuseLayout L = reuse_layout(ws, n, D, forced, lent);
   if (!ws_ok(ws, ws_bytes, L.total)) return PTC_ERR_WORKSPACE;
-  const FillRange zf[2] = {{ws, L.zero_bytes, 0u}, {L.cut, sizeof(uint32_t) * L.nwords, 0u}};
-  if (fill_many_async(zf, 2, s) != PTC_OK) return PTC_ERR_CUDA;
+  if (!lent) {
+    const FillRange zf[2] = {{ws, L.zero_bytes, 0u}, {L.cut, sizeof(uint32_t) * L.nwords, 0u}};
+    if (fill_many_async(zf, 2, s) != PTC_OK) return PTC_ERR_CUDA;
+  }
   IrArgs a;
   a.ids = ids;
   a.n = (uint32_t)n;
@@ -548,7 +557,8 @@ ptc_status reuse_by_runs(const uint32_t* ids, uint64_t n, uint64_t D, uint32_t* 
   a.max_runs = (uint32_t)(L.kcap < kNone ? L.kcap : kNone - 1);
   a.st = L.st;
   a.nd = din ? din->nd : nullptr;
-  a.ext_err = din ? din->ids_err : nullptr;
+  a.errs = din ? din->errs : nullptr;
+  a.n_errs = din ? din->n_errs : 0;
   // the count with 16-byte loads when the ids allow them (measured faster);
   // the marking pass stays one access per lane and round (the 16-byte form
   // of it measured slower: 0.77 against 0.70 ms on the mixed 10B-token trace)
@@ -615,20 +625,20 @@ ptc_status reuse_by_runs(const uint32_t* ids, uint64_t n, uint64_t D, uint32_t* 
   const uint32_t fill_blocks = ceil_div_u32(K, 256) < (uint32_t)(8 * num_sms()) ? ceil_div_u32(K, 256)
                                                                                 : (uint32_t)(8 * num_sms());
   PTC_KERNEL("k_ir_fill", s, k_ir_fill, fill_blocks, 256, 0, f);
-  if (defer_err) return defer_status(L.st, defer_err, s);
+  if (lent) return cudaGetLastError() == cudaSuccess ? PTC_OK : PTC_ERR_CUDA;
   return end_call(L.st, s, &h);
 }
 
 }  // namespace
 
 ptc_status reuse_view(const uint32_t* ids, uint64_t n, uint64_t n_distinct, uint32_t* prev_out, uint32_t* next_out,
-                      void* ws, size_t ws_bytes, cudaStream_t s, uint32_t* defer_err, const ReuseDevIn* din,
+                      void* ws, size_t ws_bytes, cudaStream_t s, const ReuseLent* lent, const ReuseDevIn* din,
                       ReuseHostOut* hout) {
   if (n >= (uint64_t)kNone) return PTC_ERR_OVERFLOW;
   if (n == 0) return PTC_OK;
   if (!ids || !prev_out || !next_out || n_distinct == 0 || n_distinct > n) return PTC_ERR_INVALID_ARG;
   if (din && !hout) return PTC_ERR_INVALID_ARG;
-  return reuse_by_runs(ids, n, n_distinct, prev_out, next_out, ws, ws_bytes, s, false, defer_err, din, hout);
+  return reuse_by_runs(ids, n, n_distinct, prev_out, next_out, ws, ws_bytes, s, false, lent, din, hout);
 }
 
 }  // namespace ptc

@@ -784,17 +784,17 @@ struct RunsLayout {
   size_t total;
 };
 
-RunsLayout runs_layout(void* ws, uint64_t n, uint64_t R) {
+RunsLayout runs_layout(void* ws, uint64_t n, uint64_t R, const StackLent* lent = nullptr) {
   RunsLayout W;
   Carver cv(ws);
   const uint64_t nn = n ? n : 1, rr = R ? R : 1;
   W.L = key_bits_n(rr + 1);  // key ranks and thresholds lie in [0, R + 1]
   W.mtiles = ceil_div_u32(nn, kMTile);
   W.rtiles = ceil_div_u32(rr, kRTile);
-  W.kwords = (uint32_t)(nn / 32 + 2);  // keys and thresholds lie in [0, n]
+  W.kwords = (uint32_t)stack_key_words(nn);  // keys and thresholds lie in [0, n]
   W.ktiles = rank_tiles(W.kwords);
   W.st = cv.take<DevStatus>(1);
-  W.done = cv.take<uint32_t>(64);
+  W.done = cv.take<uint32_t>(kStackDone);
   W.kbits = cv.take<uint32_t>(W.kwords);
   W.zero_bytes = cv.off;
   W.tcnt = cv.take<uint32_t>(W.mtiles + 1);
@@ -817,6 +817,11 @@ RunsLayout runs_layout(void* ws, uint64_t n, uint64_t R) {
   W.w1 = cv.take<uint32_t>(rr);
   W.zw = cv.take<uint2>((uint64_t)W.L * (rr + 1));
   W.total = cv.bytes();
+  if (lent) {
+    W.st = lent->st;
+    W.done = lent->done;
+    W.kbits = lent->kbits;
+  }
   return W;
 }
 
@@ -851,10 +856,10 @@ bool cluster_fits(uint32_t C, const cudaLaunchConfig_t& cfg) {
 }
 
 ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_out, void* ws, size_t ws_bytes,
-                               cudaStream_t s, int method, RunsView* view, uint32_t* defer_err = nullptr) {
-  const RunsLayout M = runs_layout(ws, n, 1);
+                               cudaStream_t s, int method, RunsView* view, const StackLent* lent = nullptr) {
+  const RunsLayout M = runs_layout(ws, n, 1, lent);
   if (!ws_ok(ws, ws_bytes, M.total)) return PTC_ERR_WORKSPACE;
-  if (begin_call(ws, M.zero_bytes, s) != PTC_OK) return PTC_ERR_CUDA;
+  if (!lent && begin_call(ws, M.zero_bytes, s) != PTC_OK) return PTC_ERR_CUDA;
   MarkArgs m;
   m.prev = prev;
   m.n = (uint32_t)n;
@@ -881,7 +886,7 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
   ptc_status rc = end_call(M.st, s, &h);
   if (rc != PTC_OK) return rc;
   const uint64_t R = h.value[1];
-  const RunsLayout W = runs_layout(ws, n, R);
+  const RunsLayout W = runs_layout(ws, n, R, lent);
   const bool fits = R >= 1 && R <= n && ws_bytes >= W.total;
   if (method == PTC_SD_AUTO && (!fits || R > n / 3)) {
     // no runs to speak of: by counting, or on the matrix over every access
@@ -894,8 +899,6 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
     return stack_distance_points(prev, n, dist_out, ws, ws_bytes, s);
   }
   if (!fits) return PTC_ERR_WORKSPACE;
-  const FillRange zf[2] = {{W.acc, W.acc_bytes, 0u}, {W.done, 64 * sizeof(uint32_t), 0u}};
-  if (fill_many_async(zf, 2, s) != PTC_OK) return PTC_ERR_CUDA;
   const uint32_t R32 = (uint32_t)R, T = W.rtiles, L = W.L;
   const size_t tstride = (size_t)T + 1;
   // one cluster when the runs fit in its shared memory, else one launch per level
@@ -943,6 +946,8 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
       (void)cudaGetLastError();
   }
   if (!built) {
+    const FillRange zf[2] = {{W.acc, W.acc_bytes, 0u}, {W.done, kStackDone * sizeof(uint32_t), 0u}};
+    if (fill_many_async(zf, 2, s) != PTC_OK) return PTC_ERR_CUDA;
     PTC_KERNEL("k_runs_init", s, k_runs_init, T, kRT, 0, W.rec_s, W.rec_a, W.kbits, W.kpre, W.k0, W.w0, W.acc, W.pre,
                &W.done[0], R32, T, L - 1);
     uint32_t* keys[2] = {W.k0, W.k1};
@@ -978,7 +983,8 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
   q.L = L;
   PTC_KERNEL("k_runs_query", s, k_runs_query, ceil_div_u32(R, 256), 256, 0, q);
   PTC_KERNEL("k_runs_expand", s, k_runs_expand, ceil_div_u32(n, kExpThreads * kExpPer), kExpThreads, 0, W.bits, W.wpre, W.sd, (uint32_t)n, dist_out, R32, W.st);
-  const ptc_status done = defer_err ? defer_status(W.st, defer_err, s) : end_call(W.st, s, &h);
+  const ptc_status done =
+      lent ? (cudaGetLastError() == cudaSuccess ? PTC_OK : PTC_ERR_CUDA) : end_call(W.st, s, &h);
   if (done == PTC_OK && view) {
     view->used = true;
     view->R = R32;
@@ -993,13 +999,13 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
 }  // namespace
 
 ptc_status stack_distance_view(const uint32_t* prev, uint64_t n, uint32_t* dist_out, int method, void* ws,
-                               size_t ws_bytes, cudaStream_t s, RunsView* view, uint32_t* defer_err) {
+                               size_t ws_bytes, cudaStream_t s, RunsView* view, const StackLent* lent) {
   *view = RunsView{};
   if (n >= (uint64_t)kNone) return PTC_ERR_OVERFLOW;
   if (n == 0) return PTC_OK;
   if (!prev || !dist_out) return PTC_ERR_INVALID_ARG;
   if (method == PTC_SD_POINTS) return stack_distance_points(prev, n, dist_out, ws, ws_bytes, s);
-  return stack_distance_runs(prev, n, dist_out, ws, ws_bytes, s, method, view, defer_err);
+  return stack_distance_runs(prev, n, dist_out, ws, ws_bytes, s, method, view, lent);
 }
 
 }  // namespace ptc

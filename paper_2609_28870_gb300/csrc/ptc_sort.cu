@@ -253,6 +253,91 @@ __global__ void __launch_bounds__(kSortThreads, 3) k_sort_scatter(ScatterArgs a)
   }
 }
 
+// The whole sort of up to kSortTile pairs in one launch of one CTA: every pass
+// of k_sort_scatter's ranking, from registers to shared memory and back.  Six
+// launches (count, row scan, scatter; two digits) of a few microseconds each
+// otherwise.
+__global__ void __launch_bounds__(kSortThreads) k_sort_one(const uint32_t* __restrict__ keys_in,
+                                                           const uint32_t* __restrict__ vals_in, uint32_t n,
+                                                           uint32_t bits, uint32_t passes,
+                                                           uint32_t* __restrict__ keys_out,
+                                                           uint32_t* __restrict__ vals_out) {
+  grid_dep_sync();
+  __shared__ uint32_t s_keys[kSortTile];
+  __shared__ uint32_t s_vals[kSortTile];
+  __shared__ uint32_t s_whist[kSortWarps][kRadix];
+  __shared__ uint32_t s_warp[kSortWarps];
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5, base = w * (32 * kSortPer);
+  uint32_t key[kSortPer], val[kSortPer], at[kSortPer];
+#pragma unroll
+  for (int j = 0; j < kSortPer; ++j) {
+    const uint32_t i = base + j * 32 + lane;
+    key[j] = i < n ? keys_in[i] : 0u;
+    val[j] = i < n ? (vals_in ? vals_in[i] : i) : 0u;
+  }
+  uint32_t shift = 0;
+  for (uint32_t p = 0; p < passes; ++p) {
+    const uint32_t width = (bits - shift + (passes - p) - 1) / (passes - p), R = 1u << width;
+    for (uint32_t x = lane; x < R; x += 32) s_whist[w][x] = 0;
+    __syncwarp();
+#pragma unroll
+    for (int j = 0; j < kSortPer; ++j) {
+      const bool valid = base + j * 32 + lane < n;
+      const uint32_t d = (key[j] >> shift) & (R - 1);
+      const uint32_t peers = digit_peers(d, width, __ballot_sync(kFull, valid));
+      const uint32_t leader = valid ? __ffs(peers) - 1 : lane;
+      uint32_t before = 0;
+      if (valid && lane == leader) {
+        before = s_whist[w][d];
+        s_whist[w][d] = before + __popc(peers);
+      }
+      at[j] = __shfl_sync(kFull, before, leader) + __popc(peers & lanemask_lt());
+      __syncwarp();
+    }
+    __syncthreads();
+    const uint32_t d = threadIdx.x;
+    uint32_t c = 0, all;
+    if (d < R) {
+#pragma unroll
+      for (int ww = 0; ww < kSortWarps; ++ww) c += s_whist[ww][d];
+    }
+    uint32_t run = block_excl_scan<uint32_t>(c, s_warp, all);
+    if (d < R) {
+#pragma unroll
+      for (int ww = 0; ww < kSortWarps; ++ww) {
+        const uint32_t v = s_whist[ww][d];
+        s_whist[ww][d] = run;
+        run += v;
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kSortPer; ++j) {
+      if (base + j * 32 + lane < n) {
+        const uint32_t q = s_whist[w][(key[j] >> shift) & (R - 1)] + at[j];
+        s_keys[q] = key[j];
+        s_vals[q] = val[j];
+      }
+    }
+    __syncthreads();
+#pragma unroll
+    for (int j = 0; j < kSortPer; ++j) {
+      const uint32_t i = base + j * 32 + lane;
+      key[j] = i < n ? s_keys[i] : 0u;
+      val[j] = i < n ? s_vals[i] : 0u;
+    }
+    shift += width;
+  }
+#pragma unroll
+  for (int j = 0; j < kSortPer; ++j) {
+    const uint32_t i = base + j * 32 + lane;
+    if (i < n) {
+      keys_out[i] = key[j];
+      vals_out[i] = val[j];
+    }
+  }
+}
+
 __device__ __forceinline__ void link_runs(const uint2* __restrict__ head_kv, const uint2* __restrict__ tail_kv,
                                           size_t row, int32_t prev_cell, uint32_t cell, uint32_t n,
                                           uint32_t* __restrict__ prev, uint32_t* __restrict__ next) {
@@ -409,6 +494,12 @@ void ptc::sort_pairs(const uint32_t* keys, const uint32_t* vals, uint32_t n, uin
   if (bits < 1) bits = 1;
   const uint32_t passes = (bits + 7) / 8;
   const uint32_t T = ceil_div_u32(n ? n : 1, kSortTile);
+  if (n <= kSortTile) {
+    PTC_KERNEL("k_sort_one", s, k_sort_one, 1, kSortThreads, 0, keys, vals, n, bits, passes, L.k0, L.v0);
+    *keys_sorted = L.k0;
+    *vals_sorted = L.v0;
+    return;
+  }
   const uint32_t* kin = keys;
   const uint32_t* vin = vals;
   uint32_t *kout = L.k0, *vout = L.v0;
