@@ -925,13 +925,19 @@ uint32_t chunks_per_block(uint32_t B) {  // G: power of two >= ceil(B / 16)
   return g;
 }
 
-// Blocks per hash tile, a power of two: as many as make up to 256 units for
-// k_hash_units, one CTA's kHashThreads / G for k_hash_local.
-uint32_t tile_blocks(uint32_t B) {
+// Blocks per hash tile for up to nb blocks, a power of two: as many as make up
+// to 256 units for k_hash_units, one CTA's kHashThreads / G for k_hash_local.
+// With few blocks a tile of units is cut down to 64 while that makes more warps
+// than half of those that fit the GPU: a warp takes its rounds of 32 units one
+// after another, and a window of 127K blocks took 20 us in tiles of 256, 13 in
+// tiles of 64.
+uint32_t tile_blocks(uint32_t B, uint64_t nb) {
   const uint32_t U = unit_tokens(B);
   if (!U) return kHashThreads / chunks_per_block(B);
+  const uint32_t g = B / U;
   uint32_t tb = kUnitTile;
-  while (tb * (B / U) > kUnitTile) tb >>= 1;
+  while (tb * g > kUnitTile) tb >>= 1;
+  while (tb > 1 && tb * g > 64 && nb / tb < 16 * 152) tb >>= 1;
   return tb;
 }
 
@@ -952,7 +958,7 @@ HashLayout hash_layout(void* ws, uint32_t n_req, uint64_t n_tok, uint32_t B, uin
   Carver cv(ws);
   const uint32_t off_tiles = ceil_div_u32(n_req, kOffTile) + 1;
   const uint64_t nb = n_tok / B < keys_cap ? n_tok / B : keys_cap;
-  const uint32_t tb = tile_blocks(B);
+  const uint32_t tb = tile_blocks(B, n_tok / B);
   const uint32_t hash_tiles = ceil_div_u32(nb, tb) + 1;
   L.st = cv.take<DevStatus>(1);
   L.lb_off = cv.take<uint64_t>(off_tiles);
@@ -975,7 +981,7 @@ size_t ptc::hash_lb_words(uint32_t n_req) { return ceil_div_u32(n_req, kOffTile)
 
 uint64_t ptc::hash_carry_tiles(uint64_t n_tok, uint32_t block_size) {
   if (block_size == 0) block_size = 1;
-  return ceil_div_u32(n_tok / block_size, tile_blocks(block_size)) + 1;
+  return ceil_div_u32(n_tok / block_size, tile_blocks(block_size, n_tok / block_size)) + 1;
 }
 
 extern "C" size_t ptc_hash_blocks_workspace_bytes(uint32_t n_req, uint64_t n_tok, uint32_t block_size) {
@@ -1013,7 +1019,7 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
   }
   const uint32_t G = chunks_per_block(block_size);
   const bool aligned = (((uintptr_t)tokens) & 15) == 0;
-  const uint32_t tb = tile_blocks(block_size), U = unit_tokens(block_size);
+  const uint32_t tb = tile_blocks(block_size, n_tok / block_size), U = unit_tokens(block_size);
   // seeded bases and their derived constants
   PowArgs pw;
   HashConsts hc;
