@@ -20,7 +20,7 @@
 //               kernels below redo the curves from scratch.
 //   k_curves    running max, bin search in shared memory, run-merged
 //               shared histograms, one global atomic per non-empty bin
-//   k_curves_runs  (ptc_pipeline) the same from stage c's runs: one thread
+//   k_curves_runs  (ptc_pipeline) the same from stage c's runs: four lanes
 //               per request, one (count, depth sum) per piece of a run that
 //               lies in the request; a fall between the runs of a request
 //               sets the flag for the scan kernels
@@ -511,24 +511,32 @@ __global__ void __launch_bounds__(256) k_curves_runs(CurveArgs a, RunsArgs ra) {
   const uint32_t G = a.G;
   s_bins.init(a.caps, G);
   __syncthreads();
+  // Four lanes per request, a run per lane and round: a request has a handful
+  // of runs.  (A thread per request reads them one after another, 17 us at any
+  // size of trace; a warp per request leaves most lanes idle, 125 us for the
+  // 291K requests of half a mixed day.)
   bool fell = false;
-  for (uint32_t q = blockIdx.x * blockDim.x + threadIdx.x; q < a.R; q += gridDim.x * blockDim.x) {
-    const uint32_t start = (uint32_t)a.blk_off[q], end = (uint32_t)a.blk_off[q + 1];
-    if (end <= start || end > a.n) continue;  // empty (bad offsets are reported by k_heads)
-    const uint32_t r0 = run_at(ra.bits, ra.wpre, start), r1 = run_at(ra.bits, ra.wpre, end - 1);
-    uint32_t prev_v = 0, last_v = 0xFFFFFFFEu, g = G;
-    for (uint32_t r = r0; r <= r1; ++r) {
-      const uint32_t s0 = max(ra.rec_s[r], start), e0 = min(ra.rec_s[r + 1], end), v = ra.sd[r];
-      if (v < prev_v) fell = true;  // the running max would bind
-      prev_v = v;
-      if (v != last_v) {
-        g = s_bins.of(v, G);
-        last_v = v;
-      }
-      const uint32_t c = e0 - s0;
+  const uint32_t sub = threadIdx.x & 3, groups = gridDim.x * (blockDim.x >> 2);
+  for (uint32_t q0 = blockIdx.x * (blockDim.x >> 2) + ((threadIdx.x >> 5) << 3); q0 < a.R; q0 += groups) {
+    const uint32_t q = q0 + ((threadIdx.x & 31) >> 2);
+    const uint32_t start = q < a.R ? (uint32_t)a.blk_off[q] : 0u, end = q < a.R ? (uint32_t)a.blk_off[q + 1] : 0u;
+    const bool some = end > start && end <= a.n;  // not empty (bad offsets are reported by k_heads)
+    const uint32_t r0 = some ? run_at(ra.bits, ra.wpre, start) : 1u, r1 = some ? run_at(ra.bits, ra.wpre, end - 1) : 0u;
+    const uint32_t rounds = __reduce_max_sync(kFull, some ? (r1 - r0) / 4 + 1 : 0u);
+    uint32_t before = 0;  // the distance of the run before this round's first
+    for (uint32_t c = 0; c < rounds; ++c) {
+      const uint32_t r = r0 + 4 * c + sub;
+      const bool live = r <= r1;
+      const uint32_t v = live ? ra.sd[r] : kNone;
+      uint32_t up = __shfl_up_sync(kFull, v, 1, 4);
+      if (sub == 0) up = before;
+      before = __shfl_sync(kFull, v, 3, 4);
+      if (!live) continue;
+      if (v < up) fell = true;  // the running max would bind
+      const uint32_t s0 = max(ra.rec_s[r], start), n = min(ra.rec_s[r + 1], end) - s0, g = s_bins.of(v, G);
       const unsigned long long k0 = s0 - start;
-      atomicAdd(&s_bins.cnt[g], c);  // few adds, of any size: no 32-bit sums
-      atomicAdd(&s_bins.ks[g], (unsigned long long)c * k0 + (unsigned long long)c * (c - 1) / 2);
+      atomicAdd(&s_bins.cnt[g], n);  // few adds, of any size: no 32-bit sums
+      atomicAdd(&s_bins.ks[g], (unsigned long long)n * k0 + (unsigned long long)n * (n - 1) / 2);
     }
   }
   if (__syncthreads_or(fell) && threadIdx.x == 0) atomicOr(a.slow, 1u);
@@ -728,8 +736,8 @@ ptc_status ptc::curves_impl(const uint32_t* dist, uint64_t n, const uint64_t* re
   };
   if (from_runs) {
     const RunsArgs ra{runs->rec_s, runs->sd, runs->bits, runs->wpre};
-    const uint32_t g_r = ceil_div_u32(n_req, 256) < (uint32_t)(2 * num_sms()) ? ceil_div_u32(n_req, 256)
-                                                                                : (uint32_t)(2 * num_sms());
+    const uint32_t want = ceil_div_u32(n_req, 64), most = (uint32_t)(4 * num_sms());
+    const uint32_t g_r = want < most ? want : most;
     PTC_KERNEL("k_curves_runs", s, k_curves_runs, g_r, 256, 0, a, ra);
   } else if (n > 0) {
     heads();

@@ -42,20 +42,15 @@
 //                  among the distinct keys, so it has ceil(log2(R + 2))
 //                  levels instead of ceil(log2(n + 1)), and a query's
 //                  threshold x becomes the number of keys below x
+// Up to kDomMax runs (2 million) the count needs no matrix:
+//   k_dom_time, k_dom_rank, k_dom_out   pair sums by blocks (see there)
+// and with more:
 //   k_runs_init    level-0 keys and weights, per-tile zero counts / weights
 //   k_runs_level   one level: (Z, W), stable partition, the next level's
 //                  per-tile zero counts (four atomics per tile)
 //   k_runs_query   one thread per run: the distance of its head
 //   k_runs_expand  every access takes its run's distance
-#include <cooperative_groups.h>
-
-#include <utility>
-
-#include <atomic>
-
 #include "ptc_internal.h"
-
-namespace cg = cooperative_groups;
 
 namespace ptc {
 namespace {
@@ -519,163 +514,174 @@ __global__ void __launch_bounds__(kRT) k_runs_level(LevelArgs a) {
   }
 }
 
-// All L levels in one launch of one thread-block cluster when the runs fit in
-// its shared memory.  CTA c owns positions [c S, c S + S) of every level's
-// order.  A level: read the slice, stable-partition it locally (zeros, then
-// ones) into the same buffer, publish the CTA's (zeros, zero weight), and
-// after a cluster barrier copy the two partitioned segments, which are
-// contiguous in the next level's order, into their owners' other buffer with
-// coalesced distributed-shared-memory stores; a second barrier ends the level.
-// Same (Z, W) arrays as k_runs_level.
-constexpr int kCT = 1024;           // threads per CTA of the cluster
-constexpr int kCPer = 8;            // most elements a thread holds (one per round)
-constexpr int kCSlice = kCT * kCPer;
-constexpr int kCMax = 16;           // largest cluster (above 8 needs the non-portable attribute)
+// ---- up to kDomMax runs: by blocks, without a matrix
+// With s_r, a_r the start and first value of run r (a_r = p + 1), the distance
+// of its head is #{ j < s_r : v_j < a_r } - p.  The accesses before s_r are whole
+// runs, and every earlier context run lies wholly below or above a_r (its values
+// are consecutive and a_r is not among them), every first access below.  So with
+// the context runs ranked by value
+//   SD_r = s_r - (length of the context runs before r)
+//              + (length of those of them with a smaller rank) - p.
+// The last term is a weighted count over pairs.  Cut time (run order) and rank
+// into blocks of kDomB: a pair lies in one time block, or in different time
+// blocks and one rank block, or differs in both.  The first two are summed by
+// brute force inside a block, half a thousand steps from shared memory; the last
+// is a prefix over the matrix of the lengths per (time block, rank block).
+// Three launches whatever R, against log2(R) levels of barriers and as many
+// dependent reads per query of a wavelet matrix over the runs: 39,800 runs of the
+// chat trace took 75 us there (one thread-block cluster, then the queries) and 30
+// here, 0.7M runs of the mixed trace 450 us and 143.
+constexpr uint32_t kDomB = 512;
+constexpr uint64_t kDomMax = 1ULL << 21;  // runs; the lengths' matrix then takes 67 MB
 
-struct BuildArgs {
+struct DomArgs {
   const uint32_t* rec_s;
   const uint32_t* rec_a;
-  const uint32_t* kbits;  // keys enter the matrix as their ranks (key_rank)
+  const uint32_t* kbits;
   const uint32_t* kpre;
-  uint2* zw;
-  uint32_t R, L, slice;
+  uint32_t* mat;    // nb x (nb + 1): lengths per (time block, rank block), and per time block
+  uint2* by_rank;   // (run, length) of every rank
+  uint32_t* in_time;   // per run: smaller ranks before it in its time block
+  uint32_t* before;    // per run: context runs' length before it in its time block
+  uint32_t* in_rank;   // per run: smaller ranks of its rank block in earlier time blocks
+  uint32_t* rank;      // per run: rank (kNone: first accesses)
+  uint32_t* sd;
+  uint32_t R, nb, kwords;
 };
 
-__global__ void __launch_bounds__(kCT) k_runs_build_cluster(BuildArgs a) {
-  grid_dep_sync();
-  extern __shared__ uint2 s_dyn[];  // two buffers of `slice` (key, weight)
-  __shared__ unsigned long long s_rw[kCPer * 32];  // per (round, warp) (zeros, zero weight)
-  __shared__ unsigned long long s_tot, s_pre, s_all;
-  cg::cluster_group cl = cg::this_cluster();
-  const uint32_t rank = cl.block_rank(), C = cl.num_blocks();
+// Sum of w over the pairs (key, w) of s[0 .. n) with key < mine: n even, two
+// pairs per load, the same for the whole warp.
+__device__ __forceinline__ uint32_t sum_below(const uint2* s, uint32_t n, uint32_t mine) {
+  const uint4* s4 = reinterpret_cast<const uint4*>(s);
+  uint32_t sum = 0;
+#pragma unroll 8
+  for (uint32_t i = 0; i < n / 2; ++i) {
+    const uint4 x = s4[i];
+    if (x.x < mine) sum += x.y;
+    if (x.z < mine) sum += x.w;
+  }
+  return sum;
+}
+
+// Exclusive prefix over a CTA of kDomB threads; *total gets the sum.
+__device__ __forceinline__ uint32_t dom_excl(uint32_t x, uint32_t* s_w, uint32_t* total) {
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint32_t S = a.slice, base = rank * S;
-  const uint32_t cnt = base < a.R ? min(S, a.R - base) : 0u;
-  const uint32_t q = (S + kCT - 1) / kCT;  // rounds (the same in every CTA)
-  const float invS = 1.0f / (float)S;
-  for (uint32_t i = threadIdx.x; i < cnt; i += kCT) {
-    const uint32_t r = base + i;
-    const uint32_t st = a.rec_s[r], e = a.rec_s[r + 1], a0 = a.rec_a[r];
-    const uint32_t len = e - st;
-    s_dyn[i] = make_uint2(key_rank(a.kbits, a.kpre, a0 ? a0 + len - 1 : 0u), len);
+  uint32_t incl = x;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kFull, incl, o);
+    if (lane >= (uint32_t)o) incl += y;
   }
-  cl.sync();
-  for (uint32_t l = 0; l < a.L; ++l) {
-    uint2* cur = s_dyn + (l & 1) * S;
-    uint2* nxt = s_dyn + ((l + 1) & 1) * S;
-    const uint32_t shift = a.L - 1 - l;
-    // round k holds positions [k * kCT, k * kCT + kCT): lane order is index order
-    uint2 el[kCPer];
-    uint32_t lz[kCPer], lw[kCPer];
+  __syncthreads();
+  if (lane == 31) s_w[w] = incl;
+  __syncthreads();
+  uint32_t pre = 0, all = 0;
 #pragma unroll
-    for (int k = 0; k < kCPer; ++k) {
-      if (k >= (int)q) break;  // q is the same for the whole CTA
-      const uint32_t i = k * kCT + threadIdx.x;
-      const bool valid = i < cnt;
-      el[k] = valid ? cur[i] : make_uint2(0u, 0u);
-      const bool zero = valid && !((el[k].x >> shift) & 1u);
-      const uint32_t m = __ballot_sync(kFull, zero);
-      uint32_t wi = zero ? el[k].y : 0u;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(kFull, wi, o);
-        if (lane >= (uint32_t)o) wi += y;
-      }
-      lz[k] = __popc(m & lanemask_lt());
-      lw[k] = wi - (zero ? el[k].y : 0u);
-      if (lane == 31 && k < (int)q) s_rw[k * 32 + w] = pack_zw(__popc(m), wi);
-    }
-    __syncthreads();
-    // exclusive scan of the q x 32 (round, warp) totals in index order, by
-    // warp 0: lane l sums the q consecutive entries [l q, l q + q)
-    if (w == 0) {
-      unsigned long long part[kCPer];
-      unsigned long long sum = 0;
-#pragma unroll
-      for (int k = 0; k < kCPer; ++k) {
-        part[k] = 0;
-        if (k < (int)q) {
-          part[k] = s_rw[lane * q + k];
-          sum += part[k];
-        }
-      }
-      unsigned long long incl = sum;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(kFull, incl, o);
-        if (lane >= (uint32_t)o) incl += y;
-      }
-      unsigned long long run = incl - sum;
-#pragma unroll
-      for (int k = 0; k < kCPer; ++k) {
-        if (k < (int)q) {
-          s_rw[lane * q + k] = run;
-          run += part[k];
-        }
-      }
-      if (lane == 31) s_tot = incl;
-    }
-    __syncthreads();
-    const uint32_t nz = (uint32_t)s_tot;
-    // local stable partition into `cur` (every element is in registers)
-#pragma unroll
-    for (int k = 0; k < kCPer; ++k) {
-      if (k >= (int)q) break;
-      const uint32_t i = k * kCT + threadIdx.x;
-      if (i < cnt) {
-        const unsigned long long rw = s_rw[k * 32 + w];
-        lz[k] += (uint32_t)rw;
-        lw[k] += (uint32_t)(rw >> 32);
-        const bool zero = !((el[k].x >> shift) & 1u);
-        cur[zero ? lz[k] : nz + (i - lz[k])] = el[k];
-      }
-    }
-    cl.sync();  // every CTA's total is published and every slice partitioned
-    if (w == 0) {
-      const unsigned long long v = lane < C ? *cl.map_shared_rank(&s_tot, lane) : 0ull;
-      unsigned long long in = v;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const unsigned long long y = __shfl_up_sync(kFull, in, o);
-        if (lane >= (uint32_t)o) in += y;
-      }
-      if (lane == rank) s_pre = in - v;
-      if (lane == 31) s_all = in;
-    }
-    __syncthreads();
-    const uint32_t Zpre = (uint32_t)s_pre, Wpre = (uint32_t)(s_pre >> 32), Zc = (uint32_t)s_all;
-    if (l + 1 < a.L) {
-      // zeros go to [Zpre, Zpre + nz), ones to [Zc + base - Zpre, ...)
-      const uint32_t one0 = Zc + (base - Zpre);
-      for (uint32_t j = threadIdx.x; j < cnt; j += kCT) {
-        const uint32_t dst = j < nz ? Zpre + j : one0 + (j - nz);
-        // dst / S through a float reciprocal (dst < 2^24, so dst is exact in
-        // a float and the estimate is off by at most one)
-        int32_t owner = (int32_t)((float)dst * invS);
-        int32_t off = (int32_t)dst - owner * (int32_t)S;
-        if (off < 0) {
-          --owner;
-          off += (int32_t)S;
-        } else if (off >= (int32_t)S) {
-          ++owner;
-          off -= (int32_t)S;
-        }
-        if (dst < a.R) *cl.map_shared_rank(&nxt[off], owner) = cur[j];
-      }
-    }
-    // the barrier orders the copies above; the (Z, W) stores, read only by
-    // the next kernel, go out while the other CTAs arrive
-    auto token = cl.barrier_arrive();
-    uint2* zl = a.zw + (size_t)l * (a.R + 1);
-#pragma unroll
-    for (int k = 0; k < kCPer; ++k) {
-      if (k >= (int)q) break;
-      const uint32_t i = k * kCT + threadIdx.x;
-      if (i < cnt) zl[base + i] = make_uint2(Zpre + lz[k], Wpre + lw[k]);
-    }
-    if (rank == 0 && threadIdx.x == 0) zl[a.R] = make_uint2(Zc, (uint32_t)(s_all >> 32));
-    cl.barrier_wait(std::move(token));  // the next level's order is in place
+  for (int k = 0; k < (int)kDomB / 32; ++k) {
+    const uint32_t v = s_w[k];
+    if (k < (int)w) pre += v;
+    all += v;
   }
+  *total = all;
+  return pre + incl - x;
+}
+
+// One CTA per time block: ranks, the pairs inside the block, the block's row of
+// lengths.
+__global__ void __launch_bounds__(kDomB) k_dom_time(DomArgs a) {
+  grid_dep_sync();
+  extern __shared__ uint32_t s_row[];  // nb
+  __shared__ __align__(16) uint2 s_run[kDomB];
+  __shared__ uint32_t s_w[kDomB / 32];
+  const uint32_t t = threadIdx.x, r = blockIdx.x * kDomB + t;
+  for (uint32_t b = t; b < a.nb; b += kDomB) s_row[b] = 0;
+  uint32_t rank = kNone, len = 0;
+  if (r < a.R) {
+    const uint32_t v = a.rec_a[r];
+    if (v) {
+      len = a.rec_s[r + 1] - a.rec_s[r];
+      rank = key_rank(a.kbits, a.kpre, v + len - 1) - 1;  // key 0 is entered too
+    }
+    a.rank[r] = rank;
+  }
+  s_run[t] = make_uint2(rank, len);
+  uint32_t all;
+  const uint32_t before = dom_excl(len, s_w, &all);  // its barriers order s_row and s_run
+  if (rank != kNone) {
+    atomicAdd(&s_row[rank / kDomB], len);
+    a.by_rank[rank] = make_uint2(r, len);
+  }
+  if (r < a.R) a.before[r] = before;
+  // earlier runs of the block: whole warps, then the warp's own earlier lanes
+  const uint32_t w0 = t & ~31u;
+  uint32_t sum = sum_below(s_run, w0, rank == kNone ? 0u : rank);
+#pragma unroll
+  for (uint32_t k = 0; k < 31; ++k) {
+    const uint2 x = s_run[w0 + k];
+    if (k < (t & 31) && x.x < rank) sum += x.y;
+  }
+  if (rank != kNone) a.in_time[r] = sum;
+  __syncthreads();
+  uint32_t* row = a.mat + (size_t)blockIdx.x * (a.nb + 1);
+  for (uint32_t b = t; b < a.nb; b += kDomB) row[b] = s_row[b];
+  if (t == 0) row[a.nb] = all;
+}
+
+// One CTA per rank block (and one for the time blocks' totals): its column of
+// lengths becomes the prefix over earlier time blocks, and the pairs inside the
+// block.
+__global__ void __launch_bounds__(kDomB) k_dom_rank(DomArgs a) {
+  grid_dep_sync();
+  __shared__ __align__(16) uint2 s_run[kDomB];
+  __shared__ uint32_t s_w[kDomB / 32];
+  const uint32_t t = threadIdx.x, b = blockIdx.x, q = b * kDomB + t;
+  uint2 x = make_uint2(kNone, 0u);
+  const uint32_t ranks = a.kpre[a.kwords - 1] + __popc(a.kbits[a.kwords - 1]) - 1;  // keys but 0
+  if (b < a.nb && q < ranks && q < a.R) x = a.by_rank[q];
+  // (time block, length) in rank order: an entry counts the earlier ones of
+  // smaller time blocks
+  const uint32_t tb = x.x == kNone ? kNone : x.x / kDomB;
+  s_run[t] = make_uint2(tb, x.y);
+  uint32_t run = 0;
+  for (uint32_t t0 = 0; t0 < a.nb; t0 += kDomB) {
+    uint32_t* cell = a.mat + (size_t)(t0 + t) * (a.nb + 1) + b;
+    const uint32_t v = t0 + t < a.nb ? *cell : 0u;
+    uint32_t all;
+    const uint32_t pre = dom_excl(v, s_w, &all);
+    if (t0 + t < a.nb) *cell = run + pre;
+    run += all;
+  }
+  if (b == a.nb) return;
+  const uint32_t w0 = t & ~31u;
+  uint32_t sum = sum_below(s_run, w0, tb == kNone ? 0u : tb);
+#pragma unroll
+  for (uint32_t k = 0; k < 31; ++k) {
+    const uint2 y = s_run[w0 + k];
+    if (k < (t & 31) && y.x < tb) sum += y.y;
+  }
+  if (x.x != kNone && x.x < a.R) a.in_rank[x.x] = sum;
+}
+
+// One CTA per time block: the row's prefix over rank blocks, and the distances.
+__global__ void __launch_bounds__(kDomB) k_dom_out(DomArgs a) {
+  grid_dep_sync();
+  extern __shared__ uint32_t s_row[];  // nb
+  __shared__ uint32_t s_w[kDomB / 32];
+  const uint32_t t = threadIdx.x, r = blockIdx.x * kDomB + t;
+  const uint32_t* row = a.mat + (size_t)blockIdx.x * (a.nb + 1);
+  uint32_t run = 0;
+  for (uint32_t b0 = 0; b0 < a.nb; b0 += kDomB) {
+    uint32_t all;
+    const uint32_t pre = dom_excl(b0 + t < a.nb ? row[b0 + t] : 0u, s_w, &all);
+    if (b0 + t < a.nb) s_row[b0 + t] = run + pre;
+    run += all;
+  }
+  __syncthreads();
+  if (r >= a.R) return;
+  const uint32_t rank = a.rank[r];
+  a.sd[r] = rank == kNone ? kNone
+                          : a.rec_s[r] - (row[a.nb] + a.before[r]) + s_row[rank / kDomB] + a.in_rank[r] +
+                                a.in_time[r] - (a.rec_a[r] - 1u);
 }
 
 struct QueryArgs {
@@ -778,7 +784,8 @@ struct RunsLayout {
   size_t zero_bytes;
   uint32_t *bits, *wpre, *rec_s, *rec_a;
   uint32_t *sd, *k0, *k1, *w0, *w1;
-  uint2 *acc, *pre, *zw;
+  uint2 *acc, *pre, *zw;  // the weighted matrix (more than kDomMax runs)
+  DomArgs dom;            // the blocks' arrays (up to kDomMax)
   uint32_t L, mtiles, rtiles;
   size_t acc_bytes;
   size_t total;
@@ -806,16 +813,29 @@ RunsLayout runs_layout(void* ws, uint64_t n, uint64_t R, const StackLent* lent =
   W.wpre = cv.take<uint32_t>(nn / 32 + 2);
   W.rec_s = cv.take<uint32_t>(nn + 1);
   W.rec_a = cv.take<uint32_t>(nn);
-  const size_t acc_off = cv.off;
-  W.acc = cv.take<uint2>((uint64_t)(W.L + 1) * (W.rtiles + 1));
-  W.acc_bytes = cv.off - acc_off;
-  W.pre = cv.take<uint2>((uint64_t)(W.L + 1) * (W.rtiles + 1));
   W.sd = cv.take<uint32_t>(rr);
-  W.k0 = cv.take<uint32_t>(rr);
-  W.k1 = cv.take<uint32_t>(rr);
-  W.w0 = cv.take<uint32_t>(rr);
-  W.w1 = cv.take<uint32_t>(rr);
-  W.zw = cv.take<uint2>((uint64_t)W.L * (rr + 1));
+  W.acc = W.pre = W.zw = nullptr;
+  W.acc_bytes = 0;
+  W.dom = DomArgs{};
+  if (rr <= kDomMax) {
+    W.dom.nb = ceil_div_u32(rr, kDomB);
+    W.dom.mat = cv.take<uint32_t>((size_t)W.dom.nb * (W.dom.nb + 1));
+    W.dom.by_rank = cv.take<uint2>(rr);
+    W.dom.in_time = cv.take<uint32_t>(rr);
+    W.dom.before = cv.take<uint32_t>(rr);
+    W.dom.in_rank = cv.take<uint32_t>(rr);
+    W.dom.rank = cv.take<uint32_t>(rr);
+  } else {
+    const size_t acc_off = cv.off;
+    W.acc = cv.take<uint2>((uint64_t)(W.L + 1) * (W.rtiles + 1));
+    W.acc_bytes = cv.off - acc_off;
+    W.pre = cv.take<uint2>((uint64_t)(W.L + 1) * (W.rtiles + 1));
+    W.k0 = cv.take<uint32_t>(rr);
+    W.k1 = cv.take<uint32_t>(rr);
+    W.w0 = cv.take<uint32_t>(rr);
+    W.w1 = cv.take<uint32_t>(rr);
+    W.zw = cv.take<uint2>((uint64_t)W.L * (rr + 1));
+  }
   W.total = cv.bytes();
   if (lent) {
     W.st = lent->st;
@@ -830,29 +850,6 @@ RunsLayout runs_layout(void* ws, uint64_t n, uint64_t R, const StackLent* lent =
 uint64_t runs_reserve(uint64_t n) {
   const uint64_t r = n / 3 + 1;
   return r < (1ULL << 24) ? r : (1ULL << 24);
-}
-
-// Whether a cluster of C CTAs of k_runs_build_cluster can be resident, asked
-// once per device and cluster size with the largest shared-memory request (a
-// smaller one fits whenever that does); the occupancy query is slow next to
-// the kernels around it.
-bool cluster_fits(uint32_t C, const cudaLaunchConfig_t& cfg) {
-  constexpr int kDevs = 64;
-  static std::atomic<int8_t> known[kDevs][kCMax + 1];  // 0 unknown, 1 yes, 2 no
-  int dev = 0;
-  if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kDevs || C > (uint32_t)kCMax) {
-    (void)cudaGetLastError();
-    return false;
-  }
-  const int8_t k = known[dev][C].load(std::memory_order_relaxed);
-  if (k) return k == 1;
-  cudaLaunchConfig_t q = cfg;
-  q.dynamicSmemBytes = 2 * kCSlice * sizeof(uint2);
-  int clusters = 0;
-  const bool ok = cudaOccupancyMaxActiveClusters(&clusters, k_runs_build_cluster, &q) == cudaSuccess && clusters >= 1;
-  if (!ok) (void)cudaGetLastError();
-  known[dev][C].store(ok ? 1 : 2, std::memory_order_relaxed);
-  return ok;
 }
 
 ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_out, void* ws, size_t ws_bytes,
@@ -899,53 +896,23 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
     return stack_distance_points(prev, n, dist_out, ws, ws_bytes, s);
   }
   if (!fits) return PTC_ERR_WORKSPACE;
-  const uint32_t R32 = (uint32_t)R, T = W.rtiles, L = W.L;
-  const size_t tstride = (size_t)T + 1;
-  // one cluster when the runs fit in its shared memory, else one launch per level
-  bool built = false;
-  static int attrs_set = -1;  // per process: the attributes belong to the device function
-  if (attrs_set < 0)
-    attrs_set = cudaFuncSetAttribute(k_runs_build_cluster, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                     (int)(2 * kCSlice * sizeof(uint2))) == cudaSuccess &&
-                cudaFuncSetAttribute(k_runs_build_cluster, cudaFuncAttributeNonPortableClusterSizeAllowed, 1) ==
-                    cudaSuccess;
-  for (uint32_t cmax = kCMax; attrs_set == 1 && !built && cmax >= 8; cmax /= 2) {
-    uint32_t C = ceil_div_u32(R, 2048);  // about two runs per thread
-    if (C > cmax) C = cmax;
-    if ((uint64_t)C * kCSlice < R) continue;
-    BuildArgs b;
-    b.rec_s = W.rec_s;
-    b.rec_a = W.rec_a;
-    b.kbits = W.kbits;
-    b.kpre = W.kpre;
-    b.zw = W.zw;
-    b.R = R32;
-    b.L = L;
-    b.slice = ceil_div_u32(R, C);
-    cudaLaunchConfig_t cfg = {};
-    cudaLaunchAttribute attr[2];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = C;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.gridDim = dim3(C);
-    cfg.blockDim = dim3(kCT);
-    cfg.dynamicSmemBytes = 2 * (size_t)b.slice * sizeof(uint2);
-    cfg.stream = s;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    if (!cluster_fits(C, cfg)) continue;
-    attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;  // as launch_pdl
-    attr[1].val.programmaticStreamSerializationAllowed = 1;
-    cfg.numAttrs = 2;
-    cudaError_t e = cudaSuccess;
-    PTC_LAUNCH("k_runs_build_cluster", s, e = cudaLaunchKernelEx(&cfg, k_runs_build_cluster, b));
-    if (e == cudaSuccess)
-      built = true;
-    else
-      (void)cudaGetLastError();
-  }
-  if (!built) {
+  const uint32_t R32 = (uint32_t)R;
+  if (R <= kDomMax) {
+    DomArgs d = W.dom;
+    d.rec_s = W.rec_s;
+    d.rec_a = W.rec_a;
+    d.kbits = W.kbits;
+    d.kpre = W.kpre;
+    d.sd = W.sd;
+    d.R = R32;
+    d.kwords = W.kwords;
+    const size_t row = sizeof(uint32_t) * d.nb;
+    PTC_KERNEL("k_dom_time", s, k_dom_time, d.nb, kDomB, row, d);
+    PTC_KERNEL("k_dom_rank", s, k_dom_rank, d.nb + 1, kDomB, 0, d);
+    PTC_KERNEL("k_dom_out", s, k_dom_out, d.nb, kDomB, row, d);
+  } else {
+    const uint32_t T = W.rtiles, L = W.L;
+    const size_t tstride = (size_t)T + 1;
     const FillRange zf[2] = {{W.acc, W.acc_bytes, 0u}, {W.done, kStackDone * sizeof(uint32_t), 0u}};
     if (fill_many_async(zf, 2, s) != PTC_OK) return PTC_ERR_CUDA;
     PTC_KERNEL("k_runs_init", s, k_runs_init, T, kRT, 0, W.rec_s, W.rec_a, W.kbits, W.kpre, W.k0, W.w0, W.acc, W.pre,
@@ -969,19 +936,19 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
       a.shift = L - 1 - l;
       PTC_KERNEL("k_runs_level", s, k_runs_level, T, kRT, 0, a);
     }
+    QueryArgs q;
+    q.rec_s = W.rec_s;
+    q.rec_a = W.rec_a;
+    q.bits = W.bits;
+    q.wpre = W.wpre;
+    q.kbits = W.kbits;
+    q.kpre = W.kpre;
+    q.zw = W.zw;
+    q.sd = W.sd;
+    q.R = R32;
+    q.L = L;
+    PTC_KERNEL("k_runs_query", s, k_runs_query, ceil_div_u32(R, 256), 256, 0, q);
   }
-  QueryArgs q;
-  q.rec_s = W.rec_s;
-  q.rec_a = W.rec_a;
-  q.bits = W.bits;
-  q.wpre = W.wpre;
-  q.kbits = W.kbits;
-  q.kpre = W.kpre;
-  q.zw = W.zw;
-  q.sd = W.sd;
-  q.R = R32;
-  q.L = L;
-  PTC_KERNEL("k_runs_query", s, k_runs_query, ceil_div_u32(R, 256), 256, 0, q);
   PTC_KERNEL("k_runs_expand", s, k_runs_expand, ceil_div_u32(n, kExpThreads * kExpPer), kExpThreads, 0, W.bits, W.wpre, W.sd, (uint32_t)n, dist_out, R32, W.st);
   const ptc_status done =
       lent ? (cudaGetLastError() == cudaSuccess ? PTC_OK : PTC_ERR_CUDA) : end_call(W.st, s, &h);

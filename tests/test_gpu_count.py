@@ -1,7 +1,7 @@
 """Stage c by counting (traces without runs) against the oracle's distances,
 bit-exact, at sizes around the edges of its warps (1,024 positions), tiles
-(8,192) and buckets (32,768 re-reads); the fallback for a prev that takes a
-value twice; and stage d's bins where a CTA walks many tiles."""
+(8,192) and buckets (32,768 re-reads); the distances of runs by blocks of 512;
+the fallback for a prev that takes a value twice; and stage d's bins where a CTA walks many tiles."""
 import numpy as np
 import pytest
 
@@ -46,6 +46,30 @@ def test_counted_distances_at_bucket_edges(ptc, rereads):
     prev = _prev(ids)
     got = ptc.u32(ptc.ptc_stack_distance(ptc.to_device_u32(prev)))
     assert np.array_equal(got, oracle.sd_fenwick(prev))
+
+
+@pytest.mark.parametrize("n", [1, 31, 511, 512, 513, 1023, 1025, 20_000, 262_145])
+def test_runs_by_blocks(ptc, n):
+    """The distances of runs around the edges of their blocks of 512: context
+    re-reads of random stretches, so that runs of every length and rank order
+    meet, and a trace without runs (every access its own)."""
+    rng = np.random.default_rng(n)
+    parts, size = [], 0
+    while size < n:
+        lo = int(rng.integers(0, max(1, n // 3)))
+        parts.append(np.arange(lo, lo + int(rng.integers(1, 9))))
+        size += len(parts[-1])
+    for ids in (np.concatenate(parts)[:n], rng.integers(0, max(1, n // 2), n)):
+        prev = _prev(ids)
+        got = ptc.u32(ptc.ptc_stack_distance(ptc.to_device_u32(prev), method=ptc.PTC_SD_RUNS))
+        assert np.array_equal(got, oracle.sd_fenwick(prev))
+
+
+def test_more_runs_than_blocks_take(ptc):
+    """Above 2^21 runs the forced run method builds its matrix level by level."""
+    rng = np.random.default_rng(1)
+    p = ptc.to_device_u32(_prev(rng.integers(0, 900_000, 2_300_000)))
+    assert np.array_equal(ptc.u32(ptc.ptc_stack_distance(p, method=ptc.PTC_SD_RUNS)), ptc.u32(ptc.ptc_stack_distance(p)))
 
 
 def test_prev_that_repeats_a_value_takes_the_matrix(ptc):
