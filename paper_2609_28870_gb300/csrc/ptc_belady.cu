@@ -35,24 +35,21 @@
 // is a plain store of whole words by one lane.
 // What bounds the replay is the latency of one run's chain of reads and
 // shuffles, hence: the summaries sit in shared memory (a bit per 32 accesses:
-// up to about 50M accesses), three other warps read the bitmap words of the
-// next 32 runs into L1 ahead of the replayer, whose own stores go through the
-// same L1, and the bitmap's last word, which the next run extends, stays in a
-// register.  Hits count with the prefix rule (Sec. 2.2): a request's accesses
-// before its first miss.
+// up to about 50M accesses), and the bitmap's last word, which the next run
+// extends, stays in a register.  Hits count with the prefix rule (Sec. 2.2): a
+// request's accesses before its first miss.
 //
 // Measured on the 9.3M-access chat trace, 64 capacities: 180 ms with the
 // summaries in L2, every update an atomic and one lane searching; 43.7 ms with
 // exact summaries in shared memory; 29 ms so (about 260 instructions a run at
-// 5.8 cycles each: instruction latency, not memory, is what is left).
+// 5.8 cycles each: instruction latency is what is left, as three more warps
+// that read the next runs' bitmap words into L1 changed nothing).
 #include "ptc_internal.h"
 
 namespace ptc {
 namespace {
 
-constexpr uint32_t kBelAhead = 3;     // warps that read ahead
-constexpr uint32_t kBelThreads = 32 * (1 + kBelAhead);
-constexpr uint32_t kBelRuns = 32 * kBelAhead;  // runs per batch, one per lane of those
+constexpr uint32_t kBelThreads = 32;  // one warp per capacity
 constexpr size_t kBelSmemMax = 200 * 1024;  // summaries in shared memory up to this size
 
 __device__ __forceinline__ uint32_t hi_bit(uint32_t v) { return 31u - __clz(v); }
@@ -249,12 +246,12 @@ __device__ __forceinline__ void add_mul(uint64_t& lo, uint64_t& hi, uint64_t a, 
   add128(lo, hi, a * b, __umul64hi(a, b));
 }
 
-// One CTA per capacity: warp 0 replays, the others read ahead.
+// One CTA of one warp per capacity.
 template <bool SMEM>
 __global__ void __launch_bounds__(kBelThreads, 1) k_bel_sim(BelArgs a, BelCaps caps) {
   extern __shared__ uint32_t s_sum[];
   grid_dep_sync();
-  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const uint32_t lane = threadIdx.x;
   const uint32_t g = blockIdx.x;
   if (g >= a.G) return;
   uint32_t* const l0 = a.lv0 + (uint64_t)g * a.s0;
@@ -263,205 +260,173 @@ __global__ void __launch_bounds__(kBelThreads, 1) k_bel_sim(BelArgs a, BelCaps c
     for (uint32_t i = threadIdx.x; i < a.s1 + a.s2 + a.s3; i += kBelThreads) sum[i] = 0;
   FreeBits fb{l0, sum, sum + a.s1, sum + a.s1 + a.s2, 0, a.s0, a.st};
   const uint32_t R = (uint32_t)*a.nruns;
-  // The words of the previous accesses of runs r0 .. r0 + kBelRuns - 1 and
-  // the 128-byte line below them (the latest free times below p tend to lie
-  // there), into L1: one run per lane, a word per 32-byte sector, eight loads
-  // in flight.  All of a batch's misses are outstanding at once: L1 answers in
-  // order, so the replayer's hits wait while any are.
-  auto read_ahead = [&](uint32_t r0) {
-    const uint32_t r = r0 + (warp - 1) * 32 + lane;
-    if (r >= R) return;
-    const uint32_t p = __ldg(&a.rec_p[r]), L = __ldg(&a.rec_start[r + 1]) - __ldg(&a.rec_start[r]);
-    if (p == kNone) return;
-    const uint32_t last = (uint32_t)(((uint64_t)p + L) >> 5), first = (p >> 8) * 8;
-    for (uint32_t w = first >= 32 ? first - 32 : 0u; w <= last; w += 64) {
-      uint32_t x[8];
-#pragma unroll
-      for (uint32_t u = 0; u < 8; ++u) {
-        x[u] = 0;
-        if (w + 8 * u <= last && w + 8 * u < a.s0)
-          asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(x[u]) : "l"(l0 + w + 8 * u));
-      }
-#pragma unroll
-      for (uint32_t u = 0; u < 8; ++u) asm volatile("" ::"r"(x[u]));
-    }
-  };
   uint64_t free_inf = caps.c[g] - 1;  // never-used tracks
   uint64_t hits = 0, raw = 0, depths = 0;  // counted hits, all hits, and the counted hits' depths
   uint32_t req_start = 0;
   uint32_t tail_w = 0, tail = 0;  // the highest word that free times were added to, as it stands
   bool missed = false;
-  if (warp) read_ahead(0);
-  __syncthreads();
-  for (uint32_t r0 = 0; r0 < R; r0 += kBelRuns) {
-    if (warp) {
-      if (R - r0 > kBelRuns) read_ahead(r0 + kBelRuns);
-      __syncthreads();
-      continue;
-    }
-    for (uint32_t q0 = r0; q0 < R && q0 < r0 + kBelRuns; q0 += 32) {
-      const uint32_t rl = q0 + lane;
-      const uint32_t my_s = rl < R ? a.rec_start[rl] : 0u;
-      const uint32_t my_e = rl < R ? a.rec_start[rl + 1] : 0u;
-      const uint32_t my_p = rl < R ? a.rec_p[rl] : kNone;
-      const uint32_t opens = __ballot_sync(kFull, rl < R && a.rec_rs[rl]);  // runs that open a request
-      const uint32_t nr = R - q0 < 32 ? R - q0 : 32;
-      for (uint32_t t = 0; t < nr; ++t) {
-        uint32_t s = __shfl_sync(kFull, my_s, t);
-        const uint32_t e = __shfl_sync(kFull, my_e, t);
-        uint32_t p = __shfl_sync(kFull, my_p, t);
-        if ((opens >> t) & 1u) {
-          req_start = s;
-          missed = false;
+  __syncwarp();
+  for (uint32_t q0 = 0; q0 < R; q0 += 32) {
+    const uint32_t rl = q0 + lane;
+    const uint32_t my_s = rl < R ? a.rec_start[rl] : 0u;
+    const uint32_t my_e = rl < R ? a.rec_start[rl + 1] : 0u;
+    const uint32_t my_p = rl < R ? a.rec_p[rl] : kNone;
+    const uint32_t opens = __ballot_sync(kFull, rl < R && a.rec_rs[rl]);  // runs that open a request
+    const uint32_t nr = R - q0 < 32 ? R - q0 : 32;
+    for (uint32_t t = 0; t < nr; ++t) {
+      uint32_t s = __shfl_sync(kFull, my_s, t);
+      const uint32_t e = __shfl_sync(kFull, my_e, t);
+      uint32_t p = __shfl_sync(kFull, my_p, t);
+      if ((opens >> t) & 1u) {
+        req_start = s;
+        missed = false;
+      }
+      uint32_t L = e - s;
+      if (p == kNone || p >= s) {  // cold accesses: misses, no track (p >= s is malformed, reported)
+        missed = true;
+        continue;
+      }
+      if (s - p == 1) {  // every step re-reads the block just accessed: busy nowhere, hits
+        raw += L;
+        if (!missed) {
+          hits += L;
+          depths += (uint64_t)L * (s - req_start) + (uint64_t)L * (L - 1) / 2;
         }
-        uint32_t L = e - s;
-        if (p == kNone || p >= s) {  // cold accesses: misses, no track (p >= s is malformed, reported)
-          missed = true;
-          continue;
-        }
-        if (s - p == 1) {  // every step re-reads the block just accessed: busy nowhere, hits
-          raw += L;
-          if (!missed) {
-            hits += L;
-            depths += (uint64_t)L * (s - req_start) + (uint64_t)L * (L - 1) / 2;
-          }
-          continue;
-        }
-        while (L > 0) {
-          const uint32_t gap = s - p, sp = p & 31;
-          uint32_t Lj = L < gap ? L : gap;
-          if (Lj > 1024 - sp) Lj = 1024 - sp;  // the 32 words from p's
-          // this lane's word of them (positions 32 (w0 + lane) ..) and of the 32 below
-          const uint32_t w0 = p >> 5, w = w0 + lane;
-          const uint32_t end = sp + Lj;  // past the last step, counted from word w0
-          uint32_t valid = lane * 32 >= end ? 0u : end - lane * 32 >= 32 ? kFull : mask_lt(end - lane * 32);
-          const bool has = valid != 0 && in_bounds(a.st, w, a.s0);
-          const uint32_t word = has ? l0[w] : 0u;
-          const uint32_t below = w0 > lane ? l0[w0 - 1 - lane] : 0u;
-          // the level-1 words of the 32 words where this chunk's free times go
-          const uint32_t v0 = (s - 1) >> 5;
-          uint32_t old0 = fb.l1[v0 >> 5], old1 = fb.l1[(v0 >> 5) + 1];
-          if (lane == 0) valid &= ~mask_lt(sp);
-          const uint32_t Bk = word & valid;
-          const bool edge = Lj >= 2 && p + Lj == s;  // the last step: decided by step 0 below
-          const uint32_t elane = (end - 1) >> 5, ebit = 1u << ((end - 1) & 31);
-          const uint32_t z = Lj - edge - __reduce_add_sync(kFull, __popc(Bk));
-          uint32_t left = word & ~valid;  // the free times of [p, p + Lj) are used up
-          uint32_t A = valid;        // steps that hit
-          uint32_t nh = Lj, f = Lj;  // hits, and hits before the first miss
-          if (z) {
-            // the other steps take the latest free times below p, then never-used tracks
-            uint32_t acc = 0;
-            if (p > fb.low) {
-              const uint32_t first = __shfl_sync(kFull, word, 0) & mask_lt(sp);  // those in p's own word
-              uint32_t sum;
-              const uint32_t c = __popc(below), n0 = __popc(first), above = n0 + lanes_excl(c, &sum);
-              if (n0 > z) {
-                const uint32_t tk = top_bits(first, z, lane);
-                if (lane == 0) left &= ~tk;
-              } else {
-                if (lane == 0) left &= ~first;
-                uint32_t take = above + c <= z ? below : 0u;
-                const uint32_t part = __ballot_sync(kFull, above < z && above + c > z);
-                if (part) {  // the word that holds the last one wanted
-                  const uint32_t src = __ffs(part) - 1;
-                  const uint32_t more = z - __shfl_sync(kFull, above, src);
-                  const uint32_t tk = top_bits(__shfl_sync(kFull, below, src), more, lane);
-                  if (lane == src) take = tk;
-                }
-                if (take) l0[w0 - 1 - lane] = below & ~take;
-              }
-              acc = n0 + sum;
-              if (acc >= z) {
-                acc = z;
-              } else {
-                if (w0 > 32) {
-                  acc += fb.pop_words(w0 - 32, z - acc, lane);
-                  old0 = fb.l1[v0 >> 5];  // it may have cleared bits there
-                  old1 = fb.l1[(v0 >> 5) + 1];
-                }
-                if (acc < z) fb.low = p;  // nothing is left below p, and free times are added above it
-              }
-            }
-            const uint32_t rest = z - acc, inf = rest < free_inf ? rest : (uint32_t)free_inf;
-            free_inf -= inf;
-            acc += inf;
-            if (acc < z) {  // the first acc of them hit
-              uint32_t zm = ~Bk & valid, sum;
-              if (edge && lane == elane) zm &= ~ebit;
-              const uint32_t zc = __popc(zm), zx = lanes_excl(zc, &sum);
-              A = (valid & ~zm) | (zx + zc <= acc ? zm : 0u);
-              const uint32_t part = __ballot_sync(kFull, zx < acc && zx + zc > acc);
-              if (part) {
-                const uint32_t src = __ffs(part) - 1;
-                const uint32_t tk = low_bits(__shfl_sync(kFull, zm, src), acc - __shfl_sync(kFull, zx, src), lane);
-                if (lane == src) A |= tk;
-              }
-              const bool hit0 = ((__shfl_sync(kFull, Bk, 0) >> sp) & 1u) || acc >= 1;
-              if (edge && !hit0 && lane == elane) A &= ~ebit;
-              const uint32_t rej = valid & ~A;
-              const uint32_t with = __ballot_sync(kFull, rej != 0);
-              nh = Lj - __reduce_add_sync(kFull, __popc(rej));
-              const uint32_t l_f = __ffs(with) - 1;
-              f = 32 * l_f + __ffs(__shfl_sync(kFull, rej, l_f)) - 1 - sp;
-            }
-          }
-          if (has && left != word) l0[w] = left;
-          // New free times s - 1 + k of the hits; with p + Lj = s the last step
-          // took step 0's.  They lie above every free time so far.
-          {
-            uint32_t T = A;
-            if (edge && lane == 0) T &= ~(1u << sp);
-            const uint32_t sq = (s - 1) & 31;
-            const uint32_t up = __shfl_up_sync(kFull, T, 1), dn = __shfl_down_sync(kFull, T, 1);
-            uint32_t out, past = 0;  // words v0 + lane, and v0 + 32 (lane 31)
-            if (sq >= sp) {
-              const uint32_t d = sq - sp;
-              out = T << d | (d && lane ? up >> (32 - d) : 0u);
-              if (d && lane == 31) past = T >> (32 - d);
+        continue;
+      }
+      while (L > 0) {
+        const uint32_t gap = s - p, sp = p & 31;
+        uint32_t Lj = L < gap ? L : gap;
+        if (Lj > 1024 - sp) Lj = 1024 - sp;  // the 32 words from p's
+        // this lane's word of them (positions 32 (w0 + lane) ..) and of the 32 below
+        const uint32_t w0 = p >> 5, w = w0 + lane;
+        const uint32_t end = sp + Lj;  // past the last step, counted from word w0
+        uint32_t valid = lane * 32 >= end ? 0u : end - lane * 32 >= 32 ? kFull : mask_lt(end - lane * 32);
+        const bool has = valid != 0 && in_bounds(a.st, w, a.s0);
+        const uint32_t word = has ? l0[w] : 0u;
+        const uint32_t below = w0 > lane ? l0[w0 - 1 - lane] : 0u;
+        // the level-1 words of the 32 words where this chunk's free times go
+        const uint32_t v0 = (s - 1) >> 5;
+        uint32_t old0 = fb.l1[v0 >> 5], old1 = fb.l1[(v0 >> 5) + 1];
+        if (lane == 0) valid &= ~mask_lt(sp);
+        const uint32_t Bk = word & valid;
+        const bool edge = Lj >= 2 && p + Lj == s;  // the last step: decided by step 0 below
+        const uint32_t elane = (end - 1) >> 5, ebit = 1u << ((end - 1) & 31);
+        const uint32_t z = Lj - edge - __reduce_add_sync(kFull, __popc(Bk));
+        uint32_t left = word & ~valid;  // the free times of [p, p + Lj) are used up
+        uint32_t A = valid;        // steps that hit
+        uint32_t nh = Lj, f = Lj;  // hits, and hits before the first miss
+        if (z) {
+          // the other steps take the latest free times below p, then never-used tracks
+          uint32_t acc = 0;
+          if (p > fb.low) {
+            const uint32_t first = __shfl_sync(kFull, word, 0) & mask_lt(sp);  // those in p's own word
+            uint32_t sum;
+            const uint32_t c = __popc(below), n0 = __popc(first), above = n0 + lanes_excl(c, &sum);
+            if (n0 > z) {
+              const uint32_t tk = top_bits(first, z, lane);
+              if (lane == 0) left &= ~tk;
             } else {
-              const uint32_t d = sp - sq;
-              out = T >> d | (lane < 31 ? dn << (32 - d) : 0u);
+              if (lane == 0) left &= ~first;
+              uint32_t take = above + c <= z ? below : 0u;
+              const uint32_t part = __ballot_sync(kFull, above < z && above + c > z);
+              if (part) {  // the word that holds the last one wanted
+                const uint32_t src = __ffs(part) - 1;
+                const uint32_t more = z - __shfl_sync(kFull, above, src);
+                const uint32_t tk = top_bits(__shfl_sync(kFull, below, src), more, lane);
+                if (lane == src) take = tk;
+              }
+              if (take) l0[w0 - 1 - lane] = below & ~take;
             }
-            // what word v0 holds already: the tail's bits, read back if this
-            // run's updates may have met that word
-            if ((p + Lj - 1) >> 5 >= v0) {
-              __syncwarp();  // the words cleared above
-              tail_w = v0;
-              tail = in_bounds(a.st, v0, a.s0) ? l0[v0] : 0u;
-              if (lane == 0 && out) out |= tail;
-              __syncwarp();
-            } else if (v0 == tail_w && lane == 0 && out) {
-              out |= tail;
-            }
-            if (out && in_bounds(a.st, v0 + lane, a.s0)) l0[v0 + lane] = out;
-            if (past && in_bounds(a.st, v0 + 32, a.s0)) l0[v0 + 32] = past;
-            const uint32_t set = __ballot_sync(kFull, out != 0);
-            fb.mark(v0, set, old0, old1, lane);
-            const uint32_t over = __shfl_sync(kFull, past, 31);
-            if (over) {
-              fb.mark(v0 + 32, 1u, fb.l1[(v0 >> 5) + 1], 0u, lane);
-              tail_w = v0 + 32;
-              tail = over;
-            } else if (set) {
-              const uint32_t l_t = hi_bit(set);
-              tail_w = v0 + l_t;
-              tail = __shfl_sync(kFull, out, l_t);
+            acc = n0 + sum;
+            if (acc >= z) {
+              acc = z;
+            } else {
+              if (w0 > 32) {
+                acc += fb.pop_words(w0 - 32, z - acc, lane);
+                old0 = fb.l1[v0 >> 5];  // it may have cleared bits there
+                old1 = fb.l1[(v0 >> 5) + 1];
+              }
+              if (acc < z) fb.low = p;  // nothing is left below p, and free times are added above it
             }
           }
-          raw += nh;
-          if (!missed) {
-            hits += f;
-            depths += (uint64_t)f * (s - req_start) + (uint64_t)f * (f ? f - 1 : 0) / 2;
-            if (f < Lj) missed = true;
+          const uint32_t rest = z - acc, inf = rest < free_inf ? rest : (uint32_t)free_inf;
+          free_inf -= inf;
+          acc += inf;
+          if (acc < z) {  // the first acc of them hit
+            uint32_t zm = ~Bk & valid, sum;
+            if (edge && lane == elane) zm &= ~ebit;
+            const uint32_t zc = __popc(zm), zx = lanes_excl(zc, &sum);
+            A = (valid & ~zm) | (zx + zc <= acc ? zm : 0u);
+            const uint32_t part = __ballot_sync(kFull, zx < acc && zx + zc > acc);
+            if (part) {
+              const uint32_t src = __ffs(part) - 1;
+              const uint32_t tk = low_bits(__shfl_sync(kFull, zm, src), acc - __shfl_sync(kFull, zx, src), lane);
+              if (lane == src) A |= tk;
+            }
+            const bool hit0 = ((__shfl_sync(kFull, Bk, 0) >> sp) & 1u) || acc >= 1;
+            if (edge && !hit0 && lane == elane) A &= ~ebit;
+            const uint32_t rej = valid & ~A;
+            const uint32_t with = __ballot_sync(kFull, rej != 0);
+            nh = Lj - __reduce_add_sync(kFull, __popc(rej));
+            const uint32_t l_f = __ffs(with) - 1;
+            f = 32 * l_f + __ffs(__shfl_sync(kFull, rej, l_f)) - 1 - sp;
           }
-          s += Lj;
-          p += Lj;
-          L -= Lj;
         }
+        if (has && left != word) l0[w] = left;
+        // New free times s - 1 + k of the hits; with p + Lj = s the last step
+        // took step 0's.  They lie above every free time so far.
+        {
+          uint32_t T = A;
+          if (edge && lane == 0) T &= ~(1u << sp);
+          const uint32_t sq = (s - 1) & 31;
+          const uint32_t up = __shfl_up_sync(kFull, T, 1), dn = __shfl_down_sync(kFull, T, 1);
+          uint32_t out, past = 0;  // words v0 + lane, and v0 + 32 (lane 31)
+          if (sq >= sp) {
+            const uint32_t d = sq - sp;
+            out = T << d | (d && lane ? up >> (32 - d) : 0u);
+            if (d && lane == 31) past = T >> (32 - d);
+          } else {
+            const uint32_t d = sp - sq;
+            out = T >> d | (lane < 31 ? dn << (32 - d) : 0u);
+          }
+          // what word v0 holds already: the tail's bits, read back if this
+          // run's updates may have met that word
+          if ((p + Lj - 1) >> 5 >= v0) {
+            __syncwarp();  // the words cleared above
+            tail_w = v0;
+            tail = in_bounds(a.st, v0, a.s0) ? l0[v0] : 0u;
+            if (lane == 0 && out) out |= tail;
+            __syncwarp();
+          } else if (v0 == tail_w && lane == 0 && out) {
+            out |= tail;
+          }
+          if (out && in_bounds(a.st, v0 + lane, a.s0)) l0[v0 + lane] = out;
+          if (past && in_bounds(a.st, v0 + 32, a.s0)) l0[v0 + 32] = past;
+          const uint32_t set = __ballot_sync(kFull, out != 0);
+          fb.mark(v0, set, old0, old1, lane);
+          const uint32_t over = __shfl_sync(kFull, past, 31);
+          if (over) {
+            fb.mark(v0 + 32, 1u, fb.l1[(v0 >> 5) + 1], 0u, lane);
+            tail_w = v0 + 32;
+            tail = over;
+          } else if (set) {
+            const uint32_t l_t = hi_bit(set);
+            tail_w = v0 + l_t;
+            tail = __shfl_sync(kFull, out, l_t);
+          }
+        }
+        raw += nh;
+        if (!missed) {
+          hits += f;
+          depths += (uint64_t)f * (s - req_start) + (uint64_t)f * (f ? f - 1 : 0) / 2;
+          if (f < Lj) missed = true;
+        }
+        s += Lj;
+        p += Lj;
+        L -= Lj;
       }
     }
-    __syncthreads();
   }
   uint64_t sv_lo = 0, sv_hi = 0;  // depths fits 64 bits: fewer than 2^32 hits at depths below 2^32
   add_mul(sv_lo, sv_hi, a.alpha, hits);
