@@ -1,7 +1,7 @@
 // Session-level LRU eviction at every capacity of a grid (Sec. 5.3: block-
 // level vs session-level eviction).  Session-level eviction is not a stack
 // algorithm (a cache of C + 1 blocks can hold a session that a cache of C
-// blocks dropped whole), so each capacity is its own replay: one warp per
+// blocks dropped whole), so each capacity is its own replay: one CTA per
 // capacity walks the trace in order.
 //
 // Readings: a block belongs to the session whose request brought it in,
@@ -23,19 +23,21 @@
 //              blocks (a passed entry never becomes valid again, so the front
 //              only moves forward).
 // The replay of one capacity is a serial chain, so what bounds it is the
-// latency of a step.  One warp (the replayer) settles a window of up to 256
-// accesses of one request per step, eight per lane: owners, then epochs, then
-// one ballot per 32 accesses.  All misses that fit settle together; a miss
-// that takes the cache past C evicts (the queue is searched 32 requests at a
-// time) and the accesses after it are tested again from the owners in
-// registers, since an eviction can drop a later block of the window.  Once
-// the current session is alone and above C, every later block of the window
-// misses, and they settle in closed form.  Eight other warps read ahead: the
-// ids of the next 4,096 accesses into shared memory, and the owner words of
-// those ids into L1, so that the replayer's owner reads hit L1 (its own
-// stores go through the same L1) instead of waiting for DRAM: the owner table
-// takes 8 bytes per block and capacity.  Epochs, counts and latest requests
-// sit in shared memory when there are at most 14,336 sessions.
+// latency of a step.  A step settles a window of up to kSesWin accesses of one
+// request: each of the replaying warps takes 32 of them (owner, epoch, one
+// ballot), a barrier counts the misses, the ballots are exchanged through shared
+// memory where there are some, and every warp draws the same conclusions from
+// them, so that the replay's state needs no other exchange.  All misses that fit
+// settle together; a miss that takes the cache past C evicts (the queue is
+// searched 32 requests at a time) and the accesses after it are tested again
+// from the owners in registers, since an eviction can drop a later block of the
+// window.  Once the current session is alone and above C, every later block of
+// the window misses, and they settle in closed form.  Eight other warps read
+// ahead: the ids of the next 4,096 accesses into shared memory, and the owner
+// words of those ids into L1, so that the owner reads hit L1 (the replayers'
+// stores go through the same L1) instead of waiting for L2 or DRAM: the owner
+// table takes 8 bytes per block and capacity.  Epochs, counts and latest
+// requests sit in shared memory when there are at most 14,336 sessions.
 //
 // Ids of prefix chains rise strictly within a request (a prefix first occurs
 // no later than its extensions), so no window holds a block twice.  Whether
@@ -43,11 +45,13 @@
 // do not, every window is settled 32 accesses at a time, a second copy of a
 // block after the first.
 //
-// Measured on the 9.3M-access chat trace, 64 capacities: 486 ms with one warp per
-// capacity, 32 accesses a step and owners read from DRAM as they came; 116 ms
-// with the windows read ahead; 55 ms with epochs read together, the check for
-// repeats made once and 4,096 accesses read ahead at a time (33 ms at the
-// largest capacity, 55 at the smallest, which evicts in every window).
+// Measured on the 9.3M-access chat trace, 64 capacities: 486 ms with one warp
+// per capacity, 32 accesses a step and owners read from DRAM as they came; 116
+// ms with 128 accesses a step and the ids read ahead; 55 ms with the epochs read
+// together and the check for repeats made once; 41 ms with 16 warps and one
+// barrier per eviction (43.9 without the owners read ahead).  The smallest
+// capacities take longest: they evict in every window (40.7 ms for 64 blocks,
+// 20.3 for 1.6M).
 #include "ptc_internal.h"
 
 namespace ptc {
@@ -101,86 +105,105 @@ __global__ void k_ses_check(const uint64_t* __restrict__ blk_off, uint32_t R, ui
 }
 
 constexpr uint32_t kSesSmemSessions = 14336;  // session state kept in shared memory up to this many
-constexpr uint32_t kSesPer = 8;                // accesses per lane and window
-constexpr uint32_t kSesWin = 32 * kSesPer;
+constexpr uint32_t kSesReplay = 16;            // warps that replay
+constexpr uint32_t kSesWin = 32 * kSesReplay;  // accesses per window, one per lane
 constexpr uint32_t kSesAhead = 8;              // warps that read ahead
 constexpr uint32_t kSesAheadPer = 16;          // accesses per lane that a batch reads ahead
 constexpr uint32_t kSesBatch = kSesAhead * 32 * kSesAheadPer;  // 4,096 accesses
-constexpr uint32_t kSesThreads = 32 * (1 + kSesAhead);
+constexpr uint32_t kSesThreads = 32 * (kSesReplay + kSesAhead);
 
-// Ids of the batch being replayed and the two after it.
+// Ids of the batch being replayed and the two after it, and what the replaying
+// warps exchange.
+struct SesShared {  // the replay's state, where one warp has moved it on alone
+  uint64_t total, hits, depths;
+  uint32_t cnt, es;
+  bool missed;
+};
 struct SesRing {
   uint32_t ids[3][kSesBatch];
+  uint32_t slots[2][32];  // exchanged ballots
+  uint32_t touched[kSesAhead];
+  SesShared state;
 };
 
-// One capacity's session state; the pointers go to shared or global memory,
-// and only the replaying warp touches them.
+// One capacity's session state, in shared or global memory.  Every replaying
+// warp reads it, the first one's lane 0 writes it.
 struct SesState {
   uint32_t *ep, *count, *last;
 };
 
-// Evict until at most C blocks are resident, after block x came in for
-// session s (whose epoch is es and which holds cnt blocks) in request r.
-// Returns true if session s itself was emptied but for x.
-__device__ __forceinline__ bool ses_evict(const SesArgs& a, const SesState& S, uint64_t* owner, uint32_t lane,
-                                          uint32_t r, uint32_t s, uint32_t x, uint64_t C, uint32_t& front,
-                                          uint64_t& total, uint32_t& cnt, uint32_t& es) {
-  while (total > C) {
-    uint32_t v = kNone;
-    while (front < r) {
-      const uint32_t f = front + lane;
-      uint32_t t = 0;
-      bool ok = f < r;
-      if (ok) {
-        t = a.ses[f];
-        ok = in_bounds(a.st, t, a.n_session) && S.last[t] == f && S.count[t] > 0;
-      }
-      const uint32_t m = __ballot_sync(kFull, ok);
-      if (m) {
-        const uint32_t b = __ffs(m) - 1;
-        v = __shfl_sync(kFull, t, b);
-        front += b + 1;
-        break;
-      }
-      front = r - front > 32 ? front + 32 : r;
+// The front of the recency queue, and the sessions of the 32 requests around
+// it, one per lane.
+struct SesFront {
+  uint32_t front = 0, base = kNone, ses = 0;
+};
+
+// A barrier of the replaying warps.
+__device__ __forceinline__ void replay_sync() { asm volatile("bar.sync 1, %0;" ::"r"(32 * kSesReplay) : "memory"); }
+
+// The least recently touched session before request r that holds blocks, or
+// kNone.  Whole warps only.
+__device__ __forceinline__ uint32_t ses_victim(const SesArgs& a, const SesState& S, uint32_t lane, uint32_t r,
+                                               SesFront& q) {
+  while (q.front < r) {
+    if ((q.front & ~31u) != q.base) {
+      q.base = q.front & ~31u;
+      q.ses = q.base + lane < a.n_req ? a.ses[q.base + lane] : 0u;
     }
-    if (v == kNone) {  // the current session alone is above C: it keeps the block just brought in
-      es += 1;
-      cnt = 1;
-      total = 1;
-      __syncwarp();
-      if (lane == 0) {
-        S.ep[s] = es;
-        owner[x] = ((uint64_t)s << 32) | es;
-      }
-      __syncwarp();
-      return true;
+    const uint32_t f = q.base + lane;
+    const bool ok =
+        f >= q.front && f < r && in_bounds(a.st, q.ses, a.n_session) && S.last[q.ses] == f && S.count[q.ses] > 0;
+    const uint32_t m = __ballot_sync(kFull, ok);
+    if (m) {
+      const uint32_t b = __ffs(m) - 1;
+      q.front = q.base + b + 1;
+      return __shfl_sync(kFull, q.ses, b);
     }
-    // the least recently touched other session goes whole
-    total -= S.count[v];
-    __syncwarp();
-    if (lane == 0) {
-      S.ep[v] = S.ep[v] + 1u;
-      S.count[v] = 0;
-    }
-    __syncwarp();
+    q.front = r - q.base > 32 ? q.base + 32 : r;
   }
-  return false;
+  return kNone;
 }
 
-// Which of the owner words in `o` name a resident block: every epoch is read
-// before any is compared, so the reads overlap.
-template <int N>
-__device__ __forceinline__ void ses_resident(const SesArgs& a, const SesState& S, const uint64_t (&o)[N],
-                                             bool (&res)[N]) {
-  uint32_t ep[N];
+// Whether owner word `o` names a resident block, where sessions v and w are
+// known to have been evicted.
+__device__ __forceinline__ bool ses_resident(const SesArgs& a, const SesState& S, uint64_t o, uint32_t v = kNone,
+                                             uint32_t w = kNone) {
+  const uint32_t t = o == kNoOwner ? 0u : (uint32_t)(o >> 32);
+  const uint32_t ep = in_bounds(a.st, t, a.n_session) ? S.ep[t] : 0u;
+  return o != kNoOwner && ep == (uint32_t)o && t != v && t != w;
+}
+
+// The misses of a window: every warp stores its ballot, and the barrier itself
+// counts them.
+__device__ __forceinline__ uint32_t ses_count(bool miss, uint32_t* slots, uint32_t warp, uint32_t lane) {
+  const uint32_t mine = __ballot_sync(kFull, miss);
+  if (lane == 0) slots[warp] = mine;
+  uint32_t all;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "setp.ne.u32 p, %1, 0;\n\t"
+      "barrier.cta.red.popc.aligned.u32 %0, 1, %2, p;\n\t}"
+      : "=r"(all)
+      : "r"((uint32_t)miss), "r"(32 * kSesReplay)
+      : "memory");
+  return all;
+}
+// Lane w < kSesReplay holds warp w's ballot and the misses of the warps before.
+struct SesMisses {
+  uint32_t mask, before;
+};
+__device__ __forceinline__ SesMisses ses_misses(const uint32_t* slots, uint32_t lane) {
+  SesMisses m;
+  m.mask = lane < kSesReplay ? slots[lane] : 0u;
+  const uint32_t c = __popc(m.mask);
+  uint32_t x = c;
 #pragma unroll
-  for (int u = 0; u < N; ++u) {
-    const uint32_t t = o[u] == kNoOwner ? 0u : (uint32_t)(o[u] >> 32);
-    ep[u] = in_bounds(a.st, t, a.n_session) ? S.ep[t] : 0u;
+  for (int o = 1; o < (int)kSesReplay; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kFull, x, o);
+    if (lane >= (uint32_t)o) x += y;
   }
-#pragma unroll
-  for (int u = 0; u < N; ++u) res[u] = o[u] != kNoOwner && ep[u] == (uint32_t)o[u];
+  m.before = x - c;
+  return m;
 }
 
 template <bool SMEM>
@@ -192,8 +215,7 @@ __global__ void __launch_bounds__(kSesThreads, 1) k_ses_sim(SesArgs a, SesCaps c
   const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t g = blockIdx.x;
   if (g >= a.G) return;
-  // malformed offsets or labels: nothing to replay (one answer for the whole
-  // CTA: another capacity may report a bad id meanwhile)
+  // malformed offsets, labels or ids: nothing to replay
   if (__syncthreads_or(threadIdx.x == 0 && ld_relaxed_u32(&a.st->err) != 0)) return;
   uint64_t* owner = a.owner + g * a.sD;
   SesState S;
@@ -216,43 +238,48 @@ __global__ void __launch_bounds__(kSesThreads, 1) k_ses_sim(SesArgs a, SesCaps c
   // together and once per batch: L1 answers in order, so the replayer's hits
   // wait while any of these misses is outstanding.
   auto read_ahead = [&](uint32_t t_owner, uint32_t t_ids) {
-    const uint32_t k0 = (warp - 1) * 32 * kSesAheadPer + lane;
+    const uint32_t k0 = (warp - kSesReplay) * 32 * kSesAheadPer + lane;
     const uint64_t owners = (uint64_t)t_owner * kSesBatch, next = (uint64_t)t_ids * kSesBatch;
-    uint32_t id[kSesAheadPer], o[kSesAheadPer];
+    uint32_t id[kSesAheadPer], touched = 0;
 #pragma unroll
     for (uint32_t u = 0; u < kSesAheadPer; ++u) {
       const uint32_t k = k0 + 32 * u;
       id[u] = next + k < n ? __ldg(&a.ids[next + k]) : 0u;
     }
+    if (t_owner != kNone) {
 #pragma unroll
-    for (uint32_t u = 0; u < kSesAheadPer; ++u) {  // the values are not used
-      const uint32_t k = k0 + 32 * u;
-      o[u] = 0;
-      if (t_owner != kNone && owners + k < n)
-        asm volatile("ld.global.ca.u32 %0, [%1];" : "=r"(o[u]) : "l"(owner + ring.ids[t_owner % 3][k]));
+      for (uint32_t u = 0; u < kSesAheadPer; ++u) {
+        const uint32_t k = k0 + 32 * u;
+        if (owners + k < n) touched ^= *reinterpret_cast<const uint32_t*>(owner + ring.ids[t_owner % 3][k]);
+      }
     }
 #pragma unroll
     for (uint32_t u = 0; u < kSesAheadPer; ++u) ring.ids[t_ids % 3][k0 + 32 * u] = id[u];
-#pragma unroll
-    for (uint32_t u = 0; u < kSesAheadPer; ++u) asm volatile("" ::"r"(o[u]));
+    // nobody reads it: without a use the loads that bring the words into L1
+    // would be removed
+    ring.touched[warp - kSesReplay] = touched;
   };
   const uint64_t C = caps.c[g];
   const uint32_t per = C < kSesWin ? (uint32_t)C : 2 * kSesWin;  // misses between two resets of a lone session
-  const uint32_t per_inv = 65536u / per + 1;  // k / per = k per_inv >> 16 for k < 256 (per <= 256), and 0 above
+  const uint32_t per_inv = (1u << 20) / per + 1;  // k / per = k per_inv >> 20 for k < kSesWin, per <= 2 kSesWin
   const bool repeats = __ldg(falls) != 0;
   uint64_t total = 0;
   uint64_t hits = 0, depths = 0;  // counted hits and their depths
-  uint32_t front = 0;
-  // the current request; 32 requests' sessions and ends at a time, one per lane
-  uint32_t r = kNone, s = 0, b = 0, e = 0, es = 0, cnt = 0, q_s = 0, q_e = 0;
+  SesFront queue;
+  // the current request; 32 requests' sessions and ends at a time, one per lane.
+  // Every replaying warp keeps all of this.
+  uint32_t r = kNone, s = kNone, b = 0, e = 0, es = 0, cnt = 0, q_s = 0, q_e = 0;
+  uint32_t turn = 0;  // which of the two sets of exchange slots is next
+  const bool writer = threadIdx.x == 0;
   bool missed = false;
   const uint32_t batches = (uint32_t)(((uint64_t)n + kSesBatch - 1) / kSesBatch);
-  if (warp) read_ahead(kNone, 0);
+  const bool ahead = warp >= kSesReplay;
+  if (ahead) read_ahead(kNone, 0);
   __syncthreads();
-  if (warp) read_ahead(0, 1);
+  if (ahead) read_ahead(0, 1);
   __syncthreads();
   for (uint32_t t = 0; t < batches; ++t) {
-    if (warp) {
+    if (ahead) {
       if (t + 1 < batches) read_ahead(t + 1, t + 2);
       __syncthreads();
       continue;
@@ -261,23 +288,35 @@ __global__ void __launch_bounds__(kSesThreads, 1) k_ses_sim(SesArgs a, SesCaps c
     const uint64_t t0 = (uint64_t)t * kSesBatch;
     const uint32_t size = n - t0 < kSesBatch ? (uint32_t)(n - t0) : kSesBatch;
     uint32_t at = 0;  // accesses of this batch settled
+    // The window in registers: this lane's id and owner word (of the whole
+    // window, whichever requests it meets), read again after a step that stored
+    // owners.  The next window's are read while this one's misses are counted.
+    uint32_t cur = kNone, id = 0, next_id = 0;
+    uint64_t o = kNoOwner, next_o = kNoOwner;
+    bool stale = false, ready = false;
     while (at < size) {
-      while (t0 + at >= e) {  // the next request (one without accesses only touches its session)
-        if (r != kNone && lane == 0) S.count[s] = cnt;
-        ++r;
-        if (r >= a.n_req) break;  // cannot happen: the offsets were checked
-        if ((r & 31) == 0) {
-          q_s = r + lane < a.n_req ? a.ses[r + lane] : 0u;
-          q_e = r + lane < a.n_req ? (uint32_t)a.blk_off[r + lane + 1] : 0u;
+      if (t0 + at >= e) {  // the next request with accesses (those without only touch their sessions)
+        uint32_t next_s = s;
+        do {
+          ++r;
+          if (r >= a.n_req) break;  // cannot happen: the offsets were checked
+          if ((r & 31) == 0) {
+            q_s = r + lane < a.n_req ? a.ses[r + lane] : 0u;
+            q_e = r + lane < a.n_req ? (uint32_t)a.blk_off[r + lane + 1] : 0u;
+          }
+          next_s = __shfl_sync(kFull, q_s, r & 31);
+          b = e;
+          e = __shfl_sync(kFull, q_e, r & 31);
+          if (writer) S.last[next_s] = r;
+        } while (t0 + at >= e);
+        // the new session's count was stored, and every epoch, before the last
+        // window's barrier
+        if (next_s != s) {
+          if (writer && s != kNone) S.count[s] = cnt;
+          s = next_s;
+          es = S.ep[s];
+          cnt = S.count[s];
         }
-        s = __shfl_sync(kFull, q_s, r & 31);
-        b = e;
-        e = __shfl_sync(kFull, q_e, r & 31);
-        __syncwarp();
-        if (lane == 0) S.last[s] = r;
-        __syncwarp();
-        es = S.ep[s];
-        cnt = S.count[s];
         missed = false;
       }
       if (t0 + at >= e) break;
@@ -288,144 +327,169 @@ __global__ void __launch_bounds__(kSesThreads, 1) k_ses_sim(SesArgs a, SesCaps c
       const uint64_t depth = t0 + at - b;
       at = w0 + hi;
       if (repeats) {
-        // ---- a block may come twice: 32 accesses at a time
-        uint64_t d0 = depth;
-        for (uint32_t c = lo & ~31u; c < hi; c += 32) {
-          const uint32_t k = c + lane;
-          const uint32_t x = ids[w0 + k];
-          uint32_t pending = __ballot_sync(kFull, k >= lo && k < hi);
-          while (pending) {
-            const bool mine = (pending >> lane) & 1u;
-            const uint64_t o1[1] = {mine ? owner[x] : kNoOwner};
-            bool r1[1];
-            ses_resident<1>(a, S, o1, r1);
-            const bool res = r1[0];
-            uint32_t same = 0;
-            if (mine) same = __match_any_sync(pending, x);
-            const uint32_t later_copy = __ballot_sync(kFull, mine && (same & lanemask_lt()) != 0);
-            const uint32_t ms = __ballot_sync(kFull, mine && !res);
-            const uint64_t room = C - total;
-            uint32_t over = 32;  // the first miss that would push the cache past C
-            if ((uint64_t)__popc(ms) > room) {
-              uint32_t m = ms;
-              for (uint64_t q = 0; q < room; ++q) m &= m - 1u;
-              over = (uint32_t)(__ffs(m) - 1);
+        // ---- a block may come twice: 32 accesses at a time, by the first warp
+        replay_sync();  // the request's state is written
+        if (warp == 0) {
+          uint64_t d0 = depth;
+          for (uint32_t c = lo & ~31u; c < hi; c += 32) {
+            const uint32_t k = c + lane;
+            const uint32_t x = ids[w0 + k];
+            uint32_t pending = __ballot_sync(kFull, k >= lo && k < hi);
+            while (pending) {
+              const bool mine = (pending >> lane) & 1u;
+              const bool res = ses_resident(a, S, mine ? owner[x] : kNoOwner);
+              uint32_t same = 0;
+              if (mine) same = __match_any_sync(pending, x);
+              const uint32_t later_copy = __ballot_sync(kFull, mine && (same & lanemask_lt()) != 0);
+              const uint32_t ms = __ballot_sync(kFull, mine && !res);
+              const uint64_t room = C - total;
+              uint32_t over = 32;  // the first miss that would push the cache past C
+              if ((uint64_t)__popc(ms) > room) {
+                uint32_t m = ms;
+                for (uint64_t q = 0; q < room; ++q) m &= m - 1u;
+                over = (uint32_t)(__ffs(m) - 1);
+              }
+              const uint32_t rep = later_copy ? (uint32_t)(__ffs(later_copy) - 1) : 32u;
+              const uint32_t stop = over < rep ? over : rep;
+              const uint32_t part = pending & (stop == 32 ? kFull : ((1u << stop) - 1u));
+              const uint32_t pm = ms & part;
+              __syncwarp();
+              if ((pm >> lane) & 1u) owner[x] = ((uint64_t)s << 32) | es;
+              total += __popc(pm);
+              cnt += __popc(pm);
+              if (!missed && part) {
+                const uint32_t f0 = __ffs(part) - 1;
+                const uint32_t f = (pm ? (uint32_t)(__ffs(pm) - 1) : 32u - __clz(part)) - f0;
+                hits += f;
+                depths += (uint64_t)f * d0 + (uint64_t)f * (f ? f - 1 : 0) / 2;
+                missed = pm != 0;
+              }
+              d0 += __popc(part);
+              pending &= ~part;
+              __syncwarp();
+              if (stop == 32 || stop == rep) continue;  // done, or a repeated block: test it again
+              const uint32_t y = __shfl_sync(kFull, x, stop);
+              // one block too many: the least recently touched other session
+              // goes whole, or, with none left, this one but for block y
+              const uint32_t v = ses_victim(a, S, lane, r, queue);
+              if (v == kNone) {
+                es += 1;
+                cnt = 1;
+                total = 1;
+              } else {
+                cnt += 1;
+                total = C + 1 - S.count[v];
+              }
+              __syncwarp();
+              if (writer) {
+                owner[y] = ((uint64_t)s << 32) | es;
+                if (v == kNone) {
+                  S.ep[s] = es;
+                } else {
+                  S.ep[v] += 1u;
+                  S.count[v] = 0;
+                }
+              }
+              __syncwarp();
+              missed = true;
+              d0 += 1;
+              pending &= ~(1u << stop);
             }
-            const uint32_t rep = later_copy ? (uint32_t)(__ffs(later_copy) - 1) : 32u;
-            const uint32_t stop = over < rep ? over : rep;
-            const uint32_t part = pending & (stop == 32 ? kFull : ((1u << stop) - 1u));
-            const uint32_t pm = ms & part;
-            __syncwarp();
-            if ((pm >> lane) & 1u) owner[x] = ((uint64_t)s << 32) | es;
-            total += __popc(pm);
-            cnt += __popc(pm);
-            if (!missed && part) {
-              const uint32_t f0 = __ffs(part) - 1;
-              const uint32_t f = (pm ? (uint32_t)(__ffs(pm) - 1) : 32u - __clz(part)) - f0;
-              hits += f;
-              depths += (uint64_t)f * d0 + (uint64_t)f * (f ? f - 1 : 0) / 2;
-              missed = pm != 0;
-            }
-            d0 += __popc(part);
-            pending &= ~part;
-            __syncwarp();
-            if (stop == 32 || stop == rep) continue;  // done, or a repeated block: test it again
-            const uint32_t y = __shfl_sync(kFull, x, stop);
-            if (lane == 0) owner[y] = ((uint64_t)s << 32) | es;
-            total += 1;
-            cnt += 1;
-            ses_evict(a, S, owner, lane, r, s, y, C, front, total, cnt, es);
-            missed = true;
-            d0 += 1;
-            pending &= ~(1u << stop);
           }
+          if (writer) ring.state = SesShared{total, hits, depths, cnt, es, missed};
+        }
+        replay_sync();
+        total = ring.state.total;
+        hits = ring.state.hits;
+        depths = ring.state.depths;
+        cnt = ring.state.cnt;
+        es = ring.state.es;
+        missed = ring.state.missed;
+        continue;
+      }
+      const uint32_t k = 32 * warp + lane;
+      const bool valid = k >= lo && k < hi;
+      if (cur != w0) {
+        id = ready ? next_id : ids[w0 + k];
+        o = ready ? next_o : w0 + k < size ? owner[id] : kNoOwner;
+        cur = w0;
+      } else if (stale) {
+        o = w0 + k < size ? owner[id] : kNoOwner;
+      }
+      bool miss = valid && !ses_resident(a, S, o);
+      ready = w0 + hi < size && hi == kSesWin;
+      if (ready) {
+        next_id = ids[w0 + kSesWin + k];
+        next_o = w0 + kSesWin + k < size ? owner[next_id] : kNoOwner;
+      }
+      uint32_t all = ses_count(miss, ring.slots[turn ^= 1], warp, lane);
+      stale = all != 0;
+      if (all == 0) {
+        if (!missed) {
+          const uint32_t f = hi - lo;
+          hits += f;
+          depths += (uint64_t)f * depth + (uint64_t)f * (f - 1) / 2;
         }
         continue;
       }
-      uint32_t id[kSesPer], miss[kSesPer];
-      uint64_t o[kSesPer];
-      bool res[kSesPer];
-#pragma unroll
-      for (uint32_t u = 0; u < kSesPer; ++u) id[u] = ids[w0 + 32 * u + lane];
-#pragma unroll
-      for (uint32_t u = 0; u < kSesPer; ++u) o[u] = 32 * u + lane >= lo && 32 * u + lane < hi ? owner[id[u]] : kNoOwner;
-      ses_resident<kSesPer>(a, S, o, res);
-      uint32_t m_all = 0, first = hi;
-#pragma unroll
-      for (int u = kSesPer - 1; u >= 0; --u) {
-        const uint32_t k = 32 * u + lane;
-        miss[u] = __ballot_sync(kFull, k >= lo && k < hi && !res[u]);
-        m_all += __popc(miss[u]);
-        if (miss[u]) first = 32 * u + __ffs(miss[u]) - 1;
-      }
+      ready = false;
       if (!missed) {  // the hits before the first miss
-        const uint32_t f = first - lo;
+        const uint32_t mask = lane < kSesReplay ? ring.slots[turn][lane] : 0u;
+        const uint32_t fw = __ffs(__ballot_sync(kFull, mask != 0)) - 1;
+        const uint32_t f = 32 * fw + __ffs(__shfl_sync(kFull, mask, fw)) - 1 - lo;
         hits += f;
         depths += (uint64_t)f * depth + (uint64_t)f * (f ? f - 1 : 0) / 2;
-        missed = m_all != 0;
+        missed = true;
       }
-      if (m_all == 0) continue;
       const uint64_t stamp = ((uint64_t)s << 32) | es;
-      while (total + m_all > C) {
+      uint32_t v = kNone;
+      while (total + all > C) {
         // the misses before the one that overflows (the room-th, from 0)
         // settle, and so does that one before it evicts
         const uint32_t room = (uint32_t)(C - total);
-        uint32_t x_u = 0, x_m = 0, before = 0, x_before = 0, x_id = 0;
-#pragma unroll
-        for (uint32_t u = 0; u < kSesPer; ++u) {
-          const uint32_t c = __popc(miss[u]);
-          if (before <= room && before + c > room) {
-            x_u = u;
-            x_m = miss[u];
-            x_before = before;
-            x_id = id[u];
-          }
-          before += c;
-        }
+        const SesMisses m = ses_misses(ring.slots[turn], lane);
+        const uint32_t xw =
+            __ffs(__ballot_sync(kFull, m.before <= room && m.before + __popc(m.mask) > room)) - 1;
+        const uint32_t x_mask = __shfl_sync(kFull, m.mask, xw), x_before = __shfl_sync(kFull, m.before, xw);
         const uint32_t x_lane =
-            __ffs(__ballot_sync(kFull, ((x_m >> lane) & 1u) && x_before + __popc(x_m & lanemask_lt()) == room)) - 1;
-        const uint32_t x_at = 32 * x_u + x_lane, x = __shfl_sync(kFull, x_id, x_lane);
-#pragma unroll
-        for (uint32_t u = 0; u < kSesPer; ++u)
-          if (((miss[u] >> lane) & 1u) && 32 * u + lane <= x_at) owner[id[u]] = stamp;
-        total += room + 1;
-        cnt += room + 1;
-        __syncwarp();
-        if (ses_evict(a, S, owner, lane, r, s, x, C, front, total, cnt, es)) {
-          // session s is alone with block x: each later block misses, and
-          // every C-th of them empties the session again
-          const uint32_t rest = hi - 1 - x_at, resets = rest * per_inv >> 16;
-#pragma unroll
-          for (uint32_t u = 0; u < kSesPer; ++u) {
-            const uint32_t k = 32 * u + lane;
-            if (k > x_at && k < hi) owner[id[u]] = ((uint64_t)s << 32) | (es + ((k - x_at) * per_inv >> 16));
-          }
+            __ffs(__ballot_sync(kFull, ((x_mask >> lane) & 1u) && x_before + __popc(x_mask & lanemask_lt()) == room)) -
+            1;
+        const uint32_t x_at = 32 * xw + x_lane;
+        const uint32_t v_last = v;
+        v = ses_victim(a, S, lane, r, queue);
+        if (v == kNone) {
+          // session s alone is above C: it keeps the block just brought in, each
+          // later one misses, and every C-th of them empties the session again
+          if (miss && k < x_at) owner[id] = stamp;
+          es += 1;
+          const uint32_t rest = hi - 1 - x_at, resets = rest * per_inv >> 20;
+          if (k >= x_at && k < hi) owner[id] = ((uint64_t)s << 32) | (es + ((k - x_at) * per_inv >> 20));
           es += resets;
           total = 1 + rest - resets * per;
           cnt = (uint32_t)total;
-          m_all = 0;
-          __syncwarp();
-          if (lane == 0) S.ep[s] = es;
-          __syncwarp();
+          all = 0;
+          if (writer) S.ep[s] = es;
           break;
         }
-        ses_resident<kSesPer>(a, S, o, res);
-        m_all = 0;
-#pragma unroll
-        for (uint32_t u = 0; u < kSesPer; ++u) {
-          const uint32_t k = 32 * u + lane;
-          miss[u] = __ballot_sync(kFull, k > x_at && k < hi && !res[u]);
-          m_all += __popc(miss[u]);
+        // the least recently touched other session goes whole.  One barrier
+        // has to do: the others may still read v's state, so it changes after
+        // the barrier, and until the one after that they know v by name.
+        if (miss && k <= x_at) owner[id] = stamp;
+        cnt += room + 1;
+        total = C + 1 - S.count[v];
+        miss = valid && k > x_at && !ses_resident(a, S, o, v, v_last);
+        all = ses_count(miss, ring.slots[turn ^= 1], warp, lane);
+        if (writer) {
+          S.ep[v] += 1u;
+          S.count[v] = 0;
         }
       }
-      if (m_all) {
-#pragma unroll
-        for (uint32_t u = 0; u < kSesPer; ++u)
-          if ((miss[u] >> lane) & 1u) owner[id[u]] = stamp;
-        total += m_all;
-        cnt += m_all;
+      if (all) {
+        if (miss) owner[id] = stamp;
+        total += all;
+        cnt += all;
       }
-      __syncwarp();
+      replay_sync();  // before the next window reads what this one stored
     }
     __syncthreads();
   }
