@@ -411,7 +411,7 @@ ptc_status ptc_belady_curves(const uint32_t* prev, uint64_t n, const uint64_t* r
  *     recently touched session other than the current one is evicted;
  *   - a session that alone holds more than C blocks keeps only the block
  *     just brought in.
- * Not a stack algorithm: each capacity is replayed on its own (one warp per
+ * Not a stack algorithm: each capacity is replayed on its own (one CTA per
  * capacity), so the time grows with n, not with the number of runs.
  *   ids          u32[n] from ptc_assign_ids, each below n_distinct
  *   req_session  u32[n_req] labels below n_session

@@ -550,7 +550,7 @@ __global__ void k_session_prior(const uint32_t* __restrict__ ses_sorted, const u
 //                  every access without a hint; with one, the depths of each
 //                  request from its lam on (a warp per request)
 //   k_pd_count     level 1: per CTA of a persistent grid, the keys of its
-//                  range of accesses per bucket (h0 bits 53..60)
+//                  stretches of accesses per bucket (h0 bits 53..60)
 //   k_pd_rows1     one CTA per bucket: the prefix of its counts over the
 //                  level-1 CTAs, and the bucket's total
 //   k_pd_scatter1  the same pass again: a 16-byte record (96 key bits,
@@ -651,7 +651,6 @@ struct PdArgs {
   const uint64_t* n_dev;
   InsCarry kc;
   PriorHint ph;        // ph.lam null: no hint
-  uint32_t per;        // accesses per level-1 CTA, a multiple of kPdRound
   uint32_t* cnt1;      // [bucket * grid + cta]
   uint32_t* off1;      // its prefix along each bucket's row
   uint32_t* tot1;      // kPdBuckets totals
@@ -705,77 +704,137 @@ __global__ void __launch_bounds__(256) k_pd_flags(PriorHint ph, uint32_t n_ub, c
   }
 }
 
-// The carries of the hash tiles that a round of kPdRound accesses from
-// `base` spans (base a multiple of kPdRound, hence of every tile size; a
-// hash tile holds 8 to 256 blocks), read once per round into shared memory:
-// entry t is tile (base >> tile_shift) + t, up to hi.
-constexpr uint32_t kPdRoundTiles = kPdRound / 8;
-__device__ __forceinline__ void pd_round_carry(const InsCarry& kc, uint64_t base, uint64_t hi, uint32_t* s_lead,
-                                               ulonglong2* s_cy) {
+// Level 1 walks the words of ubits that are not zero, kPdWords to a round: a
+// hint leaves whole stretches of accesses matched, and rounds over positions,
+// part of them idle, took as long as full ones.  The words wait in a ring in
+// shared memory, refilled kPdThreads words of the bitmap at a time.  Both
+// passes are bound by the keys' bytes and their latency: 304M accesses, 144M of
+// them to settle, took 708 us to count and 2,057 to scatter by positions, 470
+// and 1,069 so (530 and 1,260 with one range of the bitmap to a CTA); 134M, 80M
+// to settle, 329 and 993 before, 255 and 604 so.
+constexpr uint32_t kPdWords = kPdRound / 32;
+constexpr uint32_t kPdRing = 1024;  // at least kPdThreads + kPdWords, a power of two
+static_assert(kPdRing >= kPdThreads + kPdWords, "a refill must fit beside what is left");
+struct PdRing {
+  uint32_t word[kPdRing], mask[kPdRing];
+  uint32_t warp_sum[kPdThreads / 32];
+};
+// A CTA's place in its part of the bitmap: every gridDim.x-th stretch of
+// kPdWords words, since whole ranges would differ in how much a hint leaves to
+// settle.  Every thread holds the same, but for its own word of the next
+// refill.
+struct PdWalk {
+  uint32_t next, stretches;  // the next refill's first stretch, their number
+  uint32_t head, size;       // of the ring
+  uint32_t w, ahead;
+};
+__device__ __forceinline__ void pd_walk_ahead(PdWalk& k, const uint32_t* ubits, uint32_t n) {
+  const uint64_t t = k.next + (uint64_t)(threadIdx.x / kPdWords) * gridDim.x;
+  k.w = (uint32_t)(t * kPdWords + threadIdx.x % kPdWords);
+  k.ahead = t < k.stretches && 32ULL * k.w < n ? __ldg(&ubits[k.w]) : 0u;
+  if (k.ahead && 32ULL * k.w + 32 > n) k.ahead &= (1u << (n & 31)) - 1u;
+}
+__device__ __forceinline__ void pd_walk_start(PdWalk& k, const uint32_t* ubits, uint32_t n) {
+  k.next = blockIdx.x;
+  k.stretches = (uint32_t)(((uint64_t)n + kPdRound - 1) / kPdRound);
+  k.head = k.size = 0;
+  pd_walk_ahead(k, ubits, n);
+}
+// Drops the `used` words of the last round and refills; returns the words of
+// the next round (0: the range is done).  Every thread calls it; it ends with
+// a barrier if it stored anything.
+__device__ __forceinline__ uint32_t pd_walk_next(PdWalk& k, PdRing& ring, const uint32_t* ubits, uint32_t n,
+                                                 uint32_t used) {
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  k.head += used;
+  k.size -= used;
+  while (k.size < kPdWords && k.next < k.stretches) {
+    const uint32_t w = k.w, v = k.ahead;
+    const uint64_t next = k.next + (uint64_t)(kPdThreads / kPdWords) * gridDim.x;
+    k.next = next < k.stretches ? (uint32_t)next : k.stretches;
+    pd_walk_ahead(k, ubits, n);
+    const uint32_t m = __ballot_sync(kFull, v != 0);
+    if (lane == 0) ring.warp_sum[warp] = __popc(m);
+    __syncthreads();
+    const uint32_t c = lane < kPdThreads / 32 ? ring.warp_sum[lane] : 0u;
+    const uint32_t before = __reduce_add_sync(kFull, lane < warp ? c : 0u), all = __reduce_add_sync(kFull, c);
+    if (v) {
+      const uint32_t at = (k.head + k.size + before + __popc(m & lanemask_lt())) & (kPdRing - 1);
+      ring.word[at] = w;
+      ring.mask[at] = v;
+    }
+    k.size += all;
+    __syncthreads();
+  }
+  return k.size < kPdWords ? k.size : kPdWords;
+}
+
+// The carries of the hash tiles that a round's words lie in (a hash tile holds
+// 8 to 256 blocks, so a word lies in 1 to 4), read once per round into shared
+// memory: word k's at k << tw, where a word lies in 1 << tw tiles.
+constexpr uint32_t kPdRoundTiles = 4 * kPdWords;
+struct PdCarry {
+  uint32_t lead[kPdRoundTiles];
+  ulonglong2 cy[kPdRoundTiles];
+};
+__device__ __forceinline__ uint32_t pd_tiles_log2(const InsCarry& kc) {
+  return kc.tile_shift < 5 ? 5 - kc.tile_shift : 0u;
+}
+__device__ __forceinline__ void pd_round_carry(const InsCarry& kc, const PdRing& ring, uint32_t head, uint32_t words,
+                                               uint64_t n, PdCarry& s) {
   if (!kc.carry) return;
-  const uint32_t nt = kPdRound >> kc.tile_shift;
-  const uint64_t t0 = base >> kc.tile_shift;
-  for (uint32_t t = threadIdx.x; t < nt; t += blockDim.x)
-    if (((t0 + t) << kc.tile_shift) < hi) {
-      s_lead[t] = __ldg(&kc.lead[t0 + t]);
-      s_cy[t] = __ldg(&kc.carry[t0 + t]);
-    }
-}
-
-// Key i of the round from `base`, with its tile's carry added (as
-// carried_key does) from the round's shared copy.
-__device__ __forceinline__ ulonglong2 pd_key(const ulonglong2* __restrict__ keys, uint32_t i, uint64_t base,
-                                             const InsCarry& kc, const uint32_t* s_lead, const ulonglong2* s_cy) {
-  ulonglong2 k = __ldcs(&keys[i]);
-  if (kc.carry) {
-    const uint32_t t = (uint32_t)(i - base) >> kc.tile_shift;
-    if ((i & ((1u << kc.tile_shift) - 1u)) < s_lead[t] && k.x < kP61 && k.y < kP61) {
-      const ulonglong2 c = s_cy[t];
-      k = make_ulonglong2(p61_add(k.x, c.x), p61_add(k.y, c.y));
+  const uint32_t tw = pd_tiles_log2(kc);
+  for (uint32_t t = threadIdx.x; t < words << tw; t += kPdThreads) {
+    const uint64_t i = 32ULL * ring.word[(head + (t >> tw)) & (kPdRing - 1)] +
+                       ((uint64_t)(t & ((1u << tw) - 1u)) << kc.tile_shift);
+    if (i < n) {
+      s.lead[t] = __ldg(&kc.lead[i >> kc.tile_shift]);
+      s.cy[t] = __ldg(&kc.carry[i >> kc.tile_shift]);
     }
   }
-  return k;
+}
+// The carry entry of access i in the round's word k, or kNone if none applies.
+__device__ __forceinline__ uint32_t pd_carry_of(const InsCarry& kc, const PdCarry& s, uint32_t k, uint32_t i) {
+  const uint32_t t = (k << pd_tiles_log2(kc)) + (kc.tile_shift < 5 ? (i & 31) >> kc.tile_shift : 0u);
+  return kc.carry && (i & ((1u << kc.tile_shift) - 1u)) < s.lead[t] ? t : kNone;
 }
 
-// h0 of key i with the carry of its hash tile added (the first word of
-// carried_key, for a key whose second word is a field element).
-__device__ __forceinline__ uint64_t carried_h0(const ulonglong2* __restrict__ keys, uint32_t i, const InsCarry& kc) {
-  uint64_t x = __ldcs(reinterpret_cast<const unsigned long long*>(&keys[i]));
-  if (kc.carry) {
-    const uint32_t t = i >> kc.tile_shift;
-    if ((i & ((1u << kc.tile_shift) - 1u)) < __ldg(&kc.lead[t]) && x < kP61)
-      x = p61_add(x, __ldg(reinterpret_cast<const unsigned long long*>(&kc.carry[t])));
-  }
-  return x;
-}
-
-// Level 1, counting: the keys of CTA g's accesses [g per, (g + 1) per) per
-// bucket.  Only h0 is read (the bucket is in it).  The scatter below skips a
+// Level 1, counting: the keys of a CTA's accesses to settle, per bucket.  Only h0 is read (the bucket is in it).  The scatter below skips a
 // key whose h1 is not a field element as well, and raises kErrInvalid, so
 // the counts can only differ from it on input the call rejects.
-__global__ void __launch_bounds__(kPdThreads, 4) k_pd_count(PdArgs a) {
+__global__ void __launch_bounds__(kPdThreads, 3) k_pd_count(PdArgs a) {
   grid_dep_sync();
   report_keys_used(a.n_ub, a.n_dev, a.st);
   __shared__ uint32_t h[kPdBuckets];
+  __shared__ PdRing ring;
+  __shared__ PdCarry s_cy;
   for (uint32_t x = threadIdx.x; x < kPdBuckets; x += kPdThreads) h[x] = 0;
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t n = keys_used(a.n_ub, a.n_dev);
-  const uint64_t lo = (uint64_t)blockIdx.x * a.per;
-  const uint64_t hi = lo + a.per < n ? lo + a.per : n;
+  PdWalk walk;
+  pd_walk_start(walk, a.ubits, n);
+  uint32_t used = 0;
   __syncthreads();
-  for (uint64_t base = lo; base < hi; base += kPdRound) {
-    bool u[kPdPer];
+  while (const uint32_t words = pd_walk_next(walk, ring, a.ubits, n, used)) {
     uint64_t x[kPdPer];
+    uint32_t at[kPdPer];
 #pragma unroll
     for (int j = 0; j < kPdPer; ++j) {
-      const uint64_t i = base + j * kPdThreads + threadIdx.x;
-      u[j] = i < hi && ((__ldg(&a.ubits[i >> 5]) >> (i & 31)) & 1u);
+      const uint32_t k = j * (kPdThreads / 32) + warp, q = (walk.head + k) & (kPdRing - 1);
+      const bool u = k < words && ((ring.mask[q] >> lane) & 1u);
+      at[j] = u ? 32 * ring.word[q] + lane : kNone;
+      x[j] = u ? __ldcs(reinterpret_cast<const unsigned long long*>(&a.keys[at[j]])) : ~0ULL;
     }
+    pd_round_carry(a.kc, ring, walk.head, words, n, s_cy);
+    __syncthreads();
 #pragma unroll
-    for (int j = 0; j < kPdPer; ++j)
-      x[j] = u[j] ? carried_h0(a.keys, (uint32_t)(base + j * kPdThreads + threadIdx.x), a.kc) : ~0ULL;
-#pragma unroll
-    for (int j = 0; j < kPdPer; ++j)
-      if (u[j] && x[j] < kP61) atomicAdd(&h[pd_bucket(x[j])], 1u);
+    for (int j = 0; j < kPdPer; ++j) {
+      if (at[j] == kNone || x[j] >= kP61) continue;
+      const uint32_t t = pd_carry_of(a.kc, s_cy, j * (kPdThreads / 32) + warp, at[j]);
+      atomicAdd(&h[pd_bucket(t == kNone ? x[j] : p61_add(x[j], s_cy.cy[t].x))], 1u);
+    }
+    __syncthreads();
+    used = words;
   }
   __syncthreads();
   for (uint32_t x = threadIdx.x; x < kPdBuckets; x += kPdThreads) a.cnt1[x * gridDim.x + blockIdx.x] = h[x];
@@ -790,38 +849,46 @@ __global__ void __launch_bounds__(kPdThreads, 2) k_pd_scatter1(PdArgs a) {
   __shared__ uint32_t h[kPdBuckets];     // the next place in each bucket
   __shared__ uint32_t c[kPdBuckets], so[kPdBuckets];  // the round's records per bucket, their offsets
   __shared__ uint32_t s_bst[kPdBuckets + 1];
-  __shared__ uint32_t s_lead[kPdRoundTiles];
-  __shared__ ulonglong2 s_cy[kPdRoundTiles];
+  __shared__ PdRing ring;
+  __shared__ PdCarry s_cy;
   pd_bucket_bounds(a.tot1, s_bst);
   for (uint32_t x = threadIdx.x; x < kPdBuckets; x += kPdThreads) {
     h[x] = s_bst[x] + a.off1[x * gridDim.x + blockIdx.x];
     c[x] = 0;
   }
+  const uint32_t lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const uint32_t n = keys_used(a.n_ub, a.n_dev);
-  const uint64_t lo = (uint64_t)blockIdx.x * a.per;
-  const uint64_t hi = lo + a.per < n ? lo + a.per : n;
-  pd_round_carry(a.kc, lo, hi, s_lead, s_cy);
+  PdWalk walk;
+  pd_walk_start(walk, a.ubits, n);
+  uint32_t used = 0;
   __syncthreads();
-  for (uint64_t base = lo; base < hi; base += kPdRound) {
-    bool u[kPdPer];
+  while (const uint32_t words = pd_walk_next(walk, ring, a.ubits, n, used)) {
     ulonglong2 k[kPdPer];
-    uint32_t rk[kPdPer];
+    uint32_t rk[kPdPer], mine = 0;  // bit j: the j-th access is one to settle
+    auto access = [&](int j) {
+      return 32 * ring.word[(walk.head + j * (kPdThreads / 32) + warp) & (kPdRing - 1)] + lane;
+    };
 #pragma unroll
     for (int j = 0; j < kPdPer; ++j) {
-      const uint64_t i = base + j * kPdThreads + threadIdx.x;
-      u[j] = i < hi && ((__ldg(&a.ubits[i >> 5]) >> (i & 31)) & 1u);
+      const uint32_t w = j * (kPdThreads / 32) + warp;
+      const bool u = w < words && ((ring.mask[(walk.head + w) & (kPdRing - 1)] >> lane) & 1u);
+      mine |= (uint32_t)u << j;
+      k[j] = u ? __ldcs(&a.keys[access(j)]) : make_ulonglong2(0, 0);
     }
+    pd_round_carry(a.kc, ring, walk.head, words, n, s_cy);
+    __syncthreads();
 #pragma unroll
     for (int j = 0; j < kPdPer; ++j) {
-      const uint32_t i = (uint32_t)(base + j * kPdThreads + threadIdx.x);
-      k[j] = u[j] ? pd_key(a.keys, i, base, a.kc, s_lead, s_cy) : make_ulonglong2(0, 0);
-      if (u[j] && (k[j].x >= kP61 || k[j].y >= kP61)) {  // not a field element: never settled
+      if (((mine >> j) & 1u) && (k[j].x >= kP61 || k[j].y >= kP61)) {  // not a field element: never settled
         raise_err(a.st, kErrInvalid);
-        u[j] = false;
+        mine &= ~(1u << j);
       }
+      if ((mine >> j) & 1u) {
+        const uint32_t t = pd_carry_of(a.kc, s_cy, j * (kPdThreads / 32) + warp, access(j));
+        if (t != kNone) k[j] = make_ulonglong2(p61_add(k[j].x, s_cy.cy[t].x), p61_add(k[j].y, s_cy.cy[t].y));
+      }
+      rk[j] = (mine >> j) & 1u ? atomicAdd(&c[pd_bucket(k[j].x)], 1u) : 0u;
     }
-#pragma unroll
-    for (int j = 0; j < kPdPer; ++j) rk[j] = u[j] ? atomicAdd(&c[pd_bucket(k[j].x)], 1u) : 0u;
     __syncthreads();
     uint32_t nrec;
     const uint32_t ex = scan256(threadIdx.x < kPdBuckets ? c[threadIdx.x] : 0u, &nrec);
@@ -829,15 +896,14 @@ __global__ void __launch_bounds__(kPdThreads, 2) k_pd_scatter1(PdArgs a) {
     __syncthreads();
 #pragma unroll
     for (int j = 0; j < kPdPer; ++j)
-      if (u[j])
-        stage[so[pd_bucket(k[j].x)] + rk[j]] = pd_record(k[j], (uint32_t)(base + j * kPdThreads + threadIdx.x));
+      if ((mine >> j) & 1u) stage[so[pd_bucket(k[j].x)] + rk[j]] = pd_record(k[j], access(j));
     __syncthreads();
     for (uint32_t x = threadIdx.x; x < nrec; x += kPdThreads) {
       const ulonglong2 r = stage[x];
       const uint32_t d = pd_bucket(r.x);
-      const uint32_t at = h[d] + (x - so[d]);
-      if (at < a.n_ub)
-        __stcg(&a.rec1[at], r);
+      const uint32_t to = h[d] + (x - so[d]);
+      if (to < a.n_ub)
+        __stcg(&a.rec1[to], r);
       else
         raise_err(a.st, kErrInvalid);
     }
@@ -846,8 +912,8 @@ __global__ void __launch_bounds__(kPdThreads, 2) k_pd_scatter1(PdArgs a) {
       h[x] += c[x];
       c[x] = 0;
     }
-    pd_round_carry(a.kc, base + kPdRound, hi, s_lead, s_cy);  // the next round's (its reads of these are done)
     __syncthreads();
+    used = words;
   }
 }
 
@@ -1455,9 +1521,7 @@ ptc_status ptc::ids_impl(const ptc_u128* keys, uint64_t n, const uint64_t* n_dev
   auto run_pd = [&]() -> bool {
     if (hint) hint_prep();
     const uint32_t sms = (uint32_t)num_sms();
-    uint32_t g1 = std::min(ceil_div_u32(n, kPdRound), std::min(4 * sms, kPdMaxG1));
-    const uint32_t per = ceil_div_u32(ceil_div_u32(n, g1), kPdRound) * kPdRound;
-    g1 = ceil_div_u32(n, per);
+    const uint32_t g1 = std::min(ceil_div_u32(n, kPdRound), std::min(4 * sms, kPdMaxG1));
     if (cudaFuncSetAttribute(k_pd_scatter1, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPdStageSmem) !=
             cudaSuccess ||
         cudaFuncSetAttribute(k_pd_level2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPdStageSmem) !=
@@ -1467,7 +1531,7 @@ ptc_status ptc::ids_impl(const ptc_u128* keys, uint64_t n, const uint64_t* n_dev
       return false;
     PTC_KERNEL("k_pd_flags", s, k_pd_flags, hint ? ceil_div_u32(hint->n_req, 8) : ceil_div_u32(L.nwords, 256), 256,
                0, ph, n32, n_dev, L.pd_ubits, L.bits, L.nwords);
-    const PdArgs pa{k, n32, n_dev, ic, ph, per, L.pd_cnt1, L.pd_off1, L.pd_tot1, L.pd_ubits, L.pd_rec1, L.st};
+    const PdArgs pa{k, n32, n_dev, ic, ph, L.pd_cnt1, L.pd_off1, L.pd_tot1, L.pd_ubits, L.pd_rec1, L.st};
     PTC_KERNEL("k_pd_count", s, k_pd_count, g1, kPdThreads, 0, pa);
     PTC_KERNEL("k_pd_rows1", s, k_pd_rows1, kPdBuckets, 256, 0, L.pd_cnt1, g1, L.pd_off1, L.pd_tot1);
     PTC_KERNEL("k_pd_scatter1", s, k_pd_scatter1, g1, kPdThreads, kPdStageSmem, pa);
