@@ -164,7 +164,10 @@ def kernel_model_bytes(name, T, N, L, D, U=None):
         "k_pd_scatter1": 32 * U + N / 8,   # settled keys in, bucket records out
         "k_pd_count2": 16 * U,             # records in
         "k_pd_scatter2": 32 * U,           # records in, partition records out
-        "k_pd_dedup": 16 * U,              # records in
+        # records in, by the variant that runs (by the average partition)
+        "k_pd_dedup": 16 * U if U < 2561 * 65536 else 0,
+        "k_pd_dedup_large": 16 * U if 2561 * 65536 <= U < 4097 * 65536 else 0,
+        "k_pd_dedup_big": 16 * U if U >= 4097 * 65536 else 0,
     }
     return {
         "k_hash_local": 4 * T + 16 * N,   # token stream in, block keys out
@@ -203,6 +206,7 @@ KERNEL_SOURCE = {
     "k_rank_count": "ptc_abi.cu", "k_rank_words": "ptc_abi.cu", "k_pd_flags": "ptc_ids.cu",
     "k_pd_count": "ptc_ids.cu", "k_pd_rows1": "ptc_ids.cu", "k_pd_scatter1": "ptc_ids.cu",
     "k_pd_count2": "ptc_ids.cu", "k_pd_rows2": "ptc_ids.cu", "k_pd_scatter2": "ptc_ids.cu", "k_pd_dedup": "ptc_ids.cu",
+    "k_pd_dedup_large": "ptc_ids.cu", "k_pd_dedup_big": "ptc_ids.cu",
 }
 
 
@@ -460,7 +464,7 @@ def hint_matched(ptc, torch, ids, blk_off, ses):
 
 
 PD_KERNELS = ("k_pd_flags", "k_pd_count", "k_pd_rows1", "k_pd_scatter1", "k_pd_count2", "k_pd_rows2",
-              "k_pd_scatter2", "k_pd_dedup")
+              "k_pd_scatter2", "k_pd_dedup", "k_pd_dedup_large", "k_pd_dedup_big")
 
 
 def id_stage(ptc, torch, L, kernels, n_access, matched, peak, dev):

@@ -561,11 +561,11 @@ __global__ void k_session_prior(const uint32_t* __restrict__ ses_sorted, const u
 //   k_pd_rows2     one CTA per bucket: the bounds of its partitions
 //   k_pd_scatter2  every tile's records moved to their partitions
 //   k_pd_dedup     one partition at a time per CTA: every record settles its
-//                  key in a shared-memory table (key + smallest index); an
-//                  index that is never stored, or that a smaller one
-//                  replaces, is a repeat and goes to a list, whose entries
-//                  then take their key's smallest index into slot_of and
-//                  clear their bit.
+//                  key in a shared-memory table that keeps the smallest index
+//                  of every key; a record with a larger one is a repeat,
+//                  takes the smallest into slot_of and clears its bit.  Two
+//                  table sizes, and k_pd_dedup_big for partitions of more
+//                  keys than they hold
 // bits then holds exactly the first occurrences, and k_ids_gather_pd reads a
 // repeat's first occurrence from slot_of itself (slot_of is written for the
 // repeats only; ubits tells the settled accesses from the matched ones).  A partition holding more
@@ -583,11 +583,22 @@ constexpr uint32_t kPdMaxG1 = 2048;                  // largest level-1 grid
 constexpr int kPd2Threads = 512;
 constexpr int kPd2Per = 8;
 constexpr uint32_t kPdTile2 = kPd2Threads * kPd2Per;  // 4096 records per level-2 tile
-constexpr int kPdDedupThreads = 512;
-constexpr int kPdDedupPer = 4;
+constexpr int kPdBigThreads = 512;
+constexpr int kPdBigPer = 4;
 constexpr uint32_t kPdSlots = 6144;  // shared table: 96 KB
 constexpr uint32_t kPdList = 1536;   // repeats listed per partition: 12 KB
-constexpr size_t kPdDedupSmem = sizeof(ulonglong2) * kPdSlots + sizeof(uint2) * kPdList;
+constexpr size_t kPdBigSmem = sizeof(ulonglong2) * kPdSlots + sizeof(uint2) * kPdList;
+// k_pd_dedup, with T threads per CTA: partitions of up to 6 T records at once.
+constexpr int kPdFitPer = 6;
+constexpr uint32_t pd_fit(int threads) { return threads * kPdFitPer; }
+constexpr size_t pd_dedup_smem(int threads) {
+  return (sizeof(ulonglong2) + 2 * sizeof(uint32_t)) * pd_fit(threads);
+}
+// It runs where partitions average at most this many (chance takes hardly any
+// of them past what fits).
+constexpr uint32_t pd_avg(int threads) { return pd_fit(threads) - 512; }
+constexpr int kPdFitS = 512;  // 3,072 records, three CTAs per SM: up to 167.8M accesses to settle
+constexpr int kPdFitL = 768;  // 4,608 records, two CTAs per SM: up to 268.4M
 
 constexpr size_t kPdStageSmem = sizeof(ulonglong2) * kPdRound;  // 64 KB
 static_assert(kPdTile2 == kPdRound, "both scatters stage one round of records");
@@ -1129,6 +1140,9 @@ __device__ __forceinline__ void pd_repeat(uint32_t* slot_of, uint32_t* bits, uin
 struct PdDedup {
   const ulonglong2* rec2;
   const uint32_t* base2;  // kPdParts + 1 partition bounds
+  uint32_t* big;          // the partitions left to k_pd_dedup_big
+  uint32_t* nbig;
+  uint32_t* cursor;       // partitions taken
   uint32_t cap;
   uint32_t* slot_of;
   uint32_t* bits;
@@ -1136,50 +1150,267 @@ struct PdDedup {
   DevStatus* st;
 };
 
-// A partition's table takes twice its records in slots (at most kPdSlots),
-// so small partitions clear little shared memory.  The loads of the next
-// chunk of records (or of the next partition's first chunk) are issued
-// before the current chunk is inserted, so they overlap its inserts.
-__global__ void __launch_bounds__(kPdDedupThreads, 2) k_pd_dedup(PdDedup a) {
-  grid_dep_sync();
-  extern __shared__ ulonglong2 tab[];  // kPdSlots, then the repeat list
-  uint2* list = reinterpret_cast<uint2*>(tab + kPdSlots);
-  __shared__ uint32_t s_nlist;
-  constexpr uint32_t kChunk = kPdDedupThreads * kPdDedupPer;
-  const ulonglong2 empty = make_ulonglong2(~0ULL, ~0ULL);
-  auto load = [&](ulonglong2(&dst)[kPdDedupPer], uint32_t c, uint32_t end) {
+// Partitions of at most pd_fit(T) records: the records are copied to shared memory
+// whole, and the table's slots are words that name one of them (16 bits of its
+// key, its place), four per record, or two at least.  One CAS of a word claims
+// a slot or tells the record in it, whose key is compared only where the 16
+// bits agree; a record that meets its own key keeps the smallest index there.
+// At the end every record knows its key's place from a register, so repeats
+// need no list.  What bounds it is the latency of a partition's steps (copy,
+// probes, barriers), hence three CTAs per SM; and then the repeats' random
+// writes.  Measured with 80M records, 1,220 to a partition: 1,379 us with
+// tables of keys (98 KB, 128-bit CAS, two CTAs per SM), 511 so.  144M, 8M of
+// them repeats of a few thousand keys: 2,062 and 1,056, of which the repeats'
+// writes take 320.
+// (Read once: the bitmap and slot_of, which repeats write, stay in L2 longer.)
+__device__ __forceinline__ void copy16_async(ulonglong2* dst, const ulonglong2* src) {
+  uint64_t once;
+  asm("createpolicy.fractional.L2::evict_first.b64 %0, 1.0;" : "=l"(once));
+  asm volatile("cp.async.cg.shared.global.L2::cache_hint [%0], [%1], 16, %2;" ::"r"(
+                   (uint32_t)__cvta_generic_to_shared(dst)),
+               "l"(src), "l"(once)
+               : "memory");
+}
+// Whether record `o` has the key (x, y), its index aside.
+__device__ __forceinline__ bool pd_same(const ulonglong2* rec, uint32_t o, uint64_t x, uint32_t y) {
+  return rec[o].x == x && reinterpret_cast<const uint32_t*>(&rec[o])[2] == y;
+}
+
+// Record o keeps the smaller index (read first: a key repeated thousands of
+// times would queue its atomics at one address).
+__device__ __forceinline__ void pd_lower(ulonglong2* rec, uint32_t o, uint32_t i) {
+  uint32_t* at = reinterpret_cast<uint32_t*>(&rec[o]) + 3;
+  if (*reinterpret_cast<volatile uint32_t*>(at) > i) atomicMin(at, i);
+}
+
+// A partition of more than that, most of them repeats (a prompt that
+// many sessions share): its records stream past the table, and only a key not
+// met yet takes a place.  A second pass over the records then
+// finds the repeats.  False if the places run out, with nothing written.
+constexpr int kPdFlowPer = 2;
+template <int T>
+__device__ __forceinline__ bool pd_flow(const PdDedup& a, ulonglong2* rec, uint32_t* slot, uint32_t b, uint32_t e,
+                                        uint32_t* places) {
+  constexpr uint32_t kFit = pd_fit(T), ts = 2 * kFit, kChunk = T * kPdFlowPer;
+  for (uint32_t x = threadIdx.x; x < ts; x += T) slot[x] = ~0u;
+  if (threadIdx.x == 0) *places = 0;
+  __syncthreads();
+  uint32_t spare = kNone;  // a place taken but not used yet
+  bool full = false;
+  auto load = [&](ulonglong2(&v)[kPdFlowPer], uint32_t c) {
 #pragma unroll
-    for (int q = 0; q < kPdDedupPer; ++q) {
-      const uint32_t x = c + q * kPdDedupThreads + threadIdx.x;
-      dst[q] = x < end && x < a.cap ? __ldcs(&a.rec2[x]) : empty;
+    for (int q = 0; q < kPdFlowPer; ++q) {
+      const uint32_t k = c + q * T + threadIdx.x;
+      v[q] = k < e && k >= c ? __ldcg(&a.rec2[k]) : make_ulonglong2(~0ULL, ~0ULL);
     }
   };
+  ulonglong2 v[kPdFlowPer], w[kPdFlowPer];
+  load(v, b);
+  for (uint32_t c = b; c < e; c += kChunk) {
+    load(w, c + kChunk < e ? c + kChunk : e);
+#pragma unroll
+    for (int q = 0; q < kPdFlowPer; ++q) {
+      const uint64_t x = v[q].x;
+      const uint32_t y = (uint32_t)v[q].y, i = (uint32_t)(v[q].y >> 32);
+      if (x == ~0ULL || full) continue;
+      uint32_t sl = pd_home(x, ts);
+      for (uint32_t probe = 0; probe < ts; ++probe) {  // the places run out before the slots do
+        uint32_t old = *reinterpret_cast<volatile uint32_t*>(&slot[sl]);
+        if (old == ~0u) {
+          if (spare == kNone) spare = atomicAdd(places, 1u);
+          if (spare >= kFit) {
+            full = true;
+            break;
+          }
+          rec[spare] = v[q];
+          __threadfence_block();
+          old = atomicCAS(&slot[sl], ~0u, y << 16 | spare);
+          if (old == ~0u) {
+            spare = kNone;
+            break;
+          }
+        }
+        const uint32_t o = old & 0xFFFFu;
+        __threadfence_block();
+        if ((old >> 16) == (y & 0xFFFFu) && pd_same(rec, o, x, y)) {
+          pd_lower(rec, o, i);
+          break;
+        }
+        sl = sl + 1 == ts ? 0 : sl + 1;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kPdFlowPer; ++q) v[q] = w[q];
+    if (__syncthreads_or(full)) return false;
+  }
+  load(v, b);
+  for (uint32_t c = b; c < e; c += kChunk) {
+    load(w, c + kChunk < e ? c + kChunk : e);
+#pragma unroll
+    for (int q = 0; q < kPdFlowPer; ++q) {
+      const uint64_t x = v[q].x;
+      const uint32_t y = (uint32_t)v[q].y, i = (uint32_t)(v[q].y >> 32);
+      if (x == ~0ULL) continue;
+      uint32_t sl = pd_home(x, ts);
+      for (uint32_t probe = 0; probe < ts; ++probe) {
+        const uint32_t old = slot[sl], o = old & 0xFFFFu;
+        if (old == ~0u) break;  // cannot happen: every key was inserted
+        if ((old >> 16) == (y & 0xFFFFu) && pd_same(rec, o, x, y)) {
+          const uint32_t first = reinterpret_cast<const uint32_t*>(&rec[o])[3];
+          if (first < i && i < a.n_ub) pd_repeat(a.slot_of, a.bits, i, first);
+          break;
+        }
+        sl = sl + 1 == ts ? 0 : sl + 1;
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < kPdFlowPer; ++q) v[q] = w[q];
+  }
+  __syncthreads();
+  return true;
+}
+
+template <int T, int CTAS>
+__global__ void __launch_bounds__(T, CTAS) k_pd_dedup(PdDedup a) {
+  grid_dep_sync();
+  constexpr uint32_t kFit = pd_fit(T);
+  extern __shared__ ulonglong2 rec[];  // kFit records, then the slots
+  uint32_t* const slot = reinterpret_cast<uint32_t*>(rec + kFit);
+  __shared__ uint32_t s_places;
+  const uint32_t avg = a.base2[kPdParts] / kPdParts;
+  if (avg > pd_avg(T) || (T == kPdFitL && avg <= pd_avg(kPdFitS))) return;  // another variant's
+  __shared__ uint32_t s_next;
   uint32_t p = blockIdx.x, b = 0, e = 0;
   if (p < kPdParts) {
     b = a.base2[p];
     e = a.base2[p + 1];
   }
-  ulonglong2 v[kPdDedupPer];
-  load(v, b, e);
   while (p < kPdParts) {
-    const uint32_t pn = p + gridDim.x;
+    const bool bad = b > e || e > a.cap;  // bounds past the records: malformed
+    const uint32_t m = bad ? 0u : e - b;
+    const uint32_t ts = 4 * m < 2 * kFit ? 4 * m : 2 * kFit;
+    if (m <= kFit) {
+#pragma unroll
+      for (int q = 0; q < kPdFitPer; ++q) {
+        const uint32_t k = q * T + threadIdx.x;
+        if (k < m) copy16_async(&rec[k], &a.rec2[b + k]);
+      }
+      for (uint32_t x = threadIdx.x; x < ts / 4; x += T)
+        reinterpret_cast<uint4*>(slot)[x] = make_uint4(~0u, ~0u, ~0u, ~0u);
+    }
+    // the partitions go to whichever CTA is free: those that flow take longer
+    if (threadIdx.x == 0) {
+      if (bad) raise_err(a.st, kErrInvalid);
+      s_next = gridDim.x + atomicAdd(a.cursor, 1u);
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+    const uint32_t pn = s_next;
     uint32_t bn = 0, en = 0;
     if (pn < kPdParts) {
       bn = a.base2[pn];
       en = a.base2[pn + 1];
     }
+    if (m > kFit) {
+      if (!pd_flow<T>(a, rec, slot, b, e, &s_places) && threadIdx.x == 0)
+        a.big[atomicAdd(a.nbig, 1u)] = p;  // each partition once: at most kPdParts
+    } else {
+      // the first probes of all of a thread's records are in flight together
+      uint32_t idx[kPdFitPer], own[kPdFitPer], met[kPdFitPer];
+#pragma unroll
+      for (int q = 0; q < kPdFitPer; ++q) {
+        const uint32_t k = q * T + threadIdx.x;
+        met[q] = ~0u;
+        idx[q] = 0;
+        if (k < m) {
+          const uint2 y = reinterpret_cast<const uint2*>(&rec[k])[1];
+          idx[q] = y.y;
+          // a slot's word is never ~0: k < kFit
+          met[q] = atomicCAS(&slot[pd_home(rec[k].x, ts)], ~0u, y.x << 16 | k);
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < kPdFitPer; ++q) {
+        const uint32_t k = q * T + threadIdx.x;
+        own[q] = k;
+        if (met[q] == ~0u) continue;
+        const uint64_t x = rec[k].x;
+        const uint32_t y = reinterpret_cast<const uint32_t*>(&rec[k])[2], word = y << 16 | k;
+        uint32_t sl = pd_home(x, ts), old = met[q];
+        do {  // half the slots stay empty: it ends
+          const uint32_t o = old & 0xFFFFu;
+          if (((old ^ word) >> 16) == 0 && pd_same(rec, o, x, y)) {
+            own[q] = o;
+            pd_lower(rec, o, idx[q]);
+            break;
+          }
+          sl = sl + 1 == ts ? 0 : sl + 1;
+          old = atomicCAS(&slot[sl], ~0u, word);
+        } while (old != ~0u);
+      }
+      __syncthreads();
+#pragma unroll
+      for (int q = 0; q < kPdFitPer; ++q) {
+        const uint32_t k = q * T + threadIdx.x;
+        if (k >= m) continue;
+        const uint32_t first = reinterpret_cast<const uint32_t*>(&rec[own[q]])[3];
+        if (first < idx[q] && idx[q] < a.n_ub) pd_repeat(a.slot_of, a.bits, idx[q], first);
+      }
+    }
+    __syncthreads();
+    p = pn;
+    b = bn;
+    e = en;
+  }
+}
+
+// The partitions that k_pd_dedup left (too many records, of too many keys), or
+// all where the average is above what its variants take (268M to settle; with
+// 300M, half of the partitions here and half there took 4% longer): their records stream through a table of at most kPdSlots keys.  The loads of the next
+// chunk of records (or of the next partition's first chunk) are issued
+// before the current chunk is inserted, so they overlap its inserts.
+__global__ void __launch_bounds__(kPdBigThreads, 2) k_pd_dedup_big(PdDedup a) {
+  grid_dep_sync();
+  extern __shared__ ulonglong2 tab[];  // kPdSlots, then the repeat list
+  uint2* list = reinterpret_cast<uint2*>(tab + kPdSlots);
+  __shared__ uint32_t s_nlist;
+  constexpr uint32_t kChunk = kPdBigThreads * kPdBigPer;
+  const ulonglong2 empty = make_ulonglong2(~0ULL, ~0ULL);
+  auto load = [&](ulonglong2(&dst)[kPdBigPer], uint32_t c, uint32_t end) {
+#pragma unroll
+    for (int q = 0; q < kPdBigPer; ++q) {
+      const uint32_t x = c + q * kPdBigThreads + threadIdx.x;
+      dst[q] = x < end && x < a.cap ? __ldcs(&a.rec2[x]) : empty;
+    }
+  };
+  const bool all = a.base2[kPdParts] / kPdParts > pd_avg(kPdFitL);
+  const uint32_t nbig = all ? kPdParts : *a.nbig;
+  if (blockIdx.x >= nbig) return;
+  auto bounds = [&](uint32_t p, uint32_t& lo, uint32_t& hi) {
+    const uint32_t d = p >= nbig ? kPdParts : all ? p : a.big[p];
+    lo = d < kPdParts ? a.base2[d] : 0u;
+    hi = d < kPdParts ? a.base2[d + 1] : 0u;
+  };
+  uint32_t p = blockIdx.x, b, e;
+  bounds(p, b, e);
+  ulonglong2 v[kPdBigPer];
+  load(v, b, e);
+  while (p < nbig) {
+    const uint32_t pn = p + gridDim.x;
+    uint32_t bn, en;
+    bounds(pn, bn, en);
     if (b >= e || e > a.cap) {  // nothing to settle (or bounds past the records: malformed)
       if (b < e && threadIdx.x == 0) raise_err(a.st, kErrInvalid);
       load(v, bn, en);
     } else {
       const uint32_t ts = e - b < kPdSlots / 2 ? ((2 * (e - b) + 31) & ~31u) : kPdSlots;
-      for (uint32_t x = threadIdx.x; x < ts; x += kPdDedupThreads) tab[x] = empty;
+      for (uint32_t x = threadIdx.x; x < ts; x += kPdBigThreads) tab[x] = empty;
       if (threadIdx.x == 0) s_nlist = 0;
       __syncthreads();
       bool full = false;
       for (uint32_t c = b;; c += kChunk) {
         const bool more = c + kChunk < e;
-        ulonglong2 w[kPdDedupPer];
+        ulonglong2 w[kPdBigPer];
         if (more)
           load(w, c + kChunk, e);
         else
@@ -1189,7 +1420,7 @@ __global__ void __launch_bounds__(kPdDedupThreads, 2) k_pd_dedup(PdDedup a) {
         // lane's queue rather than the whole warp at every record
         uint32_t nv = 0;
 #pragma unroll
-        for (int q = 0; q < kPdDedupPer; ++q) nv += v[q].x != ~0ULL;
+        for (int q = 0; q < kPdBigPer; ++q) nv += v[q].x != ~0ULL;
         uint32_t sl = pd_home(v[0].x, ts), probes = 0;
         while (__any_sync(kFull, nv > 0)) {
           uint32_t rep = kNone, rs = 0;
@@ -1202,7 +1433,7 @@ __global__ void __launch_bounds__(kPdDedupThreads, 2) k_pd_dedup(PdDedup a) {
             if (done) {
               --nv;
 #pragma unroll
-              for (int q = 0; q + 1 < kPdDedupPer; ++q) v[q] = v[q + 1];
+              for (int q = 0; q + 1 < kPdBigPer; ++q) v[q] = v[q + 1];
               sl = pd_home(v[0].x, ts);
               probes = 0;
             } else {
@@ -1212,28 +1443,28 @@ __global__ void __launch_bounds__(kPdDedupThreads, 2) k_pd_dedup(PdDedup a) {
           pd_list_push(rep, rs, list, &s_nlist);
         }
 #pragma unroll
-        for (int q = 0; q < kPdDedupPer; ++q) v[q] = w[q];
+        for (int q = 0; q < kPdBigPer; ++q) v[q] = w[q];
         if (!more) break;
       }
       if (full) raise_err(a.st, kErrTableFull);
       __syncthreads();
       const uint32_t nl = s_nlist;
       if (nl <= kPdList) {
-        for (uint32_t x = threadIdx.x; x < nl; x += kPdDedupThreads) {
+        for (uint32_t x = threadIdx.x; x < nl; x += kPdBigThreads) {
           const uint2 rp = list[x];
           const uint32_t m = reinterpret_cast<const uint32_t*>(&tab[rp.y])[3];
           if (m < rp.x && rp.x < a.n_ub) pd_repeat(a.slot_of, a.bits, rp.x, m);
         }
       } else {  // more repeats than the list holds: look every record up again
         for (uint32_t c = b; c < e; c += kChunk) {
-          ulonglong2 r[kPdDedupPer];
+          ulonglong2 r[kPdBigPer];
 #pragma unroll
-          for (int q = 0; q < kPdDedupPer; ++q) {
-            const uint32_t x = c + q * kPdDedupThreads + threadIdx.x;
+          for (int q = 0; q < kPdBigPer; ++q) {
+            const uint32_t x = c + q * kPdBigThreads + threadIdx.x;
             r[q] = x < e ? __ldcg(&a.rec2[x]) : empty;
           }
 #pragma unroll
-          for (int q = 0; q < kPdDedupPer; ++q) {
+          for (int q = 0; q < kPdBigPer; ++q) {
             if (r[q].x == ~0ULL) continue;
             const uint32_t i = (uint32_t)(r[q].y >> 32), m = pd_find(tab, ts, r[q]);
             if (m < i && i < a.n_ub) pd_repeat(a.slot_of, a.bits, i, m);
@@ -1526,7 +1757,11 @@ ptc_status ptc::ids_impl(const ptc_u128* keys, uint64_t n, const uint64_t* n_dev
             cudaSuccess ||
         cudaFuncSetAttribute(k_pd_level2<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPdStageSmem) !=
             cudaSuccess ||
-        cudaFuncSetAttribute(k_pd_dedup, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPdDedupSmem) !=
+        cudaFuncSetAttribute(k_pd_dedup<kPdFitS, 3>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)pd_dedup_smem(kPdFitS)) != cudaSuccess ||
+        cudaFuncSetAttribute(k_pd_dedup<kPdFitL, 2>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)pd_dedup_smem(kPdFitL)) != cudaSuccess ||
+        cudaFuncSetAttribute(k_pd_dedup_big, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kPdBigSmem) !=
             cudaSuccess)
       return false;
     PTC_KERNEL("k_pd_flags", s, k_pd_flags, hint ? ceil_div_u32(hint->n_req, 8) : ceil_div_u32(L.nwords, 256), 256,
@@ -1540,8 +1775,14 @@ ptc_status ptc::ids_impl(const ptc_u128* keys, uint64_t n, const uint64_t* n_dev
     PTC_KERNEL("k_pd_count2", s, k_pd_level2<false>, g2, kPd2Threads, 0, p2);
     PTC_KERNEL("k_pd_rows2", s, k_pd_rows2, kPdBuckets, 256, 0, L.pd_tot1, L.pd_tot2, L.pd_base2, L.st);
     PTC_KERNEL("k_pd_scatter2", s, k_pd_level2<true>, g2, kPd2Threads, kPdStageSmem, p2);
-    PTC_KERNEL("k_pd_dedup", s, k_pd_dedup, std::min(kPdParts, 2 * sms), kPdDedupThreads, kPdDedupSmem,
-               PdDedup{L.pd_rec2, L.pd_base2, n32, L.slot_of, L.bits, n32, L.st});
+    // the partition totals are in the bounds now: their array takes the list of large partitions
+    const PdDedup pq{L.pd_rec2, L.pd_base2, L.pd_tot2, &L.done[1], &L.done[2], n32, L.slot_of, L.bits, n32, L.st};
+    PTC_KERNEL("k_pd_dedup", s, (k_pd_dedup<kPdFitS, 3>), std::min(kPdParts, 3 * sms), kPdFitS,
+               pd_dedup_smem(kPdFitS), pq);
+    if (n / kPdParts > pd_avg(kPdFitS))  // the number to settle, up to n, is known on the device only
+      PTC_KERNEL("k_pd_dedup_large", s, (k_pd_dedup<kPdFitL, 2>), std::min(kPdParts, 2 * sms), kPdFitL,
+                 pd_dedup_smem(kPdFitL), pq);
+    PTC_KERNEL("k_pd_dedup_big", s, k_pd_dedup_big, std::min(kPdParts, 2 * sms), kPdBigThreads, kPdBigSmem, pq);
     return finish(nullptr, 0);
   };
   const uint32_t first_log2m = full_table ? L.log2m : small_table_log2(n);
