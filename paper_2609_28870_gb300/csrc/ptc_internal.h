@@ -256,16 +256,30 @@ ptc_status ids_impl(const ptc_u128* keys, uint64_t n_ub, const uint64_t* n_dev, 
                     cudaStream_t s, const KeyCarry* kc = nullptr, DevStatus* lent = nullptr, bool full_table = false,
                     const IdsHint* hint = nullptr, int method = PTC_IDS_AUTO);
 // Stage c with the runs it found in *view; with `lent` (its zeroed status
-// block, counters and key bitmap) it does not wait at its end.
+// block, counters, bitmaps and look-back words) it does not wait at its end.
+// With `pieces` (stage b's, in order and tiling the accesses; they live in the
+// same workspace, behind what stage c writes before it is done with them) the
+// runs come from those instead of from prev.
 struct StackLent {
   DevStatus* st = nullptr;
-  uint32_t* done = nullptr;   // kStackDone counters
-  uint32_t* kbits = nullptr;  // stack_key_words(n) words
+  uint32_t* done = nullptr;  // kStackDone counters
+  uint32_t* bits = nullptr;  // run starts, then keys: stack_key_words(n) words each
+  uint64_t* lb = nullptr;    // stack_lb_words(n)
+};
+// Stretches of accesses that re-read a stretch one access to one, or that are
+// all first accesses: piece o is [ipos[o], ipos[o] + ilen[o]), the first of
+// which was last accessed at ip0[o] (none: kNone).
+struct ReusePieces {
+  uint64_t K = 0;  // 0: not known
+  const uint32_t *ipos = nullptr, *ilen = nullptr, *ip0 = nullptr;
 };
 constexpr uint32_t kStackDone = 64;
+constexpr uint32_t kPieceTile = 2048;
 inline size_t stack_key_words(uint64_t n) { return n / 32 + 2; }
+inline size_t stack_lb_words(uint64_t n) { return n / kPieceTile + 2; }
 ptc_status stack_distance_view(const uint32_t* prev, uint64_t n, uint32_t* dist_out, int method, void* ws,
-                               size_t ws_bytes, cudaStream_t s, RunsView* view, const StackLent* lent);
+                               size_t ws_bytes, cudaStream_t s, RunsView* view, const StackLent* lent,
+                               const ReusePieces& pieces);
 // Stage b as ptc_reuse_indices does it (ptc_reuse.cu); with `lent` (its zeroed
 // status block, counters and cut bitmap) it does not wait at its end.  With
 // `din`, stage a2 has not waited: n and n_distinct are upper bounds, the kernels
@@ -288,6 +302,7 @@ struct ReuseDevIn {
 struct ReuseHostOut {
   uint64_t n = 0, D = 0;
   uint32_t ids_err = 0;
+  ReusePieces pieces;  // in the call's workspace
 };
 ptc_status reuse_view(const uint32_t* ids, uint64_t n, uint64_t n_distinct, uint32_t* prev_out, uint32_t* next_out,
                       void* ws, size_t ws_bytes, cudaStream_t s, const ReuseLent* lent,

@@ -64,7 +64,8 @@ PipeLayout pipe_layout(void* ws, uint32_t n_req, uint64_t n_tok, uint32_t B, uin
   L.reuse.cut = cv.take<uint32_t>(ptc::reuse_cut_words(n));
   L.stack.st = L.st ? L.st + ptc::kStStack : nullptr;
   L.stack.done = cv.take<uint32_t>(ptc::kStackDone);
-  L.stack.kbits = cv.take<uint32_t>(ptc::stack_key_words(n));
+  L.stack.bits = cv.take<uint32_t>(2 * ptc::stack_key_words(n));
+  L.stack.lb = cv.take<uint64_t>(ptc::stack_lb_words(n));
   L.curves_bytes = ptc_curves_workspace_bytes(n_tok / B, n_req, n_cap);
   L.curves = cv.take<unsigned char>(L.curves_bytes);
   L.zero_bytes = cv.off - L.curves_bytes + ptc::curves_zero_bytes(n_tok / B) - zero_off;
@@ -162,7 +163,8 @@ extern "C" ptc_status ptc_pipeline(const uint32_t* tokens, uint64_t n_tok, const
   }
   ptc::RunsView runs;
   if (n > 0) {
-    rc = ptc::stack_distance_view(prev, n, dist, PTC_SD_AUTO, L.scratch, L.scratch_bytes, s, &runs, &L.stack);
+    rc = ptc::stack_distance_view(prev, n, dist, PTC_SD_AUTO, L.scratch, L.scratch_bytes, s, &runs, &L.stack,
+                                  hout.pieces);
     if (rc != PTC_OK) return rc;
   }
   static_assert(ptc::kStStack == ptc::kStReuse + 1, "stage d reads both");

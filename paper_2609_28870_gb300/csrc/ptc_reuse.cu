@@ -625,6 +625,7 @@ ptc_status reuse_by_runs(const uint32_t* ids, uint64_t n, uint64_t D, uint32_t* 
   const uint32_t fill_blocks = ceil_div_u32(K, 256) < (uint32_t)(8 * num_sms()) ? ceil_div_u32(K, 256)
                                                                                 : (uint32_t)(8 * num_sms());
   PTC_KERNEL("k_ir_fill", s, k_ir_fill, fill_blocks, 256, 0, f);
+  if (hout) hout->pieces = ReusePieces{K, L.ipos, L.ilen, L.ip0};
   if (lent) return cudaGetLastError() == cudaSuccess ? PTC_OK : PTC_ERR_CUDA;
   return end_call(L.st, s, &h);
 }

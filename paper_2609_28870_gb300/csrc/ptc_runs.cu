@@ -317,6 +317,82 @@ __global__ void __launch_bounds__(kMT) k_runs_mark4(MarkArgs a) {
   if (tile == a.ntiles - 1 && threadIdx.x == 0) a.rec_s[a.tpre[a.ntiles]] = a.n;
 }
 
+// ---- the runs from stage b's pieces (the pipeline): a piece starts a run
+// unless it goes on where the piece before it ended, so both passes over prev,
+// 4 bytes an access each, become one over the pieces, 12 bytes each, a few per
+// run.  One launch (look-back).  What bounds it is latency.  On 304M accesses the
+// two passes took 738 us, on 9.3M 37; so 36 and 13 (and 30 and 8 more in the
+// ranks, now of both bitmaps).
+struct PieceArgs {
+  ReusePieces p;
+  uint32_t n;
+  uint32_t *bits, *kbits, *rec_s, *rec_a;  // as MarkArgs; bits and kbits zeroed
+  uint64_t* lb;
+  DevStatus* st;
+};
+constexpr int kPT = 256;
+constexpr int kPR = kPieceTile / kPT;
+constexpr uint32_t kEpochPieces = 1;
+
+__global__ void __launch_bounds__(kPT) k_runs_pieces(PieceArgs a) {
+  grid_dep_sync();
+  __shared__ uint32_t s_wcnt[kPT / 32];
+  const uint32_t tile = next_tile(a.st, kEpochPieces), K = (uint32_t)a.p.K;
+  const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const uint32_t base = tile * kPieceTile + w * (32 * kPR);
+  // v = prev + 1 (none -> 0) of a piece's first access, and past its last one;
+  // `left` the latter of the piece before
+  uint32_t first[kPR], past[kPR], left[kPR], words[kPR], cnt = 0;
+  auto read = [&](uint32_t o, uint32_t& f, uint32_t& e) {
+    const uint32_t P = o < K ? a.p.ip0[o] : kNone;
+    f = P + 1u;
+    e = P == kNone ? 0u : P + a.p.ilen[o];
+  };
+#pragma unroll
+  for (int k = 0; k < kPR; ++k) read(base + 32 * k + lane, first[k], past[k]);
+  uint32_t carry = 0, unused;
+  if (base > 0) read(base - 1, unused, carry);
+#pragma unroll
+  for (int k = 0; k < kPR; ++k) {
+    const uint32_t o = base + 32 * k + lane;
+    const uint32_t up = __shfl_up_sync(kFull, past[k], 1);
+    left[k] = lane ? up : carry;
+    carry = __shfl_sync(kFull, past[k], 31);
+    const bool cont = o > 0 && ((first[k] == left[k] + 1 && left[k] != 0) || (first[k] == 0 && left[k] == 0));
+    words[k] = __ballot_sync(kFull, o < K && !cont);
+    cnt += __popc(words[k]);
+  }
+  if (lane == 0) s_wcnt[w] = cnt;
+  __syncthreads();
+  uint32_t before = 0, total = 0;
+#pragma unroll
+  for (uint32_t ww = 0; ww < kPT / 32; ++ww) {
+    if (ww < w) before += s_wcnt[ww];
+    total += s_wcnt[ww];
+  }
+  uint32_t run = (uint32_t)lookback_sum_cta(a.lb, tile, total, kEpochPieces, a.st) + before;
+  if (tile == 0 && threadIdx.x == 0) atomicOr(&a.kbits[0], 1u);  // key 0 is always entered
+#pragma unroll
+  for (int k = 0; k < kPR; ++k) {
+    const uint32_t o = base + 32 * k + lane;
+    if ((words[k] >> lane) & 1u) {
+      const uint32_t r = run + __popc(words[k] & lanemask_lt()), j = a.p.ipos[o];
+      if (in_bounds(a.st, r, K) && in_bounds(a.st, j, a.n)) {
+        a.rec_s[r] = j;
+        a.rec_a[r] = first[k];
+        atomicOr(&a.bits[j >> 5], 1u << (j & 31));
+      }
+      if (o > 0 && left[k] != 0) atomicOr(&a.kbits[left[k] >> 5], 1u << (left[k] & 31));
+    }
+    run += __popc(words[k]);
+    if (o + 1 == K) {
+      if (past[k] != 0) atomicOr(&a.kbits[past[k] >> 5], 1u << (past[k] & 31));
+      a.rec_s[run] = a.n;
+      a.st->value[1] = run;
+    }
+  }
+}
+
 // Keys in the bitmap below v: the rank of v when v is a key.
 __device__ __forceinline__ uint32_t key_rank(const uint32_t* __restrict__ kbits, const uint32_t* __restrict__ kpre,
                                              uint32_t v) {
@@ -390,6 +466,7 @@ struct LevelArgs {
 // per-tile zero counts of level 0.
 __global__ void __launch_bounds__(kRT) k_runs_init(const uint32_t* __restrict__ rec_s, const uint32_t* __restrict__ rec_a,
                                                   const uint32_t* __restrict__ kbits, const uint32_t* __restrict__ kpre,
+                                                  uint32_t kbase,
                                                   uint32_t* __restrict__ key, uint32_t* __restrict__ wt,
                                                   uint2* __restrict__ acc, uint2* __restrict__ pre, uint32_t* done,
                                                   uint32_t R, uint32_t ntiles, uint32_t shift) {
@@ -403,7 +480,7 @@ __global__ void __launch_bounds__(kRT) k_runs_init(const uint32_t* __restrict__ 
     if (r < R) {
       const uint32_t s = rec_s[r], e = rec_s[r + 1], a0 = rec_a[r];
       const uint32_t len = e - s;
-      const uint32_t kv = key_rank(kbits, kpre, a0 ? a0 + len - 1 : 0u);
+      const uint32_t kv = key_rank(kbits, kpre, a0 ? a0 + len - 1 : 0u) - kbase;
       key[r] = kv;
       wt[r] = len;
       if (!((kv >> shift) & 1u)) {
@@ -533,6 +610,7 @@ __global__ void __launch_bounds__(kRT) k_runs_level(LevelArgs a) {
 // here, 0.7M runs of the mixed trace 450 us and 143.
 constexpr uint32_t kDomB = 512;
 constexpr uint64_t kDomMax = 1ULL << 21;  // runs; the lengths' matrix then takes 67 MB
+constexpr uint64_t kPiecesBound = 1ULL << 19;  // the lengths' matrix takes 4 MB: it costs less than the wait
 
 struct DomArgs {
   const uint32_t* rec_s;
@@ -547,7 +625,13 @@ struct DomArgs {
   uint32_t* rank;      // per run: rank (kNone: first accesses)
   uint32_t* sd;
   uint32_t R, nb, kwords;
+  const uint64_t* Rd;  // device: the number of runs where R is a bound only, or null
+  bool keys_after;     // kpre counts the run starts too (their bitmap lies before the keys')
 };
+__device__ __forceinline__ uint32_t dom_runs(const DomArgs& a) {
+  const uint64_t r = a.Rd ? *a.Rd : a.R;
+  return r < a.R ? (uint32_t)r : a.R;
+}
 
 // Sum of w over the pairs (key, w) of s[0 .. n) with key < mine: n even, two
 // pairs per load, the same for the whole warp.
@@ -594,13 +678,14 @@ __global__ void __launch_bounds__(kDomB) k_dom_time(DomArgs a) {
   __shared__ __align__(16) uint2 s_run[kDomB];
   __shared__ uint32_t s_w[kDomB / 32];
   const uint32_t t = threadIdx.x, r = blockIdx.x * kDomB + t;
+  const uint32_t R = dom_runs(a);
   for (uint32_t b = t; b < a.nb; b += kDomB) s_row[b] = 0;
   uint32_t rank = kNone, len = 0;
-  if (r < a.R) {
+  if (r < R) {
     const uint32_t v = a.rec_a[r];
     if (v) {
       len = a.rec_s[r + 1] - a.rec_s[r];
-      rank = key_rank(a.kbits, a.kpre, v + len - 1) - 1;  // key 0 is entered too
+      rank = key_rank(a.kbits, a.kpre, v + len - 1) - (a.keys_after ? R : 0u) - 1;  // key 0 is entered too
     }
     a.rank[r] = rank;
   }
@@ -611,7 +696,7 @@ __global__ void __launch_bounds__(kDomB) k_dom_time(DomArgs a) {
     atomicAdd(&s_row[rank / kDomB], len);
     a.by_rank[rank] = make_uint2(r, len);
   }
-  if (r < a.R) a.before[r] = before;
+  if (r < R) a.before[r] = before;
   // earlier runs of the block: whole warps, then the warp's own earlier lanes
   const uint32_t w0 = t & ~31u;
   uint32_t sum = sum_below(s_run, w0, rank == kNone ? 0u : rank);
@@ -636,8 +721,10 @@ __global__ void __launch_bounds__(kDomB) k_dom_rank(DomArgs a) {
   __shared__ uint32_t s_w[kDomB / 32];
   const uint32_t t = threadIdx.x, b = blockIdx.x, q = b * kDomB + t;
   uint2 x = make_uint2(kNone, 0u);
-  const uint32_t ranks = a.kpre[a.kwords - 1] + __popc(a.kbits[a.kwords - 1]) - 1;  // keys but 0
-  if (b < a.nb && q < ranks && q < a.R) x = a.by_rank[q];
+  const uint32_t R = dom_runs(a);
+  // keys but 0
+  const uint32_t ranks = a.kpre[a.kwords - 1] + __popc(a.kbits[a.kwords - 1]) - (a.keys_after ? R : 0u) - 1;
+  if (b < a.nb && q < ranks && q < R) x = a.by_rank[q];
   // (time block, length) in rank order: an entry counts the earlier ones of
   // smaller time blocks
   const uint32_t tb = x.x == kNone ? kNone : x.x / kDomB;
@@ -659,7 +746,7 @@ __global__ void __launch_bounds__(kDomB) k_dom_rank(DomArgs a) {
     const uint2 y = s_run[w0 + k];
     if (k < (t & 31) && y.x < tb) sum += y.y;
   }
-  if (x.x != kNone && x.x < a.R) a.in_rank[x.x] = sum;
+  if (x.x != kNone && x.x < R) a.in_rank[x.x] = sum;
 }
 
 // One CTA per time block: the row's prefix over rank blocks, and the distances.
@@ -677,7 +764,7 @@ __global__ void __launch_bounds__(kDomB) k_dom_out(DomArgs a) {
     run += all;
   }
   __syncthreads();
-  if (r >= a.R) return;
+  if (r >= dom_runs(a)) return;
   const uint32_t rank = a.rank[r];
   a.sd[r] = rank == kNone ? kNone
                           : a.rec_s[r] - (row[a.nb] + a.before[r]) + s_row[rank / kDomB] + a.in_rank[r] +
@@ -694,6 +781,7 @@ struct QueryArgs {
   const uint2* zw;      // level l at zw + l * (R + 1)
   uint32_t* sd;         // distance of each run
   uint32_t R, L;
+  uint32_t kbase;       // kpre counts this many bits more
 };
 
 // Index of the run holding position j.
@@ -725,7 +813,7 @@ __global__ void __launch_bounds__(256) k_runs_query(QueryArgs a) {
   uint32_t hi = r, cnt = 0;
   const uint32_t stride = a.R + 1;
   // keys below x are the keys whose rank is below the number of keys below x
-  const uint32_t xr = key_rank(a.kbits, a.kpre, x);
+  const uint32_t xr = key_rank(a.kbits, a.kpre, x) - a.kbase;
   for (uint32_t l = 0; l < a.L && lo < hi; ++l) {
     const uint2* zl = a.zw + (size_t)l * stride;
     const uint2 zlo = zl[lo], zhi = zl[hi];
@@ -799,18 +887,18 @@ RunsLayout runs_layout(void* ws, uint64_t n, uint64_t R, const StackLent* lent =
   W.mtiles = ceil_div_u32(nn, kMTile);
   W.rtiles = ceil_div_u32(rr, kRTile);
   W.kwords = (uint32_t)stack_key_words(nn);  // keys and thresholds lie in [0, n]
-  W.ktiles = rank_tiles(W.kwords);
+  W.ktiles = rank_tiles(2 * W.kwords);
   W.st = cv.take<DevStatus>(1);
   W.done = cv.take<uint32_t>(kStackDone);
   W.kbits = cv.take<uint32_t>(W.kwords);
   W.zero_bytes = cv.off;
   W.tcnt = cv.take<uint32_t>(W.mtiles + 1);
   W.tpre = cv.take<uint32_t>(W.mtiles + 1);
-  W.kpre = cv.take<uint32_t>(W.kwords);
   W.ktcnt = cv.take<uint32_t>(W.ktiles + 1);
   W.ktpre = cv.take<uint32_t>(W.ktiles + 1);
-  W.bits = cv.take<uint32_t>(nn / 32 + 2);
-  W.wpre = cv.take<uint32_t>(nn / 32 + 2);
+  W.bits = cv.take<uint32_t>(W.kwords);
+  W.wpre = cv.take<uint32_t>(2 * (size_t)W.kwords);
+  W.kpre = W.wpre + W.kwords;  // next to each other, as the bitmaps are when lent
   W.rec_s = cv.take<uint32_t>(nn + 1);
   W.rec_a = cv.take<uint32_t>(nn);
   W.sd = cv.take<uint32_t>(rr);
@@ -840,7 +928,8 @@ RunsLayout runs_layout(void* ws, uint64_t n, uint64_t R, const StackLent* lent =
   if (lent) {
     W.st = lent->st;
     W.done = lent->done;
-    W.kbits = lent->kbits;
+    W.bits = lent->bits;
+    W.kbits = lent->bits + W.kwords;
   }
   return W;
 }
@@ -853,36 +942,52 @@ uint64_t runs_reserve(uint64_t n) {
 }
 
 ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_out, void* ws, size_t ws_bytes,
-                               cudaStream_t s, int method, RunsView* view, const StackLent* lent = nullptr) {
+                               cudaStream_t s, int method, RunsView* view, const StackLent* lent = nullptr,
+                               const ReusePieces& pieces = ReusePieces{}) {
   const RunsLayout M = runs_layout(ws, n, 1, lent);
   if (!ws_ok(ws, ws_bytes, M.total)) return PTC_ERR_WORKSPACE;
   if (!lent && begin_call(ws, M.zero_bytes, s) != PTC_OK) return PTC_ERR_CUDA;
-  MarkArgs m;
-  m.prev = prev;
-  m.n = (uint32_t)n;
-  m.ntiles = M.mtiles;
-  m.bits = M.bits;
-  m.wpre = M.wpre;
-  m.rec_s = M.rec_s;
-  m.rec_a = M.rec_a;
-  m.tcnt = M.tcnt;
-  m.tpre = M.tpre;
-  m.done = &M.done[63];
-  m.kbits = M.kbits;
-  m.max_runs = method == PTC_SD_AUTO ? (uint32_t)(n / 3) : (uint32_t)n;
-  m.st = M.st;
-  if ((reinterpret_cast<uintptr_t>(prev) & 15) == 0) {
-    PTC_KERNEL("k_runs_count", s, k_runs_count4, M.mtiles, kMT, 0, m);
-    PTC_KERNEL("k_runs_mark", s, k_runs_mark4, M.mtiles, kMT, 0, m);
+  const uint64_t K = pieces.K;
+  const bool by_pieces = lent && K > 0 && reinterpret_cast<const char*>(M.sd) <= reinterpret_cast<const char*>(pieces.ipos);
+  if (by_pieces) {
+    const PieceArgs pa{pieces, (uint32_t)n, M.bits, M.kbits, M.rec_s, M.rec_a, lent->lb, M.st};
+    PTC_KERNEL("k_runs_pieces", s, k_runs_pieces, ceil_div_u32(K, kPieceTile), kPT, 0, pa);
+    if (bitmap_ranks(M.bits, 2 * M.kwords, M.wpre, M.ktcnt, M.ktpre, &M.done[62], nullptr, s) != PTC_OK)
+      return PTC_ERR_CUDA;
   } else {
-    PTC_KERNEL("k_runs_count", s, k_runs_count, M.mtiles, kMT, 0, m);
-    PTC_KERNEL("k_runs_mark", s, k_runs_mark, M.mtiles, kMT, 0, m);
+    MarkArgs m;
+    m.prev = prev;
+    m.n = (uint32_t)n;
+    m.ntiles = M.mtiles;
+    m.bits = M.bits;
+    m.wpre = M.wpre;
+    m.rec_s = M.rec_s;
+    m.rec_a = M.rec_a;
+    m.tcnt = M.tcnt;
+    m.tpre = M.tpre;
+    m.done = &M.done[63];
+    m.kbits = M.kbits;
+    m.max_runs = method == PTC_SD_AUTO ? (uint32_t)(n / 3) : (uint32_t)n;
+    m.st = M.st;
+    if ((reinterpret_cast<uintptr_t>(prev) & 15) == 0) {
+      PTC_KERNEL("k_runs_count", s, k_runs_count4, M.mtiles, kMT, 0, m);
+      PTC_KERNEL("k_runs_mark", s, k_runs_mark4, M.mtiles, kMT, 0, m);
+    } else {
+      PTC_KERNEL("k_runs_count", s, k_runs_count, M.mtiles, kMT, 0, m);
+      PTC_KERNEL("k_runs_mark", s, k_runs_mark, M.mtiles, kMT, 0, m);
+    }
+    if (bitmap_ranks(M.kbits, M.kwords, M.kpre, M.ktcnt, M.ktpre, &M.done[62], nullptr, s) != PTC_OK)
+      return PTC_ERR_CUDA;
   }
-  if (bitmap_ranks(M.kbits, M.kwords, M.kpre, M.ktcnt, M.ktpre, &M.done[62], nullptr, s) != PTC_OK) return PTC_ERR_CUDA;
+  // Few pieces: they bound the runs well enough to go on without waiting for
+  // the number of runs (a wait leaves the GPU idle for about 10 us; the blocks'
+  // matrix grows with the square of the bound).
+  const bool bound = by_pieces && K <= kPiecesBound && K <= n / 3 && runs_layout(ws, n, K, lent).total <= ws_bytes;
   DevStatus h;
-  ptc_status rc = end_call(M.st, s, &h);
+  ptc_status rc = PTC_OK;
+  if (!bound) rc = end_call(M.st, s, &h);
   if (rc != PTC_OK) return rc;
-  const uint64_t R = h.value[1];
+  const uint64_t R = bound ? K : h.value[1];
   const RunsLayout W = runs_layout(ws, n, R, lent);
   const bool fits = R >= 1 && R <= n && ws_bytes >= W.total;
   if (method == PTC_SD_AUTO && (!fits || R > n / 3)) {
@@ -906,6 +1011,8 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
     d.sd = W.sd;
     d.R = R32;
     d.kwords = W.kwords;
+    d.Rd = bound ? &W.st->value[1] : nullptr;
+    d.keys_after = by_pieces;
     const size_t row = sizeof(uint32_t) * d.nb;
     PTC_KERNEL("k_dom_time", s, k_dom_time, d.nb, kDomB, row, d);
     PTC_KERNEL("k_dom_rank", s, k_dom_rank, d.nb + 1, kDomB, 0, d);
@@ -915,7 +1022,8 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
     const size_t tstride = (size_t)T + 1;
     const FillRange zf[2] = {{W.acc, W.acc_bytes, 0u}, {W.done, kStackDone * sizeof(uint32_t), 0u}};
     if (fill_many_async(zf, 2, s) != PTC_OK) return PTC_ERR_CUDA;
-    PTC_KERNEL("k_runs_init", s, k_runs_init, T, kRT, 0, W.rec_s, W.rec_a, W.kbits, W.kpre, W.k0, W.w0, W.acc, W.pre,
+    PTC_KERNEL("k_runs_init", s, k_runs_init, T, kRT, 0, W.rec_s, W.rec_a, W.kbits, W.kpre,
+               by_pieces ? R32 : 0u, W.k0, W.w0, W.acc, W.pre,
                &W.done[0], R32, T, L - 1);
     uint32_t* keys[2] = {W.k0, W.k1};
     uint32_t* wts[2] = {W.w0, W.w1};
@@ -947,6 +1055,7 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
     q.sd = W.sd;
     q.R = R32;
     q.L = L;
+    q.kbase = by_pieces ? R32 : 0u;
     PTC_KERNEL("k_runs_query", s, k_runs_query, ceil_div_u32(R, 256), 256, 0, q);
   }
   PTC_KERNEL("k_runs_expand", s, k_runs_expand, ceil_div_u32(n, kExpThreads * kExpPer), kExpThreads, 0, W.bits, W.wpre, W.sd, (uint32_t)n, dist_out, R32, W.st);
@@ -966,13 +1075,14 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
 }  // namespace
 
 ptc_status stack_distance_view(const uint32_t* prev, uint64_t n, uint32_t* dist_out, int method, void* ws,
-                               size_t ws_bytes, cudaStream_t s, RunsView* view, const StackLent* lent) {
+                               size_t ws_bytes, cudaStream_t s, RunsView* view, const StackLent* lent,
+                               const ReusePieces& pieces) {
   *view = RunsView{};
   if (n >= (uint64_t)kNone) return PTC_ERR_OVERFLOW;
   if (n == 0) return PTC_OK;
   if (!prev || !dist_out) return PTC_ERR_INVALID_ARG;
   if (method == PTC_SD_POINTS) return stack_distance_points(prev, n, dist_out, ws, ws_bytes, s);
-  return stack_distance_runs(prev, n, dist_out, ws, ws_bytes, s, method, view, lent);
+  return stack_distance_runs(prev, n, dist_out, ws, ws_bytes, s, method, view, lent, pieces);
 }
 
 }  // namespace ptc
