@@ -409,6 +409,21 @@ __global__ void __launch_bounds__(kInsThreads) k_ids_insert_prior(const ulonglon
   }
 }
 
+// ids[to + d] = ids[from + d] for the depths d in [lo, hi), by one warp (the two
+// stretches belong to different requests).  Eight loads in flight per lane: one
+// at a time, 160M ids took 525 us, so 350 (53M of long requests: 257, 106).
+__device__ __forceinline__ void copy_ids(uint32_t* ids, uint64_t to, uint64_t from, uint64_t lo, uint64_t hi,
+                                         uint32_t lane) {
+  for (uint64_t d0 = lo + lane; d0 < hi; d0 += 256) {
+    uint32_t v[8];
+#pragma unroll
+    for (int k = 0; k < 8; ++k) v[k] = d0 + 32 * k < hi ? ids[from + d0 + 32 * k] : 0u;
+#pragma unroll
+    for (int k = 0; k < 8; ++k)
+      if (d0 + 32 * k < hi) ids[to + d0 + 32 * k] = v[k];
+  }
+}
+
 // ids of the matched accesses, one warp per request r: its depths below
 // lam[r] equal those of prior[r]; walking the prior chain t = prior[r],
 // prior[t], ..., the depths in [lam[t], hi) are unmatched in t (their ids
@@ -434,7 +449,7 @@ __global__ void __launch_bounds__(kFoThreads) k_ids_follow(PriorHint ph, uint32_
     const uint64_t lo = ph.lam[t];  // depths [lo, n_t) of t are unmatched
     if (lo < hi) {
       if (!in_bounds(st, tb + hi - 1, b) || !in_bounds(st, b + hi - 1, ph.blk_off[ph.n_req])) return;
-      for (uint64_t d = lo + lane; d < hi; d += 32) ids[b + d] = ids[tb + d];
+      copy_ids(ids, b, tb, lo, hi, lane);
       hi = lo;
     }
     cur = t;
@@ -506,7 +521,7 @@ __global__ void __launch_bounds__(kFoThreads) k_ids_follow_win(PriorHint ph, uin
       const uint64_t lo = __shfl_sync(kFull, (uint64_t)la, src), top = __shfl_sync(kFull, hl, src);
       const uint64_t tb = __shfl_sync(kFull, ta, src);
       if (!in_bounds(st, tb + top - 1, b) || !in_bounds(st, b + top - 1, ph.blk_off[ph.n_req])) return;
-      for (uint64_t d = lo + lane; d < top; d += 32) ids[b + d] = ids[tb + d];
+      copy_ids(ids, b, tb, lo, top, lane);
     }
     const uint64_t wmin = __shfl_sync(kFull, incl, 31);
     hi = wmin < hi ? wmin : hi;
@@ -1482,7 +1497,10 @@ __global__ void __launch_bounds__(kPdBigThreads, 2) k_pd_dedup_big(PdDedup a) {
 // ids after the partitioned dedup: ubits marks the settled accesses, bits
 // their first occurrences; a settled access that is not a first occurrence
 // (a repeat) finds its first occurrence in slot_of.  Matched accesses are
-// left to k_ids_follow.
+// left to k_ids_follow.  A warp's accesses share their words, so slot_of is
+// read for repeats only, and nothing but ubits for a word without settled ones:
+// 304M accesses, 144M settled, took 461 us with all three words read for every
+// access, 373 so; 134M, 80M settled, 208 and 156.
 __global__ void __launch_bounds__(kGaThreads) k_ids_gather_pd(const uint32_t* __restrict__ slot_of,
                                                              const uint32_t* __restrict__ ubits,
                                                              const uint32_t* __restrict__ bits,
@@ -1490,37 +1508,28 @@ __global__ void __launch_bounds__(kGaThreads) k_ids_gather_pd(const uint32_t* __
                                                              const uint64_t* n_dev, uint32_t* __restrict__ ids) {
   grid_dep_sync();
   const uint32_t n = keys_used(n_ub, n_dev);
-  const uint32_t i0 = blockIdx.x * (kGaThreads * kGaPer) + threadIdx.x;
-  uint32_t f[kGaPer], own[kGaPer], uw[kGaPer];
-  // the three words of every access are read together (slot_of whether or
-  // not the access turns out to be a repeat: one coalesced stream)
+  const uint32_t i0 = blockIdx.x * (kGaThreads * kGaPer) + threadIdx.x, lane = threadIdx.x & 31;
+  uint32_t uw[kGaPer], own[kGaPer], wp[kGaPer], f[kGaPer];
 #pragma unroll
   for (int k = 0; k < kGaPer; ++k) {
     const uint32_t i = i0 + k * kGaThreads;
     uw[k] = i < n ? __ldg(&ubits[i >> 5]) : 0u;
     own[k] = i < n ? bits[i >> 5] : 0u;
-    f[k] = i < n ? __ldcs(&slot_of[i]) : 0u;
+    wp[k] = i < n ? wpre[i >> 5] : 0u;
   }
 #pragma unroll
   for (int k = 0; k < kGaPer; ++k) {
     const uint32_t i = i0 + k * kGaThreads;
-    if (!((uw[k] >> (i & 31)) & 1u))
-      f[k] = kMatchedSlot;
-    else if ((own[k] >> (i & 31)) & 1u)
-      f[k] = i;
-  }
-  uint32_t wp[kGaPer], bw[kGaPer];
-#pragma unroll
-  for (int k = 0; k < kGaPer; ++k) {
-    const uint32_t i = i0 + k * kGaThreads;
-    const bool ok = f[k] < n;
-    wp[k] = ok ? wpre[f[k] >> 5] : 0u;
-    bw[k] = f[k] == i ? own[k] : ok ? bits[f[k] >> 5] : 0u;
+    f[k] = i < n && (((uw[k] & ~own[k]) >> lane) & 1u) ? __ldcs(&slot_of[i]) : kMatchedSlot;  // a repeat
   }
 #pragma unroll
   for (int k = 0; k < kGaPer; ++k) {
     const uint32_t i = i0 + k * kGaThreads;
-    if (i < n && f[k] != kMatchedSlot) ids[i] = f[k] < n ? wp[k] + __popc(bw[k] & ((1u << (f[k] & 31)) - 1u)) : kNone;
+    if (i >= n || !((uw[k] >> lane) & 1u)) continue;
+    uint32_t id = wp[k] + __popc(own[k] & lanemask_lt());
+    if (!((own[k] >> lane) & 1u))
+      id = f[k] < n ? wpre[f[k] >> 5] + __popc(bits[f[k] >> 5] & ((1u << (f[k] & 31)) - 1u)) : kNone;
+    ids[i] = id;
   }
 }
 
