@@ -84,7 +84,11 @@ constexpr int kInsK = 1;  // keys per thread: their key and slot loads are in fl
 // only).  An index that is stored and later replaced is toggled twice, the
 // final one once, and XOR does not depend on the order in which the toggles
 // land, so once all keys are settled the set bits are exactly the smallest
-// index of every key.
+// index of every key.  settle toggles only the indices that it replaces and
+// returns whether i's own bit is to be toggled: a warp's accesses share a word,
+// which toggle_own then changes by one atomic.  (One per claim, an atomic to L2
+// each: 11.3M keys, half of them claims, took 391 us, so 311; 9.3M, a sixth of
+// them claims, 166 and 144.)
 // 96 key bits: all of h0 (61) + 35 bits of h1.  Word 0 is never all-ones
 // because h0 < 2^61 - 1, and word 1 of a filled slot holds an index below
 // 2^32 - 1, so an all-ones word marks an empty or half-written slot.
@@ -95,7 +99,7 @@ __device__ __forceinline__ bool table_outrun(const DevStatus* st) {
   return (ld_relaxed_u32(&st->err) & kErrTableFull) != 0;
 }
 
-__device__ __forceinline__ void settle(ulonglong2* table, uint64_t mask, uint64_t probe_cap, uint32_t i,
+__device__ __forceinline__ bool settle(ulonglong2* table, uint64_t mask, uint64_t probe_cap, uint32_t i,
                                        ulonglong2 k, uint64_t pos, ulonglong2 cur, uint32_t* __restrict__ slot_out,
                                        uint32_t* bits, DevStatus* st) {
   const uint64_t w0 = k.x | ((k.y & 7ULL) << 61);
@@ -106,21 +110,19 @@ __device__ __forceinline__ void settle(ulonglong2* table, uint64_t mask, uint64_
     if (cur.x == ~0ULL || cur.y == ~0ULL) {  // empty, or being filled: settle it with the CAS
       cur = cas128(&table[pos], empty, mine);
       if (cur.x == ~0ULL && cur.y == ~0ULL) {
-        toggle(bits, i);
         __stcs(slot_out, (uint32_t)pos);
-        return;
+        return true;
       }
     }
     if (cur.x == w0 && (uint32_t)cur.y == w1lo) {
+      bool own = false;
       if ((uint32_t)(cur.y >> 32) > i) {
         const uint32_t old = atomicMin(reinterpret_cast<uint32_t*>(&table[pos]) + 3, i);
-        if (old > i) {
-          toggle(bits, i);
-          toggle(bits, old);
-        }
+        own = old > i;
+        if (own) toggle(bits, old);
       }
       __stcs(slot_out, (uint32_t)pos);
-      return;
+      return own;
     }
     if (++probe > mask || probe >= probe_cap) break;
     // a table some other key has outrun is given up: nobody walks its long runs to the end
@@ -130,6 +132,14 @@ __device__ __forceinline__ void settle(ulonglong2* table, uint64_t mask, uint64_
   }
   raise_err(st, kErrTableFull);
   *slot_out = 0;
+  return false;
+}
+
+// Toggles the bits of a warp's 32 consecutive accesses (from a multiple of 32,
+// this lane's is i) where `own` is set.  Whole warps only.
+__device__ __forceinline__ void toggle_own(uint32_t* bits, uint32_t i, bool own) {
+  const uint32_t m = __ballot_sync(kFull, own);
+  if ((i & 31) == 0 && m) atomicXor(&bits[i >> 5], m);
 }
 
 // kInsK keys per thread, kInsThreads apart: all their key loads, then all
@@ -186,13 +196,14 @@ __global__ void __launch_bounds__(kInsThreads) k_ids_insert(const ulonglong2* __
 #pragma unroll
   for (int j = 0; j < kInsK; ++j) {
     const uint32_t i = i0 + j * kInsThreads;
-    if (i >= n) continue;
-    if (k[j].x >= kP61 || k[j].y >= kP61) {
+    bool own = false;
+    if (i < n && (k[j].x >= kP61 || k[j].y >= kP61)) {
       raise_err(st, kErrInvalid);
       slot_of[i] = 0;
-      continue;
+    } else if (i < n) {
+      own = settle(table, mask, probe_cap, i, k[j], pos[j], cur[j], &slot_of[i], bits, st);
     }
-    settle(table, mask, probe_cap, i, k[j], pos[j], cur[j], &slot_of[i], bits, st);
+    toggle_own(bits, i, own);
   }
 }
 
@@ -375,13 +386,14 @@ __global__ void __launch_bounds__(kInsThreads) k_ids_insert_prior(const ulonglon
   report_keys_used(n_ub, n_dev, st);
   const uint32_t n = keys_used(n_ub, n_dev);
   const uint32_t base = blockIdx.x * (kInsThreads * K) + threadIdx.x;
-  if (blockIdx.x * (kInsThreads * K) >= n || table_outrun(st)) return;
+  if (blockIdx.x * (kInsThreads * K) >= n) return;
+  const uint32_t end = table_outrun(st) ? 0u : n;  // an attempt given up: nothing is settled
   bool unm[K];
 #pragma unroll
   for (int j = 0; j < K; ++j) {
     const uint32_t i = base + j * kInsThreads;
     unm[j] = false;
-    if (i >= n) continue;
+    if (i >= end) continue;
     const uint32_t t = i >> kReqTileLog2;
     const uint32_t r = req_at(ph.blk_off, __ldg(&ph.tile_req[t]), __ldg(&ph.tile_req[t + 1]), i);
     unm[j] = i - __ldg(&ph.blk_off[r]) >= __ldg(&ph.lam[r]);
@@ -403,9 +415,10 @@ __global__ void __launch_bounds__(kInsThreads) k_ids_insert_prior(const ulonglon
   }
 #pragma unroll
   for (int j = 0; j < K; ++j) {
-    if (!unm[j]) continue;
-    settle(table, (1ULL << log2m) - 1, probe_cap, base + j * kInsThreads, k[j], pos[j], cur[j],
-           &slot_of[base + j * kInsThreads], bits, st);
+    const uint32_t i = base + j * kInsThreads;
+    const bool own =
+        unm[j] && settle(table, (1ULL << log2m) - 1, probe_cap, i, k[j], pos[j], cur[j], &slot_of[i], bits, st);
+    toggle_own(bits, i, own);
   }
 }
 
