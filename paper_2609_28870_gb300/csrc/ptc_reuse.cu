@@ -16,10 +16,11 @@
 // (run order is time order) gives prev and next of every access; on a trace
 // without runs it is the sort of every (id, i).
 //
-//   k_ir_count     id-run starts per tile (ids < D checked); last CTA: prefixes
-//                  (k_ir_count4: 16-byte loads when the ids are 16-byte aligned)
-//   k_ir_mark      id-run records (start, first id) and the cuts, as a bitmap
-//                  over [0, D]
+//   k_ir_count     id-run starts as a bitmap over the accesses, and per tile (ids
+//                  < D checked); last CTA: prefixes (k_ir_count4: 16-byte loads
+//                  when the ids are 16-byte aligned)
+//   k_ir_mark      from that bitmap: id-run records (start, first id) and the
+//                  cuts, as a bitmap over [0, D]
 //   k_bm_count / k_bm_words   ranks of the cuts (and the cut of each rank)
 //   k_ir_inc1      elementary intervals per run; last CTA: prefixes and K
 //   k_ir_inc2      the K incidences (e, r)
@@ -51,6 +52,7 @@ struct IrArgs {
   uint32_t* tcnt;
   uint32_t* tpre;     // runs before each tile; tpre[ntiles] = number of runs
   uint32_t* done;
+  uint32_t* starts;   // bitmap of the run starts, kITile / 32 words per tile
   uint32_t* rec_s;    // start of each run (rec_s[R] = n)
   uint32_t* rec_x;    // first id of each run
   uint32_t* cut;      // bitmap over [0, D]: the cuts of id-space
@@ -158,7 +160,10 @@ __global__ void __launch_bounds__(kIT) k_ir_count(IrArgs a0) {
   id_starts(a, tile * kITile + w * (32 * kIR), lane, id, left, words, bad);
   uint32_t cnt = 0;
 #pragma unroll
-  for (int k = 0; k < kIR; ++k) cnt += __popc(words[k]);
+  for (int k = 0; k < kIR; ++k) {
+    cnt += __popc(words[k]);
+    if (lane == 0) a.starts[(tile * kITile + w * (32 * kIR)) / 32 + k] = words[k];
+  }
   if (bad) raise_err(a.st, kErrInvalid);
   uint32_t total;
   cta_excl_u32(lane == 0 ? cnt : 0u, s_w, &total);
@@ -168,40 +173,58 @@ __global__ void __launch_bounds__(kIT) k_ir_count(IrArgs a0) {
   if (threadIdx.x == 0) a.st->value[1] = R;
 }
 
-__global__ void __launch_bounds__(kIT) k_ir_mark(IrArgs a0) {
+// Marks the cut at id x.  Prompts that many sessions share are cut at the same ids
+// again and again, so the word is read first (a stale one only costs the atomic).
+__device__ __forceinline__ void mark_cut(uint32_t* cut, uint32_t x) {
+  const uint32_t b = 1u << (x & 31);
+  if (!(cut[x >> 5] & b)) atomicOr(&cut[x >> 5], b);
+}
+
+// A word of the bitmap per thread, whose starts go to a list in shared memory;
+// then a start per thread: its record and cuts, from its id and the one left of
+// it, which are read again.  Bound by latency.  Marking in a
+// second pass over the ids took 376 us on 304M accesses and 158 on 134M, so 88
+// and 39 (174 and 74 with one word per thread and more CTAs; but the steps of a
+// CTA follow one another, and with few CTAs 127K accesses took 4 us longer so).
+constexpr uint32_t kMarkSteps = 4;  // words per thread at most
+__global__ void __launch_bounds__(kIT) k_ir_mark(IrArgs a0, uint32_t steps) {
   grid_dep_sync();
   __shared__ uint32_t s_w[kIT / 32];
+  __shared__ uint16_t s_at[kIT * 32];
   const IrArgs a = resolved(a0);
   // ids >= D (reported, nothing is indexed by them), or a trace without runs,
   // whose accesses are all sorted: marking its cuts, two random atomics per
   // access, took 0.6 ms of a 12M-access block trace's 5.5 for nothing
   if (*(volatile uint32_t*)&a.st->err || *(volatile uint64_t*)&a.st->value[1] > a.max_runs) return;
-  const uint32_t tile = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const uint32_t base = tile * kITile + w * (32 * kIR);
-  uint32_t id[kIR], left[kIR], words[kIR];
-  bool bad = false;
-  id_starts(a, base, lane, id, left, words, bad);
-  uint32_t cnt = 0;
+  uint32_t words[kMarkSteps];
 #pragma unroll
-  for (int k = 0; k < kIR; ++k) cnt += __popc(words[k]);
-  uint32_t total;
-  uint32_t run = a.tpre[tile] + cta_excl_u32(lane == 0 ? cnt : 0u, s_w, &total);
-  run = __shfl_sync(kFull, run, 0);
+  for (uint32_t k = 0; k < kMarkSteps; ++k) {
+    const uint64_t j0 = ((uint64_t)blockIdx.x * steps + k) * (kIT * 32) + threadIdx.x * 32;
+    words[k] = k < steps && j0 < a.n ? a.starts[j0 / 32] : 0u;
+  }
+#pragma unroll 1
+  for (uint32_t k = 0; k < steps; ++k) {
+    const uint64_t c0 = ((uint64_t)blockIdx.x * steps + k) * (kIT * 32);
+    if (c0 >= a.n) return;
+    const uint32_t first = a.tpre[c0 / kITile];
+    uint32_t m = 0, total;
 #pragma unroll
-  for (int k = 0; k < kIR; ++k) {
-    const uint32_t j = base + k * 32 + lane;
-    if ((words[k] >> lane) & 1u) {
-      const uint32_t r = run + __popc(words[k] & lanemask_lt());
-      a.rec_s[r] = j;
-      a.rec_x[r] = id[k];
-      atomicOr(&a.cut[id[k] >> 5], 1u << (id[k] & 31));
-      if (j > 0) atomicOr(&a.cut[(left[k] + 1) >> 5], 1u << ((left[k] + 1) & 31));
+    for (uint32_t q = 0; q < kMarkSteps; ++q) m = q == k ? words[q] : m;
+    uint32_t q = cta_excl_u32(__popc(m), s_w, &total);
+    for (; m; m &= m - 1) s_at[q++] = (uint16_t)(32 * threadIdx.x + __ffs(m) - 1);
+    __syncthreads();
+    for (uint32_t i = threadIdx.x; i < total; i += kIT) {
+      const uint32_t j = (uint32_t)c0 + s_at[i];
+      const uint32_t x = a.ids[j], left = j > 0 ? a.ids[j - 1] : 0u;
+      a.rec_s[first + i] = j;
+      a.rec_x[first + i] = x;
+      mark_cut(a.cut, x);
+      if (j > 0) mark_cut(a.cut, left + 1);
     }
-    if (j + 1 == a.n) {
-      atomicOr(&a.cut[(id[k] + 1) >> 5], 1u << ((id[k] + 1) & 31));
-      a.rec_s[a.tpre[a.ntiles]] = a.n;
+    if (a.n - c0 <= kIT * 32 && threadIdx.x == 0) {  // the last access is among these
+      mark_cut(a.cut, a.ids[a.n - 1] + 1);
+      a.rec_s[first + total] = a.n;
     }
-    run += __popc(words[k]);
   }
 }
 
@@ -259,7 +282,16 @@ __global__ void __launch_bounds__(kIT) k_ir_count4(IrArgs a0) {
   uint4 v[kIR4];
   uint32_t x[kIR4], il[kIR4];
   bool bad = false;
-  const uint32_t cnt = __reduce_add_sync(kFull, warp_id_starts4(a, tile * kITile + w * (32 * kIR), lane, v, x, il, bad));
+  const uint32_t base = tile * kITile + w * (32 * kIR);
+  const uint32_t cnt = __reduce_add_sync(kFull, warp_id_starts4(a, base, lane, v, x, il, bad));
+#pragma unroll
+  for (int k = 0; k < kIR4; ++k) {  // lanes 8 g .. 8 g + 7 hold the nibbles of word g
+    uint32_t word = x[k] << (4 * (lane & 7));
+    word |= __shfl_xor_sync(kFull, word, 1);
+    word |= __shfl_xor_sync(kFull, word, 2);
+    word |= __shfl_xor_sync(kFull, word, 4);
+    if ((lane & 7) == 0) a.starts[base / 32 + 4 * k + (lane >> 3)] = word;
+  }
   if (lane == 0) s_wcnt[w] = cnt;
   if (bad) raise_err(a.st, kErrInvalid);
   __syncthreads();
@@ -523,7 +555,7 @@ struct ReuseLayout {
   DevStatus* st;
   uint32_t* done;
   size_t zero_bytes;
-  uint32_t *tcnt, *tpre, *rec_s, *rec_x;
+  uint32_t *tcnt, *tpre, *starts, *rec_s, *rec_x;
   uint32_t *cut, *cwpre, *cut_at, *btcnt, *btpre;
   uint32_t *rtcnt, *rtpre;
   uint32_t *key, *val;
@@ -552,6 +584,7 @@ ReuseLayout reuse_layout(void* ws, uint64_t n, uint64_t D, bool forced, const Re
   L.zero_bytes = cv.off;
   L.tcnt = cv.take<uint32_t>(L.ntiles + 1);
   L.tpre = cv.take<uint32_t>(L.ntiles + 1);
+  L.starts = cv.take<uint32_t>((size_t)L.ntiles * (kITile / 32));
   L.rec_s = cv.take<uint32_t>(nn + 1);
   L.rec_x = cv.take<uint32_t>(nn);
   L.cut = cv.take<uint32_t>(L.nwords);
@@ -600,6 +633,7 @@ ptc_status reuse_by_runs(const uint32_t* ids, uint64_t n, uint64_t D, uint32_t* 
   a.tcnt = L.tcnt;
   a.tpre = L.tpre;
   a.done = &L.done[0];
+  a.starts = L.starts;
   a.rec_s = L.rec_s;
   a.rec_x = L.rec_x;
   a.cut = L.cut;
@@ -608,14 +642,13 @@ ptc_status reuse_by_runs(const uint32_t* ids, uint64_t n, uint64_t D, uint32_t* 
   a.nd = din ? din->nd : nullptr;
   a.errs = din ? din->errs : nullptr;
   a.n_errs = din ? din->n_errs : 0;
-  // the count with 16-byte loads when the ids allow them (measured faster);
-  // the marking pass stays one access per lane and round (the 16-byte form
-  // of it measured slower: 0.77 against 0.70 ms on the mixed 10B-token trace)
+  // the count with 16-byte loads when the ids allow them (measured faster)
   if ((reinterpret_cast<uintptr_t>(ids) & 15) == 0)
     PTC_KERNEL("k_ir_count", s, k_ir_count4, L.ntiles, kIT, 0, a);
   else
     PTC_KERNEL("k_ir_count", s, k_ir_count, L.ntiles, kIT, 0, a);
-  PTC_KERNEL("k_ir_mark", s, k_ir_mark, L.ntiles, kIT, 0, a);
+  const uint32_t steps = n / (kMarkSteps * kIT * 32) >= (uint64_t)(2 * num_sms()) ? kMarkSteps : 1;
+  PTC_KERNEL("k_ir_mark", s, k_ir_mark, ceil_div_u32(n, (uint64_t)steps * kIT * 32), kIT, 0, a, steps);
   PTC_KERNEL("k_bm_count", s, k_bm_count, L.btiles, kIT, 0, L.cut, L.nwords, L.btiles, L.btcnt, L.btpre, &L.done[1], L.st);
   PTC_KERNEL("k_bm_words", s, k_bm_words, L.btiles, kIT, 0, L.cut, L.nwords, L.btpre, L.cwpre, L.cut_at);
   IncArgs ia;

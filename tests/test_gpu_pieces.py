@@ -17,7 +17,7 @@ def _gpu():
     ptc.lib()
 
 
-@pytest.mark.parametrize("n_req", [1, 2, 300, 2047, 2048, 2049, 30000, 600000])
+@pytest.mark.parametrize("n_req", [1, 2, 300, 2047, 2048, 2049, 30000, 600000, 1300000])
 @pytest.mark.parametrize("follow", [0.0, 0.7])
 def test_pieces(n_req, follow):
     """Requests of eight one-token blocks each re-read a document whole, now and
@@ -45,6 +45,10 @@ def test_pieces(n_req, follow):
     nxt[order[:-1][again]] = order[1:][again]
     assert res["n_access"] == n and res["n_distinct"] == 8 * len(np.unique(pick))
     assert np.array_equal(ptc.u32(buf["prev"]), prev) and np.array_equal(ptc.u32(buf["next"]), nxt)
+    ids = torch.zeros(n + 1, dtype=torch.int32, device="cuda")  # not 16-byte aligned from its second entry on
+    ids[1:] = buf["ids"]
+    p1, n1 = ptc.ptc_reuse_indices(ids[1:], res["n_distinct"])
+    assert np.array_equal(ptc.u32(p1), prev) and np.array_equal(ptc.u32(n1), nxt)
     dist = ptc.ptc_stack_distance(torch.from_numpy(prev.view(np.int32)).cuda())
     assert torch.equal(buf["dist"], dist.view(torch.int32))
     c = ptc.ptc_curves(dist, ptc.to_device_u64(off), 1, caps, ptc.PTC_COST_UNIFORM)
