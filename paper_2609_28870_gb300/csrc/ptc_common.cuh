@@ -355,6 +355,37 @@ struct Carver {
   size_t bytes() const { return (off + 255) / 256 * 256; }
 };
 
+// ---- runs (stage c): run-start bitmap and the runs starting before each word
+// Index of the run holding access j.
+__device__ __forceinline__ uint32_t run_of(const uint32_t* bits, const uint32_t* wpre, uint32_t j) {
+  const uint32_t wi = j >> 5, b = j & 31;
+  const uint32_t mask_le = b == 31 ? kFull : ((2u << b) - 1u);
+  return wpre[wi] + __popc(bits[wi] & mask_le) - 1u;
+}
+
+// Every access takes its run's distance: kExpPer accesses per thread, kExpThreads
+// apart, so that each thread's dependent loads (word, then distance) for all of
+// them are in flight together.
+constexpr int kExpThreads = 256;
+constexpr int kExpPer = 8;
+__device__ __forceinline__ void expand_runs(uint32_t tile, const uint32_t* __restrict__ bits,
+                                            const uint32_t* __restrict__ wpre, const uint32_t* __restrict__ sd,
+                                            uint32_t n, uint32_t* __restrict__ dist, uint32_t nruns,
+                                            const DevStatus* st) {
+  const uint32_t j0 = tile * (kExpThreads * kExpPer) + threadIdx.x;
+  uint32_t r[kExpPer];
+#pragma unroll
+  for (int k = 0; k < kExpPer; ++k) {
+    const uint32_t j = j0 + k * kExpThreads;
+    r[k] = j < n ? run_of(bits, wpre, j) : 0u;
+  }
+#pragma unroll
+  for (int k = 0; k < kExpPer; ++k) {
+    const uint32_t j = j0 + k * kExpThreads;
+    if (j < n && in_bounds(st, r[k], nruns)) __stcs(&dist[j], __ldg(&sd[r[k]]));
+  }
+}
+
 inline uint32_t ceil_div_u32(uint64_t a, uint64_t b) { return (uint32_t)((a + b - 1) / b); }
 
 }  // namespace ptc

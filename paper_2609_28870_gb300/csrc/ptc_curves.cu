@@ -25,7 +25,7 @@
 //               lies in the request; a fall between the runs of a request
 //               sets the flag for the scan kernels
 //   k_finalize  cumulative sums over bins (a block scan); 128-bit saved and
-//               total cost
+//               total cost (after k_curves_runs its last CTA does this)
 #include "ptc_internal.h"
 
 namespace ptc {
@@ -490,12 +490,93 @@ __global__ void __launch_bounds__(kCvThreads) k_curves_fast(CurveArgs a) {
 }
 
 
-// Index of the run holding access j (stage c's run-start bitmap and the runs
-// starting before each 32-access word).
-__device__ __forceinline__ uint32_t run_at(const uint32_t* bits, const uint32_t* wpre, uint32_t j) {
-  const uint32_t wi = j >> 5, b = j & 31;
-  const uint32_t mask_le = b == 31 ? kFull : ((2u << b) - 1u);
-  return wpre[wi] + __popc(bits[wi] & mask_le) - 1u;
+struct U128 {
+  uint64_t lo, hi;
+};
+__device__ __forceinline__ U128 mul_u64(uint64_t a, uint64_t b) { return U128{a * b, __umul64hi(a, b)}; }
+__device__ __forceinline__ U128 add_u128(U128 a, U128 b) {
+  U128 r;
+  r.lo = a.lo + b.lo;
+  r.hi = a.hi + b.hi + (r.lo < a.lo ? 1 : 0);
+  return r;
+}
+
+// The results from the bins: hits[G] | saved[G] (lo, hi) | total (lo, hi) | slow.
+// The errors of the stages before join this call's; `out` and `st_host` may be
+// the mapped host stage (then the results and the status need no copies).
+struct FinishArgs {
+  const unsigned long long* cnt;
+  const unsigned long long* ksum;
+  uint32_t G;
+  uint64_t alpha, beta;
+  uint64_t* out;
+  const uint32_t* slow;
+  DevStatus* st;
+  const DevStatus* earlier;
+  uint32_t n_earlier;
+  DevStatus* st_host;
+};
+
+// By one CTA of T threads: an inclusive scan of (count, depth sum) over the bins,
+// consecutive ones per thread.
+template <int T>
+__device__ __forceinline__ void finalize_bins(const FinishArgs& f) {
+  __shared__ unsigned long long s_h[T / 32], s_k[T / 32];
+  const uint32_t t = threadIdx.x, lane = t & 31, w = t >> 5, G = f.G;
+  const uint32_t per = (G + T - 1) / T, g0 = t * per, g1 = g0 + per < G ? g0 + per : G;
+  unsigned long long h = 0, k = 0;
+  for (uint32_t g = g0; g < g1; ++g) {
+    h += __ldcg(&f.cnt[g]);
+    k += __ldcg(&f.ksum[g]);
+  }
+  const unsigned long long own_h = h, own_k = k;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long yh = __shfl_up_sync(kFull, h, o), yk = __shfl_up_sync(kFull, k, o);
+    if (lane >= (uint32_t)o) {
+      h += yh;
+      k += yk;
+    }
+  }
+  if (lane == 31) {
+    s_h[w] = h;
+    s_k[w] = k;
+  }
+  __syncthreads();
+  for (uint32_t ww = 0; ww < w; ++ww) {
+    h += s_h[ww];
+    k += s_k[ww];
+  }
+  h -= own_h;
+  k -= own_k;
+  for (uint32_t g = g0; g < g1; ++g) {
+    h += __ldcg(&f.cnt[g]);
+    k += __ldcg(&f.ksum[g]);
+    const U128 sv = add_u128(mul_u64(f.alpha, h), mul_u64(f.beta, k));
+    f.out[g] = h;
+    f.out[G + 2 * g] = sv.lo;
+    f.out[G + 2 * g + 1] = sv.hi;
+    if (g == G - 1) {  // the miss bin G joins the total
+      const uint64_t hn = h + __ldcg(&f.cnt[G]), kn = k + __ldcg(&f.ksum[G]);
+      const U128 tc = add_u128(mul_u64(f.alpha, hn), mul_u64(f.beta, kn));
+      f.out[3 * G] = tc.lo;
+      f.out[3 * G + 1] = tc.hi;
+      f.out[3 * G + 2] = __ldcg(f.slow);
+    }
+  }
+  if (t == 0) {
+    uint32_t e = f.st->err;
+    for (uint32_t q = 0; q < f.n_earlier; ++q) e |= f.earlier[q].err;
+    f.st->err = e;
+  }
+  __syncthreads();
+  if (f.st_host && t < sizeof(DevStatus) / 4)
+    reinterpret_cast<uint32_t*>(f.st_host)[t] = reinterpret_cast<const volatile uint32_t*>(f.st)[t];
+}
+
+__global__ void __launch_bounds__(1024) k_finalize(FinishArgs f) {
+  grid_dep_sync();
+  finalize_bins<1024>(f);
 }
 
 struct RunsArgs {
@@ -503,10 +584,21 @@ struct RunsArgs {
   const uint32_t* sd;
   const uint32_t* bits;
   const uint32_t* wpre;
+  uint32_t R;      // runs at most
+  uint32_t* dist;  // distances still to be written (or null)
+  uint32_t ctas;   // that take requests; those after them write the distances
+  uint32_t* done;  // zeroed
 };
 
-__global__ void __launch_bounds__(256) k_curves_runs(CurveArgs a, RunsArgs ra) {
+// The last CTA of the requests writes the results (FinishArgs), and the CTAs after
+// them the distances: nothing but the stage's end waits for these, and on a small
+// trace each launch less is 4 us.
+__global__ void __launch_bounds__(256) k_curves_runs(CurveArgs a, RunsArgs ra, FinishArgs f) {
   grid_dep_sync();
+  if (blockIdx.x >= ra.ctas) {
+    expand_runs(blockIdx.x - ra.ctas, ra.bits, ra.wpre, ra.sd, a.n, ra.dist, ra.R, a.st);
+    return;
+  }
   __shared__ Bins s_bins;
   const uint32_t G = a.G;
   s_bins.init(a.caps, G);
@@ -516,12 +608,12 @@ __global__ void __launch_bounds__(256) k_curves_runs(CurveArgs a, RunsArgs ra) {
   // size of trace; a warp per request leaves most lanes idle, 125 us for the
   // 291K requests of half a mixed day.)
   bool fell = false;
-  const uint32_t sub = threadIdx.x & 3, groups = gridDim.x * (blockDim.x >> 2);
+  const uint32_t sub = threadIdx.x & 3, groups = ra.ctas * (blockDim.x >> 2);
   for (uint32_t q0 = blockIdx.x * (blockDim.x >> 2) + ((threadIdx.x >> 5) << 3); q0 < a.R; q0 += groups) {
     const uint32_t q = q0 + ((threadIdx.x & 31) >> 2);
     const uint32_t start = q < a.R ? (uint32_t)a.blk_off[q] : 0u, end = q < a.R ? (uint32_t)a.blk_off[q + 1] : 0u;
     const bool some = end > start && end <= a.n;  // not empty (bad offsets are reported by k_heads)
-    const uint32_t r0 = some ? run_at(ra.bits, ra.wpre, start) : 1u, r1 = some ? run_at(ra.bits, ra.wpre, end - 1) : 0u;
+    const uint32_t r0 = some ? run_of(ra.bits, ra.wpre, start) : 1u, r1 = some ? run_of(ra.bits, ra.wpre, end - 1) : 0u;
     const uint32_t rounds = __reduce_max_sync(kFull, some ? (r1 - r0) / 4 + 1 : 0u);
     uint32_t before = 0;  // the distance of the run before this round's first
     for (uint32_t c = 0; c < rounds; ++c) {
@@ -541,72 +633,16 @@ __global__ void __launch_bounds__(256) k_curves_runs(CurveArgs a, RunsArgs ra) {
   }
   if (__syncthreads_or(fell) && threadIdx.x == 0) atomicOr(a.slow, 1u);
   s_bins.store(G, a.cnt, a.ksum);
-}
-
-
-struct U128 {
-  uint64_t lo, hi;
-};
-__device__ __forceinline__ U128 mul_u64(uint64_t a, uint64_t b) { return U128{a * b, __umul64hi(a, b)}; }
-__device__ __forceinline__ U128 add_u128(U128 a, U128 b) {
-  U128 r;
-  r.lo = a.lo + b.lo;
-  r.hi = a.hi + b.hi + (r.lo < a.lo ? 1 : 0);
-  return r;
-}
-
-// out layout: hits[G] | saved[G] (lo, hi) | total (lo, hi) | slow.  One CTA of
-// 1,024 threads: an inclusive block scan of (count, depth sum) over the bins.
-// The errors of the stages before join this call's; `out` and `st_host` may be
-// the mapped host stage (then the results and the status need no copies).
-__global__ void __launch_bounds__(1024) k_finalize(const unsigned long long* __restrict__ cnt,
-                                                   const unsigned long long* __restrict__ ksum, uint32_t G,
-                                                   uint64_t alpha, uint64_t beta, uint64_t* __restrict__ out,
-                                                   const uint32_t* slow, DevStatus* st, const DevStatus* earlier,
-                                                   uint32_t n_earlier, DevStatus* st_host) {
-  grid_dep_sync();
-  __shared__ unsigned long long s_h[32], s_k[32];
-  const uint32_t t = threadIdx.x, lane = t & 31, w = t >> 5;
-  unsigned long long h = t < G ? cnt[t] : 0ull, k = t < G ? ksum[t] : 0ull;
-#pragma unroll
-  for (int o = 1; o < 32; o <<= 1) {
-    const unsigned long long yh = __shfl_up_sync(kFull, h, o), yk = __shfl_up_sync(kFull, k, o);
-    if (lane >= (uint32_t)o) {
-      h += yh;
-      k += yk;
-    }
-  }
-  if (lane == 31) {
-    s_h[w] = h;
-    s_k[w] = k;
-  }
+  __shared__ uint32_t s_last;
+  __threadfence();
   __syncthreads();
-  for (uint32_t ww = 0; ww < w; ++ww) {
-    h += s_h[ww];
-    k += s_k[ww];
-  }
-  if (t < G) {
-    const U128 sv = add_u128(mul_u64(alpha, h), mul_u64(beta, k));
-    out[t] = h;
-    out[G + 2 * t] = sv.lo;
-    out[G + 2 * t + 1] = sv.hi;
-  }
-  if (t == G - 1) {  // G >= 1; the miss bin G joins the total
-    const uint64_t hn = h + cnt[G], kn = k + ksum[G];
-    const U128 tc = add_u128(mul_u64(alpha, hn), mul_u64(beta, kn));
-    out[3 * G] = tc.lo;
-    out[3 * G + 1] = tc.hi;
-    out[3 * G + 2] = *slow;
-  }
-  if (t == 0) {
-    uint32_t e = st->err;
-    for (uint32_t q = 0; q < n_earlier; ++q) e |= earlier[q].err;
-    st->err = e;
-  }
+  if (threadIdx.x == 0) s_last = atomicAdd(ra.done, 1u) == ra.ctas - 1;
   __syncthreads();
-  if (st_host && t < sizeof(DevStatus) / 4)
-    reinterpret_cast<uint32_t*>(st_host)[t] = reinterpret_cast<const volatile uint32_t*>(st)[t];
+  if (!s_last) return;
+  __threadfence();
+  finalize_bins<256>(f);
 }
+
 
 struct CurvesLayout {
   DevStatus* st;
@@ -614,6 +650,7 @@ struct CurvesLayout {
   unsigned long long* ksum;
   uint32_t* bitmap;
   uint32_t* slow;
+  uint32_t* done;
   uint32_t* tile_req;
   RunMax* lb_agg;
   uint64_t* out;
@@ -630,6 +667,7 @@ CurvesLayout curves_layout(void* ws, uint64_t n, uint32_t G) {
   L.ksum = cv.take<unsigned long long>(PTC_MAX_CAPACITIES + 1);
   L.bitmap = cv.take<uint32_t>(n / 32 + 2);
   L.slow = cv.take<uint32_t>(1);
+  L.done = cv.take<uint32_t>(1);
   L.tile_req = cv.take<uint32_t>(tiles + 1);
   L.zero_bytes = cv.off;
   L.lb_agg = cv.take<RunMax>(tiles);
@@ -726,33 +764,35 @@ ptc_status ptc::curves_impl(const uint32_t* dist, uint64_t n, const uint64_t* re
   };
   // results and status, waited for
   DevStatus h;
-  auto finish = [&]() -> ptc_status {
-    const bool staged = hs->dev != nullptr;
-    PTC_KERNEL("k_finalize", s, k_finalize, 1, 1024, 0, L.cnt, L.ksum, n_cap, alpha, beta,
-               staged ? hs->dev->out : L.out, L.slow, L.st, earlier, n_earlier, staged ? &hs->dev->st : nullptr);
+  const bool staged = hs->dev != nullptr;
+  const FinishArgs fin{L.cnt,  L.ksum, n_cap,   alpha,     beta, staged ? hs->dev->out : L.out,
+                       L.slow, L.st,   earlier, n_earlier, staged ? &hs->dev->st : nullptr};
+  auto finish = [&](bool written) -> ptc_status {
+    if (!written) PTC_KERNEL("k_finalize", s, k_finalize, 1, 1024, 0, fin);
     if (staged) return end_call_staged(s, &h);
     if (copy_to_host_async(hs->out, L.out, sizeof(uint64_t) * (3 * n_cap + 3), s) != PTC_OK) return PTC_ERR_CUDA;
     return end_call(L.st, s, &h);
   };
   if (from_runs) {
-    const RunsArgs ra{runs->rec_s, runs->sd, runs->bits, runs->wpre};
     const uint32_t want = ceil_div_u32(n_req, 64), most = (uint32_t)(4 * num_sms());
     const uint32_t g_r = want < most ? want : most;
-    PTC_KERNEL("k_curves_runs", s, k_curves_runs, g_r, 256, 0, a, ra);
+    const uint32_t g_e = runs->dist ? ceil_div_u32(n, kExpThreads * kExpPer) : 0;
+    const RunsArgs ra{runs->rec_s, runs->sd, runs->bits, runs->wpre, runs->R, runs->dist, g_r, L.done};
+    PTC_KERNEL("k_curves_runs", s, k_curves_runs, g_r + g_e, kExpThreads, 0, a, ra, fin);
   } else if (n > 0) {
     heads();
     PTC_KERNEL("k_curves_fast", s, k_curves_fast, grid, kCvThreads, 0, a);
     scans();
   }
   const uint64_t* host_out = hs->out;
-  ptc_status rc = finish();
+  ptc_status rc = finish(from_runs);
   if (rc != PTC_OK) return rc;
   if (from_runs && host_out[3 * n_cap + 2]) {
     // the distances of some request's runs fall (never so for a root-first
     // trace): the bins are void, and the scans start them afresh
     heads();
     scans();
-    rc = finish();
+    rc = finish(false);
     if (rc != PTC_OK) return rc;
   }
   for (uint32_t g = 0; g < n_cap; ++g) {

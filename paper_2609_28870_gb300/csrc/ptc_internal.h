@@ -192,6 +192,7 @@ struct RunsView {
   const uint32_t* sd = nullptr;     // distance of every run
   const uint32_t* bits = nullptr;   // run-start bitmap, one word per 32 accesses
   const uint32_t* wpre = nullptr;   // runs starting before each word
+  uint32_t* dist = nullptr;         // the distances of all accesses, left to stage d's launch
 };
 // Keys left without the carry from earlier tiles (stage a1 skips its
 // chain pass): block i of tile t = i / tile_blocks still needs carry[t] added

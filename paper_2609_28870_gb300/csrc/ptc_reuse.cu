@@ -21,7 +21,8 @@
 //                  when the ids are 16-byte aligned)
 //   k_ir_mark      from that bitmap: id-run records (start, first id) and the
 //                  cuts, as a bitmap over [0, D]
-//   k_bm_count / k_bm_words   ranks of the cuts (and the cut of each rank)
+//   k_bm_count / k_bm_words   ranks of the cuts (and the cut of each rank); of few
+//                  ids k_bm_one
 //   k_ir_inc1      elementary intervals per run; last CTA: prefixes and K
 //   k_ir_inc2      the K incidences (e, r)
 //   (sort_pairs)   stable radix sort of the incidences by e
@@ -346,6 +347,40 @@ __global__ void __launch_bounds__(kIT) k_bm_words(const uint32_t* __restrict__ b
   }
 }
 
+// Both in one CTA of 1,024 threads where the bitmap is small: up to kBmOne words,
+// a launch less (4 us of a window of 127K accesses).
+constexpr uint32_t kBmOne = 8192;
+__global__ void __launch_bounds__(1024) k_bm_one(const uint32_t* __restrict__ bits, uint32_t nwords,
+                                                 uint32_t* __restrict__ wpre, uint32_t* __restrict__ cut_at,
+                                                 DevStatus* st) {
+  grid_dep_sync();
+  __shared__ uint32_t s_w[32];
+  const uint32_t t = threadIdx.x, lane = t & 31, w = t >> 5;
+  const uint32_t per = (nwords + 1023) / 1024, w0 = t * per, w1 = w0 + per < nwords ? w0 + per : nwords;
+  uint32_t b[kBmOne / 1024], c = 0;
+#pragma unroll
+  for (uint32_t k = 0; k < kBmOne / 1024; ++k) {
+    b[k] = k < per && w0 + k < w1 ? bits[w0 + k] : 0u;
+    c += __popc(b[k]);
+  }
+  uint32_t incl = c;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const uint32_t y = __shfl_up_sync(kFull, incl, o);
+    if (lane >= (uint32_t)o) incl += y;
+  }
+  if (lane == 31) s_w[w] = incl;
+  __syncthreads();
+  const uint32_t mine = s_w[lane], before = __reduce_add_sync(kFull, lane < w ? mine : 0u);
+  if (t == 1023) st->value[2] = before + incl;
+  uint32_t r = before + incl - c;
+#pragma unroll
+  for (uint32_t k = 0; k < kBmOne / 1024; ++k) {
+    if (k < per && w0 + k < w1) wpre[w0 + k] = r;
+    for (uint32_t m = b[k]; m; m &= m - 1) cut_at[r++] = (w0 + k) * 32 + (__ffs(m) - 1);
+  }
+}
+
 // Cuts at or below y, minus one: the elementary interval holding id y.
 __device__ __forceinline__ uint32_t interval_of(const uint32_t* bits, const uint32_t* wpre, uint32_t y) {
   const uint32_t wi = y >> 5, b = y & 31;
@@ -370,7 +405,14 @@ struct IncArgs {
   uint32_t max_tiles;       // tiles of tcnt / tpre
   uint32_t max_runs;
   DevStatus* st;            // value[3] <- K
+  DevStatus* st_host;       // takes the status block at the end (the mapped host stage, or null)
 };
+
+// The status block to the host stage, by the calling CTA (after a barrier).
+__device__ __forceinline__ void publish(const DevStatus* st, DevStatus* host) {
+  if (host && threadIdx.x < sizeof(DevStatus) / 4)
+    reinterpret_cast<uint32_t*>(host)[threadIdx.x] = reinterpret_cast<const volatile uint32_t*>(st)[threadIdx.x];
+}
 
 // Intervals of run r: [first, end).
 __device__ __forceinline__ void run_intervals(const IncArgs& a, uint32_t r, uint32_t& first, uint32_t& end) {
@@ -383,9 +425,12 @@ __device__ __forceinline__ void run_intervals(const IncArgs& a, uint32_t r, uint
 __global__ void __launch_bounds__(kIT) k_ir_inc1(IncArgs a) {
   grid_dep_sync();
   __shared__ uint32_t s_w[kIT / 32];
-  if (*(volatile const uint32_t*)&a.stc->err) return;  // the records are incomplete
   const uint32_t R = (uint32_t)a.stc->value[1];
-  if (R > a.max_runs) return;  // there are no records
+  // the records are incomplete, or there are none
+  if (*(volatile const uint32_t*)&a.stc->err || R > a.max_runs) {
+    if (blockIdx.x == 0) publish(a.stc, a.st_host);
+    return;
+  }
   const uint32_t T = (R + kRunTile - 1) / kRunTile;
   for (uint32_t t = blockIdx.x; t < T; t += gridDim.x) {
     const uint32_t r0 = t * kRunTile + threadIdx.x * kRunPer;
@@ -405,6 +450,8 @@ __global__ void __launch_bounds__(kIT) k_ir_inc1(IncArgs a) {
   if (!last_cta(a.done)) return;
   const uint32_t K = tiles_prefix(a.tcnt, a.tpre, T < a.max_tiles ? T : a.max_tiles, s_w);
   if (threadIdx.x == 0) a.st->value[3] = K;
+  __syncthreads();
+  publish(a.st, a.st_host);
 }
 
 __global__ void __launch_bounds__(kIT) k_ir_inc2(IncArgs a, uint32_t R) {
@@ -649,8 +696,13 @@ ptc_status reuse_by_runs(const uint32_t* ids, uint64_t n, uint64_t D, uint32_t* 
     PTC_KERNEL("k_ir_count", s, k_ir_count, L.ntiles, kIT, 0, a);
   const uint32_t steps = n / (kMarkSteps * kIT * 32) >= (uint64_t)(2 * num_sms()) ? kMarkSteps : 1;
   PTC_KERNEL("k_ir_mark", s, k_ir_mark, ceil_div_u32(n, (uint64_t)steps * kIT * 32), kIT, 0, a, steps);
-  PTC_KERNEL("k_bm_count", s, k_bm_count, L.btiles, kIT, 0, L.cut, L.nwords, L.btiles, L.btcnt, L.btpre, &L.done[1], L.st);
-  PTC_KERNEL("k_bm_words", s, k_bm_words, L.btiles, kIT, 0, L.cut, L.nwords, L.btpre, L.cwpre, L.cut_at);
+  if (L.nwords <= kBmOne) {
+    PTC_KERNEL("k_bm_one", s, k_bm_one, 1, 1024, 0, L.cut, L.nwords, L.cwpre, L.cut_at, L.st);
+  } else {
+    PTC_KERNEL("k_bm_count", s, k_bm_count, L.btiles, kIT, 0, L.cut, L.nwords, L.btiles, L.btcnt, L.btpre, &L.done[1],
+               L.st);
+    PTC_KERNEL("k_bm_words", s, k_bm_words, L.btiles, kIT, 0, L.cut, L.nwords, L.btpre, L.cwpre, L.cut_at);
+  }
   IncArgs ia;
   ia.rec_s = L.rec_s;
   ia.rec_x = L.rec_x;
@@ -668,10 +720,12 @@ ptc_status reuse_by_runs(const uint32_t* ids, uint64_t n, uint64_t D, uint32_t* 
   ia.max_tiles = L.rtiles_max;
   ia.max_runs = a.max_runs;
   ia.st = L.st;
+  HostStage* hs = host_stage();
+  ia.st_host = hs->dev ? &hs->dev->st : nullptr;
   const uint32_t g1 = L.rtiles_max < (uint32_t)(2 * num_sms()) ? L.rtiles_max : (uint32_t)(2 * num_sms());
   PTC_KERNEL("k_ir_inc1", s, k_ir_inc1, g1, kIT, 0, ia);
   DevStatus h{};
-  ptc_status rc = end_call(L.st, s, &h);
+  ptc_status rc = ia.st_host ? end_call_staged(s, &h) : end_call(L.st, s, &h);
   if (din) {  // n and D were bounds: the real ones, and stage a2's status, arrive with this wait
     hout->n = h.value[4];
     hout->D = h.value[5];

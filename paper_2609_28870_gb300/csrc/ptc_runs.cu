@@ -784,13 +784,6 @@ struct QueryArgs {
   uint32_t kbase;       // kpre counts this many bits more
 };
 
-// Index of the run holding position j.
-__device__ __forceinline__ uint32_t run_of(const uint32_t* bits, const uint32_t* wpre, uint32_t j) {
-  const uint32_t wi = j >> 5, b = j & 31;
-  const uint32_t mask_le = b == 31 ? kFull : ((2u << b) - 1u);
-  return wpre[wi] + __popc(bits[wi] & mask_le) - 1u;
-}
-
 __global__ void __launch_bounds__(256) k_runs_query(QueryArgs a) {
   grid_dep_sync();
   const uint32_t r = blockIdx.x * blockDim.x + threadIdx.x;
@@ -830,28 +823,17 @@ __global__ void __launch_bounds__(256) k_runs_query(QueryArgs a) {
   a.sd[r] = 1u + partial + cnt;
 }
 
-// kExpPer accesses per thread, kExpThreads apart: each thread's dependent
-// loads (word, then distance) for all of them are in flight together.
-constexpr int kExpThreads = 256;
-constexpr int kExpPer = 8;
+// Up to this many accesses the pipeline leaves the distances to stage d's launch:
+// a launch less, 4 us, but CTAs beside that kernel's registers and shared memory
+// are fewer (9.3M accesses 13 us either way; 304M 295 us alone, 350 there).
+constexpr uint64_t kExpandLate = 1ULL << 24;
 __global__ void __launch_bounds__(kExpThreads) k_runs_expand(const uint32_t* __restrict__ bits,
                                                             const uint32_t* __restrict__ wpre,
                                                             const uint32_t* __restrict__ sd, uint32_t n,
                                                             uint32_t* __restrict__ dist, uint32_t nruns,
                                                             const DevStatus* st) {
   grid_dep_sync();
-  const uint32_t j0 = blockIdx.x * (kExpThreads * kExpPer) + threadIdx.x;
-  uint32_t r[kExpPer];
-#pragma unroll
-  for (int k = 0; k < kExpPer; ++k) {
-    const uint32_t j = j0 + k * kExpThreads;
-    r[k] = j < n ? run_of(bits, wpre, j) : 0u;
-  }
-#pragma unroll
-  for (int k = 0; k < kExpPer; ++k) {
-    const uint32_t j = j0 + k * kExpThreads;
-    if (j < n && in_bounds(st, r[k], nruns)) __stcs(&dist[j], __ldg(&sd[r[k]]));
-  }
+  expand_runs(blockIdx.x, bits, wpre, sd, n, dist, nruns, st);
 }
 
 uint32_t key_bits_n(uint64_t n) {  // keys and thresholds lie in [0, n]
@@ -1058,7 +1040,10 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
     q.kbase = by_pieces ? R32 : 0u;
     PTC_KERNEL("k_runs_query", s, k_runs_query, ceil_div_u32(R, 256), 256, 0, q);
   }
-  PTC_KERNEL("k_runs_expand", s, k_runs_expand, ceil_div_u32(n, kExpThreads * kExpPer), kExpThreads, 0, W.bits, W.wpre, W.sd, (uint32_t)n, dist_out, R32, W.st);
+  const bool late = lent && view && n <= kExpandLate;
+  if (!late)
+    PTC_KERNEL("k_runs_expand", s, k_runs_expand, ceil_div_u32(n, kExpThreads * kExpPer), kExpThreads, 0, W.bits, W.wpre,
+               W.sd, (uint32_t)n, dist_out, R32, W.st);
   const ptc_status done =
       lent ? (cudaGetLastError() == cudaSuccess ? PTC_OK : PTC_ERR_CUDA) : end_call(W.st, s, &h);
   if (done == PTC_OK && view) {
@@ -1068,6 +1053,7 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
     view->sd = W.sd;
     view->bits = W.bits;
     view->wpre = W.wpre;
+    view->dist = late ? dist_out : nullptr;
   }
   return done;
 }
