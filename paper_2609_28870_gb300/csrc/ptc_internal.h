@@ -260,7 +260,8 @@ ptc_status ids_impl(const ptc_u128* keys, uint64_t n_ub, const uint64_t* n_dev, 
 // block, counters, bitmaps and look-back words) it does not wait at its end.
 // With `pieces` (stage b's, in order and tiling the accesses; they live in the
 // same workspace, behind what stage c writes before it is done with them) the
-// runs come from those instead of from prev.
+// runs come from those instead of from prev.  With `runs_only` the distances of the
+// accesses are left out where there are runs (view->used).
 struct StackLent {
   DevStatus* st = nullptr;
   uint32_t* done = nullptr;  // kStackDone counters
@@ -280,7 +281,7 @@ inline size_t stack_key_words(uint64_t n) { return n / 32 + 2; }
 inline size_t stack_lb_words(uint64_t n) { return n / kPieceTile + 2; }
 ptc_status stack_distance_view(const uint32_t* prev, uint64_t n, uint32_t* dist_out, int method, void* ws,
                                size_t ws_bytes, cudaStream_t s, RunsView* view, const StackLent* lent,
-                               const ReusePieces& pieces);
+                               const ReusePieces& pieces, bool runs_only = false);
 // Stage b as ptc_reuse_indices does it (ptc_reuse.cu); with `lent` (its zeroed
 // status block, counters and cut bitmap) it does not wait at its end.  With
 // `din`, stage a2 has not waited: n and n_distinct are upper bounds, the kernels

@@ -925,7 +925,7 @@ uint64_t runs_reserve(uint64_t n) {
 
 ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_out, void* ws, size_t ws_bytes,
                                cudaStream_t s, int method, RunsView* view, const StackLent* lent = nullptr,
-                               const ReusePieces& pieces = ReusePieces{}) {
+                               const ReusePieces& pieces = ReusePieces{}, bool runs_only = false) {
   const RunsLayout M = runs_layout(ws, n, 1, lent);
   if (!ws_ok(ws, ws_bytes, M.total)) return PTC_ERR_WORKSPACE;
   if (!lent && begin_call(ws, M.zero_bytes, s) != PTC_OK) return PTC_ERR_CUDA;
@@ -1041,7 +1041,7 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
     PTC_KERNEL("k_runs_query", s, k_runs_query, ceil_div_u32(R, 256), 256, 0, q);
   }
   const bool late = lent && view && n <= kExpandLate;
-  if (!late)
+  if (!late && !runs_only)
     PTC_KERNEL("k_runs_expand", s, k_runs_expand, ceil_div_u32(n, kExpThreads * kExpPer), kExpThreads, 0, W.bits, W.wpre,
                W.sd, (uint32_t)n, dist_out, R32, W.st);
   const ptc_status done =
@@ -1053,7 +1053,7 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
     view->sd = W.sd;
     view->bits = W.bits;
     view->wpre = W.wpre;
-    view->dist = late ? dist_out : nullptr;
+    view->dist = late && !runs_only ? dist_out : nullptr;
   }
   return done;
 }
@@ -1062,13 +1062,13 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
 
 ptc_status stack_distance_view(const uint32_t* prev, uint64_t n, uint32_t* dist_out, int method, void* ws,
                                size_t ws_bytes, cudaStream_t s, RunsView* view, const StackLent* lent,
-                               const ReusePieces& pieces) {
+                               const ReusePieces& pieces, bool runs_only) {
   *view = RunsView{};
   if (n >= (uint64_t)kNone) return PTC_ERR_OVERFLOW;
   if (n == 0) return PTC_OK;
   if (!prev || !dist_out) return PTC_ERR_INVALID_ARG;
   if (method == PTC_SD_POINTS) return stack_distance_points(prev, n, dist_out, ws, ws_bytes, s);
-  return stack_distance_runs(prev, n, dist_out, ws, ws_bytes, s, method, view, lent, pieces);
+  return stack_distance_runs(prev, n, dist_out, ws, ws_bytes, s, method, view, lent, pieces, runs_only);
 }
 
 }  // namespace ptc

@@ -34,8 +34,8 @@
 //   k_var_perm    leaf-first: prev and the window ends in touch order
 //   k_var_heads   per request: run heads of the touch stream (a bitmap)
 //   k_var_rec     per request: each run's start and first prev value
-//   k_var_fix     per request: the count above, off the per-block distance
-//   k_var_unperm  leaf-first: the distances back in depth order
+//   k_var_out     the distances in depth order: from stage c's runs, per request
+//                 less the count above
 #include "ptc_internal.h"
 
 namespace ptc {
@@ -154,7 +154,6 @@ struct RunArgs {
   const unsigned long long* total;
   uint32_t* rec_start;   // R + 1 entries (rec_start[R] = n)
   uint32_t* rec_q;       // first prev value of each run (kNone: a run of first accesses)
-  uint32_t* dist;        // per-block distances in touch order, corrected in place
 };
 
 // A position starts a run if it starts its request, or its prev is not the
@@ -204,61 +203,70 @@ __global__ void __launch_bounds__(kVT) k_var_rec(const __grid_constant__ RunArgs
   if (blockIdx.x == 0 && threadIdx.x == 0) a.rec_start[*a.total] = a.n;
 }
 
-__global__ void __launch_bounds__(kVT) k_var_fix(const __grid_constant__ RunArgs a) {
+// The distances in depth order: of access i, at touch position ip (i itself unless
+// leaf-first), its distance there, from stage c's runs where it used them, and
+// with FIX (per request) less the count of its request's earlier accesses.
+// Bound by latency and L2: one pass where the distances of all touch positions
+// (14 us on 9.3M accesses), the counts (48) and the way back (27) took one each,
+// 60 together.
+struct OutArgs {
+  const uint32_t* req_of;   // leaf-first: request of every access, and the offsets
+  const uint64_t* off;
+  const uint32_t* sd;       // stage c's runs: distance of each, starts as a bitmap with ranks (null: tdist)
+  const uint32_t* bits;
+  const uint32_t* wpre;
+  const uint32_t* tdist;    // distances in touch order
+  uint32_t* dist;
+};
+template <bool LEAF, bool FIX>
+__global__ void __launch_bounds__(kVT) k_var_out(const __grid_constant__ RunArgs a, const __grid_constant__ OutArgs o) {
   grid_dep_sync();
   constexpr int kH = 4;  // positions whose loads are in flight together
 #pragma unroll 1
   for (int half = 0; half < kVPer / kH; ++half) {
     const uint64_t base = (uint64_t)blockIdx.x * kVTile + half * kH * kVT + threadIdx.x;
-    uint32_t p[kH], e[kH], t[kH], st[kH];
+    uint32_t ip[kH], d[kH], p[kH], e[kH], t[kH], st[kH];
 #pragma unroll
     for (int k = 0; k < kH; ++k) {
       const uint64_t i = base + k * kVT;
-      p[k] = i < a.n ? __ldg(a.prev + i) : kNone;
-      e[k] = i < a.n ? __ldg(a.wend + i) : 0u;
-      t[k] = p[k] != kNone ? heads_through(a, (uint32_t)i) - 1 : 0u;
-    }
-#pragma unroll
-    for (int k = 0; k < kH; ++k) st[k] = p[k] != kNone ? a.rec_start[t[k]] : 0u;
-#pragma unroll
-    for (int k = 0; k < kH; ++k) {
-      const uint64_t i = base + k * kVT;
-      if (p[k] == kNone) continue;
-      uint32_t cnt = (uint32_t)i - st[k];  // earlier positions of its own run
-      uint32_t end = st[k];
-      for (uint32_t u = t[k]; u-- > 0;) {  // earlier runs of its request
-        const uint32_t s0 = a.rec_start[u];
-        if (s0 < e[k]) break;
-        const uint32_t len = end - s0, q = a.rec_q[u];
-        cnt += q == kNone ? len : (p[k] > q ? (p[k] - q < len ? p[k] - q : len) : 0u);
-        end = s0;
+      ip[k] = i < a.n ? (uint32_t)i : kNone;
+      if (LEAF && i < a.n) {
+        const uint32_t r = o.req_of[i];
+        const uint64_t lo = __ldg(o.off + r), hi = __ldg(o.off + r + 1);
+        ip[k] = lo <= i && i < hi && hi <= a.n ? (uint32_t)(lo + hi - 1 - i) : kNone;
       }
-      a.dist[i] -= cnt;
     }
-  }
-}
-
-__global__ void __launch_bounds__(kVT) k_var_unperm(const __grid_constant__ VarArgs a) {
-  grid_dep_sync();
-  const uint64_t base = (uint64_t)blockIdx.x * kVTile + threadIdx.x;
-  uint32_t r[kVPer], ip[kVPer], d[kVPer];
 #pragma unroll
-  for (int k = 0; k < kVPer; ++k) {
-    const uint64_t i = base + k * kVT;
-    r[k] = i < a.n ? a.req_of[i] : 0u;
-  }
+    for (int k = 0; k < kH; ++k) {
+      d[k] = ip[k] == kNone ? kNone : o.sd ? run_of(o.bits, o.wpre, ip[k]) : o.tdist[ip[k]];
+      if (FIX) {
+        p[k] = ip[k] != kNone ? __ldg(a.prev + ip[k]) : kNone;
+        e[k] = ip[k] != kNone ? __ldg(a.wend + ip[k]) : 0u;
+        t[k] = p[k] != kNone ? heads_through(a, ip[k]) - 1 : 0u;
+      }
+    }
 #pragma unroll
-  for (int k = 0; k < kVPer; ++k) {
-    const uint64_t i = base + k * kVT;
-    const uint64_t lo = __ldg(a.off + r[k]), hi = __ldg(a.off + r[k] + 1);
-    ip[k] = (i < a.n && lo <= i && i < hi && hi <= a.n) ? (uint32_t)(lo + hi - 1 - i) : kNone;
-  }
+    for (int k = 0; k < kH; ++k) {
+      if (o.sd && ip[k] != kNone) d[k] = __ldg(o.sd + d[k]);
+      if (FIX) st[k] = p[k] != kNone ? a.rec_start[t[k]] : 0u;
+    }
 #pragma unroll
-  for (int k = 0; k < kVPer; ++k) d[k] = ip[k] != kNone ? a.distp[ip[k]] : kNone;
-#pragma unroll
-  for (int k = 0; k < kVPer; ++k) {
-    const uint64_t i = base + k * kVT;
-    if (i < a.n) a.dist[i] = d[k];
+    for (int k = 0; k < kH; ++k) {
+      const uint64_t i = base + k * kVT;
+      if (FIX && p[k] != kNone) {
+        uint32_t cnt = ip[k] - st[k];  // earlier positions of its own run
+        uint32_t end = st[k];
+        for (uint32_t u = t[k]; u-- > 0;) {  // earlier runs of its request
+          const uint32_t s0 = a.rec_start[u];
+          if (s0 < e[k]) break;
+          const uint32_t len = end - s0, q = a.rec_q[u];
+          cnt += q == kNone ? len : (p[k] > q ? (p[k] - q < len ? p[k] - q : len) : 0u);
+          end = s0;
+        }
+        d[k] -= cnt;
+      }
+      if (i < a.n) o.dist[i] = d[k];
+    }
   }
 }
 
@@ -266,6 +274,7 @@ struct VarLayout {
   DevStatus* st;
   uint32_t* done;             // bitmap_ranks' counter
   unsigned long long* heads;  // number of runs
+  StackLent stack;            // for the stack-distance stage: its status block is st
   size_t zero_bytes;
   uint32_t* tile_req;
   uint32_t* req_of;
@@ -285,6 +294,9 @@ VarLayout var_layout(void* ws, uint64_t n, int leaf, int request) {
   L.st = cv.take<DevStatus>(1);
   L.done = cv.take<uint32_t>(1);
   L.heads = cv.take<unsigned long long>(1);
+  L.stack.st = L.st;
+  L.stack.done = cv.take<uint32_t>(kStackDone);
+  L.stack.bits = cv.take<uint32_t>(2 * stack_key_words(n));
   L.zero_bytes = cv.off;
   L.tile_req = cv.take<uint32_t>((n + kVTile - 1) / kVTile + 1);
   L.req_of = leaf ? cv.take<uint32_t>(n) : nullptr;
@@ -349,10 +361,11 @@ extern "C" ptc_status ptc_stack_distance_variant_ex(const uint32_t* prev, uint64
   const uint32_t* tprev = leaf ? L.prevp : prev;  // the touch stream
   uint32_t* tdist = leaf ? L.distp : dist_out;
   ptc_status rc_sd = PTC_OK;
-  bool few_runs = true;
+  bool fix = request;
+  RunsView runs;
+  RunArgs ra{tprev, L.wend, (uint32_t)n, L.bits, L.pre, L.heads, L.rec_start, L.rec_q};
   if (request) {
     // runs of the touch stream, cut at request starts
-    const RunArgs ra{tprev, L.wend, (uint32_t)n, L.bits, L.pre, L.heads, L.rec_start, L.rec_q, tdist};
     PTC_KERNEL("k_var_heads", s, k_var_heads, tiles, kVT, 0, ra);
     if (bitmap_ranks(L.bits, L.nwords, L.pre, L.tcnt, L.tpre, L.done, reinterpret_cast<uint64_t*>(L.heads), s) !=
         PTC_OK)
@@ -360,18 +373,23 @@ extern "C" ptc_status ptc_stack_distance_variant_ex(const uint32_t* prev, uint64
     uint64_t* hv = &host_stage()->out[0];
     if (copy_to_host_async(hv, L.heads, sizeof(uint64_t), s) != PTC_OK) return PTC_ERR_CUDA;
     if (cudaStreamSynchronize(s) != cudaSuccess) return PTC_ERR_CUDA;
-    few_runs = method == PTC_SD_RUNS || (method == PTC_SD_AUTO && *hv <= n / 3);
-    if (few_runs) {
+    fix = method == PTC_SD_RUNS || (method == PTC_SD_AUTO && *hv <= n / 3);
+    if (fix)
       PTC_KERNEL("k_var_rec", s, k_var_rec, tiles, kVT, 0, ra);
-      rc_sd = ptc_stack_distance(tprev, n, tdist, L.sd, L.sd_bytes, s);
-      PTC_KERNEL("k_var_fix", s, k_var_fix, tiles, kVT, 0, ra);
-    } else {
+    else
       rc_sd = stack_distance_points(tprev, n, tdist, L.sd, L.sd_bytes, s, L.wend);
-    }
-  } else {
-    rc_sd = ptc_stack_distance(tprev, n, tdist, L.sd, L.sd_bytes, s);
   }
-  if (leaf) PTC_KERNEL("k_var_unperm", s, k_var_unperm, tiles, kVT, 0, a);
+  if (fix || !request)
+    rc_sd = stack_distance_view(tprev, n, tdist, PTC_SD_AUTO, L.sd, L.sd_bytes, s, &runs, &L.stack, ReusePieces{}, true);
+  const OutArgs oa{L.req_of, req_blk_off, runs.used ? runs.sd : nullptr, runs.bits, runs.wpre, tdist, dist_out};
+  if (rc_sd == PTC_OK) {
+    if (leaf && fix)
+      PTC_KERNEL("k_var_out", s, (k_var_out<true, true>), tiles, kVT, 0, ra, oa);
+    else if (leaf)
+      PTC_KERNEL("k_var_out", s, (k_var_out<true, false>), tiles, kVT, 0, ra, oa);
+    else if (fix)
+      PTC_KERNEL("k_var_out", s, (k_var_out<false, true>), tiles, kVT, 0, ra, oa);
+  }
   DevStatus h;
   const ptc_status rc = end_call(L.st, s, &h);
   return rc != PTC_OK ? rc : rc_sd;
