@@ -49,9 +49,10 @@
 // per capacity, 32 accesses a step and owners read from DRAM as they came; 116
 // ms with 128 accesses a step and the ids read ahead; 55 ms with the epochs read
 // together and the check for repeats made once; 41 ms with 16 warps and one
-// barrier per eviction (43.9 without the owners read ahead).  The smallest
-// capacities take longest: they evict in every window (40.7 ms for 64 blocks,
-// 20.3 for 1.6M).
+// barrier per eviction (43.9 without the owners read ahead); 36.6 ms with windows
+// that start where the last one or its request ended (37.3 with two accesses per
+// lane, 1,024 to a window).  The smallest capacities take longest: they evict in
+// every window (36.2 ms for 64 blocks, 18.0 for 1.6M).
 #include "ptc_internal.h"
 
 namespace ptc {
@@ -288,12 +289,13 @@ __global__ void __launch_bounds__(kSesThreads, 1) k_ses_sim(SesArgs a, SesCaps c
     const uint64_t t0 = (uint64_t)t * kSesBatch;
     const uint32_t size = n - t0 < kSesBatch ? (uint32_t)(n - t0) : kSesBatch;
     uint32_t at = 0;  // accesses of this batch settled
-    // The window in registers: this lane's id and owner word (of the whole
-    // window, whichever requests it meets), read again after a step that stored
-    // owners.  The next window's are read while this one's misses are counted.
-    uint32_t cur = kNone, id = 0, next_id = 0;
-    uint64_t o = kNoOwner, next_o = kNoOwner;
-    bool stale = false, ready = false;
+    // The window in registers: this lane's id and owner word.  The next window's
+    // are read while this one's misses are counted, the owners again after a step
+    // that stored some.
+    uint32_t next_id = 0;
+    uint64_t next_o = kNoOwner;
+    bool ready = false, stale = false;
+    auto read_id = [&](uint32_t k) { return ids[k < size ? k : size - 1]; };
     while (at < size) {
       if (t0 + at >= e) {  // the next request with accesses (those without only touch their sessions)
         uint32_t next_s = s;
@@ -320,8 +322,7 @@ __global__ void __launch_bounds__(kSesThreads, 1) k_ses_sim(SesArgs a, SesCaps c
         missed = false;
       }
       if (t0 + at >= e) break;
-      const uint32_t w0 = at & ~(kSesWin - 1);  // this window of the batch
-      const uint32_t lo = at - w0;
+      const uint32_t w0 = at;  // the window: up to kSesWin accesses of the request from here
       uint32_t hi = size - w0 < kSesWin ? size - w0 : kSesWin;
       if (e - (t0 + w0) < hi) hi = (uint32_t)(e - (t0 + w0));
       const uint64_t depth = t0 + at - b;
@@ -331,10 +332,10 @@ __global__ void __launch_bounds__(kSesThreads, 1) k_ses_sim(SesArgs a, SesCaps c
         replay_sync();  // the request's state is written
         if (warp == 0) {
           uint64_t d0 = depth;
-          for (uint32_t c = lo & ~31u; c < hi; c += 32) {
+          for (uint32_t c = 0; c < hi; c += 32) {
             const uint32_t k = c + lane;
-            const uint32_t x = ids[w0 + k];
-            uint32_t pending = __ballot_sync(kFull, k >= lo && k < hi);
+            const uint32_t x = read_id(w0 + k);
+            uint32_t pending = __ballot_sync(kFull, k < hi);
             while (pending) {
               const bool mine = (pending >> lane) & 1u;
               const bool res = ses_resident(a, S, mine ? owner[x] : kNoOwner);
@@ -408,35 +409,29 @@ __global__ void __launch_bounds__(kSesThreads, 1) k_ses_sim(SesArgs a, SesCaps c
         continue;
       }
       const uint32_t k = 32 * warp + lane;
-      const bool valid = k >= lo && k < hi;
-      if (cur != w0) {
-        id = ready ? next_id : ids[w0 + k];
-        o = ready ? next_o : w0 + k < size ? owner[id] : kNoOwner;
-        cur = w0;
-      } else if (stale) {
-        o = w0 + k < size ? owner[id] : kNoOwner;
-      }
+      const bool valid = k < hi;
+      const uint32_t id = ready ? next_id : read_id(w0 + k);
+      const uint64_t o = ready && !stale ? next_o : w0 + k < size ? owner[id] : kNoOwner;
       bool miss = valid && !ses_resident(a, S, o);
-      ready = w0 + hi < size && hi == kSesWin;
+      ready = at < size;
       if (ready) {
-        next_id = ids[w0 + kSesWin + k];
-        next_o = w0 + kSesWin + k < size ? owner[next_id] : kNoOwner;
+        next_id = read_id(at + k);
+        next_o = at + k < size ? owner[next_id] : kNoOwner;
       }
       uint32_t all = ses_count(miss, ring.slots[turn ^= 1], warp, lane);
       stale = all != 0;
       if (all == 0) {
         if (!missed) {
-          const uint32_t f = hi - lo;
+          const uint32_t f = hi;
           hits += f;
           depths += (uint64_t)f * depth + (uint64_t)f * (f - 1) / 2;
         }
         continue;
       }
-      ready = false;
       if (!missed) {  // the hits before the first miss
         const uint32_t mask = lane < kSesReplay ? ring.slots[turn][lane] : 0u;
         const uint32_t fw = __ffs(__ballot_sync(kFull, mask != 0)) - 1;
-        const uint32_t f = 32 * fw + __ffs(__shfl_sync(kFull, mask, fw)) - 1 - lo;
+        const uint32_t f = 32 * fw + __ffs(__shfl_sync(kFull, mask, fw)) - 1;
         hits += f;
         depths += (uint64_t)f * depth + (uint64_t)f * (f ? f - 1 : 0) / 2;
         missed = true;
