@@ -57,9 +57,9 @@ NOMINAL_HBM_GBS = 7900.0
 # sha256 prefix of the source file it was taken on (a changed source reads as
 # "no counters", null) and how the capture was scaled to a full launch.
 NCU_TRAFFIC: dict[tuple[str, int], tuple[float, str, str]] = {
-    ("k_hash16", 1): (6.3766e+08, "d33ef0cf44921375", "ncu dram__bytes metrics, first 6,000 requests, x 153.81 / 55.67"),
-    ("k_hash16", 3): (4.9715e+10, "d33ef0cf44921375", "ncu dram__bytes metrics, first 60,000 requests: reads x tokens "
-                      "(9984.4M / 943.9M), key writes x blocks (623.75M / 58.97M)"),
+    ("k_hash_units", 1): (6.3741e+08, "2276413f5518ab07", "ncu dram__bytes metrics, first 6,000 requests, x 153.81 / 55.67"),
+    ("k_hash_units", 3): (5.0614e+10, "2276413f5518ab07", "ncu dram__bytes metrics, first 60,000 requests: reads x tokens "
+                          "(9984.4M / 943.9M), key writes x blocks (623.75M / 58.97M)"),
 }
 
 
@@ -189,24 +189,35 @@ def kernel_model_bytes(name, T, N, L, D, U=None):
 
 
 KERNEL_SOURCE = {
-    "k_block_offsets": "ptc_hash.cu", "k_pow_tables": "ptc_hash.cu", "k_hash_local": "ptc_hash.cu",
-    "k_hash16": "ptc_hash.cu", "k_hash_units": "ptc_hash.cu", "k_fill_many": "ptc_abi.cu",
-    "k_hash_chain": "ptc_hash.cu", "k_ids_insert": "ptc_ids.cu",
-    "k_ids_gather": "ptc_ids.cu", "k_ids_insert_prior": "ptc_ids.cu", "k_ids_follow": "ptc_ids.cu",
-    "k_tile_req": "ptc_ids.cu", "k_ids_lam": "ptc_ids.cu", "k_session_prior": "ptc_ids.cu", "k_sort_count": "ptc_sort.cu", "k_sort_rowscan": "ptc_sort.cu",
-    "k_sort_scatter": "ptc_sort.cu", "k_sort_links": "ptc_sort.cu", "k_ir_count": "ptc_reuse.cu",
-    "k_ir_mark": "ptc_reuse.cu", "k_bm_count": "ptc_reuse.cu", "k_bm_words": "ptc_reuse.cu",
-    "k_ir_inc1": "ptc_reuse.cu", "k_ir_inc2": "ptc_reuse.cu", "k_ir_fill": "ptc_reuse.cu", "k_wm_count0": "ptc_wavelet.cu",
-    "k_wm_level": "ptc_wavelet.cu", "k_wm_dir": "ptc_wavelet.cu", "k_wm_heads": "ptc_wavelet.cu",
-    "k_wm_propagate": "ptc_wavelet.cu", "k_runs_mark": "ptc_runs.cu", "k_runs_count": "ptc_runs.cu", "k_runs_init": "ptc_runs.cu",
-    "k_runs_level": "ptc_runs.cu", "k_runs_build_cluster": "ptc_runs.cu", "k_runs_query": "ptc_runs.cu", "k_runs_expand": "ptc_runs.cu", "k_heads": "ptc_curves.cu", "k_curves_agg": "ptc_curves.cu",
-    "k_curves": "ptc_curves.cu", "k_finalize": "ptc_curves.cu", "k_curves_fast": "ptc_curves.cu",
-    "k_curves_runs": "ptc_curves.cu", "k_fill": "ptc_abi.cu", "k_copy_words": "ptc_abi.cu",
-    "k_copy_err": "ptc_abi.cu", "k_carry_err": "ptc_abi.cu", "k_hash_carry": "ptc_hash.cu",
-    "k_rank_count": "ptc_abi.cu", "k_rank_words": "ptc_abi.cu", "k_pd_flags": "ptc_ids.cu",
-    "k_pd_count": "ptc_ids.cu", "k_pd_rows1": "ptc_ids.cu", "k_pd_scatter1": "ptc_ids.cu",
-    "k_pd_count2": "ptc_ids.cu", "k_pd_rows2": "ptc_ids.cu", "k_pd_scatter2": "ptc_ids.cu", "k_pd_dedup": "ptc_ids.cu",
-    "k_pd_dedup_large": "ptc_ids.cu", "k_pd_dedup_big": "ptc_ids.cu",
+    "k_copy_words": "ptc_abi.cu", "k_fill": "ptc_abi.cu", "k_fill_many": "ptc_abi.cu", "k_rank_count": "ptc_abi.cu",
+    "k_rank_one": "ptc_abi.cu", "k_rank_words": "ptc_abi.cu", "k_bel_heads": "ptc_belady.cu",
+    "k_bel_records": "ptc_belady.cu", "k_bel_reqs": "ptc_belady.cu", "k_bel_sim": "ptc_belady.cu",
+    "k_cnt_bucket": "ptc_count.cu", "k_cnt_next": "ptc_count.cu", "k_cnt_out": "ptc_count.cu",
+    "k_cnt_rank": "ptc_count.cu", "k_cnt_rows": "ptc_count.cu", "k_cnt_scatter": "ptc_count.cu",
+    "k_curves": "ptc_curves.cu", "k_curves_agg": "ptc_curves.cu", "k_curves_fast": "ptc_curves.cu",
+    "k_curves_runs": "ptc_curves.cu", "k_finalize": "ptc_curves.cu", "k_heads": "ptc_curves.cu",
+    "k_block_offsets": "ptc_hash.cu", "k_hash_carry": "ptc_hash.cu", "k_hash_chain": "ptc_hash.cu",
+    "k_hash_local": "ptc_hash.cu", "k_hash_units": "ptc_hash.cu", "k_ids_follow": "ptc_ids.cu",
+    "k_ids_gather": "ptc_ids.cu", "k_ids_insert": "ptc_ids.cu", "k_ids_insert_prior": "ptc_ids.cu",
+    "k_ids_lam": "ptc_ids.cu", "k_pd_count": "ptc_ids.cu", "k_pd_count2": "ptc_ids.cu", "k_pd_dedup": "ptc_ids.cu",
+    "k_pd_dedup_big": "ptc_ids.cu", "k_pd_dedup_large": "ptc_ids.cu", "k_pd_flags": "ptc_ids.cu",
+    "k_pd_rows1": "ptc_ids.cu", "k_pd_rows2": "ptc_ids.cu", "k_pd_scatter1": "ptc_ids.cu",
+    "k_pd_scatter2": "ptc_ids.cu", "k_session_prior": "ptc_ids.cu", "k_tile_req": "ptc_ids.cu",
+    "k_verify": "ptc_ids.cu", "k_verify_first": "ptc_ids.cu", "k_probe_rmw": "ptc_probe.cu",
+    "k_bm_count": "ptc_reuse.cu", "k_bm_one": "ptc_reuse.cu", "k_bm_words": "ptc_reuse.cu",
+    "k_ir_count": "ptc_reuse.cu", "k_ir_fill": "ptc_reuse.cu", "k_ir_inc1": "ptc_reuse.cu",
+    "k_ir_inc2": "ptc_reuse.cu", "k_ir_links": "ptc_reuse.cu", "k_ir_mark": "ptc_reuse.cu",
+    "k_dom_out": "ptc_runs.cu", "k_dom_rank": "ptc_runs.cu", "k_dom_time": "ptc_runs.cu",
+    "k_runs_count": "ptc_runs.cu", "k_runs_expand": "ptc_runs.cu", "k_runs_init": "ptc_runs.cu",
+    "k_runs_level": "ptc_runs.cu", "k_runs_mark": "ptc_runs.cu", "k_runs_pieces": "ptc_runs.cu",
+    "k_runs_query": "ptc_runs.cu", "k_ses_check": "ptc_session.cu", "k_ses_sim": "ptc_session.cu",
+    "k_sort_count": "ptc_sort.cu", "k_sort_links": "ptc_sort.cu", "k_sort_one": "ptc_sort.cu",
+    "k_sort_rowscan": "ptc_sort.cu", "k_sort_scatter": "ptc_sort.cu", "k_st_access": "ptc_stats.cu",
+    "k_st_blocks": "ptc_stats.cu", "k_st_req": "ptc_stats.cu", "k_st_reuse": "ptc_stats.cu",
+    "k_var_heads": "ptc_variant.cu", "k_var_out": "ptc_variant.cu", "k_var_perm": "ptc_variant.cu",
+    "k_var_rec": "ptc_variant.cu", "k_var_reqof": "ptc_variant.cu", "k_var_tiles": "ptc_variant.cu",
+    "k_wm_count0": "ptc_wavelet.cu", "k_wm_dir": "ptc_wavelet.cu", "k_wm_heads": "ptc_wavelet.cu",
+    "k_wm_level": "ptc_wavelet.cu", "k_wm_propagate": "ptc_wavelet.cu",
 }
 
 
@@ -829,7 +840,7 @@ def chat_extras(args, ptc, tracegen, dev, timer, slowest, peak, peak_kind, rank,
         ids_t, D, rbo, ses_t, tr.n_sessions, BLOCK, caps, ws=sws)))) / args.steps
     del sws
     out["session_eviction"] = {
-        "call": "ptc_session_lru_curves on the step's ids: session-level LRU at every grid capacity, one warp per "
+        "call": "ptc_session_lru_curves on the step's ids: session-level LRU at every grid capacity, one CTA per "
                 "capacity", "ms": round(ses_ms, 3),
         "hit_ratio_at": {str(int(caps[g])): round(sesc["hits"][g] / N, 5) for g in mid},
         "block_level_hit_ratio_at": {str(int(caps[g])): round(int(plan.hits[g]) / N, 5) for g in mid}}

@@ -266,8 +266,8 @@ ptc_status ptc_reuse_indices_ex(const uint32_t* ids, uint64_t n, uint64_t n_dist
  *               = 1 + #{ j : p < j < i, prev[j] < p or prev[j] == PTC_NONE }
  * and PTC_NONE (never seen) when p == PTC_NONE.  An access hits in an LRU
  * cache of C >= 1 blocks iff dist <= C (Mattson et al. 1970).  The count is a
- * 2-D dominance count answered by N range-rank queries on a wavelet matrix
- * (Claude, Navarro, Ordonez 2015) built over v_j = prev[j] + 1.
+ * 2-D dominance count over v_j = prev[j] + 1, made over runs of re-reads where
+ * there are such runs and over every access otherwise.
  *
  *   prev      u32[n] from ptc_reuse_indices (prev[i] < i or PTC_NONE)
  *   dist_out  u32[n], 1-based; PTC_NONE for a first access
@@ -277,18 +277,21 @@ ptc_status ptc_stack_distance(const uint32_t* prev, uint64_t n, uint32_t* dist_o
                               void* stream);
 
 /*
- * ptc_stack_distance_ex — the same distances with the matrix chosen by the
- * caller.  PTC_SD_POINTS builds the wavelet matrix over every access.
- * PTC_SD_RUNS builds it over runs: maximal stretches where prev grows by one
- * from access to access, or that are all first accesses.  A run is either
- * wholly counted or wholly left out of every window (an access has at most
- * one next use), so a matrix over runs weighted by their lengths gives the
- * same counts with R points instead of n.  PTC_SD_AUTO (what
- * ptc_stack_distance does) finds the runs first and takes the matrix over
- * runs when R <= n / 3 and the workspace holds it, else the one over accesses.
+ * ptc_stack_distance_ex — the same distances with the method chosen by the
+ * caller.  PTC_SD_POINTS answers N range-rank queries on a wavelet matrix
+ * (Claude, Navarro, Ordonez 2015) over every access.  PTC_SD_RUNS counts over
+ * runs: maximal stretches where prev grows by one from access to access, or
+ * that are all first accesses.  A run is either wholly counted or wholly left
+ * out of every window (an access has at most one next use), so the R runs
+ * weighted by their lengths give the same counts as the n accesses (by blocks
+ * of pair sums up to 2^21 runs, on a weighted wavelet matrix above).
+ * PTC_SD_AUTO (what ptc_stack_distance does) finds the runs first and counts
+ * over them when R <= n / 3 and the workspace holds them, else over the
+ * accesses: in buckets of values for n up to about 33.5M, and on the matrix of
+ * PTC_SD_POINTS above.
  *   prev must come from ptc_reuse_indices, or at least satisfy prev[i] < i and
- *   take each value other than PTC_NONE at most once; the matrix over runs
- *   relies on the latter, and neither checks it.
+ *   take each value other than PTC_NONE at most once; the runs rely on the
+ *   latter, and nothing checks it.
  * Workspace: ptc_stack_distance_ex_workspace_bytes(n, method);
  * PTC_ERR_WORKSPACE when PTC_SD_RUNS finds more runs than the workspace holds.
  */
