@@ -1225,17 +1225,17 @@ __device__ __forceinline__ bool pd_flow(const PdDedup& a, ulonglong2* rec, uint3
   __syncthreads();
   uint32_t spare = kNone;  // a place taken but not used yet
   bool full = false;
-  auto load = [&](ulonglong2(&v)[kPdFlowPer], uint32_t c) {
+  auto load = [&](ulonglong2(&v)[kPdFlowPer], uint64_t c) {
 #pragma unroll
     for (int q = 0; q < kPdFlowPer; ++q) {
-      const uint32_t k = c + q * T + threadIdx.x;
-      v[q] = k < e && k >= c ? __ldcg(&a.rec2[k]) : make_ulonglong2(~0ULL, ~0ULL);
+      const uint64_t k = c + q * T + threadIdx.x;
+      v[q] = k < e ? __ldcg(&a.rec2[k]) : make_ulonglong2(~0ULL, ~0ULL);
     }
   };
   ulonglong2 v[kPdFlowPer], w[kPdFlowPer];
   load(v, b);
-  for (uint32_t c = b; c < e; c += kChunk) {
-    load(w, c + kChunk < e ? c + kChunk : e);
+  for (uint64_t c = b; c < e; c += kChunk) {
+    load(w, c + kChunk);
 #pragma unroll
     for (int q = 0; q < kPdFlowPer; ++q) {
       const uint64_t x = v[q].x;
@@ -1272,8 +1272,8 @@ __device__ __forceinline__ bool pd_flow(const PdDedup& a, ulonglong2* rec, uint3
     if (__syncthreads_or(full)) return false;
   }
   load(v, b);
-  for (uint32_t c = b; c < e; c += kChunk) {
-    load(w, c + kChunk < e ? c + kChunk : e);
+  for (uint64_t c = b; c < e; c += kChunk) {
+    load(w, c + kChunk);
 #pragma unroll
     for (int q = 0; q < kPdFlowPer; ++q) {
       const uint64_t x = v[q].x;

@@ -37,7 +37,8 @@
 //                  (both with 16-byte loads, four accesses per lane and
 //                  round, when prev is 16-byte aligned: k_runs_count4,
 //                  k_runs_mark4)
-//   bitmap_ranks   the runs' keys (marked by k_runs_mark in a bitmap over
+//   k_runs_pieces  (ptc_pipeline) the same from stage b's pieces, in one launch
+//   bitmap_ranks   the runs' keys (marked in a bitmap over
 //                  [0, n]) counted per word: the matrix holds each key's rank
 //                  among the distinct keys, so it has ceil(log2(R + 2))
 //                  levels instead of ceil(log2(n + 1)), and a query's

@@ -1,7 +1,8 @@
 """The pipeline's stage c from stage b's pieces, against the separate call (whose
 stage c reads prev), and stage b against the uses by definition: numbers of
 pieces around a tile, below and above the bound up to which the pipeline does not
-wait for the number of runs; pieces that start where a tile of accesses does."""
+wait for the number of runs, and more runs than are counted by blocks; pieces
+that start where a tile of accesses does."""
 import numpy as np
 import pytest
 
@@ -17,7 +18,7 @@ def _gpu():
     ptc.lib()
 
 
-@pytest.mark.parametrize("n_req", [1, 2, 300, 2047, 2048, 2049, 30000, 600000, 1300000])
+@pytest.mark.parametrize("n_req", [1, 2, 300, 2047, 2048, 2049, 30000, 600000, 1300000, 2900000])
 @pytest.mark.parametrize("follow", [0.0, 0.7])
 def test_pieces(n_req, follow):
     """Requests of eight one-token blocks each re-read a document whole, now and
