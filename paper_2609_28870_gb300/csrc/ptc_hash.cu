@@ -282,15 +282,16 @@ __device__ __forceinline__ void unit_sum_2(const uint32_t (&wd)[NW], const HashC
   }
 }
 
-// Congruent to (a0 + a1 2^31) mod p and below 2^61 + 3, for a0, a1 < 2^62.
+// Congruent to (a0 + a1 2^31) mod p and below 2^62 + 2^61 + 2^31, for a0 < 2^62
+// and a1 < 2^61 (sums of 16 products of a token below 2^27 and a 31- or 30-bit
+// limb).
 __device__ __forceinline__ uint64_t limbs2_lazy(uint64_t a0, uint64_t a1) {
-  const uint64_t x = (a0 & kP61) + (a0 >> 61) + ((a1 & ((1ULL << 30) - 1)) << 31) + (a1 >> 30);  // < 2^62 + 2^33
-  return (x & kP61) + (x >> 61);
+  return a0 + ((a1 & ((1ULL << 30) - 1)) << 31) + (a1 >> 30);
 }
 
-// a b mod p, reduced only below 2^61 + 5, for a < 2^63 and b < p: the
-// product is below 2^124, so hi << 3 < 2^63 and the first sum stays below
-// 2^63 + 2^61 + 8.
+// a b mod p, reduced only below 2^61 + 8, for a < 2^63 + 2^33 and b < p: the
+// product is below 2^124 + 2^94, so hi << 3 < 2^63 + 2^33 and the first sum stays
+// below 2^64.
 __device__ __forceinline__ uint64_t p61_mul_lazy(uint64_t a, uint64_t b) {
   const uint64_t lo = a * b, hi = __umul64hi(a, b);
   const uint64_t r = (lo & kP61) + (lo >> 61) + (hi << 3);
@@ -526,16 +527,21 @@ __global__ void __launch_bounds__(kHashThreads) k_hash_local(HashArgs a, const _
 // each of 256 threads one block and ran a warp scan, a scan over the warps and
 // the exchange of request starts for every block, with four CTA barriers: 562
 // instructions a block, of which the products are 64.
-// Measured (keys and tokens over the time; the form before in brackets): 844
-// us or 4.5 TB/s on 763M tokens of the agentic trace [3.7 TB/s on the whole
-// one], 186 us on the chat trace [214], 776 us on 724M tokens in blocks of 64
-// that start at an odd word [1,675], 87 us on 55M tokens in blocks of 24 [223].
+// Measured (keys and tokens over the time; the form before in brackets): 753
+// us or 5.1 TB/s on 763M tokens of the agentic trace [3.7 TB/s on the whole
+// one], 168 us on the chat trace [214], 696 us on 724M tokens in blocks of 64
+// that start at an odd word [1,675], 79 us on 55M tokens in blocks of 24 [223].
+// It pays for every instruction of a round: 844 us with the limb sums folded
+// before the multiplication, bounds tested per lane, lanes past the tile's end
+// masked and 64-bit slot and power addresses.
 // At 64 registers 32 warps an SM are half the latency hiding the loads want;
-// five or six CTAs' worth of warps with spills took 7 and 30% longer, and a
-// separate path for tiles inside one request (a quarter fewer instructions,
-// the next round's tokens loaded ahead) took as long on the agentic trace and a
-// third longer on the chat trace, where both paths' code competes for the
-// instruction cache.
+// five or six CTAs' worth of warps with spills took 7 and 30% longer, 22 warps
+// with the tokens staged in shared memory a round ahead 30%, the products on the
+// tensor cores (exact, as byte products) 36 to 47% (the bookkeeping around them
+// is more), and a separate path for tiles inside one request (a quarter fewer
+// instructions, the next round's tokens loaded ahead) as long on the agentic
+// trace and a third longer on the chat trace, where both paths' code competes for
+// the instruction cache.
 constexpr uint32_t kUnitTile = 256;                            // units per tile at most
 constexpr uint32_t kUnitWarps = 2;  // per CTA: small, so that few tiles still spread over the SMs
 constexpr uint32_t kUnitThreads = 32 * kUnitWarps;
@@ -549,7 +555,7 @@ __device__ __forceinline__ uint64_t p61_canon(uint64_t x) {
 }
 __device__ __forceinline__ uint64_t p61_part(uint64_t x) { return (x & kP61) + (x >> 61); }
 
-// h of a unit whose first token is word M of wd: below 2^62 + 3.
+// h of a unit whose first token is word M of wd: below 2^63 + 2^32.
 template <int U, int M, bool WIDE, int NW>
 __device__ __forceinline__ void unit_hash(const uint32_t (&wd)[NW], const HashConsts& c, uint64_t& h0, uint64_t& h1) {
   if (WIDE) {
@@ -571,13 +577,14 @@ __device__ __forceinline__ int64_t shfl_i64(int64_t v, uint32_t src) {
 
 // The sums of a tile: slot[v] (units' values below 2^61 + 8) becomes the
 // canonical sum of the values since the last request start.  `mine` are the
-// starts among this lane's eight units, `opens` the lanes that have one.
-__device__ __forceinline__ void unit_sums(ulonglong2* slot, uint32_t lane, uint32_t mine, uint32_t opens, bool in) {
+// starts among this lane's eight units, `opens` the lanes that have one.  (Slots
+// past the tile's last unit hold anything: sums only reach later units.)
+__device__ __forceinline__ void unit_sums(ulonglong2* slot, uint32_t lane, uint32_t mine, uint32_t opens) {
   uint64_t p0[8], p1[8];
   uint64_t s0 = 0, s1 = 0;
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
-    const ulonglong2 t = in ? slot[9 * lane + j] : make_ulonglong2(0, 0);
+    const ulonglong2 t = slot[9 * lane + j];
     if ((mine >> j) & 1u) s0 = s1 = 0;
     s0 += t.x;
     s1 += t.y;
@@ -612,7 +619,7 @@ __device__ __forceinline__ void unit_sums(ulonglong2* slot, uint32_t lane, uint3
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     if ((mine >> j) & 1u) c0 = c1 = 0;  // the carry ends at the lane's first start
-    if (in) slot[9 * lane + j] = make_ulonglong2(p61_canon(p0[j] + c0), p61_canon(p1[j] + c1));
+    slot[9 * lane + j] = make_ulonglong2(p61_canon(p0[j] + c0), p61_canon(p1[j] + c1));
   }
 }
 
@@ -650,11 +657,13 @@ __device__ __forceinline__ bool hash_units_tile(const HashArgs& a, const HashCon
   window();
   const bool one = r_first == r_last;
   bool big = false;
+  ulonglong2* out = slot + unit_slot(lane);
 #pragma unroll 1
   for (uint32_t v0 = 0; v0 < nu; v0 += 32) {
     const uint32_t v = v0 + lane;
     const bool live = v < nu;
-    int64_t e = e0, x = x0;  // of this lane's unit
+    const uint32_t vc = live ? v : nu - 1;  // a lane past the tile does its last unit again, which nobody reads
+    int64_t e = e0, x = x0;                 // of this lane's unit
     if (!one) {
       const uint32_t last = nu - v0 < 32 ? nu - 1 : v0 + 31;
       if (past <= (int64_t)last) {  // move the window to the request of this round's first unit
@@ -667,40 +676,47 @@ __device__ __forceinline__ bool hash_units_tile(const HashArgs& a, const HashCon
         for (uint32_t i = 1; i < wn; ++i) {
           const int64_t st = -shfl_i64(e0, i);
           if (st > (int64_t)last) break;
-          if (st <= (int64_t)v) idx = i;
+          if (st <= (int64_t)vc) idx = i;
         }
         e = shfl_i64(e0, idx);
         x = shfl_i64(x0, idx);
-      } else if (live) {  // more requests than the window holds (many without blocks)
-        const uint32_t r = find_request(a.blk_off, rw, r_last, b0 + v / a.g);
+      } else {  // more requests than the window holds (many without blocks)
+        const uint32_t r = find_request(a.blk_off, rw, r_last, b0 + vc / a.g);
         e = ((int64_t)b0 - (int64_t)a.blk_off[r]) * (int64_t)a.g;
         x = (int64_t)(a.tok_off[r] + mis) + U * e;
       }
     }
-    e += v;
-    x += (int64_t)U * v;
+    e += vc;
+    x += (int64_t)U * vc;
     const uint32_t st = __ballot_sync(kFull, live && e == 0);  // units that open a request
     if (lane == 0) starts[v0 >> 5] = st;
     // its words: NV aligned vectors, and for a unit that starts m words into
     // the first the next vector's m words, which the next lane holds if its
     // unit follows on
     const uint32_t m = (uint32_t)x & 3u;
-    const uint64_t x4 = (uint64_t)x - m;
-    const bool whole = live && x4 >= mis && x4 + U <= n_word;
-    const uint32_t full = __ballot_sync(kFull, whole);
-    const bool follows = lane < 31 && ((full & ~st) >> (lane + 1)) & 1u;  // the next lane has the next vector
+    const uint64_t x4 = (uint64_t)x & ~3ULL;
+    const bool follows = lane < 31 && v + 1 < nu && !((st >> (lane + 1)) & 1u);  // the next lane has the next vector
+    // A request with blocks ends at or before the array's end, and so do the
+    // unit's NV vectors; the first may begin before the array if that does not
+    // begin on a boundary itself.
+    bool inside = true;
+    if (mis) inside = __all_sync(kFull, x4 != 0);
     uint32_t wd[U + 4];
     uint4 nx = make_uint4(0, 0, 0, 0);
+    if (inside) {
 #pragma unroll
-    for (int q = 0; q < NV; ++q) {
-      uint4 t = make_uint4(0, 0, 0, 0);
-      if (whole) t = __ldcs(reinterpret_cast<const uint4*>(base + x4) + q);
-      wd[4 * q] = t.x;
-      wd[4 * q + 1] = t.y;
-      wd[4 * q + 2] = t.z;
-      wd[4 * q + 3] = t.w;
+      for (int q = 0; q < NV; ++q) {
+        const uint4 t = __ldcs(reinterpret_cast<const uint4*>(base + x4) + q);
+        wd[4 * q] = t.x;
+        wd[4 * q + 1] = t.y;
+        wd[4 * q + 2] = t.z;
+        wd[4 * q + 3] = t.w;
+      }
+    } else {
+#pragma unroll
+      for (int q = 0; q < U; ++q) wd[q] = x4 + q >= mis ? base[x4 + q] : 0u;
     }
-    if (live && m != 0 && !follows) {
+    if (m != 0 && !follows) {
       const uint64_t y = x4 + U;
       if (y + 4 <= n_word) {
         nx = __ldcs(reinterpret_cast<const uint4*>(base + y));
@@ -712,14 +728,11 @@ __device__ __forceinline__ bool hash_units_tile(const HashArgs& a, const HashCon
     }
     // the powers go out with the tokens
     const uint64_t* T = a.tables;
-    uint64_t w0 = 0, w1 = 0;
-    if (live) {
-      w0 = pow_at(T + 0 * 65536, T + 1 * 65536, (uint64_t)e);
-      w1 = pow_at(T + 2 * 65536, T + 3 * 65536, (uint64_t)e);
-    }
-    if (live && !whole) {
-#pragma unroll
-      for (int q = 0; q < U; ++q) wd[q] = x4 + q >= mis && x4 + q < n_word ? base[x4 + q] : 0u;
+    const uint32_t e_lo = (uint32_t)e & 0xFFFFu, e_hi = (uint32_t)e >> 16;  // e < 2^32: the tables reach no further
+    uint64_t w0 = __ldg(&T[e_lo]), w1 = __ldg(&T[2 * 65536 + e_lo]);
+    if (e_hi) {
+      w0 = p61_mul(w0, __ldg(&T[65536 + e_hi]));
+      w1 = p61_mul(w1, __ldg(&T[3 * 65536 + e_hi]));
     }
     if (__any_sync(kFull, m != 0)) {
       const uint32_t n0 = __shfl_down_sync(kFull, wd[0], 1), n1 = __shfl_down_sync(kFull, wd[1], 1),
@@ -736,28 +749,23 @@ __device__ __forceinline__ bool hash_units_tile(const HashArgs& a, const HashCon
       for (int q = 0; q < U + 3; ++q) any |= wd[q];
       big |= (any >> 27) != 0;
     }
-    uint64_t g0 = 0, g1 = 0;
-    if (live) {
-      uint64_t h0, h1;
-      switch (m) {
-        case 0: unit_hash<U, 0, WIDE>(wd, c, h0, h1); break;
-        case 1: unit_hash<U, 1, WIDE>(wd, c, h0, h1); break;
-        case 2: unit_hash<U, 2, WIDE>(wd, c, h0, h1); break;
-        default: unit_hash<U, 3, WIDE>(wd, c, h0, h1); break;
-      }
-      g0 = p61_mul_lazy(h0, w0);
-      g1 = p61_mul_lazy(h1, w1);
+    uint64_t h0, h1;
+    switch (m) {
+      case 0: unit_hash<U, 0, WIDE>(wd, c, h0, h1); break;
+      case 1: unit_hash<U, 1, WIDE>(wd, c, h0, h1); break;
+      case 2: unit_hash<U, 2, WIDE>(wd, c, h0, h1); break;
+      default: unit_hash<U, 3, WIDE>(wd, c, h0, h1); break;
     }
-    slot[unit_slot(v)] = make_ulonglong2(g0, g1);
+    *out = make_ulonglong2(p61_mul_lazy(h0, w0), p61_mul_lazy(h1, w1));
+    out += 36;  // unit_slot(v + 32)
   }
   if (!WIDE && __any_sync(kFull, big)) return true;
   __syncwarp();
   // ---- sums: this lane's units 8 lane .. 8 lane + 7 (values below 2^61 + 8)
   const uint32_t rounds = (nu + 31) / 32;
   const uint32_t mine = (lane >> 2) < rounds ? (starts[lane >> 2] >> (8 * (lane & 3))) & 0xFFu : 0u;
-  const bool in = 8 * lane < 32 * rounds;
   const uint32_t opens = __ballot_sync(kFull, mine != 0);
-  unit_sums(slot, lane, mine, opens, in);
+  unit_sums(slot, lane, mine, opens);
   __syncwarp();
   for (uint32_t i = lane; i < nb; i += 32) a.keys[b0 + i] = slot[unit_slot((i + 1) * a.g - 1)];
   // the tile's aggregate for the carry: its last unit's sum since its request's
