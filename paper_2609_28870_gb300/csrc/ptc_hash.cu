@@ -527,21 +527,23 @@ __global__ void __launch_bounds__(kHashThreads) k_hash_local(HashArgs a, const _
 // each of 256 threads one block and ran a warp scan, a scan over the warps and
 // the exchange of request starts for every block, with four CTA barriers: 562
 // instructions a block, of which the products are 64.
-// Measured (keys and tokens over the time; the form before in brackets): 753
-// us or 5.1 TB/s on 763M tokens of the agentic trace [3.7 TB/s on the whole
-// one], 168 us on the chat trace [214], 696 us on 724M tokens in blocks of 64
-// that start at an odd word [1,675], 79 us on 55M tokens in blocks of 24 [223].
+// Measured (keys and tokens over the time; the form before in brackets): 735
+// us or 5.2 TB/s on 763M tokens of the agentic trace [3.7 TB/s on the whole
+// one], 163 us on the chat trace [214], 679 us on 724M tokens in blocks of 64
+// that start at an odd word [1,675], 77 us on 55M tokens in blocks of 24 [223].
 // It pays for every instruction of a round: 844 us with the limb sums folded
 // before the multiplication, bounds tested per lane, lanes past the tile's end
-// masked and 64-bit slot and power addresses.
-// At 64 registers 32 warps an SM are half the latency hiding the loads want;
-// five or six CTAs' worth of warps with spills took 7 and 30% longer, 22 warps
-// with the tokens staged in shared memory a round ahead 30%, the products on the
-// tensor cores (exact, as byte products) 36 to 47% (the bookkeeping around them
-// is more), and a separate path for tiles inside one request (a quarter fewer
-// instructions, the next round's tokens loaded ahead) as long on the agentic
-// trace and a third longer on the chat trace, where both paths' code competes for
-// the instruction cache.
+// masked and 64-bit slot and power addresses, 753 without.  18 CTAs an SM are the
+// best number: 846 us with 12, 790 with 14, 753 with 16, 962 with 20 (48
+// registers) and 1,054 with 21; the sums one word at a time, in half the
+// registers, took 743 with 18 and 959 with 20.  Not kept either: 22 warps with
+// the tokens staged in shared memory a round ahead (30% longer), the products on
+// the tensor cores (exact, as byte products; 36 to 47%: the bookkeeping around
+// them is more), a separate path for tiles inside one request with the next
+// round's tokens loaded ahead (as long on the agentic trace, a third longer on the
+// chat trace, where both paths' code competes for the instruction cache), and the
+// sums without the starts' tests where a tile has none (1.4% less there, 1.8% more
+// on the chat trace).
 constexpr uint32_t kUnitTile = 256;                            // units per tile at most
 constexpr uint32_t kUnitWarps = 2;  // per CTA: small, so that few tiles still spread over the SMs
 constexpr uint32_t kUnitThreads = 32 * kUnitWarps;
@@ -791,7 +793,7 @@ __device__ __noinline__ void hash_units_wide(const HashArgs& a, const HashConsts
 }
 
 template <int U>
-__global__ void __launch_bounds__(kUnitThreads, 16) k_hash_units(const __grid_constant__ HashArgs a,
+__global__ void __launch_bounds__(kUnitThreads, 18) k_hash_units(const __grid_constant__ HashArgs a,
                                                                  const __grid_constant__ HashConsts c) {
   grid_dep_sync();
   __shared__ ulonglong2 s_slot[kUnitWarps][kUnitSlots];
