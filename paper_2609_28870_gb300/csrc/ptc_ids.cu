@@ -625,6 +625,7 @@ constexpr size_t pd_dedup_smem(int threads) {
 // It runs where partitions average at most this many (chance takes hardly any
 // of them past what fits).
 constexpr uint32_t pd_avg(int threads) { return pd_fit(threads) - 512; }
+constexpr uint32_t kPdGroupLog2 = 5;  // at most 32 partitions together: 2,048 groups still fill the GPU
 constexpr int kPdFitS = 512;  // 3,072 records, three CTAs per SM: up to 167.8M accesses to settle
 constexpr int kPdFitL = 768;  // 4,608 records, two CTAs per SM: up to 268.4M
 
@@ -1187,7 +1188,8 @@ struct PdDedup {
 // need no list.  What bounds it is the latency of a partition's steps (copy,
 // probes, barriers), hence three CTAs per SM; and then the repeats' random
 // writes.  Measured with 80M records, 1,220 to a partition: 1,379 us with
-// tables of keys (98 KB, 128-bit CAS, two CTAs per SM), 511 so.  144M, 8M of
+// tables of keys (98 KB, 128-bit CAS, two CTAs per SM), 511 so, 436 with two
+// partitions at a time (21M records, 318 to a partition: 417 one at a time).  144M, 8M of
 // them repeats of a few thousand keys: 2,062 and 1,056, of which the repeats'
 // writes take 320.
 // (Read once: the bitmap and slot_of, which repeats write, stay in L2 longer.)
@@ -1307,13 +1309,19 @@ __global__ void __launch_bounds__(T, CTAS) k_pd_dedup(PdDedup a) {
   __shared__ uint32_t s_places;
   const uint32_t avg = a.base2[kPdParts] / kPdParts;
   if (avg > pd_avg(T) || (T == kPdFitL && avg <= pd_avg(kPdFitS))) return;  // another variant's
+  // Neighbouring partitions that fit together are settled together (their records
+  // follow one another, and keys of different partitions differ anyway): a
+  // partition's steps take their latency however few its records are.
+  uint32_t gl = 0;
+  while (gl < kPdGroupLog2 && avg << (gl + 1) <= pd_avg(T)) ++gl;
+  const uint32_t groups = kPdParts >> gl;
   __shared__ uint32_t s_next;
   uint32_t p = blockIdx.x, b = 0, e = 0;
-  if (p < kPdParts) {
-    b = a.base2[p];
-    e = a.base2[p + 1];
+  if (p < groups) {
+    b = a.base2[p << gl];
+    e = a.base2[(p + 1) << gl];
   }
-  while (p < kPdParts) {
+  while (p < groups) {
     const bool bad = b > e || e > a.cap;  // bounds past the records: malformed
     const uint32_t m = bad ? 0u : e - b;
     const uint32_t ts = 4 * m < 2 * kFit ? 4 * m : 2 * kFit;
@@ -1335,13 +1343,14 @@ __global__ void __launch_bounds__(T, CTAS) k_pd_dedup(PdDedup a) {
     __syncthreads();
     const uint32_t pn = s_next;
     uint32_t bn = 0, en = 0;
-    if (pn < kPdParts) {
-      bn = a.base2[pn];
-      en = a.base2[pn + 1];
+    if (pn < groups) {
+      bn = a.base2[pn << gl];
+      en = a.base2[(pn + 1) << gl];
     }
     if (m > kFit) {
-      if (!pd_flow<T>(a, rec, slot, b, e, &s_places) && threadIdx.x == 0)
-        a.big[atomicAdd(a.nbig, 1u)] = p;  // each partition once: at most kPdParts
+      // each partition is left at most once
+      if (!pd_flow<T>(a, rec, slot, b, e, &s_places) && threadIdx.x < 1u << gl)
+        a.big[atomicAdd(a.nbig, 1u)] = (p << gl) + threadIdx.x;
     } else {
       // the first probes of all of a thread's records are in flight together
       uint32_t idx[kPdFitPer], own[kPdFitPer], met[kPdFitPer];

@@ -43,12 +43,13 @@ def _check(keys, want, blk=None, prior=None):
     assert np.array_equal(ptc.u32(ids), want)
 
 
+@pytest.mark.parametrize("apart", [3, 32])  # in 32 partitions settled together: eleven of them, or one
 @pytest.mark.parametrize("distinct", [True, False])
 @pytest.mark.parametrize("size", [1, 2, 33, 511, 512, 513, FIT - 1, FIT, FIT + 1, 2 * FIT - 1])
-def test_partition_sizes(size, distinct):
+def test_partition_sizes(size, distinct, apart):
     rng = np.random.default_rng(size)
     parts = 40  # partitions of this size, next to each other and among empty ones
-    which = np.repeat(np.arange(parts) * 3, size)
+    which = np.repeat(np.arange(parts) * apart, size)
     own = np.arange(size) if distinct else rng.integers(0, max(size // 3, 1), parts * size) if size > 1 else np.zeros(1)
     label = (np.tile(own, parts) if len(own) == size else own).astype(np.int64) + which * 4 * FIT
     order = rng.permutation(len(label))
