@@ -523,8 +523,9 @@ __global__ void __launch_bounds__(kHashThreads) k_hash_local(HashArgs a, const _
 //           where a request starts, one segmented scan over the lanes for the
 //           256 units, and the canonical residues back to shared memory
 //   store   the block ends, coalesced
-// What bounds it: integer issue, then DRAM.  The form before this one gave
-// each of 256 threads one block and ran a warp scan, a scan over the warps and
+// What bounds it: L1's data path (73% busy), the pipe that multiplies (67%),
+// issue (58%) and DRAM (75% of a copy's rate) together.  The form before this
+// one gave each of 256 threads one block and ran a warp scan, a scan over the warps and
 // the exchange of request starts for every block, with four CTA barriers: 562
 // instructions a block, of which the products are 64.
 // Measured (keys and tokens over the time; the form before in brackets): 735
