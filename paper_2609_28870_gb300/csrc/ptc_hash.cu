@@ -943,6 +943,9 @@ uint32_t chunks_per_block(uint32_t B) {  // G: power of two >= ceil(B / 16)
 // after another, and a window of 127K blocks took 20 us in tiles of 256, 13 in
 // tiles of 64.
 uint32_t tile_blocks(uint32_t B, uint64_t nb) {
+  // a block is at most 512 / 8 units, or 32 chunks
+  static_assert(PTC_MAX_BLOCK_SIZE / 8 * kCarryTileMin <= kUnitTile && 32 * kCarryTileMin <= kHashThreads,
+                "tiles without the cut below hold kCarryTileMin blocks or more");
   const uint32_t U = unit_tokens(B);
   if (!U) return kHashThreads / chunks_per_block(B);
   const uint32_t g = B / U;

@@ -812,9 +812,9 @@ __device__ __forceinline__ uint32_t pd_walk_next(PdWalk& k, PdRing& ring, const 
 }
 
 // The carries of the hash tiles that a round's words lie in (a hash tile holds
-// 8 to 256 blocks, so a word lies in 1 to 4), read once per round into shared
-// memory: word k's at k << tw, where a word lies in 1 << tw tiles.
-constexpr uint32_t kPdRoundTiles = 4 * kPdWords;
+// kCarryTileMin to 256 blocks, so a word lies in 1 to 8), read once per round
+// into shared memory: word k's at k << tw, where a word lies in 1 << tw tiles.
+constexpr uint32_t kPdRoundTiles = 32 / kCarryTileMin * kPdWords;
 struct PdCarry {
   uint32_t lead[kPdRoundTiles];
   ulonglong2 cy[kPdRoundTiles];
@@ -1777,7 +1777,9 @@ ptc_status ptc::ids_impl(const ptc_u128* keys, uint64_t n, const uint64_t* n_dev
   if (lent) L.st = lent;
   const PriorHint ph = hint ? PriorHint{hint->blk_off, hint->prior, hint->order, hint->pos, hint->n_req, L.lam, L.tile_req}
                             : PriorHint{nullptr, nullptr, nullptr, nullptr, 0, nullptr, nullptr};
-  const bool pd = pd_layout && !full_table;  // the first attempt deduplicates by partitions
+  // the first attempt deduplicates by partitions (not with smaller hash tiles
+  // than it makes room for, which traces of few blocks have)
+  const bool pd = pd_layout && !full_table && !(kc && kc->tile_blocks < kCarryTileMin);
   // the status block, the table (all ones: empty; none for the partitioned
   // dedup) and the bitmaps are cleared by one launch
   auto start = [&](uint32_t log2m, bool table) -> bool {

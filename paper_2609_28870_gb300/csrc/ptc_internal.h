@@ -204,6 +204,9 @@ struct KeyCarry {
   uint32_t* lead;
   uint32_t tile_blocks;
 };
+// The fewest blocks of a hash tile, but for a trace of few blocks (which has
+// smaller tiles): the partitioned dedup makes room for so many tiles' carries.
+constexpr uint32_t kCarryTileMin = 4;
 uint64_t hash_carry_tiles(uint64_t n_tok, uint32_t block_size);
 
 // In ptc_pipeline no stage but the last waits for its own status: the stages
