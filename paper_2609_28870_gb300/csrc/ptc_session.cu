@@ -37,7 +37,7 @@
 // words of those ids into L1, so that the owner reads hit L1 (the replayers'
 // stores go through the same L1) instead of waiting for L2 or DRAM: the owner
 // table takes 8 bytes per block and capacity.  Epochs, counts and latest
-// requests sit in shared memory when there are at most 14,336 sessions.
+// requests sit in shared memory when there are at most kSesSmemSessions sessions.
 //
 // Ids of prefix chains rise strictly within a request (a prefix first occurs
 // no later than its extensions), so no window holds a block twice.  Whether
@@ -105,7 +105,11 @@ __global__ void k_ses_check(const uint64_t* __restrict__ blk_off, uint32_t R, ui
   }
 }
 
-constexpr uint32_t kSesSmemSessions = 14336;  // session state kept in shared memory up to this many
+// Session state is kept in shared memory up to this many sessions (12 bytes each
+// beside the ring), and above it in global memory, of which L1 serves what is in
+// use: 136 ms for 14,000 sessions and 140 for 14,400 (the tiny workload's shape,
+// 16 capacities).
+constexpr uint32_t kSesSmemSessions = 14336;
 constexpr uint32_t kSesReplay = 16;            // warps that replay
 constexpr uint32_t kSesWin = 32 * kSesReplay;  // accesses per window, one per lane
 constexpr uint32_t kSesAhead = 8;              // warps that read ahead
@@ -602,6 +606,10 @@ extern "C" ptc_status ptc_session_lru_curves(const uint32_t* ids, uint64_t n, ui
     else
       PTC_KERNEL("k_ses_sim", s, k_ses_sim<true>, n_cap, kSesThreads, smem, a, caps, (uint32_t)n, L.falls);
   } else {
+    static_assert(sizeof(SesRing) > 48 * 1024, "the ids read ahead alone need more than a kernel has by default");
+    if (cudaFuncSetAttribute(k_ses_sim<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(SesRing)) !=
+        cudaSuccess)
+      return PTC_ERR_CUDA;
     PTC_KERNEL("k_ses_sim", s, k_ses_sim<false>, n_cap, kSesThreads, sizeof(SesRing), a, caps, (uint32_t)n, L.falls);
   }
   HostStage* hs = host_stage();

@@ -96,6 +96,24 @@ def test_chat_workload_prefix():
            tracegen.workload_grid(1, D))
 
 
+@pytest.mark.parametrize("S", [14336, 14337, 20000])
+@pytest.mark.parametrize("repeats", [False, True])
+def test_session_state_in_shared_and_in_global_memory(S, repeats):
+    """Labels up to the number of sessions whose state fits in shared memory, and
+    above it, a few hundred of them used; ids that rise in every request, and
+    ids that repeat inside one."""
+    rng = np.random.default_rng(S + repeats)
+    tr = tracegen.tiny(S, n_sessions=300, max_turns=5, vocab=3, max_seg=60)
+    ids, D = oracle.block_ids(tr.tokens, tr.req_tok_off, 1)
+    off = oracle.block_offsets(tr.req_tok_off, 1)
+    if repeats:
+        _, ids = np.unique(rng.integers(0, D, ids.size), return_inverse=True)
+    label = rng.permutation(S)[:300].astype(np.uint32)
+    label[0] = S - 1
+    caps = np.unique(np.geomspace(1, 2 * D, 24).astype(np.uint64))
+    _check(ids, off, label[tr.req_session], S, 1, caps, ((0, 0, 0), (1, 3, 5)))
+
+
 def test_errors():
     import paper_2609_28870_gb300 as ptc
     off = ptc.to_device_u64(np.array([0, 2, 3], np.uint64))
