@@ -595,14 +595,18 @@ void ptc_release_host_staging(void);
 /*
  * ptc_test_wait_polls — test hook for the bounded waits (no counterpart in
  * the paper: failure detection).  Kernels that wait on other CTAs (the
- * decoupled look-back of stage a1's block offsets) poll a bounded number of
- * times and then give up with PTC_ERR_TIMEOUT instead of hanging.  With
- * polls > 0, every later ptc_hash_blocks / ptc_pipeline call in the process
- * makes those waits see no predecessor as ready (a flag that nothing sets)
- * and give up after `polls` polls, so a test can drive the give-up path: the
- * call must return PTC_ERR_TIMEOUT and leave the device usable.  polls = 0
- * restores normal waits.  Process-wide; not for production use.
+ * decoupled look-backs of stage a1's block offsets and, in ptc_pipeline, of
+ * stage c's runs) poll a bounded number of times and then give up with
+ * PTC_ERR_TIMEOUT instead of hanging.  With polls > 0, every later
+ * ptc_hash_blocks / ptc_pipeline call in the process makes stage a1's waits see
+ * no predecessor as ready (a flag that nothing sets) and give up after `polls`
+ * polls, so a test can drive the give-up path: the call must return
+ * PTC_ERR_TIMEOUT and leave the device usable.  With
+ * PTC_TEST_WAIT_PIECES + polls it is stage c's wait that gives up (a call with
+ * fewer than 2,049 pieces has none).  0 restores normal waits.  Process-wide;
+ * not for production use.
  */
+#define PTC_TEST_WAIT_PIECES 0x80000000u
 void ptc_test_wait_polls(uint32_t polls);
 
 /*

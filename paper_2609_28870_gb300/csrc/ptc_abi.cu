@@ -390,7 +390,10 @@ namespace {
 std::atomic<uint32_t> g_wait_polls{0};
 }  // namespace
 
-uint32_t ptc::test_wait_polls() { return g_wait_polls.load(std::memory_order_relaxed); }
+uint32_t ptc::test_wait_polls(bool pieces) {
+  const uint32_t v = g_wait_polls.load(std::memory_order_relaxed);
+  return ((v & PTC_TEST_WAIT_PIECES) != 0) == pieces ? v & ~PTC_TEST_WAIT_PIECES : 0u;
+}
 
 void ptc::release_host_stage() {
   if (t_pinned && t_pinned != &t_fallback) {

@@ -601,6 +601,10 @@ __global__ void __launch_bounds__(256) k_curves_runs(CurveArgs a, RunsArgs ra, F
   }
   __shared__ Bins s_bins;
   const uint32_t G = a.G;
+  // an earlier stage failed: its runs are void (what the distances' CTAs read of
+  // them is in range all the same, whatever it says)
+  uint32_t failed = 0;
+  for (uint32_t q = 0; q < f.n_earlier; ++q) failed |= f.earlier[q].err;
   s_bins.init(a.caps, G);
   __syncthreads();
   // Four lanes per request, a run per lane and round: a request has a handful
@@ -609,7 +613,8 @@ __global__ void __launch_bounds__(256) k_curves_runs(CurveArgs a, RunsArgs ra, F
   // 291K requests of half a mixed day.)
   bool fell = false;
   const uint32_t sub = threadIdx.x & 3, groups = ra.ctas * (blockDim.x >> 2);
-  for (uint32_t q0 = blockIdx.x * (blockDim.x >> 2) + ((threadIdx.x >> 5) << 3); q0 < a.R; q0 += groups) {
+  const uint32_t n_req = failed ? 0 : a.R;
+  for (uint32_t q0 = blockIdx.x * (blockDim.x >> 2) + ((threadIdx.x >> 5) << 3); q0 < n_req; q0 += groups) {
     const uint32_t q = q0 + ((threadIdx.x & 31) >> 2);
     const uint32_t start = q < a.R ? (uint32_t)a.blk_off[q] : 0u, end = q < a.R ? (uint32_t)a.blk_off[q + 1] : 0u;
     const bool some = end > start && end <= a.n;  // not empty (bad offsets are reported by k_heads)

@@ -96,9 +96,9 @@ inline ptc_status begin_call(void* ws, size_t zero_bytes, cudaStream_t stream) {
   return fill_async(ws, 0u, zero_bytes, stream);
 }
 
-// The poll count set by ptc_test_wait_polls (0: normal waits), read by the
-// calls whose kernels wait on each other (stage a1's look-back).
-uint32_t test_wait_polls();
+// The poll count set by ptc_test_wait_polls (0: normal waits) for stage a1's
+// look-back or, with `pieces`, for stage c's.
+uint32_t test_wait_polls(bool pieces = false);
 
 // Words of ptc_trace_stats's results: the summary and the reach bins.
 constexpr size_t kStatsHostWords = sizeof(ptc_trace_summary) / 8 + PTC_MAX_CAPACITIES + 1;

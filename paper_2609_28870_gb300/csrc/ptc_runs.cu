@@ -626,12 +626,16 @@ struct DomArgs {
   uint32_t* rank;      // per run: rank (kNone: first accesses)
   uint32_t* sd;
   uint32_t R, nb, kwords;
-  const uint64_t* Rd;  // device: the number of runs where R is a bound only, or null
-  bool keys_after;     // kpre counts the run starts too (their bitmap lies before the keys')
+  const DevStatus* st;  // where R is a bound only: value[1] is the number of runs; else null
+  bool keys_after;      // kpre counts the run starts too (their bitmap lies before the keys')
 };
+// The runs, or none if the look-back that numbers them gave up: their records are
+// then out of order, so that lengths, and the ranks that index arrays, mean nothing.
 __device__ __forceinline__ uint32_t dom_runs(const DomArgs& a) {
-  const uint64_t r = a.Rd ? *a.Rd : a.R;
-  return r < a.R ? (uint32_t)r : a.R;
+  if (!a.st) return a.R;  // the host has seen the status
+  const uint32_t err = a.st->err;
+  const uint64_t r = a.st->value[1];
+  return err ? 0u : r < a.R ? (uint32_t)r : a.R;
 }
 
 // Sum of w over the pairs (key, w) of s[0 .. n) with key < mine: n even, two
@@ -933,6 +937,8 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
   const uint64_t K = pieces.K;
   const bool by_pieces = lent && K > 0 && reinterpret_cast<const char*>(M.sd) <= reinterpret_cast<const char*>(pieces.ipos);
   if (by_pieces) {
+    const uint32_t wait_test = test_wait_polls(true);
+    if (wait_test && fill_async(&M.st->wait_test, wait_test, sizeof(uint32_t), s) != PTC_OK) return PTC_ERR_CUDA;
     const PieceArgs pa{pieces, (uint32_t)n, M.bits, M.kbits, M.rec_s, M.rec_a, lent->lb, M.st};
     PTC_KERNEL("k_runs_pieces", s, k_runs_pieces, ceil_div_u32(K, kPieceTile), kPT, 0, pa);
     if (bitmap_ranks(M.bits, 2 * M.kwords, M.wpre, M.ktcnt, M.ktpre, &M.done[62], nullptr, s) != PTC_OK)
@@ -994,7 +1000,7 @@ ptc_status stack_distance_runs(const uint32_t* prev, uint64_t n, uint32_t* dist_
     d.sd = W.sd;
     d.R = R32;
     d.kwords = W.kwords;
-    d.Rd = bound ? &W.st->value[1] : nullptr;
+    d.st = bound ? W.st : nullptr;
     d.keys_after = by_pieces;
     const size_t row = sizeof(uint32_t) * d.nb;
     PTC_KERNEL("k_dom_time", s, k_dom_time, d.nb, kDomB, row, d);

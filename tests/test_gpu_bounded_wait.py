@@ -1,8 +1,8 @@
 """Failure detection of the bounded device waits, with no GPU fault.
 
-Kernels that wait on other CTAs (the decoupled look-back of stage a1's block
-offsets) poll a bounded number of times and then give up with
-PTC_ERR_TIMEOUT.  The test hook ptc_test_wait_polls makes those waits see no
+Kernels that wait on other CTAs (the decoupled look-backs of stage a1's block
+offsets and of stage c's runs) poll a bounded number of times and then give up
+with PTC_ERR_TIMEOUT.  The test hook ptc_test_wait_polls makes those waits see no
 predecessor as ready (a flag nothing sets) and give up after a few hundred
 polls, so the give-up path runs for real: the call must return
 PTC_ERR_TIMEOUT, nothing downstream may read through the unfinished offsets,
@@ -56,3 +56,30 @@ def test_forced_give_up_then_exact_results():
     g = ptc.ptc_pipeline(tok, off, ts, B, caps)
     assert g["n_distinct"] == D and g["hits"] == o["hits"] and g["saved"] == o["saved"]
     assert g["total_cost"] == o["total_cost"]
+
+
+@pytest.mark.parametrize("n_req", [30_000, 600_000])  # the host goes on without waiting for the runs, or waits
+def test_stage_c_gives_up_then_exact_results(n_req):
+    """Requests that each re-read a document of eight one-token blocks, a piece
+    a request: many tiles of pieces, whose wait gives up.  The records of the
+    runs are then out of order, and no kernel after may index by them."""
+    import torch
+
+    import paper_2609_28870_gb300 as ptc
+    rng = np.random.default_rng(n_req)
+    tok = (rng.integers(0, n_req // 3, n_req)[:, None] * 8 + np.arange(8)).astype(np.uint32).ravel()
+    off = ptc.to_device_u64(np.arange(n_req + 1, dtype=np.uint64) * 8)
+    plan = ptc.PipelinePlan(ptc.to_device_u32(tok), off, None, 1, [10, 1000, n_req], ptc.PTC_COST_UNIFORM)
+    want = plan.run().result()
+    L = ptc.lib()
+    L.ptc_test_wait_polls(0x80000000 + 300)
+    try:
+        with pytest.raises(ptc.PtcError) as e:
+            plan.run()
+        assert e.value.name == "PTC_ERR_TIMEOUT"
+    finally:
+        L.ptc_test_wait_polls(0)
+    torch.cuda.synchronize()  # the context is still usable
+    assert plan.run().result() == want
+    sd = oracle.sd_fenwick(oracle.reuse(*oracle.block_ids(tok, np.arange(n_req + 1, dtype=np.uint64) * 8, 1))[0])
+    assert want["hits"] == [int((sd <= c).sum()) for c in (10, 1000, n_req)]
