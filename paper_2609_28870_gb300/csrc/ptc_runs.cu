@@ -143,10 +143,17 @@ __global__ void __launch_bounds__(kMT) k_runs_count(MarkArgs a) {
   if (threadIdx.x == 0) a.st->value[1] = total;
 }
 
+// Whether pass 2 has nothing to mark: too many runs, or a previous use that does
+// not lie before its access (its key would fall outside the bitmap of keys).
+__device__ __forceinline__ bool marked_void(const MarkArgs& a) {
+  const uint32_t err = a.st->err;
+  return err != 0 || a.st->value[1] > a.max_runs;
+}
+
 // Pass 2: bitmap, run index per word, and the (start, first value) records.
 __global__ void __launch_bounds__(kMT) k_runs_mark(MarkArgs a) {
   grid_dep_sync();
-  if (a.st->value[1] > a.max_runs) return;
+  if (marked_void(a)) return;
   __shared__ uint32_t s_wcnt[kMT / 32];
   const uint32_t tile = blockIdx.x;
   const uint32_t lane = threadIdx.x & 31, w = threadIdx.x >> 5;
@@ -266,7 +273,7 @@ __global__ void __launch_bounds__(kMT) k_runs_count4(MarkArgs a) {
 
 __global__ void __launch_bounds__(kMT) k_runs_mark4(MarkArgs a) {
   grid_dep_sync();
-  if (a.st->value[1] > a.max_runs) return;
+  if (marked_void(a)) return;
   __shared__ uint32_t s_wcnt[kMT / 32];
   const uint32_t tile = blockIdx.x, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
   const uint32_t base = tile * kMTile + w * (32 * kMR);

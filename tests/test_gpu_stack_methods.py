@@ -106,9 +106,9 @@ def test_forced_runs_with_a_small_workspace_is_refused():
 
 
 def test_many_runs_take_the_per_level_build():
-    """More runs than one cluster's shared memory holds (131,072): the matrix
-    over runs is built one level per launch; a random reuse array with short
-    runs, forced onto the matrix over runs."""
+    """A random reuse array with short runs, about as many as accesses, forced
+    onto the count over runs (by blocks of pair sums; tests/test_gpu_pieces.py
+    has more runs than those take, which go to the matrix level by level)."""
     import torch
     import paper_2609_28870_gb300 as ptc
     rng = np.random.default_rng(11)
@@ -124,3 +124,50 @@ def test_many_runs_take_the_per_level_build():
     p = ptc.to_device_u32(prev)
     got = ptc.u32(ptc.ptc_stack_distance(p, method=ptc.PTC_SD_RUNS))
     assert np.array_equal(got, want)
+
+
+@pytest.mark.parametrize("shift", [0, 1])  # 16-byte loads, and prev off their alignment
+def test_previous_uses_that_do_not_lie_before(shift):
+    """A previous use at or after its access is an error, whatever it is: the key
+    of its run is not marked (the highest would lie 512 MB past the bitmap)."""
+    import torch
+    import paper_2609_28870_gb300 as ptc
+    n = 50_000
+    good = np.full(n, oracle.NONE, dtype=np.uint32)
+    good[n // 2:] = np.arange(n - n // 2)  # few runs: pass 2 marks them
+    want = oracle.sd_fenwick(good)
+    buf = torch.zeros(n + shift, dtype=torch.int32, device="cuda")
+    for at, value in ((n // 3, 0xFFFFFFFE), (n - 1, n - 1), (7, 0x80000000), (0, 0)):
+        bad = good.copy()
+        bad[at] = value
+        buf[shift:] = ptc.to_device_u32(bad)
+        for method in (None, ptc.PTC_SD_RUNS):
+            with pytest.raises(ptc.PtcError) as e:
+                ptc.ptc_stack_distance(buf[shift:], method=method)
+            assert e.value.name == "PTC_ERR_INVALID_ARG"
+    buf[shift:] = ptc.to_device_u32(good)
+    assert np.array_equal(ptc.u32(ptc.ptc_stack_distance(buf[shift:])), want)
+
+
+@pytest.mark.parametrize("order,residency", [(1, 0), (1, 1), (0, 1)])
+def test_variants_with_malformed_offsets(order, residency):
+    """Offsets that leave accesses to no request: leaf-first, their previous uses
+    in touch order are never written, and hold what the workspace held."""
+    import torch
+    import paper_2609_28870_gb300 as ptc
+    n = 50_000
+    prev = np.full(n, oracle.NONE, dtype=np.uint32)
+    prev[n // 2:] = np.arange(n - n // 2)
+    p = ptc.to_device_u32(prev)
+    L = ptc.lib()
+    ws = torch.empty(L.ptc_stack_distance_variant_workspace_bytes(n, 3, order, residency), dtype=torch.uint8,
+                     device="cuda")
+    for off in ([0, 100, 200, n - 5000], [0, 30_000, 20_000, n], [10, 100, 200, n]):
+        ws.fill_(0xFE)
+        with pytest.raises(ptc.PtcError) as e:
+            ptc.ptc_stack_distance_variant(p, ptc.to_device_u64(np.array(off, np.uint64)), order, residency, ws=ws)
+        assert e.value.name == "PTC_ERR_INVALID_ARG"
+    good = ptc.to_device_u64(np.array([0, n // 2, n // 2, n], np.uint64))
+    a = ptc.ptc_stack_distance_variant(p, good, order, residency, ws=ws)
+    b = ptc.ptc_stack_distance_variant(p, good, order, residency, method=ptc.PTC_SD_POINTS)
+    assert torch.equal(a, b)
