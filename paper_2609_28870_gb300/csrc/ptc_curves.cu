@@ -368,7 +368,10 @@ __global__ void __launch_bounds__(kCvThreads) k_curves_fast(CurveArgs a) {
   __shared__ Bins s_bins;
   __shared__ uint32_t s_off[kFtReq + 2];
   const uint32_t G = a.G;
+  // malformed offsets: a request's end may never come
+  const bool bad = ld_relaxed_u32(&a.st->err) != 0;
   s_bins.init(a.caps, G);
+  if (bad) return;
   uint32_t walked = 0;
   const uint32_t ntiles = (a.n + kCvTile - 1) / kCvTile;
   const uint32_t lane = threadIdx.x & 31;

@@ -117,3 +117,17 @@ def test_many_short_requests_in_one_tile():
         h, s, t = _curves_by_definition(dist, blk_off, caps, 4, kind)
         g = _gpu_curves(dist, blk_off, caps, 4, kind)
         assert g["hits"] == h and g["saved"] == s and g["total_cost"] == t
+
+
+@pytest.mark.parametrize("off", [[0, 5], [0, 5, 3, 20_000], [7, 20_000], [0, 20_001], [0, 2**40, 20_000], [0, 0, 0]])
+def test_malformed_offsets(off):
+    """Offsets that end early, fall, start late or run past the accesses: an
+    error, and no walk to a request's end that never comes."""
+    import torch
+    import paper_2609_28870_gb300 as ptc
+    dist = torch.ones(20_000, dtype=torch.int32, device="cuda")
+    with pytest.raises(ptc.PtcError) as e:
+        ptc.ptc_curves(dist, ptc.to_device_u64(np.array(off, np.uint64)), 16, [1, 2])
+    assert e.value.name == "PTC_ERR_INVALID_ARG"
+    g = ptc.ptc_curves(dist, ptc.to_device_u64(np.array([0, 5, 5, 20_000], np.uint64)), 16, [1, 2])
+    assert g["hits"] == [20_000, 20_000]
