@@ -1025,6 +1025,8 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
   }
   const uint32_t wait_test = test_wait_polls();
   if (wait_test && fill_async(&L.st->wait_test, wait_test, sizeof(uint32_t), s) != PTC_OK) return PTC_ERR_CUDA;
+  const uint32_t tb = tile_blocks(block_size, n_tok / block_size), U = unit_tokens(block_size);
+  if (carry) carry->tile_blocks = tb;  // the keys' reader looks carries up whether there are keys or not
   if (n_req == 0) {
     if (fill_async(req_blk_off_out, 0u, sizeof(uint64_t), s) != PTC_OK) return PTC_ERR_CUDA;
     if (lent) return cudaGetLastError() == cudaSuccess ? PTC_OK : PTC_ERR_CUDA;
@@ -1033,7 +1035,6 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
   }
   const uint32_t G = chunks_per_block(block_size);
   const bool aligned = (((uintptr_t)tokens) & 15) == 0;
-  const uint32_t tb = tile_blocks(block_size, n_tok / block_size), U = unit_tokens(block_size);
   // seeded bases and their derived constants
   PowArgs pw;
   HashConsts hc;
@@ -1104,7 +1105,6 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
     if (carry) {
       PTC_KERNEL("k_hash_carry", s, k_hash_carry, ceil_div_u32(grid, kChainWarps * kCarryPer), kChainWarps * 32, 0, L.tile_agg,
                  L.tile_lead, tb, L.st, keys_cap, grid, carry->carry, carry->lead);
-      carry->tile_blocks = tb;
     } else {
       PTC_KERNEL("k_hash_chain", s, k_hash_chain, ceil_div_u32(grid, kChainWarps), kChainWarps * 32, 0, a.keys,
                  L.tile_agg, L.tile_lead, tb, L.st, keys_cap);

@@ -113,6 +113,18 @@ def test_pipeline_degenerate_traces():
     assert r["dist"].tolist() == [0xFFFFFFFF]
 
 
+@pytest.mark.parametrize("B", [1, 16, 24])
+def test_pipeline_of_no_requests_on_a_token_buffer(B):
+    """A buffer of a million tokens none of which is a request's yet: the grids
+    follow the buffer, and what they look up lies within the workspace."""
+    import torch
+    import paper_2609_28870_gb300 as ptc
+    tok = torch.zeros(1_000_003, dtype=torch.int32, device="cuda")
+    none = torch.zeros(1, dtype=torch.int64, device="cuda")
+    r = ptc.ptc_pipeline(tok, none, None, B, [4, 9])
+    assert r["n_access"] == 0 and r["n_distinct"] == 0 and r["hits"] == [0, 0] and r["total_cost"] == 0
+
+
 def test_pipeline_rejects_bad_arguments():
     import ctypes
     import torch
