@@ -731,7 +731,7 @@ __device__ __forceinline__ bool hash_units_tile(const HashArgs& a, const HashCon
     }
     // the powers go out with the tokens
     const uint64_t* T = a.tables;
-    const uint32_t e_lo = (uint32_t)e & 0xFFFFu, e_hi = (uint32_t)e >> 16;  // e < 2^32: the tables reach no further
+    const uint32_t e_lo = (uint32_t)e & 0xFFFFu, e_hi = (uint32_t)e >> 16;  // e < 2^32 (unit_tokens)
     uint64_t w0 = __ldg(&T[e_lo]), w1 = __ldg(&T[2 * 65536 + e_lo]);
     if (e_hi) {
       w0 = p61_mul(w0, __ldg(&T[65536 + e_hi]));
@@ -924,11 +924,16 @@ void launch_hash(uint32_t grid, cudaStream_t s, const HashArgs& a, const HashCon
     PTC_KERNEL("k_hash_local", s, (k_hash_local<G, false>), grid, kHashThreads, 0, a, c);
 }
 
-// Tokens per unit of k_hash_units, or 0 for a block size that k_hash_local
-// takes.  Units are whole vectors of four tokens, so that the units of a
-// request share their alignment; the larger the unit, the fewer
-// multiplications and sums per token.
-uint32_t unit_tokens(uint32_t B) { return B % 16 == 0 ? 16 : B % 12 == 0 ? 12 : B % 8 == 0 ? 8 : 0; }
+// Tokens per unit of k_hash_units, or 0 for a trace that k_hash_local takes.
+// Units are whole vectors of four tokens, so that the units of a request share
+// their alignment; the larger the unit, the fewer multiplications and sums per
+// token.  A unit's place in its request is a 32-bit exponent: where a request
+// could hold 2^32 units (34 billion tokens or more), blocks are counted instead,
+// of which no trace has that many.
+uint32_t unit_tokens(uint32_t B, uint64_t n_tok) {
+  const uint32_t U = B % 16 == 0 ? 16 : B % 12 == 0 ? 12 : B % 8 == 0 ? 8 : 0;
+  return U && n_tok / U < 1ULL << 32 ? U : 0;
+}
 
 uint32_t chunks_per_block(uint32_t B) {  // G: power of two >= ceil(B / 16)
   uint32_t need = (B + 15) / 16, g = 1;
@@ -936,17 +941,18 @@ uint32_t chunks_per_block(uint32_t B) {  // G: power of two >= ceil(B / 16)
   return g;
 }
 
-// Blocks per hash tile for up to nb blocks, a power of two: as many as make up
+// Blocks per hash tile for n_tok tokens, a power of two: as many as make up
 // to 256 units for k_hash_units, one CTA's kHashThreads / G for k_hash_local.
 // With few blocks a tile of units is cut down to 64 while that makes more warps
 // than half of those that fit the GPU: a warp takes its rounds of 32 units one
 // after another, and a window of 127K blocks took 20 us in tiles of 256, 13 in
 // tiles of 64.
-uint32_t tile_blocks(uint32_t B, uint64_t nb) {
+uint32_t tile_blocks(uint32_t B, uint64_t n_tok) {
   // a block is at most 512 / 8 units, or 32 chunks
   static_assert(PTC_MAX_BLOCK_SIZE / 8 * kCarryTileMin <= kUnitTile && 32 * kCarryTileMin <= kHashThreads,
                 "tiles without the cut below hold kCarryTileMin blocks or more");
-  const uint32_t U = unit_tokens(B);
+  const uint32_t U = unit_tokens(B, n_tok);
+  const uint64_t nb = n_tok / B;
   if (!U) return kHashThreads / chunks_per_block(B);
   const uint32_t g = B / U;
   uint32_t tb = kUnitTile;
@@ -972,7 +978,7 @@ HashLayout hash_layout(void* ws, uint32_t n_req, uint64_t n_tok, uint32_t B, uin
   Carver cv(ws);
   const uint32_t off_tiles = ceil_div_u32(n_req, kOffTile) + 1;
   const uint64_t nb = n_tok / B < keys_cap ? n_tok / B : keys_cap;
-  const uint32_t tb = tile_blocks(B, n_tok / B);
+  const uint32_t tb = tile_blocks(B, n_tok);
   const uint32_t hash_tiles = ceil_div_u32(nb, tb) + 1;
   L.st = cv.take<DevStatus>(1);
   L.lb_off = cv.take<uint64_t>(off_tiles);
@@ -995,7 +1001,7 @@ size_t ptc::hash_lb_words(uint32_t n_req) { return ceil_div_u32(n_req, kOffTile)
 
 uint64_t ptc::hash_carry_tiles(uint64_t n_tok, uint32_t block_size) {
   if (block_size == 0) block_size = 1;
-  return ceil_div_u32(n_tok / block_size, tile_blocks(block_size, n_tok / block_size)) + 1;
+  return ceil_div_u32(n_tok / block_size, tile_blocks(block_size, n_tok)) + 1;
 }
 
 extern "C" size_t ptc_hash_blocks_workspace_bytes(uint32_t n_req, uint64_t n_tok, uint32_t block_size) {
@@ -1025,7 +1031,7 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
   }
   const uint32_t wait_test = test_wait_polls();
   if (wait_test && fill_async(&L.st->wait_test, wait_test, sizeof(uint32_t), s) != PTC_OK) return PTC_ERR_CUDA;
-  const uint32_t tb = tile_blocks(block_size, n_tok / block_size), U = unit_tokens(block_size);
+  const uint32_t tb = tile_blocks(block_size, n_tok), U = unit_tokens(block_size, n_tok);
   if (carry) carry->tile_blocks = tb;  // the keys' reader looks carries up whether there are keys or not
   if (n_req == 0) {
     if (fill_async(req_blk_off_out, 0u, sizeof(uint64_t), s) != PTC_OK) return PTC_ERR_CUDA;
