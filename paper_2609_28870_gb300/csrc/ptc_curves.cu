@@ -568,9 +568,9 @@ __device__ __forceinline__ void finalize_bins(const FinishArgs& f) {
     }
   }
   if (t == 0) {
-    uint32_t e = f.st->err;
+    uint32_t e = 0;
     for (uint32_t q = 0; q < f.n_earlier; ++q) e |= f.earlier[q].err;
-    f.st->err = e;
+    if (e) raise_err(f.st, e);  // others may raise theirs meanwhile
   }
   __syncthreads();
   if (f.st_host && t < sizeof(DevStatus) / 4)
@@ -620,7 +620,7 @@ __global__ void __launch_bounds__(256) k_curves_runs(CurveArgs a, RunsArgs ra, F
   for (uint32_t q0 = blockIdx.x * (blockDim.x >> 2) + ((threadIdx.x >> 5) << 3); q0 < n_req; q0 += groups) {
     const uint32_t q = q0 + ((threadIdx.x & 31) >> 2);
     const uint32_t start = q < a.R ? (uint32_t)a.blk_off[q] : 0u, end = q < a.R ? (uint32_t)a.blk_off[q + 1] : 0u;
-    const bool some = end > start && end <= a.n;  // not empty (bad offsets are reported by k_heads)
+    const bool some = end > start && end <= a.n;  // not empty (the offsets are stage a1's own)
     const uint32_t r0 = some ? run_of(ra.bits, ra.wpre, start) : 1u, r1 = some ? run_of(ra.bits, ra.wpre, end - 1) : 0u;
     const uint32_t rounds = __reduce_max_sync(kFull, some ? (r1 - r0) / 4 + 1 : 0u);
     uint32_t before = 0;  // the distance of the run before this round's first
@@ -777,7 +777,13 @@ ptc_status ptc::curves_impl(const uint32_t* dist, uint64_t n, const uint64_t* re
                        L.slow, L.st,   earlier, n_earlier, staged ? &hs->dev->st : nullptr};
   auto finish = [&](bool written) -> ptc_status {
     if (!written) PTC_KERNEL("k_finalize", s, k_finalize, 1, 1024, 0, fin);
+#ifdef PTC_CHECKED
+    // the CTAs that write the distances check theirs too, and may be done after
+    // the status was written
+    if (staged) return end_call(L.st, s, &h);
+#else
     if (staged) return end_call_staged(s, &h);
+#endif
     if (copy_to_host_async(hs->out, L.out, sizeof(uint64_t) * (3 * n_cap + 3), s) != PTC_OK) return PTC_ERR_CUDA;
     return end_call(L.st, s, &h);
   };
