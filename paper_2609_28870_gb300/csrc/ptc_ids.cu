@@ -1415,10 +1415,11 @@ __global__ void __launch_bounds__(kPdBigThreads, 2) k_pd_dedup_big(PdDedup a) {
   __shared__ uint32_t s_nlist;
   constexpr uint32_t kChunk = kPdBigThreads * kPdBigPer;
   const ulonglong2 empty = make_ulonglong2(~0ULL, ~0ULL);
-  auto load = [&](ulonglong2(&dst)[kPdBigPer], uint32_t c, uint32_t end) {
+  // positions have 64 bits: a chunk may reach past 2^32 records
+  auto load = [&](ulonglong2(&dst)[kPdBigPer], uint64_t c, uint32_t end) {
 #pragma unroll
     for (int q = 0; q < kPdBigPer; ++q) {
-      const uint32_t x = c + q * kPdBigThreads + threadIdx.x;
+      const uint64_t x = c + q * kPdBigThreads + threadIdx.x;
       dst[q] = x < end && x < a.cap ? __ldcs(&a.rec2[x]) : empty;
     }
   };
@@ -1447,7 +1448,7 @@ __global__ void __launch_bounds__(kPdBigThreads, 2) k_pd_dedup_big(PdDedup a) {
       if (threadIdx.x == 0) s_nlist = 0;
       __syncthreads();
       bool full = false;
-      for (uint32_t c = b;; c += kChunk) {
+      for (uint64_t c = b;; c += kChunk) {
         const bool more = c + kChunk < e;
         ulonglong2 w[kPdBigPer];
         if (more)
@@ -1495,11 +1496,11 @@ __global__ void __launch_bounds__(kPdBigThreads, 2) k_pd_dedup_big(PdDedup a) {
           if (m < rp.x && rp.x < a.n_ub) pd_repeat(a.slot_of, a.bits, rp.x, m);
         }
       } else {  // more repeats than the list holds: look every record up again
-        for (uint32_t c = b; c < e; c += kChunk) {
+        for (uint64_t c = b; c < e; c += kChunk) {
           ulonglong2 r[kPdBigPer];
 #pragma unroll
           for (int q = 0; q < kPdBigPer; ++q) {
-            const uint32_t x = c + q * kPdBigThreads + threadIdx.x;
+            const uint64_t x = c + q * kPdBigThreads + threadIdx.x;
             r[q] = x < e ? __ldcg(&a.rec2[x]) : empty;
           }
 #pragma unroll
