@@ -1691,7 +1691,12 @@ __device__ __forceinline__ uint2 requests_of(const uint64_t* __restrict__ blk_of
 // tokens' bytes.  With a block per lane, word by word until one differs, 2.3M
 // blocks of 24 tokens took 151 us, so 80 (98 with one word of any block at a time,
 // 84 with the searches one after the other).
+// Blocks of up to kVerLaneB tokens (WARP = false) keep the block per lane, with
+// the searches one after the other: 9.7M blocks of 4 tokens took 182 us by warps,
+// so 156; 5.2M of one token 76 and 66; of 8 tokens, 4.9M blocks, 109 so and 99.
 constexpr int kVerThreads = 256;
+constexpr uint32_t kVerLaneB = 4;
+template <bool WARP>
 __global__ void __launch_bounds__(kVerThreads) k_verify(const uint32_t* __restrict__ tokens, uint64_t n_tok,
                                                         const uint64_t* __restrict__ tok_off,
                                                         const uint64_t* __restrict__ blk_off, uint32_t R, uint32_t B,
@@ -1707,7 +1712,8 @@ __global__ void __launch_bounds__(kVerThreads) k_verify(const uint32_t* __restri
     if (f == kNone) {
       raise_err(st, kErrInvalid);
     } else if (f != (uint32_t)i) {
-      const uint2 r = requests_of(blk_off, R, i, f);
+      const uint2 r = WARP ? requests_of(blk_off, R, i, f)
+                           : make_uint2(req_search(blk_off, 0, R - 1, i), req_search(blk_off, 0, R - 1, f));
       const uint32_t ri = r.x, rf = r.y;
       const uint64_t ki = i - blk_off[ri], kf = f - blk_off[rf];
       const uint64_t bi = tok_off[ri], ei = tok_off[ri + 1], bf = tok_off[rf], ef = tok_off[rf + 1];
@@ -1722,9 +1728,15 @@ __global__ void __launch_bounds__(kVerThreads) k_verify(const uint32_t* __restri
       }
     }
   }
+  bool differ = false;
+  if (!WARP) {
+    if (ti != ~0ULL)
+      for (uint32_t t = 0; t < B; ++t) differ |= __ldg(&tokens[ti + t]) != __ldg(&tokens[tf + t]);
+    if (differ) raise_err(st, kErrCollision);
+    return;
+  }
   const uint32_t some = __ballot_sync(kFull, ti != ~0ULL);
   if (!some) return;
-  bool differ = false;
   // lanes a0 .. a1 repeat one stretch: its words, whichever block they lie in
   const uint32_t a0 = __ffs(some) - 1, a1 = 31 - __clz(some);
   const uint64_t ts = __shfl_sync(kFull, ti, a0), fs = __shfl_sync(kFull, tf, a0), d = (uint64_t)B * (lane - a0);
@@ -2006,7 +2018,9 @@ extern "C" ptc_status ptc_verify_ids(const uint32_t* tokens, uint64_t n_tok, con
   if (fill_async(first, ~0u, sizeof(uint32_t) * (n_distinct ? n_distinct : 1), s) != PTC_OK)
     return PTC_ERR_CUDA;
   PTC_KERNEL("k_verify_first", s, k_verify_first, ceil_div_u32(n, 256), 256, 0, ids, n, n_distinct, first, st);
-  PTC_KERNEL("k_verify", s, k_verify, ceil_div_u32(n, kVerThreads), kVerThreads, 0, tokens, n_tok, req_tok_off, req_blk_off, n_req, block_size, ids, n, n_distinct, first, st);
+  PTC_KERNEL("k_verify", s, (block_size <= kVerLaneB ? k_verify<false> : k_verify<true>),
+             ceil_div_u32(n, kVerThreads), kVerThreads, 0, tokens, n_tok, req_tok_off, req_blk_off, n_req, block_size,
+             ids, n, n_distinct, first, st);
   DevStatus h;
   return end_call(st, s, &h);
 }

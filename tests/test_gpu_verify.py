@@ -17,7 +17,7 @@ def ptc():
     return p
 
 
-@pytest.mark.parametrize("B", [1, 2, 7, 24, 31, 32, 33, 100, 512])
+@pytest.mark.parametrize("B", [1, 2, 4, 5, 7, 24, 31, 32, 33, 100, 512])
 def test_verify(ptc, B):
     rng = np.random.default_rng(B)
     doc = rng.integers(0, 150_000, 60 * B).astype(np.uint32)
