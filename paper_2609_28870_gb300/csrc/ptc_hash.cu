@@ -18,7 +18,7 @@
 //                    two levels of 65,536 entries, as far as a request can reach
 //   k_hash_units     B a multiple of 16, 12 or 8: a unit of U = 16, 12 or 8
 //                    tokens per lane, 32 units at a time, then prefix sums over
-//                    the 256 units of a warp's tile, eight units per lane
+//                    the units of a warp's tile, 8, 9 or 11 per lane
 //                    (three-limb products where a token reaches 2^27)
 //   k_hash_local     any other B: tokens
 //                    staged through padded shared memory with 16-byte
@@ -513,15 +513,15 @@ __global__ void __launch_bounds__(kHashThreads) k_hash_local(HashArgs a, const _
 // its last one of h_e u^(U e), so units are hashed and summed alike and only
 // every g-th sum is written.
 //
-// One warp per tile of tb blocks (tb g <= 256 units, tb a power of two), no
+// One warp per tile of tb blocks (tb g <= 32 PER units, tb a power of two), no
 // CTA barrier anywhere:
 //   units   32 at a time, one per lane: its 16-byte loads (a unit that does
 //           not start on a 16-byte boundary takes its last words from the next
 //           lane), the limb products, one multiplication by u^(U e); the
 //           result to shared memory
-//   sums    eight consecutive units per lane: a serial sum that starts anew
-//           where a request starts, one segmented scan over the lanes for the
-//           256 units, and the canonical residues back to shared memory
+//   sums    PER consecutive units per lane (8, 9 or 11: launch_units): a serial
+//           sum that starts anew where a request starts, one segmented scan over
+//           the lanes, and the canonical residues back to shared memory
 //   store   the block ends, coalesced
 // What bounds it: L1's data path (73% busy), the pipe that multiplies (67%),
 // issue (58%) and DRAM (75% of a copy's rate) together.  The form before this
@@ -545,11 +545,14 @@ __global__ void __launch_bounds__(kHashThreads) k_hash_local(HashArgs a, const _
 // chat trace, where both paths' code competes for the instruction cache), and the
 // sums without the starts' tests where a tile has none (1.4% less there, 1.8% more
 // on the chat trace).
-constexpr uint32_t kUnitTile = 256;                            // units per tile at most
 constexpr uint32_t kUnitWarps = 2;  // per CTA: small, so that few tiles still spread over the SMs
 constexpr uint32_t kUnitThreads = 32 * kUnitWarps;
-constexpr uint32_t kUnitSlots = kUnitTile + kUnitTile / 8;     // one slot of padding per lane's eight
-__device__ __forceinline__ uint32_t unit_slot(uint32_t v) { return v + (v >> 3); }
+// PER units per lane in the sums, 32 PER per tile at most.  A slot of padding per
+// lane's units where PER is even, so that the lanes' slots lie an odd number apart.
+template <int PER>
+__host__ __device__ constexpr uint32_t unit_slot(uint32_t v) {
+  return PER % 2 ? v : v + v / PER;
+}
 
 // x mod p for any 64-bit x.
 __device__ __forceinline__ uint64_t p61_canon(uint64_t x) {
@@ -580,20 +583,22 @@ __device__ __forceinline__ int64_t shfl_i64(int64_t v, uint32_t src) {
 
 // The sums of a tile: slot[v] (units' values below 2^61 + 8) becomes the
 // canonical sum of the values since the last request start.  `mine` are the
-// starts among this lane's eight units, `opens` the lanes that have one.  (Slots
+// starts among this lane's PER units, `opens` the lanes that have one.  (Slots
 // past the tile's last unit hold anything: sums only reach later units.)
+template <int PER>
 __device__ __forceinline__ void unit_sums(ulonglong2* slot, uint32_t lane, uint32_t mine, uint32_t opens) {
-  uint64_t p0[8], p1[8];
+  uint64_t p0[PER], p1[PER];
   uint64_t s0 = 0, s1 = 0;
+  slot += unit_slot<PER>(PER * lane);
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
-    const ulonglong2 t = slot[9 * lane + j];
+  for (int j = 0; j < PER; ++j) {
+    const ulonglong2 t = slot[j];
     if ((mine >> j) & 1u) s0 = s1 = 0;
     s0 += t.x;
     s1 += t.y;
     p0[j] = s0;  // below 5 2^61 + 64
     p1[j] = s1;
-    if (j == 3) {
+    if (j % 4 == 3 && j + 1 < PER) {
       s0 = p61_part(s0);
       s1 = p61_part(s1);
     }
@@ -620,17 +625,17 @@ __device__ __forceinline__ void unit_sums(ulonglong2* slot, uint32_t lane, uint3
   c0 = lane ? p61_part(c0) : 0;
   c1 = lane ? p61_part(c1) : 0;
 #pragma unroll
-  for (int j = 0; j < 8; ++j) {
+  for (int j = 0; j < PER; ++j) {
     if ((mine >> j) & 1u) c0 = c1 = 0;  // the carry ends at the lane's first start
-    slot[9 * lane + j] = make_ulonglong2(p61_canon(p0[j] + c0), p61_canon(p1[j] + c1));
+    slot[j] = make_ulonglong2(p61_canon(p0[j] + c0), p61_canon(p1[j] + c1));
   }
 }
 
 // One tile, by one warp.  WIDE = false: two-limb products, exact while every
 // token is below 2^27 (any vocabulary in use); a tile that holds a larger one
-// writes nothing and is left to k_hash_units_wide.  WIDE = true: three-limb
+// writes nothing and is left to hash_units_wide.  WIDE = true: three-limb
 // products, exact for every 32-bit token.
-template <int U, bool WIDE>
+template <int U, int PER, bool WIDE>
 __device__ __forceinline__ bool hash_units_tile(const HashArgs& a, const HashConsts& c, uint32_t tile, uint64_t N,
                                                 ulonglong2* slot, uint32_t* starts) {
   constexpr int NV = U / 4;
@@ -660,7 +665,7 @@ __device__ __forceinline__ bool hash_units_tile(const HashArgs& a, const HashCon
   window();
   const bool one = r_first == r_last;
   bool big = false;
-  ulonglong2* out = slot + unit_slot(lane);
+  ulonglong2* out = slot + unit_slot<PER>(lane);
 #pragma unroll 1
   for (uint32_t v0 = 0; v0 < nu; v0 += 32) {
     const uint32_t v = v0 + lane;
@@ -760,22 +765,26 @@ __device__ __forceinline__ bool hash_units_tile(const HashArgs& a, const HashCon
       default: unit_hash<U, 3, WIDE>(wd, c, h0, h1); break;
     }
     *out = make_ulonglong2(p61_mul_lazy(h0, w0), p61_mul_lazy(h1, w1));
-    out += 36;  // unit_slot(v + 32)
+    static_assert(PER % 2 || 32 % PER == 0, "32 units further, the padding has grown by whole lanes");
+    out += PER % 2 ? 32 : 32 + 32 / PER;  // unit_slot(v + 32)
   }
   if (!WIDE && __any_sync(kFull, big)) return true;
   __syncwarp();
-  // ---- sums: this lane's units 8 lane .. 8 lane + 7 (values below 2^61 + 8)
+  // ---- sums: this lane's units PER lane .. PER lane + PER - 1 (values below 2^61 + 8)
   const uint32_t rounds = (nu + 31) / 32;
-  const uint32_t mine = (lane >> 2) < rounds ? (starts[lane >> 2] >> (8 * (lane & 3))) & 0xFFu : 0u;
+  const uint32_t at = PER * lane, sw = at >> 5;  // the lane's starts begin at bit `at`
+  uint32_t mine = sw < rounds ? starts[sw] >> (at & 31) : 0u;
+  if (32 % PER != 0 && (at & 31) + PER > 32 && sw + 1 < rounds) mine |= starts[sw + 1] << (32 - (at & 31));
+  mine &= (1u << PER) - 1u;
   const uint32_t opens = __ballot_sync(kFull, mine != 0);
-  unit_sums(slot, lane, mine, opens);
+  unit_sums<PER>(slot, lane, mine, opens);
   __syncwarp();
-  for (uint32_t i = lane; i < nb; i += 32) a.keys[b0 + i] = slot[unit_slot((i + 1) * a.g - 1)];
+  for (uint32_t i = lane; i < nb; i += 32) a.keys[b0 + i] = slot[unit_slot<PER>((i + 1) * a.g - 1)];
   // the tile's aggregate for the carry: its last unit's sum since its request's
   // start, and whether a request starts in the tile; and the blocks before the
   // tile's first request start
   if (lane == 0) {
-    const ulonglong2 t = slot[unit_slot(nu - 1)];
+    const ulonglong2 t = slot[unit_slot<PER>(nu - 1)];
     uint32_t lead = nb;
     for (int q = (int)rounds - 1; q >= 0; --q)
       if (starts[q]) lead = (32 * q + __ffs(starts[q]) - 1) / a.g;
@@ -787,46 +796,32 @@ __device__ __forceinline__ bool hash_units_tile(const HashArgs& a, const HashCon
 
 // Kept out of line, so that the three-limb code is not part of every tile's
 // path (nor its registers of it).
-template <int U>
+template <int U, int PER>
 __device__ __noinline__ void hash_units_wide(const HashArgs& a, const HashConsts& c, uint32_t tile, uint64_t N,
                                              ulonglong2* slot, uint32_t* starts) {
-  hash_units_tile<U, true>(a, c, tile, N, slot, starts);
+  hash_units_tile<U, PER, true>(a, c, tile, N, slot, starts);
 }
 
-template <int U>
-__global__ void __launch_bounds__(kUnitThreads, 18) k_hash_units(const __grid_constant__ HashArgs a,
+template <int U, int PER>
+__global__ void __launch_bounds__(kUnitThreads, PER == 11 ? 16 : 18) k_hash_units(const __grid_constant__ HashArgs a,
                                                                  const __grid_constant__ HashConsts c) {
   grid_dep_sync();
-  __shared__ ulonglong2 s_slot[kUnitWarps][kUnitSlots];
-  __shared__ uint32_t s_starts[kUnitWarps][kUnitTile / 32];
+  __shared__ ulonglong2 s_slot[kUnitWarps][unit_slot<PER>(32 * PER - 1) + 1];
+  __shared__ uint32_t s_starts[kUnitWarps][PER];
   const uint32_t w = threadIdx.x >> 5, tile = blockIdx.x * kUnitWarps + w;
   const uint64_t N = blocks_live(a.st, a.keys_cap);
-  if (hash_units_tile<U, false>(a, c, tile, N, s_slot[w], s_starts[w])) {
+  if (hash_units_tile<U, PER, false>(a, c, tile, N, s_slot[w], s_starts[w])) {
     __syncwarp();
-    hash_units_wide<U>(a, c, tile, N, s_slot[w], s_starts[w]);
+    hash_units_wide<U, PER>(a, c, tile, N, s_slot[w], s_starts[w]);
   }
 }
 
-// Carry of every tile = the segmented sum of the aggregates of the tiles
-// before it, back to (and including) the nearest one where a request starts.
-// All aggregates exist before this kernel starts, so nothing waits.  One warp
-// per tile: each round reads 32 predecessors; then the carry is added to the
-// tile's leading blocks (the tail of a request that started earlier).
-constexpr int kChainWarps = 8;
-__global__ void __launch_bounds__(kChainWarps * 32) k_hash_chain(ulonglong2* __restrict__ keys,
-                                                                 const HashCarry* __restrict__ tile_agg,
-                                                                 const uint32_t* __restrict__ tile_lead, uint32_t TB,
-                                                                 const DevStatus* st, uint64_t keys_cap) {
-  grid_dep_sync();
-  const uint32_t lane = threadIdx.x & 31;
-  const uint32_t tile = blockIdx.x * kChainWarps + (threadIdx.x >> 5);
-  const uint64_t N = blocks_live(st, keys_cap);
-  const uint64_t b0 = (uint64_t)tile * TB;
-  if (b0 >= N || tile == 0) return;
-  const uint32_t lead = tile_lead[tile];
-  if (lead == 0 || !in_bounds(st, b0 + lead - 1, keys_cap)) return;
-  uint64_t c0 = 0, c1 = 0;
-  for (int64_t base = (int64_t)tile - 1; base >= 0; base -= 32) {
+// The segmented sum of the aggregates of the tiles before t0, back to (and
+// including) the nearest one where a request starts, by one warp, 32 tiles a
+// round.  All aggregates exist before the kernel starts, so nothing waits.
+__device__ __forceinline__ HashCarry carry_into(const HashCarry* __restrict__ tile_agg, uint32_t t0, uint32_t lane) {
+  HashCarry c{0, 0, 0};
+  for (int64_t base = (int64_t)t0 - 1; base >= 0; base -= 32) {
     const int64_t idx = base - (int64_t)lane;
     HashCarry g{0, 0, 0};
     if (idx >= 0) g = tile_agg[idx];
@@ -838,13 +833,77 @@ __global__ void __launch_bounds__(kChainWarps * 32) k_hash_chain(ulonglong2* __r
       v0 = p61_add(v0, __shfl_xor_sync(kFull, v0, o));
       v1 = p61_add(v1, __shfl_xor_sync(kFull, v1, o));
     }
-    c0 = p61_add(c0, v0);
-    c1 = p61_add(c1, v1);
+    c.v0 = p61_add(c.v0, v0);
+    c.v1 = p61_add(c.v1, v1);
     if (heads) break;
   }
-  for (uint32_t i = lane; i < lead; i += 32) {
-    const ulonglong2 k = keys[b0 + i];
-    keys[b0 + i] = make_ulonglong2(p61_add(k.x, c0), p61_add(k.y, c1));
+  return c;
+}
+// The carry of every tile of a warp's PER (lane q: tile t0 + q) from the one into
+// the first: a segmented scan of their aggregates over the lanes.
+template <int PER>
+__device__ __forceinline__ HashCarry lane_carries(const HashCarry* __restrict__ tile_agg, uint32_t t0, uint64_t live,
+                                                  const HashCarry& cin, uint32_t lane) {
+  const SegSumOp op;
+  const uint32_t t = t0 + lane;
+  HashCarry g{0, 0, 0};
+  if (lane < PER && t < live) g = tile_agg[t];
+#pragma unroll
+  for (int o = 1; o < PER; o <<= 1) {  // inclusive segmented sums over lanes 0 .. PER - 1
+    HashCarry y;
+    y.v0 = __shfl_up_sync(kFull, g.v0, o);
+    y.v1 = __shfl_up_sync(kFull, g.v1, o);
+    y.f = __shfl_up_sync(kFull, g.f, o);
+    if (lane >= (uint32_t)o) g = op(y, g);
+  }
+  HashCarry before;  // this warp's tiles before tile t
+  before.v0 = __shfl_up_sync(kFull, g.v0, 1);
+  before.v1 = __shfl_up_sync(kFull, g.v1, 1);
+  before.f = __shfl_up_sync(kFull, g.f, 1);
+  if (lane == 0) before = HashCarry{0, 0, 0};
+  return op(cin, before);
+}
+
+// The carry of every tile (carry_into) added to its leading blocks, the tail of a
+// request that started earlier.  A warp takes PER consecutive tiles, 256 blocks or
+// fewer: PER = 8 where a tile holds at most 32.  (With a warp per tile 1.5M blocks
+// of 272 tokens, eight to a tile, took 56 us, so, sixteen to a tile, 14.)
+constexpr int kChainWarps = 8;
+template <int PER>
+__global__ void __launch_bounds__(kChainWarps * 32) k_hash_chain(ulonglong2* __restrict__ keys,
+                                                                 const HashCarry* __restrict__ tile_agg,
+                                                                 const uint32_t* __restrict__ tile_lead, uint32_t TB,
+                                                                 const DevStatus* st, uint64_t keys_cap) {
+  grid_dep_sync();
+  const uint32_t lane = threadIdx.x & 31;
+  const uint32_t t0 = (blockIdx.x * kChainWarps + (threadIdx.x >> 5)) * PER;
+  const uint64_t N = blocks_live(st, keys_cap);
+  const uint64_t b0 = (uint64_t)t0 * TB, live = (N + TB - 1) / TB;
+  if (t0 >= live) return;
+  const uint32_t t = t0 + lane;
+  const uint32_t lead = lane < PER && t > 0 && t < live ? tile_lead[t] : 0u;
+  if (!__any_sync(kFull, lead != 0)) return;
+  HashCarry c{0, 0, 0};
+  if (__shfl_sync(kFull, lead, 0)) c = carry_into(tile_agg, t0, lane);
+  if (PER == 1) {
+    const uint32_t n = __shfl_sync(kFull, lead, 0);
+    for (uint32_t i = lane; i < n; i += 32) {
+      if (!in_bounds(st, b0 + i, keys_cap)) return;
+      const ulonglong2 k = keys[b0 + i];
+      keys[b0 + i] = make_ulonglong2(p61_add(k.x, c.v0), p61_add(k.y, c.v1));
+    }
+    return;
+  }
+  c = lane_carries<PER>(tile_agg, t0, live, c, lane);
+  const uint32_t shift = 31 - __clz(TB);
+  for (uint32_t j = lane; j < PER * TB; j += 32) {  // whole warps: TB is 4 or more
+    const uint32_t q = j >> shift;
+    const uint32_t n = __shfl_sync(kFull, lead, q);
+    const uint64_t c0 = __shfl_sync(kFull, c.v0, q), c1 = __shfl_sync(kFull, c.v1, q);
+    if ((j & (TB - 1)) < n && in_bounds(st, b0 + j, keys_cap)) {
+      const ulonglong2 k = keys[b0 + j];
+      keys[b0 + j] = make_ulonglong2(p61_add(k.x, c0), p61_add(k.y, c1));
+    }
   }
 }
 
@@ -866,43 +925,10 @@ __global__ void __launch_bounds__(kChainWarps * 32) k_hash_carry(const HashCarry
   if (t0 >= ntiles) return;
   const uint64_t N = blocks_live(st, keys_cap);
   const uint64_t live = (N + TB - 1) / TB;  // tiles that hold blocks
-  const SegSumOp op;
-  HashCarry cin{0, 0, 0};
-  if (t0 > 0 && t0 < live) {
-    for (int64_t base = (int64_t)t0 - 1; base >= 0; base -= 32) {
-      const int64_t idx = base - (int64_t)lane;
-      HashCarry g{0, 0, 0};
-      if (idx >= 0) g = tile_agg[idx];
-      const uint32_t heads = __ballot_sync(kFull, idx >= 0 && g.f);
-      const uint32_t first = heads ? (uint32_t)(__ffs(heads) - 1) : 31u;
-      uint64_t v0 = lane <= first ? g.v0 : 0, v1 = lane <= first ? g.v1 : 0;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) {
-        v0 = p61_add(v0, __shfl_xor_sync(kFull, v0, o));
-        v1 = p61_add(v1, __shfl_xor_sync(kFull, v1, o));
-      }
-      cin.v0 = p61_add(cin.v0, v0);
-      cin.v1 = p61_add(cin.v1, v1);
-      if (heads) break;
-    }
-  }
+  HashCarry c{0, 0, 0};
+  if (t0 < live) c = carry_into(tile_agg, t0, lane);
+  c = lane_carries<kCarryPer>(tile_agg, t0, live, c, lane);
   const uint32_t t = t0 + lane;
-  HashCarry g{0, 0, 0};
-  if (lane < kCarryPer && t < live) g = tile_agg[t];
-#pragma unroll
-  for (int o = 1; o < kCarryPer; o <<= 1) {  // inclusive segmented sums over lanes 0 .. kCarryPer - 1
-    HashCarry y;
-    y.v0 = __shfl_up_sync(kFull, g.v0, o);
-    y.v1 = __shfl_up_sync(kFull, g.v1, o);
-    y.f = __shfl_up_sync(kFull, g.f, o);
-    if (lane >= (uint32_t)o) g = op(y, g);
-  }
-  HashCarry before;  // this warp's tiles before tile t
-  before.v0 = __shfl_up_sync(kFull, g.v0, 1);
-  before.v1 = __shfl_up_sync(kFull, g.v1, 1);
-  before.f = __shfl_up_sync(kFull, g.f, 1);
-  if (lane == 0) before = HashCarry{0, 0, 0};
-  const HashCarry c = op(cin, before);
   if (lane < kCarryPer && t < ntiles) {
     const uint64_t b0 = (uint64_t)t * TB;
     const uint32_t lead = (b0 >= N || t == 0) ? 0u : tile_lead[t];
@@ -911,9 +937,24 @@ __global__ void __launch_bounds__(kChainWarps * 32) k_hash_carry(const HashCarry
   }
 }
 
+// Units per lane: 8, but 9 or 11 where a power of two of blocks is more than 256
+// units and up to 288 or 352 (half of them would fill 256 badly: a tile's sums and
+// its last, partial round cost as much for few units).  400M tokens: B = 144 456
+// us in tiles of 144 units, 380 in 288; B = 272 479 and 397; B = 80 422 in 160 and
+// 393 in 320; B = 336 446 in 168 and 397 in 336.  11 per lane take 16 CTAs per SM
+// (with 18, whose registers spill, B = 336 took 418); 9 take 18 (B = 272: 402 with
+// 16).
+constexpr uint32_t kUnitPer = 8, kUnitPerMost = 11;
+
 template <int U>
 void launch_units(uint32_t tiles, cudaStream_t s, const HashArgs& a, const HashConsts& c) {
-  PTC_KERNEL("k_hash_units", s, k_hash_units<U>, ceil_div_u32(tiles, kUnitWarps), kUnitThreads, 0, a, c);
+  const uint32_t grid = ceil_div_u32(tiles, kUnitWarps), units = a.tb * a.g;
+  if (units <= 32 * kUnitPer)
+    PTC_KERNEL("k_hash_units", s, (k_hash_units<U, kUnitPer>), grid, kUnitThreads, 0, a, c);
+  else if (units <= 32 * 9)
+    PTC_KERNEL("k_hash_units", s, (k_hash_units<U, 9>), grid, kUnitThreads, 0, a, c);
+  else
+    PTC_KERNEL("k_hash_units", s, (k_hash_units<U, kUnitPerMost>), grid, kUnitThreads, 0, a, c);
 }
 
 template <int G>
@@ -941,23 +982,25 @@ uint32_t chunks_per_block(uint32_t B) {  // G: power of two >= ceil(B / 16)
   return g;
 }
 
-// Blocks per hash tile for n_tok tokens, a power of two: as many as make up
-// to 256 units for k_hash_units, one CTA's kHashThreads / G for k_hash_local.
-// With few blocks a tile of units is cut down to 64 while that makes more warps
-// than half of those that fit the GPU: a warp takes its rounds of 32 units one
-// after another, and a window of 127K blocks took 20 us in tiles of 256, 13 in
-// tiles of 64.
+// Blocks per hash tile for n_tok tokens, a power of two: 256 or fewer that make up
+// to 352 units (launch_units) for k_hash_units, one CTA's kHashThreads / G for
+// k_hash_local.  With few blocks a tile of units is cut down to 64 while there are
+// fewer tiles than kUnitFewTiles, 16 warps on each of the GPU's 152 SMs (36 fit):
+// a warp takes its rounds of 32 units one after another, and a window of 127K
+// blocks took 20 us in tiles of 256, 13 in tiles of 64.  (A constant, as the size
+// of the workspace follows from it, which callers may ask for without a GPU.)
+constexpr uint32_t kUnitFewTiles = 16 * 152;
 uint32_t tile_blocks(uint32_t B, uint64_t n_tok) {
   // a block is at most 512 / 8 units, or 32 chunks
-  static_assert(PTC_MAX_BLOCK_SIZE / 8 * kCarryTileMin <= kUnitTile && 32 * kCarryTileMin <= kHashThreads,
+  static_assert(PTC_MAX_BLOCK_SIZE / 8 * kCarryTileMin <= 32 * kUnitPer && 32 * kCarryTileMin <= kHashThreads,
                 "tiles without the cut below hold kCarryTileMin blocks or more");
   const uint32_t U = unit_tokens(B, n_tok);
   const uint64_t nb = n_tok / B;
   if (!U) return kHashThreads / chunks_per_block(B);
   const uint32_t g = B / U;
-  uint32_t tb = kUnitTile;
-  while (tb * g > kUnitTile) tb >>= 1;
-  while (tb > 1 && tb * g > 64 && nb / tb < 16 * 152) tb >>= 1;
+  uint32_t tb = 32 * kUnitPer;
+  while (tb * g > 32 * kUnitPerMost) tb >>= 1;
+  while (tb > 1 && tb * g > 64 && nb / tb < kUnitFewTiles) tb >>= 1;
   return tb;
 }
 
@@ -1112,8 +1155,12 @@ ptc_status ptc::hash_impl(const uint32_t* tokens, uint64_t n_tok, const uint64_t
       PTC_KERNEL("k_hash_carry", s, k_hash_carry, ceil_div_u32(grid, kChainWarps * kCarryPer), kChainWarps * 32, 0, L.tile_agg,
                  L.tile_lead, tb, L.st, keys_cap, grid, carry->carry, carry->lead);
     } else {
-      PTC_KERNEL("k_hash_chain", s, k_hash_chain, ceil_div_u32(grid, kChainWarps), kChainWarps * 32, 0, a.keys,
-                 L.tile_agg, L.tile_lead, tb, L.st, keys_cap);
+      if (tb <= 32 && tb >= kCarryTileMin)
+        PTC_KERNEL("k_hash_chain", s, k_hash_chain<8>, ceil_div_u32(grid, kChainWarps * 8), kChainWarps * 32, 0, a.keys,
+                   L.tile_agg, L.tile_lead, tb, L.st, keys_cap);
+      else
+        PTC_KERNEL("k_hash_chain", s, k_hash_chain<1>, ceil_div_u32(grid, kChainWarps), kChainWarps * 32, 0, a.keys,
+                   L.tile_agg, L.tile_lead, tb, L.st, keys_cap);
     }
   }
   if (lent) return cudaGetLastError() == cudaSuccess ? PTC_OK : PTC_ERR_CUDA;

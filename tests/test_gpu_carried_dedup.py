@@ -26,10 +26,10 @@ def test_every_block_size_has_tiles_the_dedup_makes_room_for():
     src = open(os.path.join(ROOT, "paper_2609_28870_gb300", "csrc", "ptc_internal.h")).read()
     room = re.search(r"constexpr uint32_t kCarryTileMin = (\d+);", src)
     assert room and min(tiles.values()) >= int(room.group(1))
-    assert (tiles[280], tiles[504], tiles[136], tiles[104], tiles[16]) == (4, 4, 8, 16, 256)
+    assert (tiles[488], tiles[504], tiles[136], tiles[16]) == (4, 8, 16, 256)
 
 
-@pytest.mark.parametrize("B,U", [(40, 8), (104, 8), (280, 8)])
+@pytest.mark.parametrize("B,U", [(56, 8), (104, 8), (488, 8)])
 def test_units_only_while_their_exponents_fit(B, U):
     """A request of 2^32 units or more is hashed by blocks, in tiles of 256 chunks
     of 16 tokens (the routes differ in the blocks of a tile)."""
@@ -37,7 +37,7 @@ def test_units_only_while_their_exponents_fit(B, U):
     from paper_2609_28870_gb300 import build
     build.build()
     chunks = 1 << int(np.ceil(np.log2((B + 15) // 16)))
-    units = 1 << int(np.floor(np.log2(256 * U // B)))
+    units = 1 << int(np.floor(np.log2(352 * U // B)))
     assert units != 256 // chunks
     assert _tile_blocks(ptc.lib(), B, 2**31 * U // B) == units           # 2^31 and (nearly) 2^32 units
     assert _tile_blocks(ptc.lib(), B, 2**32 * U // B + 1) == 256 // chunks
@@ -45,7 +45,7 @@ def test_units_only_while_their_exponents_fit(B, U):
 
 @pytest.mark.gpu
 @pytest.mark.parametrize("sessions", [False, True])
-@pytest.mark.parametrize("B", [280, 504, 136, 104])
+@pytest.mark.parametrize("B", [488, 504, 136, 104])
 def test_carried_keys(B, sessions):
     """The grids follow the token buffer's length, the work its requests': a
     few long requests at the front of a buffer that the id table of L2's size

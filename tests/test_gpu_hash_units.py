@@ -35,7 +35,7 @@ def _trace(rng, lens, vocab):
     return rng.integers(0, vocab, int(off[-1])).astype(np.uint32), off
 
 
-@pytest.mark.parametrize("B", [8, 12, 16, 24, 32, 36, 40, 48, 64, 176, 264, 496, 512])
+@pytest.mark.parametrize("B", [8, 12, 16, 24, 32, 36, 40, 48, 64, 80, 108, 144, 176, 264, 272, 280, 352, 496, 512])
 @pytest.mark.parametrize("lead", [0, 1, 2, 3])
 def test_block_sizes_and_alignments(ptc, B, lead):
     rng = np.random.default_rng(100 * B + lead)
