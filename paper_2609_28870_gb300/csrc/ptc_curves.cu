@@ -604,10 +604,9 @@ __global__ void __launch_bounds__(256) k_curves_runs(CurveArgs a, RunsArgs ra, F
   }
   __shared__ Bins s_bins;
   const uint32_t G = a.G;
-  // an earlier stage failed: its runs are void (what the distances' CTAs read of
-  // them is in range all the same, whatever it says)
-  uint32_t failed = 0;
-  for (uint32_t q = 0; q < f.n_earlier; ++q) failed |= f.earlier[q].err;
+  // stage c failed: its runs are void (what the distances' CTAs read of them is in
+  // range all the same, whatever it says)
+  const uint32_t failed = f.n_earlier ? f.earlier[f.n_earlier - 1].err : 0u;
   s_bins.init(a.caps, G);
   __syncthreads();
   // Four lanes per request, a run per lane and round: a request has a handful
