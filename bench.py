@@ -172,7 +172,6 @@ def kernel_model_bytes(name, T, N, L, D, U=None):
     return {
         "k_hash_local": 4 * T + 16 * N,   # token stream in, block keys out
         "k_hash_units": 4 * T + 16 * N,   # the same, B a multiple of 16, 12 or 8
-        "k_hash16": 4 * T + 16 * N,       # the same, B = 16 path of an earlier build
         "k_ids_insert": 16 * N,           # keys in
         "k_ids_insert_prior": 16 * N,     # keys in (the same stage, prior-request hint)
         "k_ids_gather": 4 * N,            # ids out

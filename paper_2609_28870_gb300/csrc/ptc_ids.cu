@@ -1564,11 +1564,12 @@ __global__ void __launch_bounds__(kGaThreads) k_ids_gather_pd(const uint32_t* __
 // blocks (an agentic trace, D near n / 2) fills it to at most about 3/4.  At
 // n / 3 slots, up to 2^22, such a trace outran its table: 11.3M keys of an
 // agentic window took 26.7 ms there and 0.39 ms in 2^23 slots, 9.3M keys of a
-// chat trace (D = 0.17 n) 174 against 166 us plus 11 us more of fill.  Forced
+// chat trace (D = 0.17 n) 174 against 166 us plus 11 us more of fill (the whole
+// call on 12M keys, a twentieth of them distinct: 275 and 291 us).  Forced
 // beyond that size the table lives in DRAM and takes 3n / 4 slots.  If
 // a probe sequence of the first attempt runs past kSmallProbeCap slots, the
 // call redoes the stage with the full table.  A table no more than 3/4 full
-// has no runs of that length; a fuller one is slower than the redo: with
+// has hardly any runs of that length; a fuller one is slower than the redo: with
 // runs of up to 4,096 slots allowed, and walked by every thread after the
 // first had failed, 12M keys half of them distinct took 24 ms.
 constexpr uint64_t kSmallProbeCap = 256;
@@ -1630,9 +1631,7 @@ IdsLayout ids_layout(void* ws, uint64_t n, uint32_t n_req_hint, bool pd) {
   L.pd_tot1 = pd ? cv.take<uint32_t>(kPdBuckets) : nullptr;
   L.pd_rel2 = pd ? cv.take<uint32_t>((size_t)L.pd_max_tiles * 256) : nullptr;
   L.pd_base2 = pd ? cv.take<uint32_t>(kPdParts + 1) : nullptr;
-  // the table last: it starts past every other array of the stage (and past
-  // stage a1's workspace, which the pipeline checks before it has stage a1
-  // fill the table); the partitioned dedup keeps its records there
+  // the table last; the partitioned dedup keeps its records there
   L.table = cv.take<ulonglong2>(pd && 2 * nn > m ? 2 * nn : m);
   L.pd_rec1 = pd ? L.table : nullptr;
   L.pd_rec2 = pd && L.table ? L.table + nn : nullptr;

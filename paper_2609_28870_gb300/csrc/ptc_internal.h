@@ -183,7 +183,7 @@ inline bool ws_ok(const void* ws, size_t ws_bytes, size_t need) {
   return ws != nullptr && ((uintptr_t)ws & 255) == 0 && ws_bytes >= need;
 }
 
-// The runs stage c leaves in its workspace when it used the matrix over runs
+// The runs stage c leaves in its workspace when it counted over runs
 // (ptc_runs.cu); the pipeline hands them to stage d.
 struct RunsView {
   bool used = false;

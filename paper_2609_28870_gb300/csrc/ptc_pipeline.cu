@@ -2,8 +2,8 @@
 // needs one crossing of the C boundary.  Intermediate arrays live in caller
 // buffers when given, otherwise in the workspace; the stages' own scratch
 // reuses one region of the workspace because they run one after another on
-// the same stream.  Stage d has a region of its own: when stage c used the
-// matrix over runs, the curves come from those runs (still in stage c's
+// the same stream.  Stage d has a region of its own: when stage c counted
+// over runs, the curves come from those runs (still in stage c's
 // scratch) instead of a pass over every distance.
 #include <algorithm>
 

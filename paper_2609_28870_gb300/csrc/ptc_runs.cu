@@ -614,11 +614,19 @@ __global__ void __launch_bounds__(kRT) k_runs_level(LevelArgs a) {
 // is a prefix over the matrix of the lengths per (time block, rank block).
 // Three launches whatever R, against log2(R) levels of barriers and as many
 // dependent reads per query of a wavelet matrix over the runs: 39,800 runs of the
-// chat trace took 75 us there (one thread-block cluster, then the queries) and 30
+// chat trace took 75 us there (its levels in one cluster's shared memory) and 30
 // here, 0.7M runs of the mixed trace 450 us and 143.
 constexpr uint32_t kDomB = 512;
-constexpr uint64_t kDomMax = 1ULL << 21;  // runs; the lengths' matrix then takes 67 MB
-constexpr uint64_t kPiecesBound = 1ULL << 19;  // the lengths' matrix takes 4 MB: it costs less than the wait
+// Up to kDomMax runs, where the lengths' matrix takes 67 MB (it grows with the
+// square).  ptc_stack_distance on runs of eight accesses, by the levels' matrix and
+// by blocks: 0.27 and 0.13 ms with 0.3M runs, 0.52 and 0.28 with 1M, 0.89 and 0.69
+// with 2M; 1.34 and 1.26 with 3M, 1.75 and 2.02 with 4M.
+constexpr uint64_t kDomMax = 1ULL << 21;
+// Up to this many pieces the pipeline takes them as the bound on the runs instead
+// of waiting for the runs' number: 217 us with the wait and 204 without at 30,000
+// pieces of eight accesses, 492 and 484 at 300,000, 676 and 677 at 500,000 (the
+// lengths' matrix then takes 4 MB), 982 and 1,020 at 800,000.
+constexpr uint64_t kPiecesBound = 1ULL << 19;
 
 struct DomArgs {
   const uint32_t* rec_s;

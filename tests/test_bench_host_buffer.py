@@ -57,5 +57,5 @@ def test_partitioned_dedup_model_bytes():
     for name, b in want.items():
         assert bench.kernel_model_bytes(name, T, N, L, D, U) == b
         assert bench.kernel_model_bytes(name, T, N, L, D) == 0.0
-    assert bench.kernel_model_bytes("k_hash16", T, N, L, D, U) == 4 * T + 16 * N
+    assert bench.kernel_model_bytes("k_hash_units", T, N, L, D, U) == 4 * T + 16 * N
     assert set(want) <= set(bench.PD_KERNELS)

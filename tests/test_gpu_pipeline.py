@@ -206,7 +206,7 @@ def test_pipeline_plan_runs_again_and_on_refilled_buffers():
 
 def test_pipeline_redoes_stage_a2_when_the_small_table_overflows():
     """ptc_pipeline does not wait for stage a2: its first attempt uses the
-    small table (N/3 slots); when every block is distinct that table
+    small table (0.6 N slots); when every block is distinct that table
     overflows, stage b's wait reports it, and the pipeline redoes a2 with the
     full table and b with the host's N and D."""
     from tests import gpu_util as gu

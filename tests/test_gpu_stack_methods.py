@@ -1,6 +1,6 @@
-"""Both wavelet matrices of the stack-distance stage (over every access and
-over runs) against the oracle's distances, bit-exact, on traces with short
-and with long runs."""
+"""The methods of the stack-distance stage (the wavelet matrix over every
+access, the count over runs, the automatic choice) against the oracle's
+distances, bit-exact, on traces with short and with long runs."""
 import numpy as np
 import pytest
 
@@ -89,7 +89,7 @@ def test_forced_runs_with_a_small_workspace_is_refused():
     p = ptc.to_device_u32(prev)
     L = ptc.lib()
     ws = torch.empty(L.ptc_stack_distance_workspace_bytes(prev.size), dtype=torch.uint8, device="cuda")
-    # the automatic choice falls back to the matrix over accesses
+    # the automatic choice counts over the accesses instead
     assert np.array_equal(ptc.u32(ptc.ptc_stack_distance(p, ws=ws)), want)
     dist = torch.empty(prev.size, dtype=torch.int32, device="cuda")
     stream = torch.cuda.current_stream().cuda_stream
