@@ -57,8 +57,8 @@ NOMINAL_HBM_GBS = 7900.0
 # sha256 prefix of the source file it was taken on (a changed source reads as
 # "no counters", null) and how the capture was scaled to a full launch.
 NCU_TRAFFIC: dict[tuple[str, int], tuple[float, str, str]] = {
-    ("k_hash_units", 1): (6.3734e+08, "31df697892c6f7e0", "ncu dram__bytes metrics, first 6,000 requests, x 153.81 / 55.67"),
-    ("k_hash_units", 3): (5.0640e+10, "31df697892c6f7e0", "ncu dram__bytes metrics, first 60,000 requests: reads x tokens "
+    ("k_hash_units", 1): (6.3658e+08, "c27d7bbe711b9b01", "ncu dram__bytes metrics, first 6,000 requests, x 153.81 / 55.67"),
+    ("k_hash_units", 3): (5.0646e+10, "c27d7bbe711b9b01", "ncu dram__bytes metrics, first 60,000 requests: reads x tokens "
                           "(9984.4M / 943.9M), key writes x blocks (623.75M / 58.97M)"),
 }
 
