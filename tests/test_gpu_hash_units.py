@@ -80,3 +80,25 @@ def test_pipeline_carries(ptc, B):
     o = oracle.run(tr.tokens, tr.req_tok_off, B, np.asarray([10, 1000, 10**6], dtype=np.uint64))
     got = ptc.ptc_pipeline(tok, off, None, B, [10, 1000, 10**6])
     assert got["n_access"] == o["n_access"] and got["n_distinct"] == o["n_distinct"] and got["hits"] == o["hits"]
+
+
+@pytest.mark.parametrize("lead", [0, 3])
+@pytest.mark.parametrize("wide", [False, True])
+@pytest.mark.parametrize("B", [40, 60, 80, 88, 108, 136, 144, 204, 272, 336])
+def test_tiles_of_more_units(ptc, B, wide, lead):
+    """9 or 11 units per lane, which token counts with many tiles take: a buffer
+    of that length whose requests lie in its front."""
+    import torch
+    rng = np.random.default_rng(10 * B + lead)
+    lens = np.concatenate([[0, B - 1, B, 33 * B + 5, 700 * B + 3], np.where(rng.random(900) < 0.7, rng.integers(0, B, 900),
+                          rng.integers(B, 6 * B, 900)), rng.integers(0, 90 * B, 40), [0, 2 * B + 1]])
+    tokens, off = _trace(rng, lens, 151_936)
+    if wide:
+        at = rng.integers(0, len(tokens), 9)
+        tokens[at] = rng.integers(2**27, 2**32, 9).astype(np.uint32)
+        tokens[0] = tokens[-1] = 0xFFFFFFFF
+    n_tok = 16 * 152 * 64 * B + 7
+    buf = torch.zeros(lead + n_tok, dtype=torch.int32, device="cuda")
+    buf[lead: lead + len(tokens)] = ptc.to_device_u32(tokens)
+    keys, _, n = ptc.ptc_hash_blocks(buf[lead:], ptc.to_device_u64(off), None, B, 3)
+    assert np.array_equal(ptc.u64(keys).reshape(-1, 2)[:n], oracle.prefix_hash(tokens, off, B, 3))
